@@ -295,15 +295,15 @@ def run_reference(args, w, world, rank):
 def launches_per_step(tfmm, plan, R, dev):
     """Kernels one aggregate + disaggregate pair launches: one persistent kernel per stage
     for one RHS (three per stage on the split path, taken by plans with fewer work items
-    than twice the SMs), the tensor-core chain for many (operand prep and four kernels
-    for aggregation, four for disaggregation)."""
+    than twice the SMs), the tensor-core chain for many (operand prep and three kernels
+    for aggregation; four and the reordering of y for disaggregation)."""
     import torch
     t = tfmm.tfmm_plan_tuning_get(plan)
     if R == 1:
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
         split = t["single_rhs_split"] == 1 or (t["single_rhs_split"] == 0 and 2 * plan.info["n_groups"] < 2 * sms)
         return 6 if split else 2
-    return 8
+    return 9
 
 
 def traffic_record(kernel, factor_bytes):

@@ -178,6 +178,10 @@ struct TcPlan {             // per (R, terms): problem lists of the 8 steps and 
     size_t dg1a_smem = 0;
     DeviceBuffer dg1a_items, dg1a_tiles;
     CatPlan cat1a, cat1b;   // the stacked-term forms of DG1a / DG1b, when they fit
+    DeviceBuffer x_tiles;   // prep_x work list
+    int n_xtiles = 0;
+    DeviceBuffer ybuf;      // DG3 output in group order (R x N complex)
+    DeviceBuffer y_pos;     // position of every RWG in group order
     // per item: element offsets of its M' and V'' / P'' scratch planes (for re-planning)
     std::vector<int64_t> m_off, v_off;
     ~TcPlan();

@@ -71,10 +71,8 @@ struct TcCtx {
     const float2* spec_in;  // DG1a input (spectra; null: A from prepared planes)
     const float* w;         // DG1a quadrature weights (null: none)
     float2* spec;        // AG4 output (spectra)
-    float2* y;           // DG3 output
-    const int* grp_rwg;
-    int64_t ld;          // ldy (DG3)
-    float2 beta;         // DG3
+    float2* ybuf;        // DG3 output in group order, [r][position]
+    int64_t N;
     int R, G, n_theta, n_dir;
     int* err;            // set when a wait gives up
 };
@@ -282,16 +280,9 @@ __device__ __forceinline__ void epilogue(const TcCtx& c, const TcProb& p, int i,
         case TDG2:  // S stored [r][c]; i = c, j = r
             store_planes<T>(o, p.o_ps, (int64_t)j * p.o_ld + i, v);
             break;
-        case TDG3: {  // y = beta y + conj(v); i = n, j = r
-            float2* dst = c.y + (int64_t)c.grp_rwg[p.rwg + i] + c.ld * j;
-            float2 r = make_float2(v.x, -v.y);
-            if (c.beta.x != 0.f || c.beta.y != 0.f) {
-                const float2 old = *dst;
-                r.x += c.beta.x * old.x - c.beta.y * old.y;
-                r.y += c.beta.x * old.y + c.beta.y * old.x;
-            }
-            *dst = r;
-        } break;
+        case TDG3:  // conj(v) in group order; i = n, j = r
+            c.ybuf[(int64_t)j * c.N + p.rwg + i] = make_float2(v.x, -v.y);
+            break;
     }
 }
 
@@ -1384,21 +1375,85 @@ __global__ void planes_kernel(const float2* __restrict__ src, int rows, int cols
     }
 }
 
-// X_g planes [r][n] for every group: x[grp_rwg[off_g + n] + ldx r].
+// X_g planes [r][n] for every group: x[grp_rwg[off_g + n] + ldx r].  One block per tile
+// of kXTile members of a group and kXCols right-hand sides, the tiles of one column block
+// before those of the next.  The gather reads 8 bytes of each 32-byte sector, so what
+// bounds it is whether a sector is still in L2 when its other three members are read:
+// kXCols columns of 972,000 RWGs are 31 MB of the 129 MB.  With the columns of a group
+// together, the whole block of x (1 GB) was in flight and every sector came from HBM up to
+// four times.  A thread takes two neighbouring members, whose terms share a 32-bit store.
+// 972,000 RWGs in random order x 128 columns: 2.53 -> 0.72 ms (floor 0.37 ms: 1.0 GB read,
+// 1.5 GB written).
+constexpr int kXTile = 512, kXCols = 4;
 template <int T>
-__global__ void prep_x_kernel(const float2* __restrict__ x, int64_t ldx, const int* __restrict__ grp_rwg,
-                              const TcProb* __restrict__ probs, int n_probs, int R) {
-    for (int q = blockIdx.y; q < n_probs; q += gridDim.y) {
-        const TcProb& p = probs[q];  // AG1 problem of (g, alpha = 0): B0 points at the group's X planes
-        if (p.alpha != 0) continue;
-        bf16* dst = const_cast<bf16*>(p.B0);
-        const int nb = p.K0;
-        const int64_t total = (int64_t)R * nb;
-        for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-            const int r = (int)(e / nb), n = (int)(e % nb);
-            store_planes<T>(dst, p.b_ps0, (int64_t)r * p.b_ld0 + n, x[(int64_t)grp_rwg[p.rwg + n] + ldx * r]);
+__global__ void __launch_bounds__(kXTile / 2) prep_x_kernel(const float2* __restrict__ x, int64_t ldx,
+                                                            const int* __restrict__ grp_rwg,
+                                                            const TcProb* __restrict__ probs,
+                                                            const MrTile* __restrict__ tiles, int R) {
+    const MrTile t = tiles[blockIdx.x];
+    const TcProb& p = probs[t.prob];  // AG1 problem of (g, alpha = 0): B0 points at the group's X planes
+    const int nb = p.K0, n = t.n0 + 2 * (int)threadIdx.x, r0 = blockIdx.y * kXCols;
+    if (n >= nb) return;
+    const int64_t ld = p.b_ld0, ps = p.b_ps0;
+    bf16* dst = const_cast<bf16*>(p.B0);
+    const bool two = n + 1 < nb;  // the second value of an odd tail is the planes' zero padding
+    const int64_t i0 = grp_rwg[p.rwg + n], i1 = two ? grp_rwg[p.rwg + n + 1] : i0;
+    float2 v0[kXCols], v1[kXCols];
+#pragma unroll
+    for (int c = 0; c < kXCols; ++c) {
+        const int64_t col = ldx * min(r0 + c, R - 1);
+        v0[c] = x[i0 + col];
+        v1[c] = two ? x[i1 + col] : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int c = 0; c < kXCols; ++c) {
+        if (r0 + c >= R) break;
+        uint32_t wr[3], wi[3];
+        split_pack<T>(v0[c].x, v1[c].x, wr);
+        split_pack<T>(v0[c].y, v1[c].y, wi);
+        bf16* o = dst + (r0 + c) * ld + n;  // n even, ld a multiple of 8: 4-byte aligned
+#pragma unroll
+        for (int q = 0; q < T; ++q) {
+            *reinterpret_cast<uint32_t*>(o + q * ps) = wr[q];
+            *reinterpret_cast<uint32_t*>(o + (T + q) * ps) = wi[q];
         }
     }
+}
+
+// y[n + ldy r] = beta y + ybuf[r][pos[n]]: DG3's result from group order to the RWGs' own
+// numbering, kXCols columns at a time for the same reason as in prep_x_kernel.  A DG3 tile
+// holds all columns of 128 members; storing them straight to y touches 8 bytes of a sector
+// per column, and once the block of y outgrows L2 each goes to HBM as a sector of its own.
+// Here the reads are the scattered side (sectors shared in L2) and y is written in order; the
+// other way round (ybuf in order, scattered stores) took 1.33 ms.  972,000 RWGs in random
+// order x 128 columns: DG3 5.55 ms -> 2.64 + 0.52 ms; 108,000 x 37 (y fits L2): 0.389 ->
+// 0.210 + 0.020 ms; 432,000 x 16: 1.22 -> 1.16 + 0.03 ms, so every size takes this way.
+__global__ void __launch_bounds__(256) order_y_kernel(const float2* __restrict__ ybuf, const int* __restrict__ pos,
+                                                      int64_t N, int R, float2 beta, float2* __restrict__ y,
+                                                      int64_t ldy) {
+    const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (n >= N) return;
+    const int r0 = blockIdx.y * kXCols, nc = min(kXCols, R - r0);
+    const float2* src = ybuf + (int64_t)r0 * N + pos[n];
+    float2* dst = y + n + ldy * r0;
+    float2 v[kXCols], o[kXCols];
+    const bool old = beta.x != 0.f || beta.y != 0.f;
+#pragma unroll
+    for (int c = 0; c < kXCols; ++c)
+        if (c < nc) v[c] = src[(int64_t)c * N];
+    if (old) {
+#pragma unroll
+        for (int c = 0; c < kXCols; ++c)
+            if (c < nc) o[c] = dst[ldy * c];
+#pragma unroll
+        for (int c = 0; c < kXCols; ++c) {
+            v[c].x += beta.x * o[c].x - beta.y * o[c].y;
+            v[c].y += beta.x * o[c].y + beta.y * o[c].x;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < kXCols; ++c)
+        if (c < nc) dst[ldy * c] = v[c];
 }
 
 // G' planes [i_phi + n_phi r][i_theta] = conj(W g) for every (g, alpha).
@@ -1902,8 +1957,16 @@ TcPlan* get_tc_plan(Plan& P, int R, int T, cudaStream_t s) {
         o.m = sz[BM]; sz[BM] += (int64_t)2 * T * std::max<int64_t>((int64_t)d.rt * R * r8(d.rp), (int64_t)R * r8(m));
         // V'' ([i_phi + n_phi r][a]) and P'' ([a + r_t r][i_phi]) share a buffer
         o.v = sz[BV]; sz[BV] += (int64_t)2 * T * std::max<int64_t>((int64_t)np * R * r8(d.rt), (int64_t)d.rt * R * r8(np));
-        o.ldg = r8(nt); o.g = sz[BG]; sz[BG] += (int64_t)2 * T * np * R * o.ldg;
+        o.ldg = r8(nt); o.g = fused_enabled() ? 0 : sz[BG]; sz[BG] += (int64_t)2 * T * np * R * o.ldg;
         for (int b = 0; b < NB; ++b) sz[b] = (sz[b] + 63) & ~int64_t(63);
+    }
+    if (fused_enabled()) sz[BG] = 0;  // DG1a reads the FP32 spectra itself: no G' planes
+    TFMM_CUDA_CHECK(device_malloc(&M.ybuf.p, sizeof(float2) * R * P.N));
+    {
+        std::vector<int> pos(P.N);
+        for (int64_t q = 0; q < P.N; ++q) pos[P.grp_rwg[q]] = (int)q;
+        TFMM_CUDA_CHECK(device_malloc(&M.y_pos.p, sizeof(int) * P.N));
+        TFMM_CUDA_CHECK(cudaMemcpy(M.y_pos.p, pos.data(), sizeof(int) * P.N, cudaMemcpyHostToDevice));
     }
     for (int b = 0; b < NB; ++b) {
         TFMM_CUDA_CHECK(device_malloc(&M.buf[b], sizeof(bf16) * std::max<int64_t>(sz[b], 1)));
@@ -1993,6 +2056,14 @@ TcPlan* get_tc_plan(Plan& P, int R, int T, cudaStream_t s) {
         upload_tc_stage(M.st[st], pr[st], tl[st]);
         if (st == TAG1 || st == TAG2 || st == TDG2 || st == TDG3) build_stage_maps(M.st[st], pr[st], T);
     }
+    {
+        std::vector<MrTile> xt;  // prep_x: members of every group, kXTile at a time
+        for (int g = 0; g < P.G; ++g)
+            for (int n0 = 0; n0 < P.items[2 * g].n_beta; n0 += kXTile) xt.push_back(MrTile{2 * g, 0, n0});
+        M.n_xtiles = (int)xt.size();
+        TFMM_CUDA_CHECK(device_malloc(&M.x_tiles.p, sizeof(MrTile) * xt.size()));
+        TFMM_CUDA_CHECK(cudaMemcpy(M.x_tiles.p, xt.data(), sizeof(MrTile) * xt.size(), cudaMemcpyHostToDevice));
+    }
     M.m_off.resize(nI);
     M.v_off.resize(nI);
     for (int q = 0; q < nI; ++q) {
@@ -2037,11 +2108,11 @@ namespace {
 template <int T>
 void tc_aggregate_t(Plan& P, TcPlan& M, const float2* x, int R, int64_t ldx, float2* spec, cudaStream_t s) {
     TcCtx c{};
-    c.grp_rwg = P.d_grp_rwg; c.R = R; c.G = P.G; c.n_theta = P.n_theta; c.n_dir = P.n_dir; c.err = static_cast<int*>(P.tc_err.p);
+    c.R = R; c.G = P.G; c.n_theta = P.n_theta; c.n_dir = P.n_dir; c.err = static_cast<int*>(P.tc_err.p);
     c.spec = spec;
-    dim3 gx(64, std::min(P.G * 2, 4096));
-    prep_x_kernel<T><<<gx, 256, 0, s>>>(x, ldx, P.d_grp_rwg, reinterpret_cast<const TcProb*>(M.st[TAG1].d_probs),
-                                        M.st[TAG1].n_probs, R);
+    const dim3 gx(M.n_xtiles, (R + kXCols - 1) / kXCols);
+    prep_x_kernel<T><<<gx, kXTile / 2, 0, s>>>(x, ldx, P.d_grp_rwg, reinterpret_cast<const TcProb*>(M.st[TAG1].d_probs),
+                                               static_cast<const MrTile*>(M.x_tiles.p), R);
     TFMM_CUDA_CHECK(cudaGetLastError());
     launch_tc<T, TAG1>(M.st[TAG1], c, s);
     launch_tc<T, TAG2>(M.st[TAG2], c, s);
@@ -2057,9 +2128,7 @@ template <int T>
 void tc_disaggregate_t(Plan& P, TcPlan& M, const float2* spec, int R, int weights, float2 beta, float2* y,
                        int64_t ldy, cudaStream_t s) {
     TcCtx c{};
-    c.grp_rwg = P.d_grp_rwg; c.R = R; c.G = P.G; c.n_theta = P.n_theta; c.n_dir = P.n_dir; c.err = static_cast<int*>(P.tc_err.p);
-    c.ld = ldy; c.beta = beta;
-    c.y = y;
+    c.R = R; c.G = P.G; c.n_theta = P.n_theta; c.n_dir = P.n_dir; c.err = static_cast<int*>(P.tc_err.p);
     if (fused_enabled()) {  // DG1a reads the FP32 spectra itself
         c.spec_in = spec;
         c.w = weights ? P.d_weights : nullptr;
@@ -2081,7 +2150,12 @@ void tc_disaggregate_t(Plan& P, TcPlan& M, const float2* spec, int R, int weight
     else
         launch_tc<T, TDG1B>(M.st[TDG1B], c, s);
     launch_tc<T, TDG2>(M.st[TDG2], c, s);
+    c.ybuf = static_cast<float2*>(M.ybuf.p);
+    c.N = P.N;
     launch_tc<T, TDG3>(M.st[TDG3], c, s);
+    const dim3 gy((unsigned)((P.N + 255) / 256), (R + kXCols - 1) / kXCols);
+    order_y_kernel<<<gy, 256, 0, s>>>(c.ybuf, static_cast<const int*>(M.y_pos.p), P.N, R, beta, y, ldy);
+    TFMM_CUDA_CHECK(cudaGetLastError());
 }
 
 }  // namespace
