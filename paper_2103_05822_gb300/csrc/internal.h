@@ -193,6 +193,7 @@ struct TransPlan {
     int N[3] = {1, 1, 1};    // FFT grid N_x, N_y, N_z >= 2K - 1
     int64_t Ns = 0;          // grid points
     int nb = 0;              // interleaved transforms per right-hand side: 2 N_dir
+    int cube = 0, K = 0;     // side of the cube kernel's grid (0: cuFFT) and of its occupied corner
     int fft = 0;             // cufftHandle (C2C, nb transforms)
     DeviceBuffer That;       // N_dir x Ns FP32 complex: transform of (-jk/16 pi^2) T_L over the grid
     DeviceBuffer grid;       // nb x Ns FP32 complex work array (one transform after the other)

@@ -6,10 +6,13 @@ those of ``test_gpu_kernels.py``: the FP64 oracle on the same factors, 1e-5 for 
 and the Tucker tolerance 1e-6 for the three-term tensor-core chain, per output vector in l2 and
 element-wise.
 """
+import math
+
 import numpy as np
 import pytest
 
-from oracle import apply, hosvd
+import oracle
+from oracle import apply, hosvd, translation
 from paper_2103_05822_gb300.inputs import complex_gaussian, synthetic_tucker
 
 torch = pytest.importorskip("torch")
@@ -70,3 +73,39 @@ def test_gather_and_order_kernels_at_their_tile_edges(R):
     nbetas = [9, 511, 512, 513, 1025]
     ranks = [[(5, 6, min(nb, 20))] * 2 for nb in nbetas]
     _check(2100 + R, 9, 18, nbetas, ranks, R, 3, 1e-6, pad=3)
+
+
+# box counts (K_x, K_y, K_z): 2K - 1 below, at and above the sides the one-CTA transforms take
+# (4 ... 36), cubes that are not full, a plate and a side past the last (cuFFT)
+@pytest.mark.parametrize("K", [(1, 1, 1), (2, 2, 2), (3, 3, 3), (4, 4, 4), (5, 4, 5), (6, 6, 6), (8, 8, 8), (9, 8, 7),
+                               (9, 9, 9), (10, 10, 10), (12, 12, 12), (13, 13, 13), (15, 15, 15), (16, 15, 14),
+                               (18, 18, 18), (12, 12, 1), (19, 19, 19)])
+def test_translation_over_box_grids(K):
+    """Incoming spectra against the oracle's direct sums, one small patch (one RWG) per occupied box."""
+    from paper_2103_05822_gb300 import tfmm
+    box, rng = 0.5, np.random.default_rng(sum(K))
+    cells = np.unique(np.vstack([[0, 0, 0], np.array(K) - 1, rng.integers(0, K, (12, 3))]), axis=0)
+    mid = box * (cells + 0.25 + 0.5 * rng.uniform(0.1, 1.0, (len(cells), 3)))
+    mid[0] = 0.25 * box  # the lowest corner anchors the grid
+    v, f = [], []
+    for m in mid:
+        f += [[len(v), len(v) + 1, len(v) + 2], [len(v) + 1, len(v), len(v) + 3]]
+        v += [m - [0.02, 0, 0], m + [0.02, 0, 0], m + [0, 0.03, 0], m + [0, -0.02, 0.02]]
+    v, f = np.array(v), np.array(f)
+    P = oracle.problem.build(v, f, k=2 * math.pi, box=box, digits=1, tol=1e-2, compress=False)
+    prm = tfmm.tfmm_params_default(box=box, digits=1.0, tol=1e-2, max_rhs=2)
+    plan = tfmm.tfmm_plan_create(tfmm.tfmm_mesh_create(v, f), prm)
+    assert plan.info["K"] == list(K) and plan.info["n_groups"] == len(cells) == P.groups.n_groups
+    G, nd = len(cells), P.grid.n_dir
+    F = complex_gaussian((2, G, 2, nd), 5).astype(np.complex64)
+    out = torch.full((2, G, 2, nd), float("nan"), dtype=torch.complex64, device="cuda")
+    tfmm.tfmm_translate(plan, torch.from_numpy(F).cuda(), out)
+    got = out.cpu().numpy()
+    for r in range(2):
+        ref = translation.translate(F[r].astype(np.complex128), P.groups, P.grid, P.k)
+        top = np.abs(ref).max()
+        if max(K) < 3:
+            assert top == 0 and np.abs(got[r]).max() <= 1e-6 * np.abs(F[r]).max()  # touching boxes only
+        else:
+            assert np.linalg.norm(got[r] - ref) <= 1e-5 * np.linalg.norm(ref)
+            assert np.abs(got[r] - ref).max() <= 1e-5 * top
