@@ -209,6 +209,31 @@ __global__ void to_f32_kernel(const double2* __restrict__ in, int64_t n, int64_t
 }
 
 // --------------------------------------------------------- plane-wave RHS
+// V_m = -sum_sides s l sum_q W_q (rho_q . pol) exp(-j k khat . (p + rho_q)), rho = x' e1 + y' e2
+// with e1 = q1 - p, e2 = q2 - p and the rule's points x' = u, y' = v (1 - u).
+//
+// FP64 runs at 1/64 of the FP32 rate here, and a sincos per point (50 per RWG and incidence)
+// made the kernel wait for nothing else: 61.8 ms for 108,000 RWGs x 128.  So the sum over the
+// points is expanded about the rule's mean point c: with x = x' - mean, y = y' - mean,
+// t1 = k khat . e1, t2 = k khat . e2,
+//   sum_q = exp(-j k khat . c) sum_n (-j)^n / n! sum_q W_q (amplitude_q) (x t1 + y t2)^n,
+// whose inner sums are the rule's moments (the same points and weights, so the same result),
+// one set for the whole mesh.  What decides the accuracy stays FP64: the phase at c, its
+// reduction to 1/256 turn and the table value there, and the terms n = 0 (amplitude at c) and
+// n = 1 (bilinear in khat and pol, a symmetric 3 x 3 matrix per side).  Terms n = 2 .. 8, at
+// most a few percent of the sum, and the rotation by the rest of the phase (under 0.0123 rad) are FP32.
+// Against 64 bits the unrounded sum is off by 7e-10 on a lambda/10 mesh (rounding V to FP32:
+// 2.55e-8, as before) and 1.3e-9 at the limit kPWSpread.  1.8 ms for the same block (0.02 ms
+// for the bytes); the 28 FP64 operations left per side and incidence are what bounds it.
+constexpr int kPWDegree = 8;
+constexpr int kPWTerms = (kPWDegree - 1) * (kPWDegree + 4) / 2;  // (n, k), 2 <= n <= 8, 0 <= k <= n
+constexpr int kPWTable = 256;    // steps per turn of the phase table
+constexpr int kPWCols = 64;      // incidences per block: a side's constants cost as much FP64 as three of them
+constexpr int kPWThreads = 128;
+// largest |phase - phase at c| over a triangle for the expansion (0.40 on a lambda/10 mesh); a
+// triangle that spreads further takes the points one by one
+constexpr float kPWSpread = 0.5f;
+
 struct PWArgs {
     const RwgGeom* geom;
     const double* khat;  // R x 3
@@ -217,20 +242,19 @@ struct PWArgs {
     double k;
     int64_t n;
     int R, nq;
+    double u, v, m00, m20, m11, m02;  // mean point and central moments of the rule
+    float cp[kPWTerms], cq[kPWTerms], cr[kPWTerms];  // (-1)^(n/2) C(n, k) / n! times m(k, n-k), m(k+1, n-k), m(k, n-k+1)
 };
 
-__global__ void planewave_kernel(const PWArgs a) {
-    const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int r = blockIdx.y;
-    if (m >= a.n) return;
-    const RwgGeom g = a.geom[m];
-    const double* kh = a.khat + 3 * r;
-    const double* p = a.pol + 3 * r;
+// The points one by one, all FP64.
+__device__ __noinline__ double2 planewave_points(const RwgGeom* gp, const double* kh, const double* p, double k,
+                                                 int nq) {
+    const RwgGeom g = *gp;
     double vr = 0.0, vi = 0.0;
     for (int side = 0; side < 2; ++side) {
         const double* pv = side ? g.pm : g.pp;
         const double sgn = side ? -1.0 : 1.0;
-        for (int q = 0; q < a.nq; ++q) {
+        for (int q = 0; q < nq; ++q) {
             const double u = c_qu[q], v = c_qv[q], w = c_qw[q];
             double r3[3], dot = 0.0, ph = 0.0;
             for (int c = 0; c < 3; ++c) {
@@ -239,12 +263,225 @@ __global__ void planewave_kernel(const PWArgs a) {
                 ph += kh[c] * r3[c];
             }
             double sn, cs;
-            sincos(-a.k * ph, &sn, &cs);
+            sincos(-k * ph, &sn, &cs);
             vr -= dot * cs;
             vi -= dot * sn;
         }
     }
-    a.V[m + a.n * r] = make_float2((float)vr, (float)vi);
+    return make_double2(vr, vi);
+}
+
+struct PWSide {        // one triangle of an RWG
+    double c[3];       // mean point
+    double w[3];       // n = 0: s l m00 (u e1 + v e2)
+    double b[6];       // n = 1: s l k (m20 e1 e1 + m11 (e1 e2 + e2 e1) + m02 e2 e2), xx yy zz xy xz yz
+    float e1[3], e2[3];  // k e1, k e2
+    float l;           // s l / k
+};
+
+__device__ __forceinline__ void planewave_side(PWSide& s, const PWArgs& a, const double* p, const double* q1,
+                                               const double* q2, double sl) {
+    double e1[3], e2[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        e1[c] = q1[c] - p[c];
+        e2[c] = q2[c] - p[c];
+        const double rho = a.u * e1[c] + a.v * e2[c];
+        s.c[c] = p[c] + rho;
+        s.w[c] = sl * a.m00 * rho;
+        s.e1[c] = (float)(a.k * e1[c]);
+        s.e2[c] = (float)(a.k * e2[c]);
+    }
+    s.l = (float)(sl / a.k);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        const int x = i < 3 ? i : i == 5 ? 1 : 0, y = i < 3 ? i : i == 3 ? 1 : 2;
+        s.b[i] = sl * a.k * (a.m20 * e1[x] * e1[y] + a.m11 * (e1[x] * e2[y] + e1[y] * e2[x]) + a.m02 * e2[x] * e2[y]);
+    }
+}
+
+struct PWInc {          // one incidence
+    double kt[3];       // khat k / 2 pi in table steps
+    double p[3];
+    double o[6];        // p_x k_x, p_y k_y, p_z k_z, p_x k_y + p_y k_x, ...
+    float kf[3], pf[3];
+};
+
+// One side's sum; false when the expansion does not hold.
+__device__ __forceinline__ bool planewave_side_sum(const PWSide& s, const PWInc& v, const PWArgs& a,
+                                                   const double2* tab, const float2* tabf, double& re,
+                                                   double& im) {
+    const float t1 = s.e1[0] * v.kf[0] + s.e1[1] * v.kf[1] + s.e1[2] * v.kf[2];
+    const float t2 = s.e2[0] * v.kf[0] + s.e2[1] * v.kf[1] + s.e2[2] * v.kf[2];
+    const float uf = (float)a.u, vf = (float)a.v, at = uf * t1 + vf * t2;
+    const float spread = fmaxf(fabsf(at), fmaxf(fabsf(t1 - at), fabsf(t2 - at)));
+    const double t = v.kt[0] * s.c[0] + v.kt[1] * s.c[1] + v.kt[2] * s.c[2];
+    // (the phase, in table steps, below 2^40: read off the exponent, which spares an FP64 comparison)
+    if (!(spread <= kPWSpread) || (__double2hiint(t) & 0x7ff00000) >= (1023 + 40) << 20) return false;
+    // n >= 2: even n to the real part, odd n to the imaginary (times -j)
+    float x1[kPWDegree + 1], x2[kPWDegree + 1];
+    x1[0] = x2[0] = 1.f;
+#pragma unroll
+    for (int n = 1; n <= kPWDegree; ++n) {
+        x1[n] = x1[n - 1] * t1;
+        x2[n] = x2[n - 1] * t2;
+    }
+    float P[2] = {0.f, 0.f}, Q[2] = {0.f, 0.f}, S[2] = {0.f, 0.f};
+    int i = kPWTerms;
+#pragma unroll
+    for (int n = kPWDegree; n >= 2; --n)
+#pragma unroll
+        for (int k = n; k >= 0; --k) {
+            --i;
+            const float m = x1[k] * x2[n - k];
+            P[n & 1] = fmaf(a.cp[i], m, P[n & 1]);
+            Q[n & 1] = fmaf(a.cq[i], m, Q[n & 1]);
+            S[n & 1] = fmaf(a.cr[i], m, S[n & 1]);
+        }
+    const float c1 = s.l * (s.e1[0] * v.pf[0] + s.e1[1] * v.pf[1] + s.e1[2] * v.pf[2]);
+    const float c2 = s.l * (s.e2[0] * v.pf[0] + s.e2[1] * v.pf[1] + s.e2[2] * v.pf[2]);
+    const float c0 = uf * c1 + vf * c2;
+    const float hr = c0 * P[0] + c1 * Q[0] + c2 * S[0], hi = -(c0 * P[1] + c1 * Q[1] + c2 * S[1]);
+    // n = 0 and 1
+    const double ar = s.w[0] * v.p[0] + s.w[1] * v.p[1] + s.w[2] * v.p[2];
+    const double ai = -(s.b[0] * v.o[0] + s.b[1] * v.o[1] + s.b[2] * v.o[2] + s.b[3] * v.o[3] + s.b[4] * v.o[4] +
+                        s.b[5] * v.o[5]);
+    // exp(-j phase) = T (1 + (cos d - 1) - j sin d), T the table value at the nearest step
+    const double magic = 6755399441055744.0;  // 1.5 2^52: the sum's low bits are the nearest integer
+    const double sh = t + magic;
+    const float d = (float)(t - (sh - magic)) * (float)(2.0 * 3.14159265358979323846 / kPWTable);
+    const int step = __double2loint(sh) & (kPWTable - 1);
+    const double2 T = tab[step];
+    const float2 Tf = tabf[step];
+    const float d2 = d * d, sd = d - d * d2 * (1.f / 6.f), cm = d2 * fmaf(d2, 1.f / 24.f, -0.5f);
+    const float er = Tf.x * cm + Tf.y * sd, ei = Tf.y * cm - Tf.x * sd;  // T (cm - j sd)
+    const float af = (float)ar, bf = (float)ai, gx = Tf.x + er, gy = Tf.y + ei;
+    const float fr = af * er - bf * ei + (hr * gx - hi * gy), fi = af * ei + bf * er + (hr * gy + hi * gx);
+    re = ar * T.x + ((double)fr - ai * T.y);
+    im = ar * T.y + ((double)fi + ai * T.x);
+    return true;
+}
+
+// One side of an RWG per thread (two neighbouring lanes an RWG: both sides in one thread
+// spilled), kPWCols incidences per block, their table in shared memory.
+__global__ void __launch_bounds__(kPWThreads, 4) planewave_kernel(const __grid_constant__ PWArgs a) {
+    __shared__ double2 tab[kPWTable];
+    __shared__ float2 tabf[kPWTable];
+    __shared__ PWInc inc[kPWCols];
+    const int r0 = blockIdx.y * kPWCols, nr = min(kPWCols, a.R - r0);
+    for (int i = threadIdx.x; i < kPWTable; i += kPWThreads) {
+        double sn, cs;
+        sincospi(2.0 * i / kPWTable, &sn, &cs);
+        tab[i] = make_double2(cs, -sn);
+        tabf[i] = make_float2((float)cs, (float)-sn);
+    }
+    if (threadIdx.x < nr) {
+        PWInc& v = inc[threadIdx.x];
+        const double* kh = a.khat + 3 * (r0 + threadIdx.x);
+        const double* p = a.pol + 3 * (r0 + threadIdx.x);
+        for (int c = 0; c < 3; ++c) {
+            v.kt[c] = kh[c] * (a.k * (kPWTable / (2.0 * 3.14159265358979323846)));
+            v.p[c] = p[c];
+            v.kf[c] = (float)kh[c];
+            v.pf[c] = (float)p[c];
+            v.o[c] = p[c] * kh[c];
+        }
+        v.o[3] = p[0] * kh[1] + p[1] * kh[0];
+        v.o[4] = p[0] * kh[2] + p[2] * kh[0];
+        v.o[5] = p[1] * kh[2] + p[2] * kh[1];
+    }
+    __syncthreads();
+    const int64_t m = blockIdx.x * (int64_t)(kPWThreads / 2) + threadIdx.x / 2;
+    const bool live = m < a.n;
+    const int minus = threadIdx.x & 1;
+    const RwgGeom* gp = a.geom + (live ? m : a.n - 1);
+    PWSide side;
+    {
+        const RwgGeom g = *gp;
+        double p[3];
+        for (int c = 0; c < 3; ++c) p[c] = minus ? g.pm[c] : g.pp[c];
+        planewave_side(side, a, p, g.q1, g.q2, minus ? -g.l : g.l);
+    }
+    for (int r = 0; r < nr; ++r) {
+        double re = 0.0, im = 0.0;
+        bool ok = planewave_side_sum(side, inc[r], a, tab, tabf, re, im);
+        re = -(re + __shfl_xor_sync(0xffffffffu, re, 1));
+        im = -(im + __shfl_xor_sync(0xffffffffu, im, 1));
+        ok = __shfl_xor_sync(0xffffffffu, (int)ok, 1) && ok;
+        if (live && !minus) {
+            if (!ok) {
+                const double2 v = planewave_points(gp, a.khat + 3 * (r0 + r), a.pol + 3 * (r0 + r), a.k, a.nq);
+                re = v.x;
+                im = v.y;
+            }
+            a.V[m + a.n * (r0 + r)] = make_float2((float)re, (float)im);
+        }
+    }
+}
+
+// The rule's points on the triangle's (u, v (1 - u)) and their weights (sum 1/2).
+void triangle_rule(int order, std::vector<double>& qu, std::vector<double>& qv, std::vector<double>& qw) {
+    std::vector<double> x, w;
+    gauss_legendre(order, x, w);
+    for (int a = 0; a < order; ++a)
+        for (int b = 0; b < order; ++b) {
+            const double u = 0.5 * (x[a] + 1.0), v = 0.5 * (x[b] + 1.0);
+            qu.push_back(u);
+            qv.push_back(v);
+            qw.push_back(0.25 * w[a] * w[b] * (1.0 - u));  // sum = 1/2: int_T f = 2A sum w f
+        }
+}
+
+void launch_planewave(const Plan& P, const double* khat, const double* pol, int R, float2* V, cudaStream_t s) {
+    PWArgs a{};
+    a.geom = P.d_geom;
+    a.khat = khat;
+    a.pol = pol;
+    a.V = V;
+    a.k = P.k;
+    a.n = P.N;
+    a.R = R;
+    a.nq = P.params.quad_order * P.params.quad_order;
+    std::vector<double> qu, qv, qw;
+    triangle_rule(P.params.quad_order, qu, qv, qw);
+    double su = 0.0, sv = 0.0;
+    for (int q = 0; q < a.nq; ++q) {
+        a.m00 += qw[q];
+        su += qw[q] * qu[q];
+        sv += qw[q] * qv[q] * (1.0 - qu[q]);
+    }
+    a.u = su / a.m00;
+    a.v = sv / a.m00;
+    auto moment = [&](int j, int k) {
+        double m = 0.0;
+        for (int q = 0; q < a.nq; ++q) m += qw[q] * std::pow(qu[q] - a.u, j) * std::pow(qv[q] * (1.0 - qu[q]) - a.v, k);
+        return m;
+    };
+    a.m20 = moment(2, 0);
+    a.m11 = moment(1, 1);
+    a.m02 = moment(0, 2);
+    int i = 0;
+    for (int n = 2; n <= kPWDegree; ++n) {
+        double binom = 1.0;  // C(n, k)
+        for (int k = 0; k <= n; ++k) {
+            const double f = binom / std::tgamma(n + 1.0) * ((n / 2) % 2 ? -1.0 : 1.0);
+            a.cp[i] = (float)(f * moment(k, n - k));
+            a.cq[i] = (float)(f * moment(k + 1, n - k));
+            a.cr[i] = (float)(f * moment(k, n - k + 1));
+            binom = binom * (n - k) / (k + 1);
+            ++i;
+        }
+    }
+    for (int c0 = 0; c0 < R; c0 += 65535 * kPWCols) {  // grid.y limit
+        PWArgs b = a;
+        b.khat += 3 * (int64_t)c0;
+        b.pol += 3 * (int64_t)c0;
+        b.V += a.n * c0;
+        b.R = std::min(R - c0, 65535 * kPWCols);
+        const dim3 grid((unsigned)((2 * P.N + kPWThreads - 1) / kPWThreads), (unsigned)((b.R + kPWCols - 1) / kPWCols));
+        planewave_kernel<<<grid, kPWThreads, 0, s>>>(b);
+        TFMM_CUDA_CHECK(cudaGetLastError());
+    }
 }
 
 int grid1d(int64_t total, int threads = 256) {
@@ -253,16 +490,8 @@ int grid1d(int64_t total, int threads = 256) {
 }
 
 void upload_quadrature(int order, cudaStream_t s) {
-    std::vector<double> x, w;
-    gauss_legendre(order, x, w);
     std::vector<double> qu, qv, qw;
-    for (int a = 0; a < order; ++a)
-        for (int b = 0; b < order; ++b) {
-            const double u = 0.5 * (x[a] + 1.0), v = 0.5 * (x[b] + 1.0);
-            qu.push_back(u);
-            qv.push_back(v);
-            qw.push_back(0.25 * w[a] * w[b] * (1.0 - u));  // sum = 1/2: int_T f = 2A sum w f
-        }
+    triangle_rule(order, qu, qv, qw);
     TFMM_CUDA_CHECK(cudaMemcpyToSymbolAsync(c_qu, qu.data(), qu.size() * sizeof(double), 0,
                                             cudaMemcpyHostToDevice, s));
     TFMM_CUDA_CHECK(cudaMemcpyToSymbolAsync(c_qv, qv.data(), qv.size() * sizeof(double), 0,
@@ -1063,18 +1292,7 @@ void planewave_rhs(const Plan& P, const double* khat, const double* pol, int R, 
     DevBuf d_k(sizeof(double) * 3 * R), d_p(sizeof(double) * 3 * R);
     TFMM_CUDA_CHECK(cudaMemcpyAsync(d_k.p, khat, sizeof(double) * 3 * R, cudaMemcpyHostToDevice, s));
     TFMM_CUDA_CHECK(cudaMemcpyAsync(d_p.p, pol, sizeof(double) * 3 * R, cudaMemcpyHostToDevice, s));
-    PWArgs a;
-    a.geom = P.d_geom;
-    a.khat = d_k.as<double>();
-    a.pol = d_p.as<double>();
-    a.V = V;
-    a.k = P.k;
-    a.n = P.N;
-    a.R = R;
-    a.nq = P.params.quad_order * P.params.quad_order;
-    dim3 grid((unsigned)((P.N + 255) / 256), R);
-    planewave_kernel<<<grid, 256, 0, s>>>(a);
-    TFMM_CUDA_CHECK(cudaGetLastError());
+    launch_planewave(P, d_k.as<double>(), d_p.as<double>(), R, V, s);
     TFMM_CUDA_CHECK(cudaStreamSynchronize(s));
 }
 
@@ -1134,18 +1352,7 @@ void planewave_rhs_noalloc(const Plan& P, const double* khat, const double* pol,
         TFMM_CUDA_CHECK(cudaMemcpyAsync(table + 3 * kNoAllocMaxIncidences, g_pw_stage + 3 * kNoAllocMaxIncidences,
                                         sizeof(double) * 3 * R, cudaMemcpyHostToDevice, s));
     }
-    PWArgs a;
-    a.geom = P.d_geom;
-    a.khat = table;
-    a.pol = table + 3 * kNoAllocMaxIncidences;
-    a.V = V;
-    a.k = P.k;
-    a.n = P.N;
-    a.R = R;
-    a.nq = P.params.quad_order * P.params.quad_order;
-    dim3 grid((unsigned)((P.N + 255) / 256), R);
-    planewave_kernel<<<grid, 256, 0, s>>>(a);
-    TFMM_CUDA_CHECK(cudaGetLastError());
+    launch_planewave(P, table, table + 3 * kNoAllocMaxIncidences, R, V, s);
 }
 
 }  // namespace tfmm

@@ -109,3 +109,38 @@ def test_translation_over_box_grids(K):
         else:
             assert np.linalg.norm(got[r] - ref) <= 1e-5 * np.linalg.norm(ref)
             assert np.abs(got[r] - ref).max() <= 1e-5 * top
+
+
+@pytest.mark.parametrize("order", [1, 2, 5, 10])
+@pytest.mark.parametrize("nu,R", [(2, 65), (3, 64), (4, 1), (7, 130)])
+def test_planewave_expansion_and_its_limit(nu, R, order):
+    """V against the same rule point by point in FP64: meshes whose triangles all, partly or never
+    spread the phase past the expansion's limit, low and high rules, R around the 64 incidences of a
+    block.  Bound: rounding V to FP32 (6e-8 an entry) and half as much again for the expansion."""
+    from paper_2103_05822_gb300 import tfmm
+    from paper_2103_05822_gb300.inputs import icosphere
+    v, f = icosphere(1.0, nu, center=(3.0, -2.0, 11.0))
+    mesh = tfmm.tfmm_mesh_create(v, f)
+    plan = tfmm.tfmm_plan_create(mesh, tfmm.tfmm_params_default(box=0.5, digits=1.0, tol=1e-2, quad_order=order))
+    edge, _, free = tfmm.tfmm_mesh_rwg(mesh)
+    rng = np.random.default_rng(order)
+    kh = rng.standard_normal((R, 3))
+    kh /= np.linalg.norm(kh, axis=1)[:, None]
+    pol = np.cross(kh, rng.standard_normal((R, 3)))
+    V = torch.full((R, len(edge)), float("nan"), dtype=torch.complex64, device="cuda")
+    tfmm.tfmm_planewave(plan, kh, pol, V)
+    x, w = np.polynomial.legendre.leggauss(order)
+    u, w = 0.5 * (x + 1), 0.5 * w
+    q1, q2 = v[edge[:, 0]], v[edge[:, 1]]
+    length = np.linalg.norm(q1 - q2, axis=1)
+    ref = np.zeros((R, len(edge)), complex)
+    for side, sign in ((0, 1.0), (1, -1.0)):
+        p = v[free[:, side]]
+        for a in range(order):
+            for b in range(order):
+                rho = u[a] * (q1 - p) + u[b] * (1 - u[a]) * (q2 - p)
+                amp = sign * w[a] * w[b] * (1 - u[a]) * length[:, None] * rho
+                ref -= (pol @ amp.T) * np.exp(-2j * math.pi * (kh @ (p + rho).T))
+    got = V.cpu().numpy()
+    assert np.linalg.norm(got - ref) <= 9e-8 * np.linalg.norm(ref)
+    assert np.abs(got - ref).max() <= 9e-8 * np.abs(ref).max()
