@@ -294,8 +294,9 @@ def run_reference(args, w, world, rank):
 # --------------------------------------------------------------------- ours
 def launches_per_step(tfmm, plan, R, dev):
     """Kernels one aggregate + disaggregate pair launches: one persistent kernel per stage
-    for one RHS (three per stage on the split path, taken by plans with fewer work items
-    than twice the SMs), the tensor-core chain for many (operand prep and three kernels
+    or one per stage with small groups wholly in shared memory (at least; by size class when
+    there are many) for one RHS (three per stage on the split path, taken by plans with fewer
+    work items than twice the SMs whose groups are larger), the tensor-core chain for many (operand prep and three kernels
     for aggregation; four and the reordering of y for disaggregation)."""
     import torch
     t = tfmm.tfmm_plan_tuning_get(plan)

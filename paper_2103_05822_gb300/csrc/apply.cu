@@ -909,6 +909,7 @@ void finalize_hot_layout(Plan& P, cudaStream_t s) {
     P.d_items = nullptr;
     TFMM_CUDA_CHECK(device_malloc(&P.d_items, sizeof(TuckerItem) * nI));
     TFMM_CUDA_CHECK(cudaMemcpyAsync(P.d_items, P.items.data(), sizeof(TuckerItem) * nI, cudaMemcpyHostToDevice, s));
+    configure_small(P, s);
     configure_hot(P, P.tuning, s);
 }
 

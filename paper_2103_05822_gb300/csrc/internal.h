@@ -218,6 +218,14 @@ struct SplitPlan {
     size_t smem_ag1 = 0, smem_ag2 = 0, smem_ag34 = 0, smem_dg1 = 0, smem_dg2 = 0, smem_dg3 = 0;
 };
 
+// Groups that one launch of the small-group kernels covers, and the sizes that its shared
+// memory is laid out for.
+struct SmallClass {
+    int first = 0, groups = 0;  // range of the plan's small_order
+    int elems = 0;              // complex elements of the largest item's factors
+    int max_nb = 0, max_rt = 0, max_rb = 0, max_m = 0;  // m: r_theta r_phi
+};
+
 struct Schedule {
     int threads = 512;
     int blocks = 0;       // persistent grid
@@ -266,6 +274,11 @@ struct Plan {
     int tc_f34_n1 = 0;                 // cap on r_theta x RHS per CTA of the fused AG3+AG4 kernel (0: largest that fits)
     int tc_dg1a_pairs = 0;             // (i_phi, r) pairs per CTA of the DG1a kernel (0: 128 when it fits, else 64)
     bool hot_ok = false;               // the single-RHS kernels fit (shared memory of the largest item)
+    bool small_ok = false;             // every item's factors and one column fit one CTA's shared memory
+    bool small_one = false;            // and that is the faster way for one right-hand side
+    std::vector<SmallClass> small_classes;
+    DeviceBuffer small_order;          // group ids, largest factors first
+    size_t small_room = 0;             // dynamic shared memory one CTA may have
     std::unique_ptr<SplitPlan> split;  // set when the single-RHS stages run the split path
     double tuned_ms[2] = {0, 0};       // autotuner's best aggregate / disaggregate times
     int live_graphs = 0;               // captured graphs that still point into this plan
@@ -339,6 +352,11 @@ void launch_dense_disaggregate(const Plan& P, const float2* spec, int R, int wei
                                int64_t ldy, cudaStream_t s);
 void pack_factors_fp32(Plan& P, cudaStream_t s);  // from P.f64 into P.d_factors
 void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s);  // orders and schedules of the 1-RHS kernels
+// small.cu
+void configure_small(Plan& P, cudaStream_t s);  // after the items are known
+void launch_small_aggregate(const Plan& P, const float2* x, int R, int64_t ldx, float2* spec, cudaStream_t s);
+void launch_small_disaggregate(const Plan& P, const float2* spec, int R, int weights, float2 beta, float2* y,
+                               int64_t ldy, cudaStream_t s);
 // mrhs_tc.cu
 void build_tc_factors(Plan& P, int T, cudaStream_t s);
 TcPlan* get_tc_plan(Plan& P, int R, int T, cudaStream_t s);

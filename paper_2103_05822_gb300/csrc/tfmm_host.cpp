@@ -164,18 +164,22 @@ void check_params(const tfmm_params& p) {
 }
 
 // The engine that applies one call with R columns:
+//   small:   one CTA per (group, component) with everything in shared memory, for plans whose
+//            every item fits (small.cu), in place of columns and chain unless the tuning
+//            asks for one of the single-RHS paths;
 //   columns: the persistent single-RHS kernels, one column after the other (R = 1, or
 //            mrhs_precision 1, or TFMM_MR=loop);
 //   chain:   the grouped-GEMM chain on FP32 CUDA cores (mrhs_precision 0), also the
 //            fallback when a work item does not fit the single-RHS kernels;
 //   tc:      the split-BF16 tensor-core chain with `terms` terms (mrhs_precision 2, 3).
-enum class Engine { columns, chain, tc };
+enum class Engine { small, columns, chain, tc };
 
 Engine engine_for(const Plan& P, int R, int* terms) {
     *terms = 0;
     const int p = P.params.mrhs_precision;
     const char* e = std::getenv("TFMM_MR");
     const bool loop = e && std::strcmp(e, "loop") == 0;
+    if (P.tuning.split == 0 && !loop && (R <= 1 ? P.small_one : P.small_ok && p <= 1)) return Engine::small;
     if (P.hot_ok && (R <= 1 || loop || p == 1 || plan_is_svd(P))) return Engine::columns;
     if (R > 1 && (p == 2 || p == 3)) {
         *terms = p;
@@ -194,6 +198,7 @@ void run_aggregate(Plan& P, const float2* x, int R, int64_t ldx, float2* spec, c
     NvtxRange nvtx("tfmm_aggregate");
     int T = 0;
     switch (engine_for(P, R, &T)) {
+        case Engine::small: launch_small_aggregate(P, x, R, ldx, spec, s); break;
         case Engine::tc: launch_tc_aggregate(P, T, x, R, ldx, spec, s); break;
         case Engine::chain: launch_mr_aggregate(P, x, R, ldx, spec, s); break;
         default: launch_tucker_aggregate(P, x, R, ldx, spec, s);
@@ -205,6 +210,7 @@ void run_disaggregate(Plan& P, const float2* spec, int R, int weights, float2 be
     NvtxRange nvtx("tfmm_disaggregate");
     int T = 0;
     switch (engine_for(P, R, &T)) {
+        case Engine::small: launch_small_disaggregate(P, spec, R, weights, beta, y, ldy, s); break;
         case Engine::tc: launch_tc_disaggregate(P, T, spec, R, weights, beta, y, ldy, s); break;
         case Engine::chain: launch_mr_disaggregate(P, spec, R, weights, beta, y, ldy, s); break;
         default: launch_tucker_disaggregate(P, spec, R, weights, beta, y, ldy, s);

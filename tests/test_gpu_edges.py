@@ -144,3 +144,30 @@ def test_planewave_expansion_and_its_limit(nu, R, order):
     got = V.cpu().numpy()
     assert np.linalg.norm(got - ref) <= 9e-8 * np.linalg.norm(ref)
     assert np.abs(got - ref).max() <= 9e-8 * np.abs(ref).max()
+
+
+def _small_ranks(rng, nt, npf, nb, top):
+    return [(int(rng.integers(1, nt + 1)), int(rng.integers(1, npf + 1)), int(rng.integers(1, min(nb, top) + 1)))
+            for _ in range(2)]
+
+
+@pytest.mark.parametrize("R", [1, 2, 5, 16, 17, 33])
+@pytest.mark.parametrize("nt,npf", [(5, 10), (8, 15), (14, 28)])
+def test_small_groups_in_shared_memory(nt, npf, R):
+    """Everything of a group in one CTA: column blocks of 1, 4, 8 and 16 and what is left of them, full and
+    rank-1 factors, odd and even sizes, the bank padding's steps."""
+    rng = np.random.default_rng(31 * nt + R)
+    nbetas = [2, 3, 8, 15, 16, 31, 64, 65, 100]
+    ranks = [_small_ranks(rng, nt, npf, nb, 30) for nb in nbetas]
+    ranks[1], ranks[3] = [(1, 1, 1), (nt, 1, 2)], [(nt, npf, 15), (1, npf, 1)]
+    _check(3000 + 40 * nt + R, nt, npf, nbetas, ranks, R, 0, 1e-5, pad=2)
+
+
+@pytest.mark.parametrize("R", [1, 6])
+def test_small_groups_by_size_class(R):
+    """Enough groups for several launches by size (four per SM)."""
+    rng = np.random.default_rng(77)
+    G = 4 * torch.cuda.get_device_properties(0).multi_processor_count + 3
+    nbetas = [int(n) for n in rng.integers(2, 40, G)]
+    ranks = [_small_ranks(rng, 4, 8, nb, 12) for nb in nbetas]
+    _check(3700 + R, 4, 8, nbetas, ranks, R, 0, 1e-5, betas=(0.5 - 0.25j,))
