@@ -217,7 +217,7 @@ __device__ __forceinline__ void load_g_tile(uint8_t* st, const TcCtx& c, const T
 // stage, NTHR threads sharing the copies.
 template <int T, int S, int NTHR = TTHREADS>
 __device__ __forceinline__ void load_stage(uint8_t* st, const TcCtx& c, const TcProb& p, int m0, int n0, int kt,
-                                           int kt0) {
+                                           int kt0, int b_plane = PLANE_TILE) {
     const bool seg1 = kt >= kt0;
     const int k0 = (seg1 ? kt - kt0 : kt) * TBK;
     const int K = seg1 ? p.K1 : p.K0;
@@ -245,7 +245,7 @@ __device__ __forceinline__ void load_stage(uint8_t* st, const TcCtx& c, const Tc
         const int n = n0 + r, k = k0 + kc * 8;
         const bool ok = n < p.N && k < K8;
         const bf16* src = ok ? B + pl * bps + (int64_t)n * bld + k : B;
-        cp16(sb + pl * PLANE_TILE + (r >> 3) * 512 + kc * 128 + (r & 7) * 16, src, ok ? 16 : 0);
+        cp16(sb + pl * b_plane + (r >> 3) * 512 + kc * 128 + (r & 7) * 16, src, ok ? 16 : 0);
     }
 }
 
@@ -256,7 +256,7 @@ __device__ __forceinline__ void epilogue(const TcCtx& c, const TcProb& p, int i,
         case TAG1:  // T stored [r][c]: row j (= r), column i (= c)
             store_planes<T>(o, p.o_ps, (int64_t)j * p.o_ld + i, v);
             break;
-        case TAG2: {  // M' stored [a + r_t r][b]; i = b + r_p a (the order of the C_(3)^T planes), j = r
+        case TAG2: {  // M' stored [a + r_t r][b]; i = b + r_p a (the order of the C_(3)^T planes, r_p even), j = r
             const int rp = p.M / p.rt, a = i / rp, b = i % rp;
             store_planes<T>(o, p.o_ps, (int64_t)(a + p.rt * j) * p.o_ld + b, v);
         } break;
@@ -306,6 +306,59 @@ __device__ __forceinline__ void drain_add(float (&ar)[64], float (&ai)[64], uint
     }
 }
 
+// The same for the stacked form (see stacked_products): hc columns (a multiple of 8) from col of
+// (L_(T-1) + ... + L_1) + L_0, the real block at `base`, the imaginary one T bn columns on.
+template <int T>
+__device__ __forceinline__ void drain_stacked(float (&ar)[64], float (&ai)[64], uint32_t base, int bn, int col,
+                                              int hc) {
+#pragma unroll
+    for (int c0 = 0; c0 < 64; c0 += 8) {
+        if (c0 < hc) {  // warp-uniform
+            uint32_t vr[T][8], vi[T][8];
+#pragma unroll
+            for (int q = 0; q < T; ++q) {
+                tmem_ld8(vr[q], base + q * bn + col + c0);
+                tmem_ld8(vi[q], base + (T + q) * bn + col + c0);
+            }
+            asm volatile("tcgen05.wait::ld.sync.aligned;");
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                float re = __uint_as_float(vr[T - 1][j]), im = __uint_as_float(vi[T - 1][j]);
+#pragma unroll
+                for (int q = T - 2; q >= 0; --q) {
+                    re += __uint_as_float(vr[q][j]);
+                    im += __uint_as_float(vi[q][j]);
+                }
+                ar[c0 + j] += re;
+                ai[c0 + j] += im;
+            }
+        }
+    }
+}
+
+// One K step of the stacked form: the rows of B's term planes follow one another in shared
+// memory (re terms, then im terms, bn rows each), so that term p of A meets the first T - p terms
+// of B in one MMA of N = (T - p) bn columns, into the levels L_p .. L_(T-1) of an accumulator of T
+// levels of bn columns (real) and T more (imaginary).  Level L_q collects the products whose
+// term orders add up to q: 4 T MMAs instead of 4 n_products, each wide enough to run at rate
+// (an MMA takes as long at N = 16 as at N = 64), and the same products.  a(p, im) and b(im) are
+// the descriptors of A's term planes and of B's first re / im plane; `fresh` restarts all levels.
+template <int T, class DA, class DB>
+__device__ __forceinline__ void stacked_products(uint32_t d, int bn, bool fresh, DA a, DB b) {
+    const uint64_t br = b(0), bi = b(1);
+#pragma unroll
+    for (int p = 0; p < T; ++p) {
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((T - p) * bn >> 3) << 17) |
+                               ((uint32_t)(TBM >> 4) << 24);
+        const uint64_t ar = a(p, 0), ai = a(p, 1);
+        const uint32_t dr = d + p * bn, di = d + (T + p) * bn, acc = (fresh && p == 0) ? 0u : 1u;
+        mma_bf16(dr, ar, br, idesc, acc);
+        mma_bf16(dr, ai, bi, idesc | (1u << 13), 1u);
+        mma_bf16(di, ar, bi, idesc, acc);
+        mma_bf16(di, ai, br, idesc, 1u);
+    }
+}
+
 // nst: stages of the shared-memory ring (1 .. NST_MAX); tcols: TMEM columns allocated
 // (Cr at column 0, Ci at column cofs).
 //
@@ -320,7 +373,7 @@ __device__ __forceinline__ void drain_add(float (&ar)[64], float (&ai)[64], uint
 template <int T, int S, bool CH>
 __global__ void __launch_bounds__(CH ? 2 * TTHREADS : TTHREADS)
     tc_gemm_kernel(const TcCtx c, const TcProb* __restrict__ probs, const MrTile* __restrict__ tiles, int nst,
-                   int tcols, int cofs, int hsplit, int chunk) {
+                   int tcols, int cofs, int hsplit, int chunk, int stack) {
     constexpr int NST_MAX = (T == 2) ? 3 : 2;
     constexpr int STAGE = 2 * 2 * T * PLANE_TILE;
     constexpr int NTHR = CH ? 2 * TTHREADS : TTHREADS;
@@ -348,8 +401,10 @@ __global__ void __launch_bounds__(CH ? 2 * TTHREADS : TTHREADS)
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.BN >> 3) << 17) | ((uint32_t)(TBM >> 4) << 24);
     const uint32_t idesc_neg = idesc | (1u << 13);
     // CH: this warp's TMEM lanes and 64 columns, and their running FP32 sums
+    // (stack: half of the BN columns)
     const uint32_t q_lanes = (uint32_t)((warp & 3) * 32) << 16;
-    const int q_col = (warp >> 2) * 64;
+    const int q_cols = CH && stack ? p.BN / 2 : 64, q_col = (warp >> 2) * q_cols;
+    const int b_plane = CH && stack ? p.BN * 64 : PLANE_TILE;
     float accr[CH ? 64 : 1], acci[CH ? 64 : 1];
     if constexpr (CH) {
 #pragma unroll
@@ -358,7 +413,7 @@ __global__ void __launch_bounds__(CH ? 2 * TTHREADS : TTHREADS)
     bool ok = true;
     // prologue: k-tiles 0 .. NST-2
     for (int s = 0; s < NST - 1; ++s) {
-        if (s < KT) load_stage<T, S, NTHR>(smem + s * STAGE, c, p, t.m0, t.n0, s, kt0);
+        if (s < KT) load_stage<T, S, NTHR>(smem + s * STAGE, c, p, t.m0, t.n0, s, kt0, b_plane);
         asm volatile("cp.async.commit_group;");
     }
     (void)STAGE;
@@ -366,7 +421,7 @@ __global__ void __launch_bounds__(CH ? 2 * TTHREADS : TTHREADS)
         const int b = kt % NST;
         if (NST == 1) {  // single buffer: reload it once the previous k-tile's MMAs are done
             if (kt >= 1) ok = ok && mbar_wait(&mbar[0], (kt - 1) & 1);
-            if (ok) load_stage<T, S, NTHR>(smem, c, p, t.m0, t.n0, kt, kt0);
+            if (ok) load_stage<T, S, NTHR>(smem, c, p, t.m0, t.n0, kt, kt0, b_plane);
             asm volatile("cp.async.commit_group;");
             asm volatile("cp.async.wait_group 0;");
         } else if (NST == 2) {
@@ -384,10 +439,18 @@ __global__ void __launch_bounds__(CH ? 2 * TTHREADS : TTHREADS)
             const int kseg = kt >= kt0 ? p.K1 : p.K0, koff = (kt >= kt0 ? kt - kt0 : kt) * TBK;
             const int nsteps = min(2, (kseg - koff + 15) / 16);
             const bool fresh = CH && (kt % chunk) == 0;  // first k-tile of a chunk
+            if constexpr (CH)
+                if (stack)
+                    for (int s16 = 0; s16 < nsteps; ++s16)
+                        stacked_products<T>(
+                            tm, p.BN, fresh && s16 == 0,
+                            [&](int q, int im) { return make_desc(base + (im * T + q) * PLANE_TILE + s16 * 256); },
+                            [&](int im) { return make_desc(base + 2 * T * PLANE_TILE + im * T * b_plane + s16 * 256); });
 #pragma unroll
             for (int s16 = 0; s16 < 2; ++s16)
 #pragma unroll
                 for (int q = 0; q < n_products<T>(); ++q) {
+                    if (CH && stack) break;
                     if (s16 >= nsteps) break;
                     const uint32_t ar = base + PI[q] * PLANE_TILE + s16 * 256;
                     const uint32_t ai = base + (T + PI[q]) * PLANE_TILE + s16 * 256;
@@ -412,7 +475,7 @@ __global__ void __launch_bounds__(CH ? 2 * TTHREADS : TTHREADS)
             const int nk = kt + NST - 1;
             if (nk < KT) {
                 if (kt >= 1) ok = ok && mbar_wait(&mbar[(kt - 1) % NST], ((kt - 1) / NST) & 1);
-                if (ok) load_stage<T, S, NTHR>(smem + (nk % NST) * STAGE, c, p, t.m0, t.n0, nk, kt0);
+                if (ok) load_stage<T, S, NTHR>(smem + (nk % NST) * STAGE, c, p, t.m0, t.n0, nk, kt0, b_plane);
             }
             asm volatile("cp.async.commit_group;");
         }
@@ -423,7 +486,10 @@ __global__ void __launch_bounds__(CH ? 2 * TTHREADS : TTHREADS)
                 ok = mbar_wait(&mbar[b], (kt / NST) & 1) && ok;
                 ok = __syncthreads_and(ok);
                 asm volatile("tcgen05.fence::after_thread_sync;");
-                if (ok) drain_add(accr, acci, tm + q_lanes, cofs, q_col, p.BN);
+                if (ok) {
+                    if (stack) drain_stacked<T>(accr, acci, tm + q_lanes, p.BN, q_col, q_cols);
+                    else drain_add(accr, acci, tm + q_lanes, cofs, q_col, p.BN);
+                }
                 asm volatile("tcgen05.fence::before_thread_sync;");
             }
         }
@@ -438,14 +504,19 @@ __global__ void __launch_bounds__(CH ? 2 * TTHREADS : TTHREADS)
         if (tid == 0) atomicAdd(c.err, 1);
     } else if constexpr (CH) {
         // the last chunk and the correction products, then the outputs from registers
-        drain_add(accr, acci, tm + q_lanes, cofs, q_col, p.BN);
-        drain_add(accr, acci, tm + q_lanes + 2 * cofs, cofs, q_col, p.BN);
+        if (stack) {
+            drain_stacked<T>(accr, acci, tm + q_lanes, p.BN, q_col, q_cols);
+        } else {
+            drain_add(accr, acci, tm + q_lanes, cofs, q_col, p.BN);
+            drain_add(accr, acci, tm + q_lanes + 2 * cofs, cofs, q_col, p.BN);
+        }
         const int row = t.m0 + (warp & 3) * 32 + lane;
         if (row < p.M) {
 #pragma unroll
             for (int jj = 0; jj < 64; ++jj) {
                 const int cc = q_col + jj, col = t.n0 + cc;
-                if (cc < p.BN && col < p.N) epilogue<T, S>(c, p, row, col, make_float2(accr[jj], acci[jj]));
+                if (jj < q_cols && cc < p.BN && col < p.N)
+                    epilogue<T, S>(c, p, row, col, make_float2(accr[jj], acci[jj]));
             }
         }
     } else {
@@ -591,176 +662,272 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 }
 
 // ------------------------------------------- stage kernel with a TMA-fed ring
-// The long-K stages (AG1, AG2, DG2, DG3) as tc_gemm_kernel<T, S, true>, the same MMAs in
-// the same order and the same chunked accumulation, but with the operands fed by the
-// tensor-memory accelerator: one thread keeps `nst` K steps of 16 in flight (two 3-D
-// boxes of 8 K x rows x 2T planes per operand and K step, zero-filled past the matrix
-// edges by the copy engine), issues the MMAs of a K step as soon as its bytes have
-// arrived and refills the stage of the previous K step once those MMAs are done; the
-// other threads only take part in the chunk drains and the epilogue.  A box lands in
-// shared memory as [8-element K chunk][plane][row][8 elements], i.e. 8 x 16-byte core
-// matrices with the next 8 rows 128 bytes on and the next K chunk one box on, which is
-// what the MMA descriptors below describe.
+// The long-K stages (AG1, AG2, DG2, DG3): the MMAs of tc_gemm_kernel<T, S, true> in the order that
+// gives the same bits, by a persistent CTA per SM whose warps have a task each:
+//   producer   keeps `nst` k-tiles of 32 in flight, two 3-D TMA boxes (32 K x rows x 2T planes)
+//              each, zero-filled past the matrix edges by the copy engine;
+//   MMA warp   issues a k-tile's products when its bytes have arrived;
+//   8 drain warps add a chunk's accumulator into FP32 registers (lane quarter w & 3, half of the
+//              columns each) and write a finished tile's outputs while the next one is multiplied.
+// Boxes land as rows of 64 bytes in the 64-byte swizzle, atoms of 8 rows (512 bytes).  An earlier
+// form took boxes of 8 K (the no-swizzle core matrices): the copy engine works row by row, and its
+// 16-byte rows held a K step of 16 to 4100 cycles at 16 columns, against 1368 for its MMAs.
+// `stack` runs the stacked products, whose accumulator has room for `nset` = 2 copies when
+// 4 T BN <= 512 columns: a chunk goes to one while the other drains.  Otherwise the corrections of
+// a chunk's first K step, which have columns of their own, run while the last chunk's leading
+// products drain.
 constexpr int NST_TMA_MAX = 8;
+constexpr int TMA_DRAIN = 2 * TTHREADS;           // drain threads
+constexpr int TMA_THREADS = TMA_DRAIN + 64;       // + producer warp + MMA warp
 
-__device__ __forceinline__ uint64_t make_desc_lbo(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+// 64-byte swizzle, K-major: 8-row groups 512 bytes apart (the leading offset is unused)
+__device__ __forceinline__ uint64_t make_desc_sw64(uint32_t addr) {
     uint64_t d = 0;
     d |= (uint64_t)((addr >> 4) & 0x3FFF);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;   // next core matrix along K
-    d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;   // next 8-row group
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(512 >> 4) << 32;
     d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;
     return d;
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
 
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
-            "r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
+            "r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
         : "memory");
 }
 
+// Outputs of a finished tile from the drain warps' registers: this thread's row, q_cols columns
+// from q_col.  Every stage's output element (i, j) lies at base(i) + j step.  The BF16 outputs go
+// in pairs of neighbouring rows, neighbours in memory too (for AG2 because its rows b + r_p a run
+// over an even number of b): two lanes swap a column, so that each splits and stores both rows of
+// one column, 4 bytes a plane; rows past M are the zeros of the planes' padding.  With a
+// 2-byte store per element and plane and 64-bit addresses each, the unrolled epilogue was 50 KB of
+// instructions and most of AG2's time (10-lambda sphere, 37 columns: 272 -> 162 us).
 template <int T, int S>
-__global__ void __launch_bounds__(2 * TTHREADS)
+__device__ __forceinline__ void store_tile(const TcCtx& c, const TcProb& p, int row, int n0, int q_col, int q_cols,
+                                           const float (&re)[64], const float (&im)[64]) {
+    const int ncol = min(min(q_cols, p.BN - q_col), p.N - n0 - q_col), j0 = n0 + q_col;
+    if constexpr (S == TDG3) {  // conj(v) in group order
+        if (row < p.M) {
+            float2* o = c.ybuf + p.rwg + row + (int64_t)j0 * c.N;
+#pragma unroll
+            for (int jj = 0; jj < 64; ++jj)
+                if (jj < ncol) o[(int64_t)jj * c.N] = make_float2(re[jj], -im[jj]);
+        }
+    } else {
+        const int odd = row & 1, i = row & ~1;
+        uint32_t base, step;
+        if (S == TAG2) {  // M' [a + r_t r][b], i = b + r_p a
+            const int rp = p.M / p.rt, a = i / rp;
+            base = (uint32_t)(a * p.o_ld + (i - rp * a));
+            step = (uint32_t)(p.rt * p.o_ld);
+        } else {  // AG1: T [r][c], DG2: S [r][c]
+            base = (uint32_t)i;
+            step = (uint32_t)p.o_ld;
+        }
+        base += (uint32_t)(j0 + odd) * step;
+        uint32_t* plane[2 * T];
+#pragma unroll
+        for (int q = 0; q < 2 * T; ++q) plane[q] = reinterpret_cast<uint32_t*>(reinterpret_cast<bf16*>(p.out) + q * p.o_ps);
+#pragma unroll
+        for (int jj = 0; jj < 64; jj += 2) {
+            const float xr = __shfl_xor_sync(0xffffffffu, odd ? re[jj] : re[jj + 1], 1);
+            const float xi = __shfl_xor_sync(0xffffffffu, odd ? im[jj] : im[jj + 1], 1);
+            uint32_t wr[3], wi[3];
+            split_pack<T>(odd ? xr : re[jj], odd ? re[jj + 1] : xr, wr);
+            split_pack<T>(odd ? xi : im[jj], odd ? im[jj + 1] : xi, wi);
+            if (i < p.M && jj + odd < ncol) {
+                const uint32_t e = (base + (uint32_t)jj * step) >> 1;
+#pragma unroll
+                for (int q = 0; q < T; ++q) {
+                    plane[q][e] = wr[q];
+                    plane[T + q][e] = wi[q];
+                }
+            }
+        }
+    }
+}
+
+template <int T, int S>
+__global__ void __launch_bounds__(TMA_THREADS, 1)
     tc_gemm_tma_kernel(const TcCtx c, const TcProb* __restrict__ probs, const CUtensorMap* __restrict__ maps,
-                       const MrTile* __restrict__ tiles, int nst, int tcols, int cofs, int chunk) {
-    extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ __align__(8) uint64_t full[NST_TMA_MAX], empty[NST_TMA_MAX];
+                       const MrTile* __restrict__ tiles, int n_tiles, int nst, int tcols, int cofs, int chunk,
+                       int stack, int nset) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full[NST_TMA_MAX], empty[NST_TMA_MAX], chunk_full[2], drained[2], fin;
     __shared__ uint32_t tmem_base;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const MrTile t = tiles[blockIdx.x];
-    const TcProb p = probs[t.prob];
-    const CUtensorMap* mp = maps + 4 * (int64_t)t.prob;  // A0, B0, A1, B1
-    const int BN = p.BN;
-    const int abox = 8 * TBM * 2 * T * 2, bbox = 8 * BN * 2 * T * 2;
-    const int stage_bytes = 2 * abox + 2 * bbox;  // one K step of 16
+    const uint32_t ring = (smem_u32(smem_raw) + 1023) & ~1023u;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
                      "r"(tcols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    if (tid == 0)
+    if (tid == 0) {
+        auto init = [](uint64_t* bar, int count) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
+        };
         for (int s = 0; s < nst; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[s])), "r"(1));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&empty[s])), "r"(1));
+            init(&full[s], 1);
+            init(&empty[s], 1);
         }
+        for (int s = 0; s < 2; ++s) {
+            init(&chunk_full[s], 1);
+            init(&drained[s], TMA_DRAIN);
+        }
+        init(&fin, 1);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;");
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tm = tmem_base;
-    const int ks0 = (p.K0 + 15) / 16, kt0 = (p.K0 + 31) / 32;
-    const int KS = ks0 + (p.K1 > 0 ? (p.K1 + 15) / 16 : 0);
-    // chunks of `chunk` k-tiles of 32 as in tc_gemm_kernel (a segment's last k-tile may hold
-    // one K step), so that both kernels round alike: k-tile of a K step, and its first / last
-    auto ktile = [&](int ks) { return ks < ks0 ? ks / 2 : kt0 + (ks - ks0) / 2; };
-    auto kt_first = [&](int ks) { return ks < ks0 ? (ks % 2) == 0 : ((ks - ks0) % 2) == 0; };
-    auto kt_last = [&](int ks) { return ks + 1 == KS || ks + 1 == ks0 || ktile(ks + 1) != ktile(ks); };
-    auto produce = [&](int ks) {
-        uint8_t* base = smem + (ks % nst) * stage_bytes;
-        const bool seg1 = ks >= ks0;
-        const int koff = (seg1 ? ks - ks0 : ks) * 16;
-        const CUtensorMap* ma = mp + (seg1 ? 2 : 0);
-        const CUtensorMap* mb = mp + (seg1 ? 3 : 1);
-        uint64_t* bar = &full[ks % nst];
-        mbar_expect_tx(bar, (uint32_t)stage_bytes);
-        tma_load_3d(base, ma, koff, t.m0, 0, bar);
-        tma_load_3d(base + abox, ma, koff + 8, t.m0, 0, bar);
-        tma_load_3d(base + 2 * abox, mb, koff, t.n0, 0, bar);
-        tma_load_3d(base + 2 * abox + bbox, mb, koff + 8, t.n0, 0, bar);
-    };
-    int produced = 0, consumed = 0;
-    if (tid == 0)
-        for (; produced < min(nst, KS); ++produced) produce(produced);
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TBM >> 4) << 24);
-    const uint32_t idesc_neg = idesc | (1u << 13);
-    const uint32_t q_lanes = (uint32_t)((warp & 3) * 32) << 16;
-    const int q_col = (warp >> 2) * 64;
-    float accr[64], acci[64];
-#pragma unroll
-    for (int j = 0; j < 64; ++j) accr[j] = acci[j] = 0.f;
     bool ok = true;
-    for (int ks = 0; ks < KS; ++ks) {
-        const int st = ks % nst;
-        const uint32_t ph = (uint32_t)(ks / nst) & 1u;
-        if (tid == 0 && ok) {
-            ok = mbar_wait(&full[st], ph);
-            if (ok) {
-                consumed = ks + 1;
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const uint32_t base = smem_u32(smem + st * stage_bytes);
-                constexpr int PI[6] = {0, 0, 1, 0, 1, 2}, PJ[6] = {0, 1, 0, 2, 1, 0};
-                const bool fresh = (ktile(ks) % chunk) == 0 && kt_first(ks);  // first K step of a chunk
-#pragma unroll
-                for (int q = 0; q < n_products<T>(); ++q) {
-                    const uint64_t ar = make_desc_lbo(base + PI[q] * TBM * 16, abox, 128);
-                    const uint64_t ai = make_desc_lbo(base + (T + PI[q]) * TBM * 16, abox, 128);
-                    const uint64_t br = make_desc_lbo(base + 2 * abox + PJ[q] * BN * 16, bbox, 128);
-                    const uint64_t bi = make_desc_lbo(base + 2 * abox + (T + PJ[q]) * BN * 16, bbox, 128);
-                    // the leading product (hi x hi) restarts its accumulator every chunk; the
-                    // correction products accumulate apart over the whole K (columns 2 cofs on)
-                    const bool lo = q > 0;
-                    const uint32_t acc = lo ? ((ks > 0 || q > 1) ? 1u : 0u) : (fresh ? 0u : 1u);
-                    const uint32_t d = tm + (lo ? 2 * cofs : 0);
-                    mma_bf16(d, ar, br, idesc, acc);
-                    mma_bf16(d, ai, bi, idesc_neg, 1u);
-                    mma_bf16(d + cofs, ar, bi, idesc, acc);
-                    mma_bf16(d + cofs, ai, br, idesc, 1u);
-                }
-                mma_commit(&empty[st]);
-                // refill the stage of K step ks - 1 once its MMAs are done (those of ks keep
-                // the tensor pipe busy meanwhile)
-                if (ks >= 1 && produced < KS) {
-                    ok = mbar_wait(&empty[(ks - 1) % nst], (uint32_t)((ks - 1) / nst) & 1u);
-                    if (ok) produce(produced++);
+    // every role walks the same tiles; k-tiles (`it`) and chunks (`cc`) count over all of them
+    if (warp == TMA_DRAIN / 32) {
+        // ---- producer
+        if (lane == 0) {
+            int it = 0;
+            for (int ti = blockIdx.x; ok && ti < n_tiles; ti += gridDim.x) {
+                const MrTile t = tiles[ti];
+                const TcProb& p = probs[t.prob];
+                const CUtensorMap* mp = maps + 4 * (int64_t)t.prob;  // A0, B0, A1, B1
+                const int kt0 = (p.K0 + 31) / 32, KT = kt0 + (p.K1 + 31) / 32;
+                const uint32_t a_bytes = 64 * TBM * 2 * T, bytes = a_bytes + 64 * (uint32_t)p.BN * 2 * T;
+                for (int kt = 0; kt < KT; ++kt, ++it) {
+                    const int st = it % nst;
+                    if (it >= nst) ok = mbar_wait(&empty[st], (uint32_t)(it / nst - 1) & 1u);
+                    if (!ok) break;
+                    const bool seg1 = kt >= kt0;
+                    const int koff = (seg1 ? kt - kt0 : kt) * 32;
+                    const uint32_t base = ring + st * bytes;
+                    mbar_expect_tx(&full[st], bytes);
+                    tma_load_3d(base, mp + (seg1 ? 2 : 0), koff, t.m0, 0, &full[st]);
+                    tma_load_3d(base + a_bytes, mp + (seg1 ? 3 : 1), koff, t.n0, 0, &full[st]);
                 }
             }
+            for (int k = max(0, it - nst); k < it; ++k)  // copies in flight land before the CTA exits
+                ok = mbar_wait(&full[k % nst], (uint32_t)(k / nst) & 1u) && ok;
         }
-        if (kt_last(ks) && (ktile(ks) % chunk) == chunk - 1 && ks + 1 < KS) {
-            // end of a chunk: once its MMAs are done, add the leading-product accumulator
-            // into the registers; the next K step restarts it
-            ok = mbar_wait(&empty[st], ph) && ok;
-            ok = __syncthreads_and(ok);
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            if (ok) drain_add(accr, acci, tm + q_lanes, cofs, q_col, BN);
-            asm volatile("tcgen05.fence::before_thread_sync;");
-            __syncthreads();
+        __syncwarp();
+    } else if (warp == TMA_DRAIN / 32 + 1) {
+        // ---- MMA warp
+        if (lane == 0) {
+            int it = 0, cc = 0;
+            for (int ti = blockIdx.x; ok && ti < n_tiles; ti += gridDim.x) {
+                const TcProb& p = probs[tiles[ti].prob];
+                const int BN = p.BN, K0 = p.K0, K1 = p.K1, kt0 = (K0 + 31) / 32, KT = kt0 + (K1 + 31) / 32;
+                const uint32_t a_plane = 64 * TBM, b_plane = 64 * (uint32_t)BN, bytes = 2 * T * (a_plane + b_plane);
+                const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
+                                       ((uint32_t)(TBM >> 4) << 24);
+                const uint32_t idesc_neg = idesc | (1u << 13);
+                for (int kt = 0; kt < KT; ++kt, ++it) {
+                    const int st = it % nst, set = cc % nset;
+                    const bool first = kt % chunk == 0, last = kt % chunk == chunk - 1 || kt + 1 == KT;
+                    const bool free_set = !first || cc < nset;
+                    auto wait_set = [&] {  // the set's previous chunk has been added up
+                        const bool w = free_set || mbar_wait(&drained[set], (uint32_t)(cc / nset - 1) & 1u);
+                        asm volatile("tcgen05.fence::after_thread_sync;");
+                        return w;
+                    };
+                    ok = mbar_wait(&full[st], (uint32_t)(it / nst) & 1u);
+                    if (ok && (stack || kt == 0)) ok = wait_set();  // a new tile restarts the corrections too
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint32_t A = ring + st * bytes, B = A + 2 * T * a_plane;
+                    const int kseg = kt >= kt0 ? K1 - (kt - kt0) * 32 : K0 - kt * 32, nsteps = kseg > 16 ? 2 : 1;
+                    for (int s16 = 0; s16 < nsteps; ++s16) {
+                        if (stack) {
+                            stacked_products<T>(
+                                tm + set * (2 * T * BN), BN, first && s16 == 0,
+                                [&](int q, int im) { return make_desc_sw64(A + (im * T + q) * a_plane + s16 * 32); },
+                                [&](int im) { return make_desc_sw64(B + im * T * b_plane + s16 * 32); });
+                            continue;
+                        }
+                        constexpr int PI[6] = {0, 0, 1, 0, 1, 2}, PJ[6] = {0, 1, 0, 2, 1, 0};
+#pragma unroll
+                        for (int i = 0; i < n_products<T>(); ++i) {
+                            // corrections first (over the whole K, columns 2 cofs on), the leading product
+                            // (restarting with the chunk) last
+                            const int q = i + 1 < n_products<T>() ? i + 1 : 0;
+                            if (q == 0 && s16 == 0 && first && kt > 0) ok = wait_set();
+                            if (!ok) break;
+                            const uint64_t ar = make_desc_sw64(A + PI[q] * a_plane + s16 * 32);
+                            const uint64_t ai = make_desc_sw64(A + (T + PI[q]) * a_plane + s16 * 32);
+                            const uint64_t br = make_desc_sw64(B + PJ[q] * b_plane + s16 * 32);
+                            const uint64_t bi = make_desc_sw64(B + (T + PJ[q]) * b_plane + s16 * 32);
+                            const uint32_t acc = q > 0 ? ((kt > 0 || s16 > 0 || q > 1) ? 1u : 0u)
+                                                       : ((first && s16 == 0) ? 0u : 1u);
+                            const uint32_t d = tm + (q > 0 ? 2 * cofs : 0);
+                            mma_bf16(d, ar, br, idesc, acc);
+                            mma_bf16(d, ai, bi, idesc_neg, 1u);
+                            mma_bf16(d + cofs, ar, bi, idesc, acc);
+                            mma_bf16(d + cofs, ai, br, idesc, 1u);
+                        }
+                    }
+                    mma_commit(&empty[st]);
+                    if (last) {
+                        mma_commit(&chunk_full[set]);
+                        ++cc;
+                    }
+                    if (!ok) break;
+                }
+            }
+            mma_commit(&fin);  // no MMA may still use TMEM when it is freed
+            ok = mbar_wait(&fin, 0) && ok;
         }
-    }
-    // always wait (bounded) for the last commit: no MMA may still read TMEM when it is freed
-    if (KS > 0 && !mbar_wait(&empty[(KS - 1) % nst], (uint32_t)((KS - 1) / nst) & 1u)) ok = false;
-    if (tid == 0)  // copies still in flight after a wait gave up land before the CTA exits
-        for (int ks = consumed; ks < produced; ++ks) mbar_wait(&full[ks % nst], (uint32_t)(ks / nst) & 1u);
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    ok = __syncthreads_and(ok);
-    if (!ok) {
-        if (tid == 0) atomicAdd(c.err, 1);
+        __syncwarp();
     } else {
-        drain_add(accr, acci, tm + q_lanes, cofs, q_col, BN);
-        drain_add(accr, acci, tm + q_lanes + 2 * cofs, cofs, q_col, BN);
-        const int row = t.m0 + (warp & 3) * 32 + lane;
-        if (row < p.M) {
+        // ---- drain warps
+        const uint32_t q_lanes = (uint32_t)((warp & 3) * 32) << 16;
+        int cc = 0;
+        for (int ti = blockIdx.x; ok && ti < n_tiles; ti += gridDim.x) {
+            const MrTile t = tiles[ti];
+            const TcProb p = probs[t.prob];
+            const int BN = p.BN, KT = (p.K0 + 31) / 32 + (p.K1 + 31) / 32;
+            const int q_cols = stack ? BN / 2 : 64, q_col = (warp >> 2) * q_cols;
+            float accr[64], acci[64];
 #pragma unroll
-            for (int jj = 0; jj < 64; ++jj) {
-                const int cc = q_col + jj, col = t.n0 + cc;
-                if (cc < BN && col < p.N) epilogue<T, S>(c, p, row, col, make_float2(accr[jj], acci[jj]));
+            for (int j = 0; j < 64; ++j) accr[j] = acci[j] = 0.f;
+            for (int kt = 0; kt < KT; kt += chunk, ++cc) {
+                const int set = cc % nset;
+                ok = __all_sync(0xffffffffu, mbar_wait(&chunk_full[set], (uint32_t)(cc / nset) & 1u));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                if (stack) {
+                    drain_stacked<T>(accr, acci, tm + set * (2 * T * BN) + q_lanes, BN, q_col, q_cols);
+                } else {
+                    drain_add(accr, acci, tm + q_lanes, cofs, q_col, BN);
+                    if (kt + chunk >= KT) drain_add(accr, acci, tm + q_lanes + 2 * cofs, cofs, q_col, BN);
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;");
+                mbar_arrive(&drained[set]);
+                if (KT - kt <= chunk) {
+                    ++cc;
+                    break;
+                }
             }
+            if (ok) store_tile<T, S>(c, p, t.m0 + (warp & 3) * 32 + lane, t.n0, q_col, q_cols, accr, acci);
         }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
+    const int bad = __syncthreads_or(ok ? 0 : 1);
+    if (bad && tid == 0) atomicAdd(c.err, 1);
+    asm volatile("tcgen05.fence::after_thread_sync;");
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm), "r"(tcols));
 }
 
 constexpr int F34_WORKERS = 512;               // 16 warps, four per TMEM lane quarter
 constexpr int F34_THREADS = F34_WORKERS + 32;  // and one warp that only issues MMAs
-
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 
 __device__ __forceinline__ void workers_sync() {
     asm volatile("bar.sync 1, %0;" ::"n"(F34_WORKERS) : "memory");
@@ -1363,13 +1530,15 @@ __global__ void __launch_bounds__(CAT_THREADS) tc_cat_kernel(const TcCtx c, cons
 // Split planes of an FP32 complex matrix: dst[p][r][k] for r < rows, k < cols,
 // src element (r, k) at src[r * sr + k * sk]; entries k in [cols, ld) stay as they are.
 // inner > 0: row r of the planes is source row (r / inner) + outer (r % inner) (the rows
-// of C_(3)^T, index a + r_t b, taken in the order b + r_p a).
+// of C_(3)^T, index a + r_t b, taken in the order b + r_p a); rows with r % inner >= inner_valid
+// (r_p rounded up to even) stay zero.
 template <int T>
 __global__ void planes_kernel(const float2* __restrict__ src, int rows, int cols, int64_t sr, int64_t sk,
-                              bf16* __restrict__ dst, int64_t ld, int64_t ps, int inner, int outer) {
+                              bf16* __restrict__ dst, int64_t ld, int64_t ps, int inner, int outer, int inner_valid) {
     const int64_t total = (int64_t)rows * cols;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int r = (int)(e / cols), k = (int)(e % cols);
+        if (inner > 0 && r % inner >= inner_valid) continue;
         const int rs = inner > 0 ? r / inner + outer * (r % inner) : r;
         store_planes<T>(dst, ps, (int64_t)r * ld + k, src[(int64_t)rs * sr + (int64_t)k * sk]);
     }
@@ -1516,44 +1685,50 @@ int tc_chunk_ktiles() {
 // Stages whose K is longer than one chunk (AG1, AG2, DG1b, DG2, DG3) run the chunked
 // accumulation.
 template <int T, int S>
-void launch_tc(const TcStagePlan& st, const TcCtx& c, cudaStream_t s) {
+void launch_tc(const TcStagePlan& st, const TcCtx& c, int sms, cudaStream_t s) {
     if (st.n_tiles == 0) return;
     constexpr int NST_MAX = (T == 2) ? 3 : 2;
     constexpr size_t STAGE = (size_t)2 * 2 * T * PLANE_TILE;
     const int nst = std::max(1, std::min(NST_MAX, st.max_kt));
     const int cofs = (st.max_bn + 31) / 32 * 32;
-    const int hsplit = tc_split_accumulators() ? 1 : 0;
+    const int hsplit = tc_split_accumulators() ? 1 : 0, chunk = tc_chunk_ktiles();
     int tcols = 32;
     while (tcols < (hsplit ? 4 : 2) * cofs) tcols *= 2;
+    // the stacked products when their widest MMA and their accumulator's levels fit (81 columns and
+    // more run the products one by one: their MMAs are at rate anyway)
+    constexpr bool kLong = S == TAG1 || S == TAG2 || S == TDG2 || S == TDG3;
+    const int stack = kLong && hsplit && chunk > 0 && T * st.max_bn <= 256 && 2 * T * st.max_bn <= 512;
+    int scols = 32;
+    while (scols < 2 * T * st.max_bn) scols *= 2;
+    if (stack && !st.d_maps) tcols = std::max(tcols, scols);
     // at most 512 / tcols CTAs per SM: pad the shared memory request so that no more fit
     const int ctas_tmem = 512 / tcols;
     constexpr size_t kSmemSM = 228 * 1024, kMaxDyn = 225 * 1024;
     size_t smem = nst * STAGE;
     if (kSmemSM / (smem + 2048) > (size_t)ctas_tmem) smem = std::min(kMaxDyn, kSmemSM / ctas_tmem - 2048);
-    const int chunk = tc_chunk_ktiles();
     const TcProb* probs = reinterpret_cast<const TcProb*>(st.d_probs);
     if (st.d_maps && hsplit) {
-        // TMA-fed ring of K steps of 16: as many stages as fit next to nothing else
-        const size_t stage = (size_t)2 * 8 * 2 * T * 2 * (TBM + st.max_bn);
-        const int nst_tma = (int)std::min<size_t>(NST_TMA_MAX, kMaxDyn / stage);
+        const size_t stage = (size_t)64 * 2 * T * (TBM + st.max_bn);
+        const int nst_tma = (int)std::min<size_t>(NST_TMA_MAX, (kMaxDyn - 1024) / stage);
+        const int nset = stack && 2 * scols <= 512 ? 2 : 1;
         allow_dyn_smem(reinterpret_cast<const void*>(tc_gemm_tma_kernel<T, S>), kMaxDyn);
-        tc_gemm_tma_kernel<T, S><<<st.n_tiles, 2 * TTHREADS, nst_tma * stage, s>>>(
-            c, probs, static_cast<const CUtensorMap*>(st.d_maps), st.d_tiles, nst_tma, tcols, cofs,
-            chunk > 0 ? chunk : 1 << 30);
+        tc_gemm_tma_kernel<T, S><<<std::min(st.n_tiles, sms), TMA_THREADS, nst_tma * stage + 1024, s>>>(
+            c, probs, static_cast<const CUtensorMap*>(st.d_maps), st.d_tiles, st.n_tiles, nst_tma,
+            stack ? nset * scols : tcols, cofs, chunk > 0 ? chunk : 1 << 30, stack, nset);
         TFMM_CUDA_CHECK(cudaGetLastError());
         return;
     }
     if constexpr (S == TAG1 || S == TAG2 || S == TDG1B || S == TDG2 || S == TDG3) {
-        if (hsplit && chunk > 0 && st.max_kt > chunk) {
+        if (hsplit && chunk > 0 && (st.max_kt > chunk || stack)) {
             allow_dyn_smem(reinterpret_cast<const void*>(tc_gemm_kernel<T, S, true>), kMaxDyn);
-            tc_gemm_kernel<T, S, true><<<st.n_tiles, 2 * TTHREADS, smem, s>>>(c, probs, st.d_tiles, nst, tcols, cofs,
-                                                                             hsplit, chunk);
+            tc_gemm_kernel<T, S, true><<<st.n_tiles, 2 * TTHREADS, smem, s>>>(
+                c, probs, st.d_tiles, nst, tcols, cofs, hsplit, chunk, stack);
             TFMM_CUDA_CHECK(cudaGetLastError());
             return;
         }
     }
     allow_dyn_smem(reinterpret_cast<const void*>(tc_gemm_kernel<T, S, false>), kMaxDyn);
-    tc_gemm_kernel<T, S, false><<<st.n_tiles, TTHREADS, smem, s>>>(c, probs, st.d_tiles, nst, tcols, cofs, hsplit, 1);
+    tc_gemm_kernel<T, S, false><<<st.n_tiles, TTHREADS, smem, s>>>(c, probs, st.d_tiles, nst, tcols, cofs, hsplit, 1, 0);
     TFMM_CUDA_CHECK(cudaGetLastError());
 }
 
@@ -1590,7 +1765,7 @@ void build_tc_factors(Plan& P, int T, cudaStream_t s) {
         const int m = d.rt * d.rp;
         add(t.ubT, d.rb, d.n_beta);   // [c][n]
         add(t.ub, d.n_beta, d.rb);    // [n][c]
-        add(t.c3T, m, d.rb);          // [ab][c], rows in the order b + r_p a
+        add(t.c3T, d.rt * ((d.rp + 1) & ~1), d.rb);  // [ab][c], rows in the order b + r_p a, r_p rounded up to even
         add(t.c3, d.rb, m);           // [c][ab]
         add(t.uphT, np, d.rp);        // [i_phi][b]
         add(t.uph, d.rp, np);         // [b][i_phi]
@@ -1601,14 +1776,14 @@ void build_tc_factors(Plan& P, int T, cudaStream_t s) {
     TFMM_CUDA_CHECK(cudaMemsetAsync(P.tc_fac[T].p, 0, sizeof(bf16) * std::max<int64_t>(off, 1), s));
     bf16* base = reinterpret_cast<bf16*>(P.tc_fac[T].p);
     auto conv = [&](const float2* src, int rows, int cols, int64_t sr, int64_t sk, const TcMat& m, int inner = 0,
-                    int outer = 0) {
+                    int outer = 0, int inner_valid = 0) {
         const int64_t ps = (int64_t)m.rows * m.ld;
         if (T == 2)
             planes_kernel<2><<<g1d((int64_t)rows * cols), 256, 0, s>>>(src, rows, cols, sr, sk, base + m.off, m.ld, ps,
-                                                                       inner, outer);
+                                                                       inner, outer, inner_valid);
         else
             planes_kernel<3><<<g1d((int64_t)rows * cols), 256, 0, s>>>(src, rows, cols, sr, sk, base + m.off, m.ld, ps,
-                                                                       inner, outer);
+                                                                       inner, outer, inner_valid);
     };
     for (size_t q = 0; q < P.items.size(); ++q) {
         const TuckerItem& d = P.items[q];
@@ -1620,7 +1795,8 @@ void build_tc_factors(Plan& P, int T, cudaStream_t s) {
         const float2* ut = P.d_factors + d.uth;     // U_theta:       (i_theta, a) at i_theta + n_theta a
         conv(ub, d.rb, d.n_beta, d.ld_nb, 1, t.ubT);
         conv(ub, d.n_beta, d.rb, 1, d.ld_nb, t.ub);
-        conv(cc, m, d.rb, 1, d.ld_ab, t.c3T, d.rp, d.rt);  // rows b + r_p a: AG2 writes M' in runs of b
+        const int rpe = (d.rp + 1) & ~1;
+        conv(cc, d.rt * rpe, d.rb, 1, d.ld_ab, t.c3T, rpe, d.rt, d.rp);  // rows b + r_p a: AG2 writes M' in runs of b
         conv(cc, d.rb, m, d.ld_ab, 1, t.c3);
         conv(up, np, d.rp, 1, np, t.uphT);
         conv(up, d.rp, np, np, 1, t.uph);
@@ -1658,8 +1834,8 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     return fn;
 }
 
-// 3-D map of the 2T planes of a K-major matrix (K x rows x planes, boxes of 8 K x
-// box_rows x 2T); false when the layout breaks a rule of the copy engine.
+// 3-D map of the 2T planes of a K-major matrix (K x rows x planes, boxes of 32 K x
+// box_rows x 2T, 64-byte swizzle); false when the layout breaks a rule of the copy engine.
 bool encode_planes(CUtensorMap* m, const bf16* base, int64_t K, int64_t rows, int64_t ld, int64_t ps, int T,
                    int box_rows) {
     const auto fn = tensor_map_encoder();
@@ -1668,10 +1844,10 @@ bool encode_planes(CUtensorMap* m, const bf16* base, int64_t K, int64_t rows, in
         return false;
     cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)(2 * T)};
     cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)ps * 2};
-    cuuint32_t box[3] = {8, (cuuint32_t)box_rows, (cuuint32_t)(2 * T)};
+    cuuint32_t box[3] = {32, (cuuint32_t)box_rows, (cuuint32_t)(2 * T)};
     cuuint32_t es[3] = {1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16*>(base), dims, strides, box, es,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -1998,7 +2174,7 @@ TcPlan* get_tc_plan(Plan& P, int R, int T, cudaStream_t s) {
         add_tc_tiles(tl[TAG1], (int)pr[TAG1].size(), p.M, p.N); pr[TAG1].push_back(p);
         // AG2: M = C_(3)^T T ; out M' planes [a + r_t r][b]
         p = b;
-        p.M = m; p.N = R; p.K0 = d.rb; p.BN = bn_of(R);
+        p.M = d.rt * ((d.rp + 1) & ~1); p.N = R; p.K0 = d.rb; p.BN = bn_of(R);
         mat(f.c3T, p.A0, p.a_ld0, p.a_ps0);
         p.B0 = Tb + o.t; p.b_ld0 = o.ldt; p.b_ps0 = (int64_t)R * o.ldt;
         p.out = Mb + o.m; p.o_ld = r8(d.rp); p.o_ps = (int64_t)d.rt * R * r8(d.rp);
@@ -2053,6 +2229,10 @@ TcPlan* get_tc_plan(Plan& P, int R, int T, cudaStream_t s) {
         add_tc_tiles(tl[TDG3], (int)pr[TDG3].size(), p.M, p.N); pr[TDG3].push_back(p);
     }
     for (int st = 0; st < 8; ++st) {
+        // longest K first: the persistent CTAs of the TMA-fed stages take every sms-th tile
+        std::stable_sort(tl[st].begin(), tl[st].end(), [&](const MrTile& x, const MrTile& y) {
+            return pr[st][x.prob].K0 + pr[st][x.prob].K1 > pr[st][y.prob].K0 + pr[st][y.prob].K1;
+        });
         upload_tc_stage(M.st[st], pr[st], tl[st]);
         if (st == TAG1 || st == TAG2 || st == TDG2 || st == TDG3) build_stage_maps(M.st[st], pr[st], T);
     }
@@ -2114,13 +2294,13 @@ void tc_aggregate_t(Plan& P, TcPlan& M, const float2* x, int R, int64_t ldx, flo
     prep_x_kernel<T><<<gx, kXTile / 2, 0, s>>>(x, ldx, P.d_grp_rwg, reinterpret_cast<const TcProb*>(M.st[TAG1].d_probs),
                                                static_cast<const MrTile*>(M.x_tiles.p), R);
     TFMM_CUDA_CHECK(cudaGetLastError());
-    launch_tc<T, TAG1>(M.st[TAG1], c, s);
-    launch_tc<T, TAG2>(M.st[TAG2], c, s);
+    launch_tc<T, TAG1>(M.st[TAG1], c, P.num_sms, s);
+    launch_tc<T, TAG2>(M.st[TAG2], c, P.num_sms, s);
     if (M.fused34) {
         launch_ag34<T>(P, M, c, s);
     } else {
-        launch_tc<T, TAG3>(M.st[TAG3], c, s);
-        launch_tc<T, TAG4>(M.st[TAG4], c, s);
+        launch_tc<T, TAG3>(M.st[TAG3], c, P.num_sms, s);
+        launch_tc<T, TAG4>(M.st[TAG4], c, P.num_sms, s);
     }
 }
 
@@ -2144,15 +2324,15 @@ void tc_disaggregate_t(Plan& P, TcPlan& M, const float2* spec, int R, int weight
     else if (M.dg1a)
         launch_dg1a<T>(P, M, c, s);
     else
-        launch_tc<T, TDG1A>(M.st[TDG1A], c, s);
+        launch_tc<T, TDG1A>(M.st[TDG1A], c, P.num_sms, s);
     if (M.cat1b.on)
         launch_cat<T, CAT_DG1B>(P, M.cat1b, c, s);
     else
-        launch_tc<T, TDG1B>(M.st[TDG1B], c, s);
-    launch_tc<T, TDG2>(M.st[TDG2], c, s);
+        launch_tc<T, TDG1B>(M.st[TDG1B], c, P.num_sms, s);
+    launch_tc<T, TDG2>(M.st[TDG2], c, P.num_sms, s);
     c.ybuf = static_cast<float2*>(M.ybuf.p);
     c.N = P.N;
-    launch_tc<T, TDG3>(M.st[TDG3], c, s);
+    launch_tc<T, TDG3>(M.st[TDG3], c, P.num_sms, s);
     const dim3 gy((unsigned)((P.N + 255) / 256), (R + kXCols - 1) / kXCols);
     order_y_kernel<<<gy, 256, 0, s>>>(c.ybuf, static_cast<const int*>(M.y_pos.p), P.N, R, beta, y, ldy);
     TFMM_CUDA_CHECK(cudaGetLastError());

@@ -171,3 +171,13 @@ def test_small_groups_by_size_class(R):
     nbetas = [int(n) for n in rng.integers(2, 40, G)]
     ranks = [_small_ranks(rng, 4, 8, nb, 12) for nb in nbetas]
     _check(3700 + R, 4, 8, nbetas, ranks, R, 0, 1e-5, betas=(0.5 - 0.25j,))
+
+
+@pytest.mark.parametrize("R", [16, 17, 40, 48, 80, 81, 129])
+def test_stage_kernel_forms(R):
+    """Stacked products with two accumulator copies, one, and products one by one; a second column tile;
+    K of one step, one and two k-tiles, odd r_phi, rows around 128."""
+    nbetas = [15, 33, 64, 127, 129, 300]
+    ranks = [[(5, 7, 15), (3, 5, 14)], [(8, 16, 33), (1, 1, 1)], [(9, 13, 64), (6, 3, 31)],
+             [(12, 11, 127), (12, 10, 96)], [(12, 22, 129), (2, 2, 4)], [(11, 19, 200), (10, 20, 128)]]
+    _check(4000 + R, 12, 24, nbetas, ranks, R, 3, 1e-6, betas=(0.5 - 0.25j,))
