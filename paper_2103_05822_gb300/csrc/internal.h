@@ -163,6 +163,14 @@ struct CatPlan {
     DeviceBuffer items, tiles;
 };
 
+// DG1a and DG1b in one kernel (tc_dg1_kernel)
+struct Dg1Plan {
+    bool on = false;
+    int PC = 0, NS = 0, K1 = 0, KP = 0, n8max = 0, n16max = 0, w_smem = 0, tcols = 0, n_units = 0;
+    size_t smem = 0;
+    DeviceBuffer items, units;
+};
+
 struct TcPlan {             // per (R, terms): problem lists of the 8 steps and scratch planes
     int R = 0, T = 0;
     TcStagePlan st[8];
@@ -177,6 +185,7 @@ struct TcPlan {             // per (R, terms): problem lists of the 8 steps and 
     int dg1a_K = 0, dg1a_NP = 0, dg1a_AR = 0, dg1a_ntiles = 0;
     size_t dg1a_smem = 0;
     DeviceBuffer dg1a_items, dg1a_tiles;
+    Dg1Plan dg1;            // both DG1 factors at once, when they fit
     CatPlan cat1a, cat1b;   // the stacked-term forms of DG1a / DG1b, when they fit
     DeviceBuffer x_tiles;   // prep_x work list
     int n_xtiles = 0;

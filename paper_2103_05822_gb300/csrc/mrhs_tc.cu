@@ -117,6 +117,37 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t ad, uint64_t bd
         "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
 }
 
+// The same for a warp that runs its loop convergently and lets one lane (`lead`) issue: descriptors
+// as two words, of which only the low one (address >> 4, leading offset) moves.  The instruction
+// takes its operands from uniform registers; computed by a lone thread in a divergent branch
+// they were moved there one by one, with the full descriptor rebuilt each time, which held
+// the issue to 120-160 cycles an MMA (66 at N = 128 by the tensor pipe).
+struct Desc {
+    uint32_t lo, hi;
+};
+__device__ __forceinline__ Desc desc_words(uint64_t d) { return Desc{(uint32_t)d, (uint32_t)(d >> 32)}; }
+__device__ __forceinline__ void mma_lead(uint32_t lead, uint32_t tmem, uint32_t alo, uint32_t ahi, uint32_t blo,
+                                         uint32_t bhi, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\tmov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+        "setp.ne.b32 p, %6, 0;\n\tsetp.ne.b32 q, %7, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}\n" ::"r"(tmem),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc), "r"(lead));
+}
+__device__ __forceinline__ void commit_lead(uint32_t lead, uint64_t* bar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(
+            (uint32_t)__cvta_generic_to_shared(bar)),
+        "r"(lead));
+}
+__device__ __forceinline__ uint32_t elect_lane() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     uint32_t done = 0;
     for (long it = 0; it < kWaitLimit && !done; ++it)
@@ -341,21 +372,23 @@ __device__ __forceinline__ void drain_stacked(float (&ar)[64], float (&ai)[64], 
 // of B in one MMA of N = (T - p) bn columns, into the levels L_p .. L_(T-1) of an accumulator of T
 // levels of bn columns (real) and T more (imaginary).  Level L_q collects the products whose
 // term orders add up to q: 4 T MMAs instead of 4 n_products, each wide enough to run at rate
-// (an MMA takes as long at N = 16 as at N = 64), and the same products.  a(p, im) and b(im) are
-// the descriptors of A's term planes and of B's first re / im plane; `fresh` restarts all levels.
-template <int T, class DA, class DB>
-__device__ __forceinline__ void stacked_products(uint32_t d, int bn, bool fresh, DA a, DB b) {
-    const uint64_t br = b(0), bi = b(1);
+// (an MMA takes as long at N = 16 as at N = 64), and the same products.  a, b: descriptors of the first
+// planes; a_plane, b_plane: from one plane to the next in units of 16 bytes; `fresh` restarts all
+// levels; IDESC: further bits of the instruction descriptor.
+template <int T, uint32_t IDESC = 0>
+__device__ __forceinline__ void stacked_products(uint32_t lead, uint32_t d, int bn, bool fresh, Desc a, uint32_t a_plane,
+                                                 Desc b, uint32_t b_plane) {
+    const uint32_t br = b.lo, bi = b.lo + T * b_plane;
 #pragma unroll
     for (int p = 0; p < T; ++p) {
-        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((T - p) * bn >> 3) << 17) |
+        const uint32_t idesc = IDESC | (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((T - p) * bn >> 3) << 17) |
                                ((uint32_t)(TBM >> 4) << 24);
-        const uint64_t ar = a(p, 0), ai = a(p, 1);
+        const uint32_t ar = a.lo + p * a_plane, ai = a.lo + (T + p) * a_plane;
         const uint32_t dr = d + p * bn, di = d + (T + p) * bn, acc = (fresh && p == 0) ? 0u : 1u;
-        mma_bf16(dr, ar, br, idesc, acc);
-        mma_bf16(dr, ai, bi, idesc | (1u << 13), 1u);
-        mma_bf16(di, ar, bi, idesc, acc);
-        mma_bf16(di, ai, br, idesc, 1u);
+        mma_lead(lead, dr, ar, a.hi, br, b.hi, idesc, acc);
+        mma_lead(lead, dr, ai, a.hi, bi, b.hi, idesc | (1u << 13), 1u);
+        mma_lead(lead, di, ar, a.hi, bi, b.hi, idesc, acc);
+        mma_lead(lead, di, ai, a.hi, br, b.hi, idesc, 1u);
     }
 }
 
@@ -442,10 +475,9 @@ __global__ void __launch_bounds__(CH ? 2 * TTHREADS : TTHREADS)
             if constexpr (CH)
                 if (stack)
                     for (int s16 = 0; s16 < nsteps; ++s16)
-                        stacked_products<T>(
-                            tm, p.BN, fresh && s16 == 0,
-                            [&](int q, int im) { return make_desc(base + (im * T + q) * PLANE_TILE + s16 * 256); },
-                            [&](int im) { return make_desc(base + 2 * T * PLANE_TILE + im * T * b_plane + s16 * 256); });
+                        stacked_products<T>(1, tm, p.BN, fresh && s16 == 0, desc_words(make_desc(base + s16 * 256)),
+                                            PLANE_TILE / 16,
+                                            desc_words(make_desc(base + 2 * T * PLANE_TILE + s16 * 256)), b_plane / 16);
 #pragma unroll
             for (int s16 = 0; s16 < 2; ++s16)
 #pragma unroll
@@ -766,7 +798,7 @@ __global__ void __launch_bounds__(TMA_THREADS, 1)
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full[NST_TMA_MAX], empty[NST_TMA_MAX], chunk_full[2], drained[2], fin;
     __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
     const uint32_t ring = (smem_u32(smem_raw) + 1023) & ~1023u;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
@@ -791,7 +823,7 @@ __global__ void __launch_bounds__(TMA_THREADS, 1)
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
-    const uint32_t tm = tmem_base;
+    const uint32_t tm = (uint32_t)uniform((int)tmem_base);
     bool ok = true;
     // every role walks the same tiles; k-tiles (`it`) and chunks (`cc`) count over all of them
     if (warp == TMA_DRAIN / 32) {
@@ -821,72 +853,76 @@ __global__ void __launch_bounds__(TMA_THREADS, 1)
         }
         __syncwarp();
     } else if (warp == TMA_DRAIN / 32 + 1) {
-        // ---- MMA warp
-        if (lane == 0) {
-            int it = 0, cc = 0;
-            for (int ti = blockIdx.x; ok && ti < n_tiles; ti += gridDim.x) {
-                const TcProb& p = probs[tiles[ti].prob];
-                const int BN = p.BN, K0 = p.K0, K1 = p.K1, kt0 = (K0 + 31) / 32, KT = kt0 + (K1 + 31) / 32;
-                const uint32_t a_plane = 64 * TBM, b_plane = 64 * (uint32_t)BN, bytes = 2 * T * (a_plane + b_plane);
-                const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                                       ((uint32_t)(TBM >> 4) << 24);
-                const uint32_t idesc_neg = idesc | (1u << 13);
-                for (int kt = 0; kt < KT; ++kt, ++it) {
-                    const int st = it % nst, set = cc % nset;
-                    const bool first = kt % chunk == 0, last = kt % chunk == chunk - 1 || kt + 1 == KT;
-                    const bool free_set = !first || cc < nset;
-                    auto wait_set = [&] {  // the set's previous chunk has been added up
-                        const bool w = free_set || mbar_wait(&drained[set], (uint32_t)(cc / nset - 1) & 1u);
-                        asm volatile("tcgen05.fence::after_thread_sync;");
-                        return w;
-                    };
-                    ok = mbar_wait(&full[st], (uint32_t)(it / nst) & 1u);
-                    if (ok && (stack || kt == 0)) ok = wait_set();  // a new tile restarts the corrections too
-                    if (!ok) break;
+        // ---- MMA warp (convergent; one lane issues)
+        const uint32_t lead = elect_lane();
+        auto wait = [&](uint64_t* bar, uint32_t parity) { return (bool)__all_sync(0xffffffffu, mbar_wait(bar, parity)); };
+        int it = 0, st = 0, cc = 0;
+        uint32_t ring_par = 0;
+        const Desc d0 = desc_words(make_desc_sw64(ring));
+        for (int ti = blockIdx.x; ok && ti < n_tiles; ti += gridDim.x) {
+            const TcProb& p = probs[tiles[ti].prob];
+            const int BN = uniform(p.BN), K0 = uniform(p.K0), K1 = uniform(p.K1);
+            const int kt0 = (K0 + 31) / 32, KT = kt0 + (K1 + 31) / 32;
+            // plane and stage sizes in 16 bytes
+            constexpr uint32_t a_plane = 64 * TBM / 16;
+            const uint32_t b_plane = 4 * (uint32_t)BN, stage = 2 * T * (a_plane + b_plane);
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
+                                   ((uint32_t)(TBM >> 4) << 24);
+            const uint32_t idesc_neg = idesc | (1u << 13);
+            for (int kt = 0; kt < KT; ++kt, ++it) {
+                const int set = nset == 2 ? cc & 1 : 0;
+                const bool first = kt % chunk == 0, last = kt % chunk == chunk - 1 || kt + 1 == KT;
+                const bool free_set = !first || cc < nset;
+                auto wait_set = [&] {  // the set's previous chunk has been added up
+                    const bool w = free_set || wait(&drained[set], (uint32_t)((nset == 2 ? cc >> 1 : cc) - 1) & 1u);
                     asm volatile("tcgen05.fence::after_thread_sync;");
-                    const uint32_t A = ring + st * bytes, B = A + 2 * T * a_plane;
-                    const int kseg = kt >= kt0 ? K1 - (kt - kt0) * 32 : K0 - kt * 32, nsteps = kseg > 16 ? 2 : 1;
-                    for (int s16 = 0; s16 < nsteps; ++s16) {
-                        if (stack) {
-                            stacked_products<T>(
-                                tm + set * (2 * T * BN), BN, first && s16 == 0,
-                                [&](int q, int im) { return make_desc_sw64(A + (im * T + q) * a_plane + s16 * 32); },
-                                [&](int im) { return make_desc_sw64(B + im * T * b_plane + s16 * 32); });
-                            continue;
-                        }
-                        constexpr int PI[6] = {0, 0, 1, 0, 1, 2}, PJ[6] = {0, 1, 0, 2, 1, 0};
+                    return w;
+                };
+                ok = wait(&full[st], ring_par);
+                if (ok && (stack || kt == 0)) ok = wait_set();  // a new tile restarts the corrections too
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t A = d0.lo + st * stage, B = A + 2 * T * a_plane;
+                const int kseg = kt >= kt0 ? K1 - (kt - kt0) * 32 : K0 - kt * 32, nsteps = kseg > 16 ? 2 : 1;
+                for (int s16 = 0; s16 < nsteps; ++s16) {
+                    const uint32_t As = A + 2 * s16, Bs = B + 2 * s16;  // 32 bytes on in the swizzled rows
+                    if (stack) {
+                        stacked_products<T>(lead, tm + set * (2 * T * BN), BN, first && s16 == 0, Desc{As, d0.hi},
+                                            a_plane, Desc{Bs, d0.hi}, b_plane);
+                        continue;
+                    }
+                    constexpr int PI[6] = {0, 0, 1, 0, 1, 2}, PJ[6] = {0, 1, 0, 2, 1, 0};
 #pragma unroll
-                        for (int i = 0; i < n_products<T>(); ++i) {
-                            // corrections first (over the whole K, columns 2 cofs on), the leading product
-                            // (restarting with the chunk) last
-                            const int q = i + 1 < n_products<T>() ? i + 1 : 0;
-                            if (q == 0 && s16 == 0 && first && kt > 0) ok = wait_set();
-                            if (!ok) break;
-                            const uint64_t ar = make_desc_sw64(A + PI[q] * a_plane + s16 * 32);
-                            const uint64_t ai = make_desc_sw64(A + (T + PI[q]) * a_plane + s16 * 32);
-                            const uint64_t br = make_desc_sw64(B + PJ[q] * b_plane + s16 * 32);
-                            const uint64_t bi = make_desc_sw64(B + (T + PJ[q]) * b_plane + s16 * 32);
-                            const uint32_t acc = q > 0 ? ((kt > 0 || s16 > 0 || q > 1) ? 1u : 0u)
-                                                       : ((first && s16 == 0) ? 0u : 1u);
-                            const uint32_t d = tm + (q > 0 ? 2 * cofs : 0);
-                            mma_bf16(d, ar, br, idesc, acc);
-                            mma_bf16(d, ai, bi, idesc_neg, 1u);
-                            mma_bf16(d + cofs, ar, bi, idesc, acc);
-                            mma_bf16(d + cofs, ai, br, idesc, 1u);
-                        }
+                    for (int i = 0; i < n_products<T>(); ++i) {
+                        // corrections first (over the whole K, columns 2 cofs on), the leading product
+                        // (restarting with the chunk) last
+                        const int q = i + 1 < n_products<T>() ? i + 1 : 0;
+                        if (q == 0 && s16 == 0 && first && kt > 0) ok = wait_set();
+                        const uint32_t ar = As + PI[q] * a_plane, ai = ar + T * a_plane;
+                        const uint32_t br = Bs + PJ[q] * b_plane, bi = br + T * b_plane;
+                        const uint32_t acc = q > 0 ? ((kt > 0 || s16 > 0 || q > 1) ? 1u : 0u)
+                                                   : ((first && s16 == 0) ? 0u : 1u);
+                        const uint32_t d = tm + (q > 0 ? 2 * cofs : 0);
+                        mma_lead(lead, d, ar, d0.hi, br, d0.hi, idesc, acc);
+                        mma_lead(lead, d, ai, d0.hi, bi, d0.hi, idesc_neg, 1u);
+                        mma_lead(lead, d + cofs, ar, d0.hi, bi, d0.hi, idesc, acc);
+                        mma_lead(lead, d + cofs, ai, d0.hi, br, d0.hi, idesc, 1u);
                     }
-                    mma_commit(&empty[st]);
-                    if (last) {
-                        mma_commit(&chunk_full[set]);
-                        ++cc;
-                    }
-                    if (!ok) break;
                 }
+                commit_lead(lead, &empty[st]);
+                if (last) {
+                    commit_lead(lead, &chunk_full[set]);
+                    ++cc;
+                }
+                if (++st == nst) {
+                    st = 0;
+                    ring_par ^= 1u;
+                }
+                if (!ok) break;
             }
-            mma_commit(&fin);  // no MMA may still use TMEM when it is freed
-            ok = mbar_wait(&fin, 0) && ok;
         }
-        __syncwarp();
+        commit_lead(lead, &fin);  // no MMA may still use TMEM when it is freed
+        ok = wait(&fin, 0) && ok;
     } else {
         // ---- drain warps
         const uint32_t q_lanes = (uint32_t)((warp & 3) * 32) << 16;
@@ -1368,9 +1404,9 @@ __device__ __forceinline__ void cat_load_planes(uint8_t* sA, const CatItem& it, 
 // B: row n of slot j, depth k, from the factor (zero past its rank and K)
 template <int T>
 __device__ __forceinline__ void cat_build_b(uint8_t* sBp, uint8_t* sBn, const CatItem& it, int K, int kc8,
-                                            uint32_t sbo) {
+                                            uint32_t sbo, int tid) {
     const int n8 = (it.rank + 7) & ~7;
-    for (int task = threadIdx.x; task < n8 * kc8; task += CAT_THREADS) {
+    for (int task = tid; task < n8 * kc8; task += CAT_THREADS) {
         const int n = task / kc8, kc = task % kc8;
         uint32_t wr[T][4], wi[T][4];
 #pragma unroll
@@ -1496,11 +1532,11 @@ __global__ void __launch_bounds__(CAT_THREADS) tc_cat_kernel(const TcCtx c, cons
     if constexpr (MODE == CAT_DG1A) {
         float2 v[CAT_ITER][8];
         cat_load_g(v, c, it, t.p0, kc8, n_phi);
-        cat_build_b<T>(sBp, sBn, it, K, kc8, sbo);
+        cat_build_b<T>(sBp, sBn, it, K, kc8, sbo, threadIdx.x);
         cat_store_g<T>(sA, v, kc8, sbo, planeA);
     } else {
         cat_load_planes<T>(sA, it, t.p0, kc8, sbo, planeA);
-        cat_build_b<T>(sBp, sBn, it, K, kc8, sbo);
+        cat_build_b<T>(sBp, sBn, it, K, kc8, sbo, threadIdx.x);
         asm volatile("cp.async.wait_group 0;");
     }
     asm volatile("fence.proxy.async.shared::cta;");
@@ -1524,6 +1560,434 @@ __global__ void __launch_bounds__(CAT_THREADS) tc_cat_kernel(const TcCtx c, cons
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm), "r"(tcols));
+}
+
+// --------------------------------------------------------------- fused DG1a + DG1b
+// H_r = U_theta^T conj(W G_r) U_phi (Fig. 3b step 1) without the P'' planes: written and read back
+// they were 12 of the 22 GB that 128 columns of the 30-lambda sphere moved here, and the two
+// kernels that ran the factors apart (tc_cat_kernel) went through load, split, multiply and
+// store one after the other with 16 warps an SM.  A persistent CTA per SM takes units (item, range
+// of columns), builds the unit's factor operands once and streams tiles of PC phi directions x
+// RB columns, PC RB = 128, PC = r_theta rounded up to 16 or 32:
+//   8 loader warps   spectra -> conj(W g) -> BF16 terms, slabs of 16 theta (128 (i_phi, r) rows) in a
+//                    ring; the next slab's loads are in registers, the tile after next on its way to L2
+//   MMA warp         S1: P = slab x U_theta, the terms stacked along N as in tc_cat_kernel;
+//                    S2: H += P x U_phi, contraction over the tile's PC directions, stacked_products
+//   4 P warps        P from TMEM (lane = (i_phi, r)) -> terms -> shared memory as the A operand of S2 with
+//                    (a, r) as its rows: an MN-major operand, 16 bytes = 8 values of a at one i_phi
+//   4 H warps        H from TMEM (lane = (a, r)) -> the planes [r][a + r_t b] that DG2 reads
+// S1 of a tile runs while P of the one before is split, S2 while the next P leaves TMEM.
+// What bounds it: the tensor pipe (narrow N: r_theta, r_phi <= 48) and the splits' issue.
+// 30-lambda sphere, 128 columns: DG1a + DG1b 8.6 + 3.3 ms -> 5.0 ms (1.4 ms for the bytes).
+struct Dg1Item {
+    const float2* uth;                        // U_theta, n_theta x r_theta column-major (FP32)
+    const bf16* uph; int64_t u_ld, u_ps;      // U_phi planes [b][i_phi]
+    bf16* out; int64_t o_ld, o_ps;            // H planes [r][a + r_t b]
+    int g, alpha, rt, rp;
+};
+struct Dg1Unit { int item, r0, nr; };
+struct Dg1Shape {
+    int PC, NS;             // phi directions per tile (rows of an item in M of S2), slabs in the ring
+    int K1, KP;             // n_theta and n_phi rounded up to 16
+    int n8max, n16max;      // largest r_theta to 8, r_phi to 16
+    int w_smem;             // the quadrature weights are kept in shared memory
+    int tcols;
+};
+
+constexpr int DG1_THREADS = 20 * 32;  // five warpgroups: P, H, two of loaders, MMA (one warp of it works)
+constexpr int DG1_REGS = 96;          // registers a thread at launch, redistributed by setmaxnreg:
+constexpr int DG1_REGS_P = 120, DG1_REGS_H = 128, DG1_REGS_L = 88, DG1_REGS_M = 56;
+static_assert(DG1_REGS_P + DG1_REGS_H + 2 * DG1_REGS_L + DG1_REGS_M <= 5 * DG1_REGS, "more than the launch holds");
+template <int N>
+__device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void regs_down() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+constexpr int DG1_SLABS = 3;
+
+// MN-major operand without swizzle: 8 x 8 core matrices whose 16-byte rows run along M; `lbo` to the
+// next 8 of K, `sbo` to the next 8 of M
+__device__ __forceinline__ uint64_t make_desc_mn(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+    uint64_t d = 0;
+    d |= (uint64_t)((addr >> 4) & 0x3FFF);
+    d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
+    d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
+    d |= (uint64_t)1 << 46;
+    return d;
+}
+
+// The BF16 terms of 8 values, 16 bytes a plane.  (Real and imaginary parts go one after the other here
+// and below: both at once spilled, and next to 220 KB of shared memory spills live in L2.)
+template <int T>
+__device__ __forceinline__ void store_terms(uint8_t* dst, int plane, const float* x) {
+    uint32_t w[T][4];
+#pragma unroll
+    for (int e = 0; e < 8; e += 2) {
+        uint32_t t[3];
+        split_pack<T>(x[e], x[e + 1], t);
+#pragma unroll
+        for (int q = 0; q < T; ++q) w[q][e / 2] = t[q];
+    }
+#pragma unroll
+    for (int q = 0; q < T; ++q) *reinterpret_cast<uint4*>(dst + q * plane) = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
+}
+
+// 8 columns of (L_(T-1) + ... + L_1) + L_0, the levels `step` TMEM columns apart
+template <int T>
+__device__ __forceinline__ void sum_levels(float* x, uint32_t taddr, int step) {
+    uint32_t v[T][8];
+#pragma unroll
+    for (int q = 0; q < T; ++q) tmem_ld8(v[q], taddr + (uint32_t)(q * step));
+    asm volatile("tcgen05.wait::ld.sync.aligned;");
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        x[e] = __uint_as_float(v[T - 1][e]);
+#pragma unroll
+        for (int q = T - 2; q >= 0; --q) x[e] += __uint_as_float(v[q][e]);
+    }
+}
+
+template <int T>
+__global__ void __launch_bounds__(DG1_THREADS, 1)
+    tc_dg1_kernel(const TcCtx c, const Dg1Item* __restrict__ items, const Dg1Unit* __restrict__ units, int n_units,
+                  const Dg1Shape sh, int n_phi, int aligned) {
+    extern __shared__ __align__(1024) uint8_t smem[];
+    __shared__ __align__(8) uint64_t slab_full[DG1_SLABS], slab_empty[DG1_SLABS], d1_full, d1_empty, a2_full, a2_empty,
+        d2_full, d2_empty, b_full, unit_done, fin;
+    __shared__ uint32_t tmem_base;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
+    const int nt = c.n_theta, PC = sh.PC, RB = TBM / PC, nch = (n_phi + PC - 1) / PC, nslab = sh.K1 / 16;
+    constexpr int SLAB_PLANE = TBM * 16 * 2;                   // 128 rows x 16 K
+    const int a2_plane = TBM * PC * 2, b1_bytes = 2 * T * sh.n8max * sh.K1 * 2;
+    uint8_t* sA1 = smem;
+    uint8_t* sA2 = sA1 + sh.NS * 2 * T * SLAB_PLANE;
+    uint8_t* sB1p = sA2 + 2 * T * a2_plane;
+    uint8_t* sB1n = sB1p + b1_bytes;
+    uint8_t* sB2 = sB1n + b1_bytes;                            // [plane][n16 rows][KP], K-major
+    bf16* sH = reinterpret_cast<bf16*>(sB2 + 2 * T * sh.n16max * sh.KP * 2);  // 4 warps x T planes x 256
+    float* sW = reinterpret_cast<float*>(sH + 4 * T * 256);
+    if (warp == 0) tmem_alloc(&tmem_base, sh.tcols);
+    if (tid == 0) {
+        auto init = [](uint64_t* bar, int count) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
+        };
+        for (int s = 0; s < sh.NS; ++s) {
+            init(&slab_full[s], 256);
+            init(&slab_empty[s], 1);
+        }
+        init(&d1_full, 1); init(&d1_empty, 128);
+        init(&a2_full, 128); init(&a2_empty, 1);
+        init(&d2_full, 1); init(&d2_empty, 128);
+        init(&b_full, 256); init(&unit_done, 1); init(&fin, 1);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;");
+    if (sh.w_smem)
+        for (int i = tid; i < c.n_dir; i += DG1_THREADS) sW[i] = c.w ? c.w[i] : 1.0f;
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tm = (uint32_t)uniform((int)tmem_base), d1 = tm, d2 = tm + (uint32_t)(2 * T * sh.n8max);
+    const uint32_t q_lanes = (uint32_t)((warp & 3) * 32) << 16;
+    bool ok = true;
+    if (warp < 4) {
+        // ---- P warps
+        regs_up<DG1_REGS_P>();
+        int t = 0;
+        const int row = warp * 32 + lane, k = row % PC, rl = row / PC;
+        const uint32_t sbo2 = (uint32_t)(PC / 8) * 128;
+        for (int ui = blockIdx.x; ok && ui < n_units; ui += gridDim.x) {
+            const Dg1Unit u = units[ui];
+            const int n8 = (items[u.item].rt + 7) & ~7, ntile = (u.nr + RB - 1) / RB * nch;
+            for (int tt = 0; tt < ntile; ++tt, ++t) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&d1_full, (uint32_t)t & 1u));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                float pr[32], pi[32];  // (L_2 + L_1) + L_0 of this row's r_theta values
+#pragma unroll
+                for (int c0 = 0; c0 < 32; c0 += 8)
+                    if (c0 < n8) {
+                        sum_levels<T>(pr + c0, d1 + q_lanes + (uint32_t)c0, 2 * n8);
+                        sum_levels<T>(pi + c0, d1 + q_lanes + (uint32_t)(n8 + c0), 2 * n8);
+                    }
+                asm volatile("tcgen05.fence::before_thread_sync;");
+                mbar_arrive(&d1_empty);
+                if (t >= 1) ok = __all_sync(0xffffffffu, mbar_wait(&a2_empty, (uint32_t)(t - 1) & 1u));
+                if (!ok) break;
+                uint8_t* dst = sA2 + (uint32_t)(rl * PC / 8) * sbo2 + (k >> 3) * 128 + (k & 7) * 16;
+#pragma unroll
+                for (int c0 = 0; c0 < 32; c0 += 8)
+                    if (c0 < n8) {
+                        store_terms<T>(dst + (c0 / 8) * sbo2, a2_plane, pr + c0);
+                        store_terms<T>(dst + T * a2_plane + (c0 / 8) * sbo2, a2_plane, pi + c0);
+                    }
+                asm volatile("fence.proxy.async.shared::cta;");
+                mbar_arrive(&a2_full);
+            }
+        }
+    } else if (warp < 8) {
+        // ---- H warps
+        regs_up<DG1_REGS_H>();
+        int bk = 0;
+        const int row = (warp & 3) * 32 + lane, a = row % PC, rl = row / PC;
+        bf16* stage_h = sH + (warp & 3) * (T * 256);
+        for (int ui = blockIdx.x; ok && ui < n_units; ui += gridDim.x) {
+            const Dg1Unit u = units[ui];
+            const Dg1Item it = items[u.item];
+            const int n16 = (it.rp + 15) & ~15;
+            for (int b0 = 0; b0 < u.nr; b0 += RB, ++bk) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&d2_full, (uint32_t)bk & 1u));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                // Eight columns b of a column r are 8 r_t neighbours in memory, starting on 16 bytes:
+                // they go through shared memory and leave as one 16-byte store per plane (2-byte
+                // stores straight from the registers, eight times as many, took 5.66 ms).
+                const int rq = lane / PC, vec = lane % PC;  // this lane's 16 bytes of column b0 + rw + rq
+                const int rw = (warp & 3) * 32 / PC;
+                const bool writes = vec < it.rt && b0 + rw + rq < u.nr;
+                bf16* out = it.out + (int64_t)(u.r0 + b0 + rw + rq) * it.o_ld + vec * 8;
+                auto put = [&](int c0, int im, const float* x) {  // columns c0 .. c0 + 7, real or imaginary
+                    bf16* o = stage_h + rl % (32 / PC) * (PC * 8) + a;
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2) {  // zeros to the next 8 elements past r_p
+                        uint32_t w[3];
+                        split_pack<T>(c0 + e < it.rp ? x[e] : 0.f, c0 + e + 1 < it.rp ? x[e + 1] : 0.f, w);
+                        if (a < it.rt)
+#pragma unroll
+                            for (int q = 0; q < T; ++q) {
+                                o[q * 256] = __ushort_as_bfloat16((unsigned short)(w[q] & 0xffffu));
+                                o[q * 256 + it.rt] = __ushort_as_bfloat16((unsigned short)(w[q] >> 16));
+                            }
+                        o += 2 * it.rt;
+                    }
+                    __syncwarp();
+                    if (writes && vec * 8 < min(8, it.rp - c0) * it.rt)
+#pragma unroll
+                        for (int q = 0; q < T; ++q)
+                            *reinterpret_cast<uint4*>(out + (im * T + q) * it.o_ps + c0 * it.rt) =
+                                *reinterpret_cast<const uint4*>(stage_h + q * 256 + rq * (PC * 8) + vec * 8);
+                    __syncwarp();
+                };
+                // the first 32 columns come out of TMEM at once, so that S2 may start over while they are
+                // split and stored; the few past them before that
+                for (int c0 = 32; c0 < it.rp; c0 += 8)
+#pragma unroll 1
+                    for (int im = 0; im < 2; ++im) {
+                        float x[8];
+                        sum_levels<T>(x, d2 + q_lanes + (uint32_t)(im * T * n16 + c0), n16);
+                        put(c0, im, x);
+                    }
+                float xs[4][2][8];
+#pragma unroll
+                for (int g = 0; g < 4; ++g)
+                    if (8 * g < it.rp) {
+                        sum_levels<T>(xs[g][0], d2 + q_lanes + (uint32_t)(8 * g), n16);
+                        sum_levels<T>(xs[g][1], d2 + q_lanes + (uint32_t)(T * n16 + 8 * g), n16);
+                    }
+                asm volatile("tcgen05.fence::before_thread_sync;");
+                mbar_arrive(&d2_empty);
+#pragma unroll
+                for (int g = 0; g < 4; ++g)
+                    if (8 * g < it.rp) {
+                        put(8 * g, 0, xs[g][0]);
+                        put(8 * g, 1, xs[g][1]);
+                    }
+            }
+        }
+    } else if (warp < 16) {
+        // ---- loader warps
+        regs_down<DG1_REGS_L>();
+        // Eight lanes share a row's 16 theta (128 bytes of spectra, two theta a lane), a warp 16 rows of one
+        // column, four at a time.  (One row's 64 bytes per lane touched every sector twice and waited
+        // 1700 cycles a slab for it.)
+        const int lt = tid - 256, sub = lane & 7, row0 = (warp & 7) * 16 + (lane >> 3), pl = row0 % PC, rl = row0 / PC;
+        int n = 0, un = 0;
+        for (int ui = blockIdx.x; ok && ui < n_units; ui += gridDim.x, ++un) {
+            const Dg1Unit u = units[ui];
+            const Dg1Item it = items[u.item];
+            const int ntile = (u.nr + RB - 1) / RB * nch;
+            const float2* spec = c.spec_in + ((int64_t)it.g * 2 + it.alpha) * c.n_dir;
+            const int64_t rs = (int64_t)c.G * 2 * c.n_dir;
+            // Two walks over the unit's slabs (tile by tile, 16 theta at a time): `at` loads this thread's
+            // theta pair of rows row0, row0 + 4, + 8, + 12, `now`, one slab behind, splits them.
+            struct Walk {
+                int s = 0, ch = 0, blk = 0;
+                __device__ __forceinline__ void next(int nslab, int nch) {
+                    if (++s == nslab) {
+                        s = 0;
+                        if (++ch == nch) {
+                            ch = 0;
+                            ++blk;
+                        }
+                    }
+                }
+            } at, now;
+            const float2* src = nullptr;  // row0 of the tile `at` is in
+            int rows = 0;                 // of the four, those that hold directions and columns
+            auto load = [&](float4 (&x)[4]) {
+                if (at.s == 0) {
+                    const int ip = at.ch * PC + pl, r = at.blk * RB + rl;
+                    rows = r < u.nr ? min(4, (n_phi - ip + 3) >> 2) : 0;
+                    src = spec + rs * (u.r0 + r) + nt * ip + 2 * sub;
+                }
+                const int th = at.s * 16 + 2 * sub;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2* p = src + at.s * 16 + 4 * j * nt;
+                    x[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (j < rows && th < nt) {
+                        if (aligned) {  // n_theta even
+                            x[j] = __ldcs(reinterpret_cast<const float4*>(p));
+                        } else {
+                            const float2 p0 = p[0], p1 = th + 1 < nt ? p[1] : make_float2(0.f, 0.f);
+                            x[j] = make_float4(p0.x, p0.y, p1.x, p1.y);
+                        }
+                    }
+                }
+                at.next(nslab, nch);
+            };
+            auto to_l2 = [&](int tt) {  // the rows of one column of a tile are contiguous
+                const int r = tt / nch * RB + lt, p0 = tt % nch * PC;
+                if (!aligned || tt >= ntile || lt >= RB || r >= u.nr) return;
+                const uint32_t bytes = (uint32_t)(min(PC, n_phi - p0) * nt * 8) & ~15u;
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(spec + rs * (u.r0 + r) + nt * p0),
+                             "r"(bytes)
+                             : "memory");
+            };
+            float4 va[4], vb[4];
+            to_l2(1);
+            load(va);
+            // the unit's factor operands, once the last unit's MMAs are done with theirs
+            if (un >= 1) ok = __all_sync(0xffffffffu, mbar_wait(&unit_done, (uint32_t)(un - 1) & 1u));
+            if (!ok) break;
+            CatItem ci{};
+            ci.fac = it.uth;
+            ci.rank = it.rt;
+            cat_build_b<T>(sB1p, sB1n, ci, nt, sh.K1 / 8, (uint32_t)sh.K1 * 16, lt);
+            {
+                const int n16 = (it.rp + 15) & ~15, kc8 = sh.KP / 8, k8v = (n_phi + 7) / 8;
+                for (int e = lt; e < 2 * T * n16 * kc8; e += 256) {
+                    const int q = e / (n16 * kc8), rem = e % (n16 * kc8), b = rem / kc8, kk = rem % kc8;
+                    const bool in = b < it.rp && kk < k8v;
+                    const bf16* src = in ? it.uph + q * it.u_ps + (int64_t)b * it.u_ld + kk * 8 : it.uph;
+                    cp16(sB2 + canon_off(q * n16 + b, kk, (uint32_t)sh.KP * 16), src, in ? 16 : 0);
+                }
+                asm volatile("cp.async.commit_group;");
+                asm volatile("cp.async.wait_group 0;");
+            }
+            asm volatile("fence.proxy.async.shared::cta;");
+            mbar_arrive(&b_full);
+            auto emit = [&](float4 (&v)[4]) {
+                if (now.s == 0) to_l2(now.blk * nch + now.ch + 2);
+                const int st = n % sh.NS, th = now.s * 16 + 2 * sub;
+                if (n >= sh.NS) ok = __all_sync(0xffffffffu, mbar_wait(&slab_empty[st], (uint32_t)(n / sh.NS - 1) & 1u));
+                if (!ok) return;
+                uint8_t* dst = sA1 + st * 2 * T * SLAB_PLANE + (sub >> 2) * 128 + (sub & 3) * 4;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int row = row0 + 4 * j, i = min(now.ch * PC + pl + 4 * j, n_phi - 1) * nt;
+                    // (past n_theta and n_phi the loads left zeros: any finite weight)
+                    const int i0 = i + min(th, nt - 1), i1 = i + min(th + 1, nt - 1);
+                    const float w0 = sh.w_smem ? sW[i0] : c.w ? __ldg(c.w + i0) : 1.0f;
+                    const float w1 = sh.w_smem ? sW[i1] : c.w ? __ldg(c.w + i1) : 1.0f;
+                    uint32_t wr[3], wi[3];
+                    split_pack<T>(w0 * v[j].x, w1 * v[j].z, wr);
+                    split_pack<T>(-w0 * v[j].y, -w1 * v[j].w, wi);
+                    uint8_t* o = dst + (row >> 3) * 256 + (row & 7) * 16;
+#pragma unroll
+                    for (int q = 0; q < T; ++q) {
+                        *reinterpret_cast<uint32_t*>(o + q * SLAB_PLANE) = wr[q];
+                        *reinterpret_cast<uint32_t*>(o + (T + q) * SLAB_PLANE) = wi[q];
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;");
+                mbar_arrive(&slab_full[st]);
+                now.next(nslab, nch);
+                ++n;
+            };
+            // by twos, so that each set of registers is loaded a whole slab ahead of its use
+            const int total = ntile * nslab;
+            for (int i = 0; ok && i < total; i += 2) {
+                if (i + 1 < total) load(vb);
+                emit(va);
+                if (!ok || i + 1 >= total) break;
+                if (i + 2 < total) load(va);
+                emit(vb);
+            }
+        }
+    } else {
+        // ---- MMA warp
+        regs_down<DG1_REGS_M>();
+        if (warp == 16) {
+            const uint32_t lead = elect_lane();
+            auto wait = [&](uint64_t* bar, uint32_t parity) { return (bool)__all_sync(0xffffffffu, mbar_wait(bar, parity)); };
+            int n = 0, st = 0, t = 0, bk = 0, un = 0;
+            uint32_t ring_par = 0;
+            const uint32_t sbo1 = (uint32_t)sh.K1 * 16, sbo2 = (uint32_t)sh.KP * 16;
+            const Desc a1 = desc_words(make_desc_sbo(smem_u32(sA1), 256));
+            const Desc b1p = desc_words(make_desc_sbo(smem_u32(sB1p), sbo1)), b1n = desc_words(make_desc_sbo(smem_u32(sB1n), sbo1));
+            const Desc a2 = desc_words(make_desc_mn(smem_u32(sA2), 128, (uint32_t)(PC / 8) * 128));
+            const Desc b2 = desc_words(make_desc_sbo(smem_u32(sB2), sbo2));
+            for (int ui = blockIdx.x; ok && ui < n_units; ui += gridDim.x, ++un) {
+                const Dg1Unit u = units[ui];
+                const int n8 = (uniform(items[u.item].rt) + 7) & ~7, n16 = (uniform(items[u.item].rp) + 15) & ~15;
+                const int ntile = (uniform(u.nr) + RB - 1) / RB * nch;
+                ok = wait(&b_full, (uint32_t)un & 1u);
+                int ch2 = 0, t2 = t;  // direction chunk and number of the tile whose P x U_phi is next
+                auto s2 = [&] {
+                    ok = ok && wait(&a2_full, (uint32_t)t2 & 1u);
+                    if (ch2 == 0 && bk >= 1) ok = ok && wait(&d2_empty, (uint32_t)(bk - 1) & 1u);
+                    if (!ok) return;
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    for (int ks = 0; ks < PC / 16; ++ks) {
+                        const int k0 = ch2 * PC + ks * 16;  // directions past n_phi multiply zeros: left out
+                        if (k0 >= n_phi) break;
+                        // (K chunk k0 / 8 of B2 lies 128 bytes a chunk on)
+                        stacked_products<T, 1u << 15>(lead, d2, n16, ch2 == 0 && ks == 0, Desc{a2.lo + ks * 16, a2.hi},
+                                                      (uint32_t)a2_plane / 16, Desc{b2.lo + k0, b2.hi},
+                                                      (uint32_t)n16 * sbo2 / 128);
+                    }
+                    commit_lead(lead, &a2_empty);
+                    ++t2;
+                    if (++ch2 == nch) {
+                        ch2 = 0;
+                        commit_lead(lead, &d2_full);
+                        ++bk;
+                    }
+                };
+                for (int tt = 0; ok && tt < ntile; ++tt, ++t) {
+                    if (t >= 1) ok = wait(&d1_empty, (uint32_t)(t - 1) & 1u);
+                    for (int s = 0; ok && s < nslab; ++s, ++n) {
+                        ok = wait(&slab_full[st], ring_par);
+                        if (!ok) break;
+                        asm volatile("tcgen05.fence::after_thread_sync;");
+                        const uint32_t da = a1.lo + (uint32_t)st * (2 * T * SLAB_PLANE / 16), kb = (uint32_t)s * 16;
+#pragma unroll
+                        for (int p = 0; p < T; ++p) {
+                            const uint32_t idesc = idesc_bf16(2 * (T - p) * n8), d = d1 + (uint32_t)(2 * p * n8);
+                            mma_lead(lead, d, da + p * (SLAB_PLANE / 16), a1.hi, b1p.lo + kb, b1p.hi, idesc,
+                                     (s > 0 || p > 0) ? 1u : 0u);
+                            mma_lead(lead, d, da + (T + p) * (SLAB_PLANE / 16), a1.hi, b1n.lo + kb, b1n.hi, idesc, 1u);
+                        }
+                        commit_lead(lead, &slab_empty[st]);
+                        if (++st == sh.NS) {
+                            st = 0;
+                            ring_par ^= 1u;
+                        }
+                    }
+                    if (!ok) break;
+                    commit_lead(lead, &d1_full);
+                    if (tt >= 1) s2();
+                }
+                if (ok) s2();
+                commit_lead(lead, &unit_done);
+            }
+            commit_lead(lead, &fin);  // no MMA may still use TMEM when it is freed
+            ok = wait(&fin, 0) && ok;
+        }
+    }
+    const int bad = __syncthreads_or(ok ? 0 : 1);
+    if (bad && tid == 0) atomicAdd(c.err, 1);
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm), "r"(sh.tcols));
 }
 
 // ------------------------------------------------------------ operand prep
@@ -2091,6 +2555,82 @@ void plan_cat(const Plan& P, TcPlan& M, int mode, bf16* Vb, VOff voff, bf16* Mb,
     C.on = true;
 }
 
+// The fused DG1a + DG1b when r_theta <= 32, both accumulators fit TMEM and the operands shared
+// memory (every workload up to 2-lambda boxes); larger ranks keep the two kernels, as do
+// TFMM_TC_CAT=0 and a DG1a pair count set by the tuning.
+template <class MOff>
+void plan_dg1(const Plan& P, TcPlan& M, const bf16* F, const std::vector<TcItem>& tci, bf16* Mb, MOff moff) {
+    Dg1Plan& D = M.dg1;
+    D.on = false;
+    if (const char* e = std::getenv("TFMM_TC_CAT"); e && e[0] == '0') return;
+    if (P.tc_dg1a_pairs != 0 || !fused_enabled() || !tc_split_accumulators()) return;
+    const int T = M.T, R = M.R, nt = P.n_theta, np = P.n_phi;
+    if (P.max_rank[0] > 32) return;
+    Dg1Shape sh{};
+    sh.PC = P.max_rank[0] <= 16 ? 16 : 32;
+    sh.NS = DG1_SLABS;
+    sh.K1 = (nt + 15) & ~15;
+    sh.KP = (np + 15) & ~15;
+    sh.n8max = (int)r8(P.max_rank[0]);
+    sh.n16max = (P.max_rank[1] + 15) & ~15;
+    if (T * sh.n16max > 256) return;
+    sh.tcols = 32;
+    while (sh.tcols < 2 * T * (sh.n8max + sh.n16max)) sh.tcols *= 2;
+    if (sh.tcols > 512) return;
+    size_t smem = (size_t)2 * T * (sh.NS * TBM * 32 + TBM * sh.PC * 2 + 2 * sh.n8max * sh.K1 * 2 + sh.n16max * sh.KP * 2) +
+                  (size_t)4 * T * 256 * 2;
+    if (smem + sizeof(float) * P.n_dir <= kMaxDynSmem) {
+        sh.w_smem = 1;
+        smem += sizeof(float) * P.n_dir;
+    }
+    if (smem > kMaxDynSmem) return;
+    std::vector<Dg1Item> items(P.items.size());
+    std::vector<Dg1Unit> units;
+    // whole items while there are enough for every SM, else shares of at least two column blocks
+    const int RB = TBM / sh.PC, nI = (int)P.items.size();
+    const int shares = std::max(1, std::min((4 * P.num_sms + nI - 1) / nI, R / (2 * RB)));
+    const int per = ((R + shares - 1) / shares + RB - 1) / RB * RB;
+    std::vector<int> order(nI);
+    std::iota(order.begin(), order.end(), 0);
+    for (int q = 0; q < nI; ++q) {
+        const TuckerItem& d = P.items[q];
+        const TcMat& u = tci[q].uph;
+        Dg1Item& it = items[q];
+        it.uth = P.d_factors + d.uth;
+        it.uph = F + u.off; it.u_ld = u.ld; it.u_ps = (int64_t)u.rows * u.ld;
+        const int64_t ldh = r8((int64_t)d.rt * d.rp);
+        it.out = Mb + moff(q); it.o_ld = ldh; it.o_ps = (int64_t)R * ldh;
+        it.g = d.g; it.alpha = d.alpha; it.rt = d.rt; it.rp = d.rp;
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return P.items[a].rp > P.items[b].rp; });
+    for (int q : order)
+        for (int r0 = 0; r0 < R; r0 += per) units.push_back(Dg1Unit{q, r0, std::min(per, R - r0)});
+    TFMM_CUDA_CHECK(device_malloc(&D.items.p, sizeof(Dg1Item) * items.size()));
+    TFMM_CUDA_CHECK(device_malloc(&D.units.p, sizeof(Dg1Unit) * units.size()));
+    TFMM_CUDA_CHECK(cudaMemcpy(D.items.p, items.data(), sizeof(Dg1Item) * items.size(), cudaMemcpyHostToDevice));
+    TFMM_CUDA_CHECK(cudaMemcpy(D.units.p, units.data(), sizeof(Dg1Unit) * units.size(), cudaMemcpyHostToDevice));
+    D.n_units = (int)units.size();
+    D.PC = sh.PC; D.NS = sh.NS; D.K1 = sh.K1; D.KP = sh.KP; D.n8max = sh.n8max; D.n16max = sh.n16max;
+    D.w_smem = sh.w_smem; D.tcols = sh.tcols;
+    D.smem = smem;
+    D.on = true;
+}
+
+template <int T>
+void launch_dg1(const Plan& P, const Dg1Plan& D, const TcCtx& c, cudaStream_t s) {
+    allow_dyn_smem(reinterpret_cast<const void*>(tc_dg1_kernel<T>), kMaxDynSmem);
+    cudaFuncAttributes fa{};  // the register split needs what the launch was compiled for
+    TFMM_CUDA_CHECK(cudaFuncGetAttributes(&fa, tc_dg1_kernel<T>));
+    if (fa.numRegs < DG1_REGS) fail(TFMM_CUDA, "tc_dg1_kernel: fewer registers at launch than its warps share out");
+    const Dg1Shape sh{D.PC, D.NS, D.K1, D.KP, D.n8max, D.n16max, D.w_smem, D.tcols};
+    // 16-byte loads and L2 prefetches of the spectra: every row of theta starts on 16 bytes
+    const int aligned = reinterpret_cast<uintptr_t>(c.spec_in) % 16 == 0 && P.n_theta % 2 == 0;
+    tc_dg1_kernel<T><<<std::min(D.n_units, P.num_sms), DG1_THREADS, D.smem, s>>>(
+        c, static_cast<const Dg1Item*>(D.items.p), static_cast<const Dg1Unit*>(D.units.p), D.n_units, sh, P.n_phi,
+        aligned);
+    TFMM_CUDA_CHECK(cudaGetLastError());
+}
+
 template <int T, int MODE>
 void launch_cat(const Plan& P, const CatPlan& C, const TcCtx& c, cudaStream_t s) {
     allow_dyn_smem(reinterpret_cast<const void*>(tc_cat_kernel<T, MODE>), kMaxDynSmem);
@@ -2253,6 +2793,7 @@ TcPlan* get_tc_plan(Plan& P, int R, int T, cudaStream_t s) {
     plan_fused34(P, M, F, tci, Mb, [&](int q) { return M.m_off[q]; });
     const auto voff = [&](int q) { return M.v_off[q]; };
     const auto moff = [&](int q) { return M.m_off[q]; };
+    plan_dg1(P, M, F, tci, Mb, moff);
     plan_cat(P, M, CAT_DG1A, Vb, voff, Mb, moff);
     if (!M.cat1a.on) plan_dg1a(P, M, F, tci, Vb, voff);
     plan_cat(P, M, CAT_DG1B, Vb, voff, Mb, moff);
@@ -2266,7 +2807,7 @@ void tc_replan_shapes(Plan& P) {
     for (auto& mp : P.tc) {
         TcPlan& M = *mp;
         for (DeviceBuffer* b : {&M.f34_items, &M.f34_tiles, &M.dg1a_items, &M.dg1a_tiles, &M.cat1a.items,
-                                &M.cat1a.tiles}) {
+                                &M.cat1a.tiles, &M.dg1.items, &M.dg1.units}) {
             if (b->p) cudaFree(b->p);
             b->p = nullptr;
         }
@@ -2277,6 +2818,7 @@ void tc_replan_shapes(Plan& P) {
         plan_fused34(P, M, F, tci, Mb, [&](int q) { return M.m_off[q]; });
         const auto voff = [&](int q) { return M.v_off[q]; };
         const auto moff = [&](int q) { return M.m_off[q]; };
+        plan_dg1(P, M, F, tci, Mb, moff);
         plan_cat(P, M, CAT_DG1A, Vb, voff, Mb, moff);
         M.dg1a = false;
         if (!M.cat1a.on) plan_dg1a(P, M, F, tci, Vb, voff);
@@ -2319,13 +2861,17 @@ void tc_disaggregate_t(Plan& P, TcPlan& M, const float2* spec, int R, int weight
                                             R, P.G, P.n_theta, P.n_phi);
         TFMM_CUDA_CHECK(cudaGetLastError());
     }
-    if (M.cat1a.on)
+    if (M.dg1.on)
+        launch_dg1<T>(P, M.dg1, c, s);
+    else if (M.cat1a.on)
         launch_cat<T, CAT_DG1A>(P, M.cat1a, c, s);
     else if (M.dg1a)
         launch_dg1a<T>(P, M, c, s);
     else
         launch_tc<T, TDG1A>(M.st[TDG1A], c, P.num_sms, s);
-    if (M.cat1b.on)
+    if (M.dg1.on)
+        ;  // both factors are applied
+    else if (M.cat1b.on)
         launch_cat<T, CAT_DG1B>(P, M.cat1b, c, s);
     else
         launch_tc<T, TDG1B>(M.st[TDG1B], c, P.num_sms, s);

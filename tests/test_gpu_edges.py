@@ -181,3 +181,16 @@ def test_stage_kernel_forms(R):
     ranks = [[(5, 7, 15), (3, 5, 14)], [(8, 16, 33), (1, 1, 1)], [(9, 13, 64), (6, 3, 31)],
              [(12, 11, 127), (12, 10, 96)], [(12, 22, 129), (2, 2, 4)], [(11, 19, 200), (10, 20, 128)]]
     _check(4000 + R, 12, 24, nbetas, ranks, R, 3, 1e-6, betas=(0.5 - 0.25j,))
+
+
+@pytest.mark.parametrize("R", [2, 9])
+@pytest.mark.parametrize("nt,npf,top", [(16, 31, (16, 31)), (17, 32, (17, 30)), (32, 64, (32, 48)), (33, 48, (32, 40)),
+                                        (33, 66, (33, 49)), (40, 75, (9, 49))])
+def test_disaggregation_first_step_forms(nt, npf, top, R):
+    """Tiles of 16 and 32 directions and ranks past both (the separate kernels), n_theta odd, below and above
+    a slab's 16, n_phi off the tiles, r_phi around the 32 columns held in registers and 48."""
+    rt, rp = top
+    nbetas = [40, 120, 90]
+    ranks = [[(rt, rp, 24), (max(1, rt - 1), max(1, rp - 1), 20)], [(rt, min(rp, 33), 100), (max(1, rt // 2), rp, 9)],
+             [(max(1, rt - 3), min(rp, 8), 64), (rt, max(1, rp // 2), 90)]]
+    _check(5000 + 10 * nt + R, nt, npf, nbetas, ranks, R, 3, 1e-6, betas=(0.5 - 0.25j,))
