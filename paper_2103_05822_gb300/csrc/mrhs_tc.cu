@@ -592,7 +592,10 @@ __global__ void __launch_bounds__(CH ? 2 * TTHREADS : TTHREADS)
 // TMEM -> registers -> shared memory (split into BF16 terms) as the A operand of
 // AG4, F_r[i_phi][i_theta] = sum_a V_r[i_phi][a] U_theta[i_theta][a] (Fig. 2b
 // steps 3-4), which leaves TMEM straight for the spectra.  The MMAs of r overlap
-// the spectra stores of r - 1 (two D2 accumulators).
+// the spectra stores of r - 1 (two D2 accumulators).  What bounds it: one CTA per SM, whose
+// operand loads and AG3 nothing overlaps, and the chain V -> A operand -> MMA -> spectra of each r.
+// 30-lambda sphere, 128 columns: 6.45 ms with a lone issuing thread, 5.88 with the convergent MMA
+// warp (1.4 ms for the bytes); 10-lambda, 37 columns: 0.591 -> 0.443 ms.
 struct F34Item {
     const bf16* uph; int64_t uph_ld, uph_ps;  // U_phi planes [i_phi][b]
     const bf16* uth; int64_t uth_ld, uth_ps;  // U_theta planes [i_theta][a]
@@ -637,25 +640,25 @@ __device__ __forceinline__ int product_order(int i) {  // corrections first, hi 
 }
 
 template <int T>
-__device__ __forceinline__ void issue_products(uint32_t d_re, uint32_t d_im, uint32_t a, int a_plane, uint32_t b,
-                                               int b_plane, uint32_t sbo_a, uint32_t sbo_b, int ksteps,
+__device__ __forceinline__ void issue_products(uint32_t lead, uint32_t d_re, uint32_t d_im, uint32_t a, int a_plane,
+                                               uint32_t b, int b_plane, uint32_t sbo_a, uint32_t sbo_b, int ksteps,
                                                uint32_t idesc) {
     constexpr int PI[6] = {0, 0, 1, 0, 1, 2}, PJ[6] = {0, 1, 0, 2, 1, 0};
     const uint32_t idesc_neg = idesc | (1u << 13);
     // the start-address field holds addr >> 4 (shared memory < 256 KB): offsets add to it
-    const uint64_t da = make_desc_sbo(a, sbo_a), db = make_desc_sbo(b, sbo_b);
-    const uint32_t ta = (uint32_t)T * a_plane >> 4, tb = (uint32_t)T * b_plane >> 4;
+    const Desc da = desc_words(make_desc_sbo(a, sbo_a)), db = desc_words(make_desc_sbo(b, sbo_b));
+    const uint32_t pa = (uint32_t)a_plane >> 4, pb = (uint32_t)b_plane >> 4;
 #pragma unroll
     for (int i = 0; i < n_products<T>(); ++i) {
         const int q = product_order<T>(i);
         for (int ks = 0; ks < ksteps; ++ks) {
-            const uint64_t ar = da + (uint32_t)(PI[q] * a_plane + ks * 256) / 16, ai = ar + ta;
-            const uint64_t br = db + (uint32_t)(PJ[q] * b_plane + ks * 256) / 16, bi = br + tb;
+            const uint32_t ar = da.lo + PI[q] * pa + ks * 16, ai = ar + T * pa;
+            const uint32_t br = db.lo + PJ[q] * pb + ks * 16, bi = br + T * pb;
             const uint32_t acc = (ks > 0 || i > 0) ? 1u : 0u;
-            mma_bf16(d_re, ar, br, idesc, acc);
-            mma_bf16(d_re, ai, bi, idesc_neg, 1u);
-            mma_bf16(d_im, ar, bi, idesc, acc);
-            mma_bf16(d_im, ai, br, idesc, 1u);
+            mma_lead(lead, d_re, ar, da.hi, br, db.hi, idesc, acc);
+            mma_lead(lead, d_re, ai, da.hi, bi, db.hi, idesc_neg, 1u);
+            mma_lead(lead, d_im, ar, da.hi, bi, db.hi, idesc, acc);
+            mma_lead(lead, d_im, ai, da.hi, br, db.hi, idesc, 1u);
         }
     }
 }
@@ -666,21 +669,21 @@ __device__ __forceinline__ void issue_products(uint32_t d_re, uint32_t d_im, uin
 // 2N-row operand.  d0 += Ar [Br | Bi], d1 += Ai [-Bi | Br]; d0 + d1 is the
 // product (d1 may equal d0).
 template <int T>
-__device__ __forceinline__ void issue_products_cat(uint32_t d0, uint32_t d1, uint32_t a, int a_plane, uint32_t b,
-                                                   int b_slot, uint32_t sbo_a, uint32_t sbo_b, int ksteps,
+__device__ __forceinline__ void issue_products_cat(uint32_t lead, uint32_t d0, uint32_t d1, uint32_t a, int a_plane,
+                                                   uint32_t b, int b_slot, uint32_t sbo_a, uint32_t sbo_b, int ksteps,
                                                    uint32_t idesc) {
     constexpr int PI[6] = {0, 0, 1, 0, 1, 2}, PJ[6] = {0, 1, 0, 2, 1, 0};
-    const uint64_t da = make_desc_sbo(a, sbo_a), db = make_desc_sbo(b, sbo_b);
-    const uint32_t ta = (uint32_t)T * a_plane >> 4;
+    const Desc da = desc_words(make_desc_sbo(a, sbo_a)), db = desc_words(make_desc_sbo(b, sbo_b));
+    const uint32_t pa = (uint32_t)a_plane >> 4, pb = (uint32_t)b_slot >> 4;
 #pragma unroll
     for (int i = 0; i < n_products<T>(); ++i) {  // corrections first, hi x hi last (see issue_products)
         const int q = product_order<T>(i);
         for (int ks = 0; ks < ksteps; ++ks) {
-            const uint64_t ar = da + (uint32_t)(PI[q] * a_plane + ks * 256) / 16, ai = ar + ta;
-            const uint64_t bneg = db + (uint32_t)(3 * PJ[q] * b_slot + ks * 256) / 16, bpos = bneg + b_slot / 16;
+            const uint32_t ar = da.lo + PI[q] * pa + ks * 16, ai = ar + T * pa;
+            const uint32_t bneg = db.lo + 3 * PJ[q] * pb + ks * 16, bpos = bneg + pb;
             const uint32_t acc = (ks > 0 || i > 0) ? 1u : 0u;
-            mma_bf16(d0, ar, bpos, idesc, acc);
-            mma_bf16(d1, ai, bneg, idesc, d1 == d0 ? 1u : acc);
+            mma_lead(lead, d0, ar, da.hi, bpos, db.hi, idesc, acc);
+            mma_lead(lead, d1, ai, da.hi, bneg, db.hi, idesc, d1 == d0 ? 1u : acc);
         }
     }
 }
@@ -981,7 +984,7 @@ __global__ void __launch_bounds__(F34_THREADS) tc_ag34_kernel(const TcCtx c, con
     // F34_EMPTY + b: D2[b] read out
     __shared__ __align__(8) uint64_t mbar[F34_NBAR];
     __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
     const F34Tile t = tiles[blockIdx.x];
     const F34Item it = items[t.item];
     const int K1 = sh.K1, K2 = sh.K2, nt = c.n_theta;
@@ -1027,30 +1030,30 @@ __global__ void __launch_bounds__(F34_THREADS) tc_ag34_kernel(const TcCtx c, con
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
-    const uint32_t tm = tmem_base;
+    const uint32_t tm = (uint32_t)uniform((int)tmem_base);
     // AG4 accumulator set b at d2 + b set: [re | im] of d0, then (two accumulators) of d1
     const uint32_t d2 = tm + 2 * sh.N1s;
     const int nbuf = sh.nbuf, set = 2 * sh.nacc * sh.ntp;
     bool ok = true;
     if (warp == F34_WORKERS / 32) {
-        // ---- MMA warp: AG3 once, then AG4 for every r as soon as its A2 is written
-        if (lane == 0) {
-            issue_products<T>(tm, tm + sh.N1s, smem_u32(sA1), a1p, smem_u32(sB1), b1p, K1 * 16, K1 * 16, K1 / 16,
-                              idesc_bf16(n1p));
-            mma_commit(&mbar[F34_D1]);
-            for (int j = 0; j < t.nr; ++j) {
-                const int a = j & 1, b = j % nbuf;
-                ok = mbar_wait(&mbar[F34_A2 + a], (j >> 1) & 1) && ok;
-                if (j >= nbuf) ok = mbar_wait(&mbar[F34_EMPTY + b], ((j - nbuf) / nbuf) & 1) && ok;
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const uint32_t dr = d2 + b * set;
-                issue_products_cat<T>(dr, dr + (sh.nacc - 1) * 2 * sh.ntp, smem_u32(sA2b + a * 2 * T * a2p), a2p,
-                                      smem_u32(sB2), b2p,
-                                      K2 * 16, K2 * 16, K2 / 16, idesc_bf16(2 * sh.ntp));
-                mma_commit(&mbar[F34_D2 + b]);
-            }
+        // ---- MMA warp (convergent, one lane issues): AG3 once, then AG4 for every r as soon as its
+        // A2 is written
+        const uint32_t lead = elect_lane();
+        const int nr = uniform(t.nr), n1u = uniform(n1p);
+        auto wait = [&](uint64_t* bar, uint32_t parity) { return (bool)__all_sync(0xffffffffu, mbar_wait(bar, parity)); };
+        issue_products<T>(lead, tm, tm + sh.N1s, smem_u32(sA1), a1p, smem_u32(sB1), b1p, K1 * 16, K1 * 16, K1 / 16,
+                          idesc_bf16(n1u));
+        commit_lead(lead, &mbar[F34_D1]);
+        for (int j = 0; j < nr; ++j) {
+            const int a = j & 1, b = nbuf == 2 ? j & 1 : 0;
+            ok = wait(&mbar[F34_A2 + a], (j >> 1) & 1) && ok;
+            if (j >= nbuf) ok = wait(&mbar[F34_EMPTY + b], ((nbuf == 2 ? j >> 1 : j) - 1) & 1) && ok;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const uint32_t dr = d2 + b * set;
+            issue_products_cat<T>(lead, dr, dr + (sh.nacc - 1) * 2 * sh.ntp, smem_u32(sA2b + a * 2 * T * a2p), a2p,
+                                  smem_u32(sB2), b2p, K2 * 16, K2 * 16, K2 / 16, idesc_bf16(2 * sh.ntp));
+            commit_lead(lead, &mbar[F34_D2 + b]);
         }
-        __syncwarp();
     } else {
         // ---- workers: warps w, w + 4, ... share lane quarter w & 3 and split the columns
         const int phi = (warp & 3) * 32 + lane, grp = warp >> 2, ngrp = F34_WORKERS / 128;
@@ -1236,7 +1239,7 @@ __global__ void __launch_bounds__(D1_THREADS) tc_dg1a_kernel(const TcCtx c, cons
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tm = tmem_base;
     if (tid == 0) {
-        issue_products<T>(tm, tm + NP, smem_u32(sA), ap, smem_u32(sB), bp, K * 16, K * 16, K / 16, idesc_bf16(NP));
+        issue_products<T>(1, tm, tm + NP, smem_u32(sA), ap, smem_u32(sB), bp, K * 16, K * 16, K / 16, idesc_bf16(NP));
         mma_commit(&mbar);
     }
     bool ok = mbar_wait(&mbar, 0);
