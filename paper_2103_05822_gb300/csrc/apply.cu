@@ -104,7 +104,57 @@ __device__ __forceinline__ int next_item(unsigned* ctr, unsigned* done, int n_it
     return *s_item;
 }
 
-// out[c] = sum_j M[c][j] v[j] (CONJ: conj(M)); rows of ld2 float4 (2 complex each)
+// One float4 of ROWS rows (nw rows apart) times v, into their sums.
+template <bool CONJ, int ROWS>
+__device__ __forceinline__ void dot_step(float2 (&acc)[ROWS], const float4 (&m)[ROWS], float4 x) {
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+        if (CONJ) {
+            cfma_conj(acc[i], make_float2(m[i].x, m[i].y), make_float2(x.x, x.y));
+            cfma_conj(acc[i], make_float2(m[i].z, m[i].w), make_float2(x.z, x.w));
+        } else {
+            cfma(acc[i], make_float2(m[i].x, m[i].y), make_float2(x.x, x.y));
+            cfma(acc[i], make_float2(m[i].z, m[i].w), make_float2(x.z, x.w));
+        }
+    }
+}
+
+// ROWS rows of out[c] = sum_j M[c][j] v[j] by one warp, c = c0 + nw i.
+template <bool CONJ, int ROWS, class Emit>
+__device__ __forceinline__ void rowdot_group(const float4* __restrict__ M, int ld2, int c0, int nw, const float4* v,
+                                             Emit emit) {
+    const int lane = threadIdx.x & 31;
+    const float4* row = M + (int64_t)c0 * ld2;
+    const int64_t step = (int64_t)nw * ld2;
+    float2 a0[ROWS], a1[ROWS];
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) a0[i] = a1[i] = make_float2(0.f, 0.f);
+    int j = lane;
+    for (; j + 32 < ld2; j += 64) {
+        float4 m0[ROWS], m1[ROWS];
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) {
+            m0[i] = ld_stream(row + i * step + j);
+            m1[i] = ld_stream(row + i * step + j + 32);
+        }
+        dot_step<CONJ, ROWS>(a0, m0, v[j]);
+        dot_step<CONJ, ROWS>(a1, m1, v[j + 32]);
+    }
+    if (j < ld2) {
+        float4 m0[ROWS];
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) m0[i] = ld_stream(row + i * step + j);
+        dot_step<CONJ, ROWS>(a0, m0, v[j]);
+    }
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+        const float2 s = warp_sum(make_float2(a0[i].x + a1[i].x, a0[i].y + a1[i].y));
+        if (lane == 0) emit(c0 + nw * i, s);
+    }
+}
+
+// out[c] = sum_j M[c][j] v[j] (CONJ: conj(M)); rows of ld2 float4 (2 complex each), one row per
+// warp at a time: for long rows, and for kernels that live on many warps (split path, dense).
 template <bool CONJ, class Emit>
 __device__ __forceinline__ void rowdot(const float4* __restrict__ M, int ld2, int nrows, const float4* v, Emit emit) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -123,9 +173,30 @@ __device__ __forceinline__ void rowdot(const float4* __restrict__ M, int ld2, in
                 cfma(a1, make_float2(m.z, m.w), make_float2(x.z, x.w));
             }
         }
-        float2 s = warp_sum(make_float2(a0.x + a1.x, a0.y + a1.y));
+        const float2 s = warp_sum(make_float2(a0.x + a1.x, a0.y + a1.y));
         if (lane == 0) emit(c, s);
     }
+}
+
+// The same, kDotRows rows per warp at a time (persistent kernels).  What a row of a few
+// hundred RWGs costs is the latency of its first loads and of its last, partly filled one: four rows
+// share them, and x is read from shared memory once for all four.  With this and eight loads in
+// flight in rowaxpy, two CTAs of 64 registers beat three of 40: 10-lambda sphere (rows of 260)
+// aggregation 106 -> 81 us, disaggregation 132 -> 87; 30-lambda (rows of 940) 792 -> 777, 868 -> 814.
+// (Drawing the next item early and pulling its first array into L2 meanwhile: slower, 85 / 95 and
+// 808 / 861; the prefetch competes with the running item's own loads.)
+constexpr int kDotRows = 4;
+template <bool CONJ, class Emit>
+__device__ __forceinline__ void rowdot_rows(const float4* __restrict__ M, int ld2, int nrows, const float4* v,
+                                            Emit emit) {
+    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int c = warp;
+    for (; c + (kDotRows - 1) * nw < nrows; c += kDotRows * nw) rowdot_group<CONJ, kDotRows>(M, ld2, c, nw, v, emit);
+    if (c + nw < nrows) {
+        rowdot_group<CONJ, 2>(M, ld2, c, nw, v, emit);
+        c += 2 * nw;
+    }
+    if (c < nrows) rowdot_group<CONJ, 1>(M, ld2, c, nw, v, emit);
 }
 
 // out[j] (float4 = two complex columns) = sum_c M[c][j] s[c]; `part` holds
@@ -134,28 +205,31 @@ template <class Emit>
 __device__ __forceinline__ void rowaxpy(const float4* __restrict__ M, int ld2, int nrows, const float2* s,
                                         float4* part, Emit emit) {
     const int NT = blockDim.x, tid = threadIdx.x;
-    if (2 * ld2 >= NT) {
-        for (int j = tid; j < ld2; j += NT) {
-            float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
-            int c = 0;
-#pragma unroll 4
-            for (; c + 1 < nrows; c += 2) {
-                const float4 m0 = ld_stream(M + (int64_t)c * ld2 + j);
-                const float4 m1 = ld_stream(M + (int64_t)(c + 1) * ld2 + j);
-                cfma2(a0, m0, s[c]);
-                cfma2(a1, m1, s[c + 1]);
+    // rows c0, c0 + st, ... of column j, eight loads in flight
+    auto column = [&](int j, int c0, int st) {
+        float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
+        const float4* col = M + j;
+        int c = c0;
+        for (; c + 7 * st < nrows; c += 8 * st) {
+            float4 m[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) m[i] = ld_stream(col + (int64_t)(c + i * st) * ld2);
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+                cfma2(a0, m[i], s[c + i * st]);
+                cfma2(a1, m[i + 1], s[c + (i + 1) * st]);
             }
-            if (c < nrows) cfma2(a0, ld_stream(M + (int64_t)c * ld2 + j), s[c]);
-            emit(j, add4(a0, a1));
         }
+#pragma unroll 4
+        for (; c < nrows; c += st) cfma2(a0, ld_stream(col + (int64_t)c * ld2), s[c]);
+        return add4(a0, a1);
+    };
+    if (2 * ld2 >= NT) {
+        for (int j = tid; j < ld2; j += NT) emit(j, column(j, 0, 1));
     } else {
         const int S = NT / ld2;  // >= 2 slices of rows
         const int j = tid % ld2, sl = tid / ld2;
-        if (sl < S) {
-            float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int c = sl; c < nrows; c += S) cfma2(a0, ld_stream(M + (int64_t)c * ld2 + j), s[c]);
-            part[sl * ld2 + j] = a0;
-        }
+        if (sl < S) part[sl * ld2 + j] = column(j, sl, S);
         __syncthreads();
         for (int jj = tid; jj < ld2; jj += NT) {
             float4 a = part[jj];
@@ -229,7 +303,7 @@ struct AggArgs {
 // format with identity theta / phi factors, core C_(3) = (U Sigma)^T and U_beta =
 // conj(V): the spectrum is AG1 followed by AG2 written straight to it.
 template <bool SVD>
-__global__ void __launch_bounds__(512, 3) tucker_aggregate_kernel(const AggArgs a) {
+__global__ void __launch_bounds__(512, 2) tucker_aggregate_kernel(const AggArgs a) {
     extern __shared__ float4 smem4[];
     float2* sm = reinterpret_cast<float2*>(smem4);
     __shared__ int s_item;
@@ -263,7 +337,7 @@ __global__ void __launch_bounds__(512, 3) tucker_aggregate_kernel(const AggArgs 
                 s_x[n] = n < d.n_beta ? a.x[(int64_t)a.grp_rwg[d.rwg + n] + a.ldx * r] : make_float2(0.f, 0.f);
             __syncthreads();
             // AG1: t[c] = sum_n U_beta[n, c] x_n
-            rowdot<false>(reinterpret_cast<const float4*>(Ub), d.ld_nb / 2, d.rb, reinterpret_cast<const float4*>(s_x),
+            rowdot_rows<false>(reinterpret_cast<const float4*>(Ub), d.ld_nb / 2, d.rb, reinterpret_cast<const float4*>(s_x),
                           [&](int c, float2 v) { s_t[c] = v; });
             __syncthreads();
             if (SVD) {
@@ -321,7 +395,7 @@ struct DisArgs {
 // Disaggregation (Fig. 3b) of one group (both alpha) per work item.  SVD (see the
 // aggregation): H is conj(W g) itself, then DG2 and DG3.
 template <bool SVD>
-__global__ void __launch_bounds__(512, 3) tucker_disaggregate_kernel(const DisArgs a) {
+__global__ void __launch_bounds__(512, 2) tucker_disaggregate_kernel(const DisArgs a) {
     extern __shared__ float4 smem4[];
     float2* sm = reinterpret_cast<float2*>(smem4);
     __shared__ int s_item;
@@ -388,7 +462,7 @@ __global__ void __launch_bounds__(512, 3) tucker_disaggregate_kernel(const DisAr
                 __syncthreads();
                 }
                 // DG2: s[c] = sum_ab C_(3)[c, ab] H[ab]
-                rowdot<false>(reinterpret_cast<const float4*>(Cc), d.ld_ab / 2, d.rb,
+                rowdot_rows<false>(reinterpret_cast<const float4*>(Cc), d.ld_ab / 2, d.rb,
                               reinterpret_cast<const float4*>(s_H), [&](int c, float2 v) { s_s[c] = v; });
                 __syncthreads();
                 if (tid == 0 && al == 0) {  // the next component's C while this one's U_beta streams
@@ -910,6 +984,15 @@ void finalize_hot_layout(Plan& P, cudaStream_t s) {
     TFMM_CUDA_CHECK(device_malloc(&P.d_items, sizeof(TuckerItem) * nI));
     TFMM_CUDA_CHECK(cudaMemcpyAsync(P.d_items, P.items.data(), sizeof(TuckerItem) * nI, cudaMemcpyHostToDevice, s));
     configure_small(P, s);
+    // CTAs of 256 threads, four per SM, for plans of many small items: a short item leaves half of
+    // 16 warps idle in most phases, and four CTAs in different phases fill DRAM better than two.
+    // Measured 512 / 256 threads (us): aggregation, 3646 items of 0.18 MB 167 / 136, 5130 of 0.11 MB
+    // 187 / 143, 1264 of 0.25 MB 82 / 73, 3646 of 0.45 MB 313 / 293, but 832 of 0.49 MB 81 / 82 and 832 of
+    // 1.2 MB 169 / 192; disaggregation, 1823 groups of 0.18 MB items 173 / 147, 632 of 0.25 MB 96 / 89,
+    // but 1823 of 0.45 MB 322 / 327 and 416 of 0.49 MB (less than a CTA per slot) 87 / 112.
+    const int64_t item = (int64_t)sizeof(float2) * P.factor_elems / nI;
+    P.tuning.agg_threads = item <= 448 * 1024 && nI >= 4 * P.num_sms ? 256 : 512;
+    P.tuning.dis_threads = item <= 300 * 1024 && P.G >= 4 * P.num_sms ? 256 : 512;
     configure_hot(P, P.tuning, s);
 }
 

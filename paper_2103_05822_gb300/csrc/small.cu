@@ -441,14 +441,12 @@ void configure_small(Plan& P, cudaStream_t s) {
     TFMM_CUDA_CHECK(cudaMemcpyAsync(P.small_order.p, order.data(), sizeof(int) * P.G, cudaMemcpyHostToDevice, s));
     TFMM_CUDA_CHECK(cudaStreamSynchronize(s));
     P.small_ok = true;
-    // One column: taken while two CTAs fit an SM (one loads while the other computes), or while
-    // there are so few items that the SMs hold nearly all at once.  Measured (aggregation +
-    // disaggregation in graphs, persistent kernels / this): 7240 groups of 60 KB items 578 / 425 us,
-    // 631 groups 66 / 41, 56 groups 31 / 21; 120 KB items, one CTA per SM: 271 groups 46 / 39, 1147
-    // groups 123 / 144, 7240 groups 697 / 1130.
-    const SmallClass& k = P.small_classes[0];
-    const size_t one = sizeof(float2) * std::max(agg_work(P, k, 1).total, dis_work(P, k, 1).total);
-    P.small_one = one <= kHalfSM || 2 * P.G <= 4 * P.num_sms;
+    // One column: taken while the SMs hold all items in at most a round and a half, where one launch
+    // with everything requested at once wins; with more, the persistent kernels keep DRAM busy through
+    // each other's phases.  Measured (aggregation + disaggregation, persistent kernels / this, us): 56
+    // groups of up to 90 KB 27 / 20, 271 of 120 KB 36 / 37, 631 of 60 KB 50 / 76, 1391 of 120 KB 105 / 193,
+    // 7240 of 60 KB 440 / 448.
+    P.small_one = 2 * P.G <= 3 * P.num_sms;
 }
 
 void launch_small_aggregate(const Plan& P, const float2* x, int R, int64_t ldx, float2* spec, cudaStream_t s) {

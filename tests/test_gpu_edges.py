@@ -194,3 +194,22 @@ def test_disaggregation_first_step_forms(nt, npf, top, R):
     ranks = [[(rt, rp, 24), (max(1, rt - 1), max(1, rp - 1), 20)], [(rt, min(rp, 33), 100), (max(1, rt // 2), rp, 9)],
              [(max(1, rt - 3), min(rp, 8), 64), (rt, max(1, rp // 2), 90)]]
     _check(5000 + 10 * nt + R, nt, npf, nbetas, ranks, R, 3, 1e-6, betas=(0.5 - 0.25j,))
+
+
+@pytest.mark.parametrize("threads", [64, 256, 512])
+def test_persistent_row_groups(threads, monkeypatch):
+    """Rows taken four, two and one at a time by 2, 8 and 16 warps, row lengths around 64 and 128
+    complex numbers, core columns split into slices and not."""
+    from paper_2103_05822_gb300 import tfmm
+    made = tfmm.tfmm_plan_from_tucker
+
+    def persistent(*args, **kw):
+        plan = made(*args, **kw)
+        tfmm.tfmm_plan_tuning_set(plan, agg_threads=threads, dis_threads=threads, single_rhs_split=2)
+        return plan
+
+    monkeypatch.setattr(tfmm, "tfmm_plan_from_tucker", persistent)
+    nbetas = [8, 63, 64, 66, 127, 130, 260, 515]
+    rb = [2, 15, 16, 17, 47, 64, 65, 130]
+    ranks = [[(5, 4, r), (7, 13, max(2, r - 1))] for r in rb]
+    _check(6000 + threads, 10, 20, nbetas, ranks, 1, 0, 1e-5, pad=1)
