@@ -681,8 +681,8 @@ SmemLayout dis_layout(const Plan& P, int NT) {
 // plan-owned scratch (t / s: r_beta, M / H: ld_ab complex per item):
 //   aggregation     SA1: t = U_beta^T x_g, blocks of kSplitRows rows per CTA (Fig. 2b step 1)
 //                   SA2: M = C_(3)^T t, blocks of kSplitCols column pairs per CTA
-//                   SA3: AG3 + AG4 from M, one CTA per item (Fig. 2b steps 2-4)
-//   disaggregation  SD1: H = U_theta^T conj(W g) U_phi, one CTA per item (Fig. 3b step 1)
+//                   SA3: AG3 + AG4 from M, blocks of phi directions (Fig. 2b steps 2-4)
+//   disaggregation  SD1: H = U_theta^T (conj(W g) U_phi), blocks of U_phi's columns (Fig. 3b step 1)
 //                   SD2: s = C_(3) vec(H), blocks of rows (step 2)
 //                   SD3: y_g = beta y_g + conj(sum_alpha U_beta s), blocks of column pairs of
 //                        U_beta^T covering both components of a group (step 3)
@@ -707,6 +707,7 @@ struct SplitArgs {
     float2* scratch;      // per item: [r_beta slot | ld_ab slot] (offsets in TuckerItem order)
     const int64_t* scr_off;
     int n_theta, n_phi, n_dir, G, r;
+    int blk;              // SA3: phi directions, SD1: columns of U_phi per CTA
     SmemLayout L;
 };
 
@@ -721,14 +722,17 @@ __device__ __forceinline__ void colblock_axpy(const float4* __restrict__ M, int6
     if (j < cbv && sl < S) {
         const float4* col = M + j0 + j;
         int c = sl;
-#pragma unroll 2
-        for (; c + S < nrows; c += 2 * S) {
-            const float4 m0 = ld_stream(col + (int64_t)c * ld2);
-            const float4 m1 = ld_stream(col + (int64_t)(c + S) * ld2);
-            cfma2(a0, m0, s[c]);
-            cfma2(a1, m1, s[c + S]);
+        for (; c + 3 * S < nrows; c += 4 * S) {  // four loads in flight (eight cost a resident CTA: slower)
+            float4 m[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) m[i] = ld_stream(col + (int64_t)(c + i * S) * ld2);
+#pragma unroll
+            for (int i = 0; i < 4; i += 2) {
+                cfma2(a0, m[i], s[c + i * S]);
+                cfma2(a1, m[i + 1], s[c + (i + 1) * S]);
+            }
         }
-        if (c < nrows) cfma2(a0, ld_stream(col + (int64_t)c * ld2), s[c]);
+        for (; c < nrows; c += S) cfma2(a0, ld_stream(col + (int64_t)c * ld2), s[c]);
     }
     if (sl < S) part[sl * kSplitCols + j] = add4(a0, a1);
     __syncthreads();
@@ -745,17 +749,19 @@ __global__ void __launch_bounds__(512) split_ag1_kernel(const SplitArgs a) {
     float2* s_x = reinterpret_cast<float2*>(smem4);
     const SplitTile t = a.tiles[blockIdx.x];
     const TuckerItem d = a.items[t.item];
+    const int rows = min(kSplitRows, d.rb - t.start);
+    if (threadIdx.x == 0)  // the rows start towards L2 while x is gathered
+        prefetch_head_l2(a.fac + d.ub + (int64_t)t.start * d.ld_nb, (int64_t)rows * d.ld_nb * 8);
     for (int n = threadIdx.x; n < d.ld_nb; n += blockDim.x)
         s_x[n] = n < d.n_beta ? a.x[(int64_t)a.grp_rwg[d.rwg + n] + a.ldx * a.r] : make_float2(0.f, 0.f);
     __syncthreads();
     float2* tout = a.scratch + a.scr_off[t.item];
-    const int rows = min(kSplitRows, d.rb - t.start);
     rowdot<false>(reinterpret_cast<const float4*>(a.fac + d.ub) + (int64_t)t.start * (d.ld_nb / 2), d.ld_nb / 2, rows,
                   reinterpret_cast<const float4*>(s_x), [&](int c, float2 v) { tout[t.start + c] = v; });
 }
 
 // SA2: M[ab] = sum_c C_(3)[c, ab] t[c] for the column pairs of one tile
-__global__ void __launch_bounds__(512) split_ag2_kernel(const SplitArgs a) {
+__global__ void __launch_bounds__(512, 3) split_ag2_kernel(const SplitArgs a) {
     extern __shared__ float4 smem4[];
     float4* s_part = smem4;
     float2* s_t = reinterpret_cast<float2*>(smem4 + blockDim.x);
@@ -770,7 +776,9 @@ __global__ void __launch_bounds__(512) split_ag2_kernel(const SplitArgs a) {
                   s_t, s_part, [&](int j, float4 v) { mout[j] = v; });
 }
 
-// SA3: AG3 + AG4 of one item from its M (one CTA per item)
+// SA3: AG3 + AG4 of a.blk phi directions of one item from its M.  The directions are
+// independent, so a plan of few items spreads them over the SMs: with one CTA per item the trihedral's 38
+// items took 14 us for latency alone (SA3 and SD1 alike), in blocks 9 and 12 us.
 __global__ void __launch_bounds__(512) split_ag34_kernel(const SplitArgs a) {
     extern __shared__ float4 smem4[];
     float2* sm = reinterpret_cast<float2*>(smem4);
@@ -778,60 +786,65 @@ __global__ void __launch_bounds__(512) split_ag34_kernel(const SplitArgs a) {
     float2* s_up = sm + a.L.o_b;
     float2* s_V = sm + a.L.o_c;
     float2* s_M = sm + a.L.o_e;
-    const int q = blockIdx.x, NT = blockDim.x, tid = threadIdx.x;
+    const SplitTile t = a.tiles[blockIdx.x];
+    const int q = t.item, p0 = t.start, np = min(a.blk, a.n_phi - p0), NT = blockDim.x, tid = threadIdx.x;
     const TuckerItem d = a.items[q];
     const float2* Ut = a.fac + d.uth;
-    const float2* Up = a.fac + d.uphi;
+    const float2* Up = a.fac + d.uphi + p0;
     const float2* min_ = a.scratch + a.scr_off[q] + round_up_dev(d.rb, 2);
     for (int e = tid; e < a.n_theta * d.rt; e += NT) s_ut[(e % a.n_theta) + a.L.ldt * (e / a.n_theta)] = Ut[e];
-    for (int e = tid; e < a.n_phi * d.rp; e += NT) s_up[(e % a.n_phi) + a.L.ldp * (e / a.n_phi)] = Up[e];
+    for (int e = tid; e < np * d.rp; e += NT) s_up[(e % np) + a.L.ldp * (e / np)] = Up[(e % np) + (int64_t)a.n_phi * (e / np)];
     for (int e = tid; e < d.rt * d.rp; e += NT) s_M[e] = min_[e];
     __syncthreads();
     {
         const int ldp = a.L.ldp, ldv = a.L.ldv, rt = d.rt;
-        smem_gemm<2, 2>(a.n_phi, rt, d.rp, [&](int ip, int b) { return s_up[ip + ldp * b]; },
+        smem_gemm<1, 2>(np, rt, d.rp, [&](int ip, int b) { return s_up[ip + ldp * b]; },
                         [&](int b, int aa) { return s_M[aa + rt * b]; },
                         [&](int ip, int aa, float2 v) { s_V[ip + ldv * aa] = v; });
     }
     __syncthreads();
-    float2* out = a.spec_out + (((int64_t)a.r * a.G + d.g) * 2 + d.alpha) * a.n_dir;
+    float2* out = a.spec_out + (((int64_t)a.r * a.G + d.g) * 2 + d.alpha) * a.n_dir + (int64_t)a.n_theta * p0;
     const int ldt = a.L.ldt, ldv = a.L.ldv, nth = a.n_theta;
-    smem_gemm<2, 4>(nth, a.n_phi, d.rt, [&](int it, int aa) { return s_ut[it + ldt * aa]; },
+    smem_gemm<1, 2>(nth, np, d.rt, [&](int it, int aa) { return s_ut[it + ldt * aa]; },
                     [&](int aa, int ip) { return s_V[ip + ldv * aa]; },
                     [&](int it, int ip, float2 v) { out[it + nth * ip] = v; });
 }
 
-// SD1: H = U_theta^T conj(W g) U_phi of one item (one CTA per item), zero-padded to ld_ab
+// SD1: columns b of H = U_theta^T (conj(W g) U_phi) for a.blk columns of U_phi of one item; the
+// last block zero-pads H to ld_ab.  (U_phi first: a block then needs all of g but a share of the work.)
 __global__ void __launch_bounds__(512) split_dg1_kernel(const SplitArgs a) {
     extern __shared__ float4 smem4[];
     float2* sm = reinterpret_cast<float2*>(smem4);
     float2* s_ut = sm + a.L.o_a;
     float2* s_up = sm + a.L.o_b;
     float2* s_G = sm + a.L.o_f;
-    float2* s_P = sm + a.L.o_g;
-    const int q = blockIdx.x, NT = blockDim.x, tid = threadIdx.x;
+    float2* s_Q = sm + a.L.o_g;  // [i_theta][b - b0]
+    const SplitTile t = a.tiles[blockIdx.x];
+    const int q = t.item, b0 = t.start, NT = blockDim.x, tid = threadIdx.x;
     const TuckerItem d = a.items[q];
+    const int nb = min(a.blk, d.rp - b0);
     const float2* Ut = a.fac + d.uth;
-    const float2* Up = a.fac + d.uphi;
+    const float2* Up = a.fac + d.uphi + (int64_t)a.n_phi * b0;
     const float2* gin = a.spec + (((int64_t)a.r * a.G + d.g) * 2 + d.alpha) * a.n_dir;
-    for (int e = tid; e < a.n_theta * d.rt; e += NT) s_ut[(e % a.n_theta) + a.L.ldt * (e / a.n_theta)] = Ut[e];
-    for (int e = tid; e < a.n_phi * d.rp; e += NT) s_up[(e % a.n_phi) + a.L.ldp * (e / a.n_phi)] = Up[e];
     for (int o = tid; o < a.n_dir; o += NT) {
         const float2 v = gin[o];
         const float wt = a.w ? a.w[o] : 1.0f;
         s_G[(o % a.n_theta) + a.L.ldg * (o / a.n_theta)] = make_float2(wt * v.x, -wt * v.y);
     }
+    for (int e = tid; e < a.n_theta * d.rt; e += NT) s_ut[(e % a.n_theta) + a.L.ldt * (e / a.n_theta)] = Ut[e];
+    for (int e = tid; e < a.n_phi * nb; e += NT) s_up[(e % a.n_phi) + a.L.ldp * (e / a.n_phi)] = Up[e];
     __syncthreads();
-    const int ldt = a.L.ldt, ldg = a.L.ldg, ldp = a.L.ldp, rt = d.rt;
-    smem_gemm<2, 4>(rt, a.n_phi, a.n_theta, [&](int aa, int it) { return s_ut[it + ldt * aa]; },
-                    [&](int it, int ip) { return s_G[it + ldg * ip]; },
-                    [&](int aa, int ip, float2 v) { s_P[aa + rt * ip] = v; });
+    const int ldt = a.L.ldt, ldg = a.L.ldg, ldp = a.L.ldp, rt = d.rt, ldq = a.L.ldv;
+    smem_gemm<1, 1>(a.n_theta, nb, a.n_phi, [&](int it, int ip) { return s_G[it + ldg * ip]; },
+                    [&](int ip, int b) { return s_up[ip + ldp * b]; },
+                    [&](int it, int b, float2 v) { s_Q[it + ldq * b] = v; });
     __syncthreads();
     float2* hout = a.scratch + a.scr_off[q] + round_up_dev(d.rb, 2);
-    smem_gemm<2, 2>(rt, d.rp, a.n_phi, [&](int aa, int ip) { return s_P[aa + rt * ip]; },
-                    [&](int ip, int b) { return s_up[ip + ldp * b]; },
-                    [&](int aa, int b, float2 v) { hout[aa + rt * b] = v; });
-    for (int o = rt * d.rp + tid; o < d.ld_ab; o += NT) hout[o] = make_float2(0.f, 0.f);
+    smem_gemm<1, 1>(rt, nb, a.n_theta, [&](int aa, int it) { return s_ut[it + ldt * aa]; },
+                    [&](int it, int b) { return s_Q[it + ldq * b]; },
+                    [&](int aa, int b, float2 v) { hout[aa + rt * (b0 + b)] = v; });
+    if (b0 + nb == d.rp)
+        for (int o = rt * d.rp + tid; o < d.ld_ab; o += NT) hout[o] = make_float2(0.f, 0.f);
 }
 
 // SD2: s[c] = sum_ab C_(3)[c, ab] H[ab] for the rows c of one tile
@@ -851,7 +864,7 @@ __global__ void __launch_bounds__(512) split_dg2_kernel(const SplitArgs a) {
 
 // SD3: y = beta y + conj(U_beta^(0) s^(0) + U_beta^(1) s^(1)) for the column pairs of one
 // tile of group t.item (both components)
-__global__ void __launch_bounds__(512) split_dg3_kernel(const SplitArgs a) {
+__global__ void __launch_bounds__(512, 3) split_dg3_kernel(const SplitArgs a) {
     extern __shared__ float4 smem4[];
     float4* s_part = smem4;
     float4* s_acc = smem4 + blockDim.x;
@@ -885,6 +898,33 @@ __global__ void __launch_bounds__(512) split_dg3_kernel(const SplitArgs a) {
         }
         *dst = v;
     }
+}
+
+// Shared memory of SA3 (a block of phi directions) and SD1 (a block of U_phi's columns).
+SmemLayout split_ag34_layout(const Plan& P, int blk) {
+    SmemLayout L{};
+    L.ldt = odd_ld(P.n_theta);
+    L.ldp = L.ldv = odd_ld(blk);
+    int o = 0;
+    L.o_a = o; o += al16(L.ldt * P.max_rank[0]);
+    L.o_b = o; o += al16(L.ldp * P.max_rank[1]);
+    L.o_c = o; o += al16(L.ldv * P.max_rank[0]);
+    L.o_e = o; o += al16(P.max_ldab);
+    L.total = o;
+    return L;
+}
+
+SmemLayout split_dg1_layout(const Plan& P, int blk) {
+    SmemLayout L{};
+    L.ldt = L.ldg = L.ldv = odd_ld(P.n_theta);
+    L.ldp = odd_ld(P.n_phi);
+    int o = 0;
+    L.o_a = o; o += al16(L.ldt * P.max_rank[0]);
+    L.o_b = o; o += al16(L.ldp * blk);
+    L.o_f = o; o += al16(L.ldg * P.n_phi);
+    L.o_g = o; o += al16(L.ldv * blk);
+    L.total = o;
+    return L;
 }
 
 template <class K>
@@ -997,6 +1037,7 @@ void finalize_hot_layout(Plan& P, cudaStream_t s) {
 }
 
 void configure_split(Plan& P, cudaStream_t s);
+bool split_fits(const Plan& P);
 
 // Queue orders (0: most factor bytes first, the LPT rule; 1: group order) and
 // persistent grids (threads per CTA, CTAs per SM capped by occupancy) of the
@@ -1041,8 +1082,14 @@ void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s) {
                                     t.dis_ctas_per_sm);
     }
     P.tuning = t;
-    P.hot_ok = P.agg_sched.blocks > 0 && P.dis_sched.blocks > 0;
-    const bool want_split = !plan_is_svd(P) && P.hot_ok && (t.split == 1 || (t.split == 0 && nI < 2 * P.num_sms));
+    // The split path needs less shared memory than the persistent kernels (a block of the theta /
+    // phi work at a time), so it also takes the plans whose items do not fit those: 4-lambda boxes, which
+    // ran the grouped-GEMM chain on 64-column tiles for one column (50 groups of up to 7273 RWGs, both
+    // stages: 5.26 -> 0.55 ms).
+    P.persistent_ok = P.agg_sched.blocks > 0 && P.dis_sched.blocks > 0;
+    const bool want_split = !plan_is_svd(P) && split_fits(P) &&
+                            (t.split == 1 || (t.split == 0 && (nI < 2 * P.num_sms || !P.persistent_ok)));
+    P.hot_ok = P.persistent_ok || want_split;
     if (want_split != (bool)P.split) {  // captured graphs point into the split path's scratch
         TFMM_REQUIRE(P.live_graphs == 0, "destroy the plan's graphs before changing the single-RHS path");
         P.split.reset();
@@ -1051,11 +1098,36 @@ void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s) {
     TFMM_CUDA_CHECK(cudaStreamSynchronize(s));
 }
 
+// Block sizes and shared memory of the split path's kernels.
+void split_smem(const Plan& P, SplitPlan& S) {
+    const int nI = P.G * 2, NT = 512;
+    // blocks of SA3 and SD1: about two CTAs per SM over all items, at least 8 directions or 4 columns each
+    const int parts = std::max(4, (2 * P.num_sms + nI - 1) / nI);
+    S.blk_phi = std::max(8, (P.n_phi + parts - 1) / parts);
+    S.blk_b = std::max(4, (P.max_rank[1] + parts - 1) / parts);
+    S.smem_ag1 = sizeof(float2) * al16(P.max_ldnb);
+    S.smem_ag2 = sizeof(float4) * NT + sizeof(float2) * al16(P.max_rank[2]);
+    S.smem_ag34 = sizeof(float2) * split_ag34_layout(P, S.blk_phi).total;
+    S.smem_dg1 = sizeof(float2) * split_dg1_layout(P, S.blk_b).total;
+    S.smem_dg2 = sizeof(float2) * al16(P.max_ldab);
+    S.smem_dg3 = sizeof(float4) * (NT + kSplitCols) + sizeof(float2) * al16(P.max_rank[2]);
+}
+
+bool split_fits(const Plan& P) {
+    SplitPlan S;
+    split_smem(P, S);
+    int dev = 0, opt_in = 0;
+    TFMM_CUDA_CHECK(cudaGetDevice(&dev));
+    TFMM_CUDA_CHECK(cudaDeviceGetAttribute(&opt_in, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    return std::max({S.smem_ag1, S.smem_ag2, S.smem_ag34, S.smem_dg1, S.smem_dg2, S.smem_dg3}) <= (size_t)opt_in;
+}
+
 // Tile lists, scratch and shared-memory sizes of the split path.
 void configure_split(Plan& P, cudaStream_t s) {
     auto SP = std::make_unique<SplitPlan>();
-    const int nI = P.G * 2, NT = 512;
-    std::vector<SplitTile> a1, a2, d2, d3;
+    const int nI = P.G * 2;
+    split_smem(P, *SP);
+    std::vector<SplitTile> a1, a2, a3, d1, d2, d3;
     std::vector<int64_t> off(nI);
     int64_t tot = 0;
     for (int q = 0; q < nI; ++q) {
@@ -1067,9 +1139,23 @@ void configure_split(Plan& P, cudaStream_t s) {
             d2.push_back(SplitTile{q, c});
         }
         for (int j = 0; j < d.ld_ab / 2; j += kSplitCols) a2.push_back(SplitTile{q, j});
+        for (int p0 = 0; p0 < P.n_phi; p0 += SP->blk_phi) a3.push_back(SplitTile{q, p0});
+        for (int b = 0; b < d.rp; b += SP->blk_b) d1.push_back(SplitTile{q, b});
     }
     for (int g = 0; g < P.G; ++g)
         for (int j = 0; j < P.items[2 * g].ld_nb / 2; j += kSplitCols) d3.push_back(SplitTile{g, j});
+    // Most bytes first: nearly all tiles of a launch are resident at once, dealt to the SMs in order,
+    // so that each SM gets its share of the long rows (a tile of the trihedral's streams 10 to 600 KB).
+    auto by_bytes = [&](std::vector<SplitTile>& v, auto bytes) {
+        std::stable_sort(v.begin(), v.end(), [&](const SplitTile& x, const SplitTile& y) { return bytes(x) > bytes(y); });
+    };
+    by_bytes(a1, [&](const SplitTile& t) { return (int64_t)std::min(kSplitRows, P.items[t.item].rb - t.start) * P.items[t.item].ld_nb; });
+    by_bytes(d2, [&](const SplitTile& t) { return (int64_t)std::min(kSplitRows, P.items[t.item].rb - t.start) * P.items[t.item].ld_ab; });
+    by_bytes(a2, [&](const SplitTile& t) { return (int64_t)std::min(kSplitCols, P.items[t.item].ld_ab / 2 - t.start) * P.items[t.item].rb; });
+    by_bytes(d3, [&](const SplitTile& t) {
+        const TuckerItem &x = P.items[2 * t.item], &y = P.items[2 * t.item + 1];
+        return (int64_t)std::min(kSplitCols, x.ld_nb / 2 - t.start) * (x.rb + y.rb);
+    });
     auto up = [&](DeviceBuffer& b, const std::vector<SplitTile>& v, int& n) {
         n = (int)v.size();
         TFMM_CUDA_CHECK(device_malloc(&b.p, sizeof(SplitTile) * std::max<size_t>(v.size(), 1)));
@@ -1077,17 +1163,13 @@ void configure_split(Plan& P, cudaStream_t s) {
     };
     up(SP->t_ag1, a1, SP->n_ag1);
     up(SP->t_ag2, a2, SP->n_ag2);
+    up(SP->t_ag34, a3, SP->n_ag34);
+    up(SP->t_dg1, d1, SP->n_dg1);
     up(SP->t_dg2, d2, SP->n_dg2);
     up(SP->t_dg3, d3, SP->n_dg3);
     TFMM_CUDA_CHECK(device_malloc(&SP->scratch.p, sizeof(float2) * std::max<int64_t>(tot, 1)));
     TFMM_CUDA_CHECK(device_malloc(&SP->scr_off.p, sizeof(int64_t) * nI));
     TFMM_CUDA_CHECK(cudaMemcpyAsync(SP->scr_off.p, off.data(), sizeof(int64_t) * nI, cudaMemcpyHostToDevice, s));
-    SP->smem_ag1 = sizeof(float2) * al16(P.max_ldnb);
-    SP->smem_ag2 = sizeof(float4) * NT + sizeof(float2) * al16(P.max_rank[2]);
-    SP->smem_ag34 = sizeof(float2) * agg_layout(P, NT).total;
-    SP->smem_dg1 = sizeof(float2) * dis_layout(P, NT).total;
-    SP->smem_dg2 = sizeof(float2) * al16(P.max_ldab);
-    SP->smem_dg3 = sizeof(float4) * (NT + kSplitCols) + sizeof(float2) * al16(P.max_rank[2]);
     auto allow = [](const void* k, size_t bytes) {
         if (bytes > 48 * 1024) TFMM_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
     };
@@ -1166,8 +1248,10 @@ void launch_split_aggregate(const Plan& P, const float2* x, int R, int64_t ldx, 
         split_ag1_kernel<<<S.n_ag1, 512, S.smem_ag1, s>>>(a);
         a.tiles = static_cast<const SplitTile*>(S.t_ag2.p);
         split_ag2_kernel<<<S.n_ag2, 512, S.smem_ag2, s>>>(a);
-        a.L = agg_layout(P, 512);
-        split_ag34_kernel<<<P.G * 2, 512, S.smem_ag34, s>>>(a);
+        a.tiles = static_cast<const SplitTile*>(S.t_ag34.p);
+        a.blk = S.blk_phi;
+        a.L = split_ag34_layout(P, S.blk_phi);
+        split_ag34_kernel<<<S.n_ag34, 512, S.smem_ag34, s>>>(a);
         TFMM_CUDA_CHECK(cudaGetLastError());
     }
 }
@@ -1182,8 +1266,10 @@ void launch_split_disaggregate(const Plan& P, const float2* spec, int R, int wei
         a.y = y;
         a.ldy = ldy;
         a.beta = beta;
-        a.L = dis_layout(P, 512);
-        split_dg1_kernel<<<P.G * 2, 512, S.smem_dg1, s>>>(a);
+        a.tiles = static_cast<const SplitTile*>(S.t_dg1.p);
+        a.blk = S.blk_b;
+        a.L = split_dg1_layout(P, S.blk_b);
+        split_dg1_kernel<<<S.n_dg1, 512, S.smem_dg1, s>>>(a);
         a.tiles = static_cast<const SplitTile*>(S.t_dg2.p);
         split_dg2_kernel<<<S.n_dg2, 512, S.smem_dg2, s>>>(a);
         a.tiles = static_cast<const SplitTile*>(S.t_dg3.p);

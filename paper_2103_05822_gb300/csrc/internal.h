@@ -220,8 +220,9 @@ struct HotTuning {
 // Split path of the single-RHS stages (plans with few, large items): tile lists of the
 // row- and column-block launches and the items' intermediates.
 struct SplitPlan {
-    DeviceBuffer t_ag1, t_ag2, t_dg2, t_dg3;  // SplitTile lists
-    int n_ag1 = 0, n_ag2 = 0, n_dg2 = 0, n_dg3 = 0;
+    DeviceBuffer t_ag1, t_ag2, t_ag34, t_dg1, t_dg2, t_dg3;  // SplitTile lists
+    int n_ag1 = 0, n_ag2 = 0, n_ag34 = 0, n_dg1 = 0, n_dg2 = 0, n_dg3 = 0;
+    int blk_phi = 0, blk_b = 0;               // phi directions per SA3 tile, columns of U_phi per SD1 tile
     DeviceBuffer scratch;                     // per item: r_beta (padded to 2) + ld_ab complex
     DeviceBuffer scr_off;                     // per item: offset of its slot (complex elements)
     size_t smem_ag1 = 0, smem_ag2 = 0, smem_ag34 = 0, smem_dg1 = 0, smem_dg2 = 0, smem_dg3 = 0;
@@ -282,7 +283,8 @@ struct Plan {
     HotTuning tuning;
     int tc_f34_n1 = 0;                 // cap on r_theta x RHS per CTA of the fused AG3+AG4 kernel (0: largest that fits)
     int tc_dg1a_pairs = 0;             // (i_phi, r) pairs per CTA of the DG1a kernel (0: 128 when it fits, else 64)
-    bool hot_ok = false;               // the single-RHS kernels fit (shared memory of the largest item)
+    bool persistent_ok = false;        // the persistent single-RHS kernels fit (shared memory of the largest item)
+    bool hot_ok = false;               // they or the split path run
     bool small_ok = false;             // every item's factors and one column fit one CTA's shared memory
     bool small_one = false;            // and that is the faster way for one right-hand side
     std::vector<SmallClass> small_classes;

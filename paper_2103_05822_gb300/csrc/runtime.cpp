@@ -399,9 +399,9 @@ tfmm_status tfmm_plan_tuning_set(tfmm_plan* plan, const tfmm_tuning* t, void* st
         h.dis_threads = t->dis_threads; h.dis_ctas_per_sm = t->dis_ctas_per_sm; h.dis_order = t->dis_order;
         h.split = t->single_rhs_split;
         const HotTuning old = plan->p.tuning;
-        const bool was_ok = plan->p.hot_ok;
+        const bool was_ok = plan->p.persistent_ok;
         configure_hot(plan->p, h, (cudaStream_t)stream);
-        if (was_ok && !plan->p.hot_ok) {
+        if (was_ok && !plan->p.persistent_ok) {
             configure_hot(plan->p, old, (cudaStream_t)stream);
             fail(TFMM_INVALID_ARG, "launch shape leaves no room for the largest work item");
         }

@@ -213,3 +213,29 @@ def test_persistent_row_groups(threads, monkeypatch):
     rb = [2, 15, 16, 17, 47, 64, 65, 130]
     ranks = [[(5, 4, r), (7, 13, max(2, r - 1))] for r in rb]
     _check(6000 + threads, 10, 20, nbetas, ranks, 1, 0, 1e-5, pad=1)
+
+
+@pytest.mark.parametrize("split", [0, 1])
+def test_split_path_blocks(split):
+    """Blocks of phi directions and of U_phi's columns with remainders; with `split` 0 the items are too
+    large for the persistent kernels' shared memory, so that the split path takes them by itself."""
+    from paper_2103_05822_gb300 import tfmm
+    nbetas = [9, 700, 12000] if split == 0 else [9, 33, 700]
+    nt, npf = (66, 131) if split == 0 else (11, 23)
+    top = [(5, 7, 9), (20, 41, 30), (11, 40, 17)] if split == 0 else [(3, 5, 9), (11, 23, 33), (7, 10, 65)]
+    ranks = [[r, (max(1, r[0] - 2), max(1, r[1] - 3), r[2])] for r in top]
+    made, seen = tfmm.tfmm_plan_from_tucker, []
+
+    def tuned(*args, **kw):
+        plan = made(*args, **kw)
+        if split:
+            tfmm.tfmm_plan_tuning_set(plan, single_rhs_split=1)
+        seen.append(tfmm.tfmm_plan_tuning_get(plan)["dis_blocks"])
+        return plan
+
+    tfmm.tfmm_plan_from_tucker = tuned
+    try:
+        _check(7000 + split, nt, npf, nbetas, ranks, 1, 0, 1e-5, pad=1)
+    finally:
+        tfmm.tfmm_plan_from_tucker = made
+    assert (seen[0] == 0) == (split == 0)
