@@ -97,6 +97,7 @@ struct MrStage {
     MrProb* d_probs = nullptr;
     MrTile* d_tiles = nullptr;
     int n_tiles = 0;
+    int bm = 0, bn = 0;     // tile shape
     ~MrStage();
 };
 struct MrPlan {             // per R: problem / tile lists of the 8 stages and scratch

@@ -3,8 +3,8 @@
 //
 // For R right-hand sides every step of the Tucker procedures becomes a small
 // dense matrix product per (group, alpha).  Each step is one launch over all
-// groups: a flat list of 64 x 64 output tiles, one CTA per tile.  Intermediates
-// live in plan-owned scratch, in layouts chosen so that the next step reads
+// groups: a flat list of output tiles (64 or 32 by 64, 32 or 16, by stage), one CTA
+// per tile.  Intermediates live in plan-owned scratch, in layouts chosen so that the next step reads
 // them with plain strides:
 //
 //   aggregation, per (g, alpha):
@@ -26,7 +26,7 @@ namespace tfmm {
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, NTH = 256;
+constexpr int BK = 16, NTH = 256;
 
 enum Stage { AG1, AG2, AG3, AG4, DG1A, DG1B, DG2, DG3 };
 
@@ -117,29 +117,32 @@ __device__ __forceinline__ void store_c(const Ctx& c, const MrProb& p, int i, in
     }
 }
 
-// One 64 x 64 complex output tile per CTA; 256 threads, 4 x 4 outputs each.
-template <Stage S>
+// One BM x BN complex output tile per CTA; 256 threads, BM / 16 x BN / 16 outputs each.
+template <Stage S, int BM, int BN>
 __global__ void __launch_bounds__(NTH) mr_gemm_kernel(const Ctx c, const MrProb* __restrict__ probs,
                                                       const MrTile* __restrict__ tiles) {
+    constexpr int TM = BM / 16, TN = BN / 16;
     __shared__ float2 As[BK][BM + 1];
     __shared__ float2 Bs[BK][BN + 1];
     const MrTile t = tiles[blockIdx.x];
     const MrProb p = probs[t.prob];
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    float2 acc[4][4];
+    float2 acc[TM][TN];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < TM; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
+        for (int b = 0; b < TN; ++b) acc[a][b] = make_float2(0.f, 0.f);
     // consecutive threads walk the operand's contiguous index
     constexpr bool a_k = (S == AG1 || S == DG1A || S == DG2);
     constexpr bool b_k = !(S == AG3 || S == AG4);
     for (int k0 = 0; k0 < p.K; k0 += BK) {
+#pragma unroll
         for (int e = tid; e < BM * BK; e += NTH) {
             const int ii = a_k ? e / BK : e % BM, kk = a_k ? e % BK : e / BM;
             const int i = t.m0 + ii, k = k0 + kk;
             As[kk][ii] = (i < p.M && k < p.K) ? load_a<S>(c, p, i, k) : make_float2(0.f, 0.f);
         }
+#pragma unroll
         for (int e = tid; e < BN * BK; e += NTH) {
             const int jj = b_k ? e / BK : e % BN, kk = b_k ? e % BK : e / BN;
             const int j = t.n0 + jj, k = k0 + kk;
@@ -148,15 +151,15 @@ __global__ void __launch_bounds__(NTH) mr_gemm_kernel(const Ctx c, const MrProb*
         __syncthreads();
 #pragma unroll 4
         for (int kk = 0; kk < BK; ++kk) {
-            float2 av[4], bv[4];
+            float2 av[TM], bv[TN];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) av[a] = As[kk][ty + 16 * a];
+            for (int a = 0; a < TM; ++a) av[a] = As[kk][ty + 16 * a];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) bv[b] = Bs[kk][tx + 16 * b];
+            for (int b = 0; b < TN; ++b) bv[b] = Bs[kk][tx + 16 * b];
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int a = 0; a < TM; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) {
+                for (int b = 0; b < TN; ++b) {
                     acc[a][b].x = fmaf(av[a].x, bv[b].x, acc[a][b].x);
                     acc[a][b].x = fmaf(-av[a].y, bv[b].y, acc[a][b].x);
                     acc[a][b].y = fmaf(av[a].x, bv[b].y, acc[a][b].y);
@@ -166,23 +169,51 @@ __global__ void __launch_bounds__(NTH) mr_gemm_kernel(const Ctx c, const MrProb*
         __syncthreads();
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < TM; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
+        for (int b = 0; b < TN; ++b) {
             const int i = t.m0 + ty + 16 * a, j = t.n0 + tx + 16 * b;
             if (i < p.M && j < p.N) store_c<S>(c, p, i, j, acc[a][b]);
         }
 }
 
-void add_tiles(std::vector<MrTile>& tiles, int prob, int M, int N) {
-    for (int m0 = 0; m0 < M; m0 += BM)
-        for (int n0 = 0; n0 < N; n0 += BN) tiles.push_back(MrTile{prob, m0, n0});
+// Tile shapes and what a multiply-add costs in each, against 64 x 64 (shared-memory loads per
+// multiply-add, 1 / TM + 1 / TN, next to the issue of the product itself).
+struct Shape {
+    int bm, bn;
+    double cost;
+};
+constexpr Shape kShapes[] = {{64, 64, 1.0}, {64, 32, 1.25}, {32, 64, 1.25}, {32, 32, 1.5}, {64, 16, 1.75}, {32, 16, 2.0}};
+
+// A stage's tiles in the shape that wastes least: for 16 columns (N of AG1, AG2, DG2, DG3) or r_theta
+// <= 32 rows (M of DG1a) most of a 64 x 64 tile was padding.  20-lambda sphere in 2-lambda boxes, 16
+// columns: aggregation 5.08 -> 2.17 ms, disaggregation 5.01 -> 2.25; 10-lambda sphere, 32 columns 1.71 -> 1.00,
+// 1.98 -> 1.15.
+void make_tiles(MrStage& st, const std::vector<MrProb>& probs, std::vector<MrTile>& tiles) {
+    double best = 0.0;
+    for (const Shape& s : kShapes) {
+        double c = 0.0;
+        for (const MrProb& p : probs)
+            c += s.cost * ((p.M + s.bm - 1) / s.bm * s.bm) * (double)((p.N + s.bn - 1) / s.bn * s.bn) * p.K;
+        if (st.bm == 0 || c < best) {
+            best = c;
+            st.bm = s.bm;
+            st.bn = s.bn;
+        }
+    }
+    for (int q = 0; q < (int)probs.size(); ++q)
+        for (int m0 = 0; m0 < probs[q].M; m0 += st.bm)
+            for (int n0 = 0; n0 < probs[q].N; n0 += st.bn) tiles.push_back(MrTile{q, m0, n0});
 }
 
 template <Stage S>
 void launch_stage(const Plan& P, const MrStage& st, Ctx c, cudaStream_t s) {
     if (st.n_tiles == 0) return;
-    mr_gemm_kernel<S><<<st.n_tiles, NTH, 0, s>>>(c, st.d_probs, st.d_tiles);
+    auto run = [&](auto kernel) { kernel<<<st.n_tiles, NTH, 0, s>>>(c, st.d_probs, st.d_tiles); };
+    if (st.bm == 64)
+        run(st.bn == 64 ? mr_gemm_kernel<S, 64, 64> : st.bn == 32 ? mr_gemm_kernel<S, 64, 32> : mr_gemm_kernel<S, 64, 16>);
+    else
+        run(st.bn == 64 ? mr_gemm_kernel<S, 32, 64> : st.bn == 32 ? mr_gemm_kernel<S, 32, 32> : mr_gemm_kernel<S, 32, 16>);
     TFMM_CUDA_CHECK(cudaGetLastError());
     (void)P;
 }
@@ -232,7 +263,6 @@ MrPlan* get_mr_plan(Plan& P, int R) {
     TFMM_CUDA_CHECK(device_malloc(&M.buf[1], sizeof(float2) * std::max<int64_t>(off2, 1)));
     TFMM_CUDA_CHECK(device_malloc(&M.buf[2], sizeof(float2) * std::max<int64_t>(off3, 1)));
     std::vector<MrProb> pr[8];
-    std::vector<MrTile> tl[8];
     for (int q = 0; q < P.G * 2; ++q) {
         const TuckerItem& d = P.items[q];
         const int m = d.rt * d.rp;
@@ -246,31 +276,31 @@ MrPlan* get_mr_plan(Plan& P, int R) {
         // AG1: T = U_beta^T X_g
         MrProb p = b;
         p.M = d.rb; p.N = R; p.K = d.n_beta; p.a0 = d.ub; p.lda = d.ld_nb; p.c0 = o1[q];
-        add_tiles(tl[AG1], (int)pr[AG1].size(), p.M, p.N); pr[AG1].push_back(p);
+        pr[AG1].push_back(p);
         // AG2: M = C_(3)^T T
         p = b;
         p.M = m; p.N = R; p.K = d.rb; p.a0 = d.core; p.lda = d.ld_ab; p.b0 = o1[q]; p.c0 = o2[q];
-        add_tiles(tl[AG2], (int)pr[AG2].size(), p.M, p.N); pr[AG2].push_back(p);
+        pr[AG2].push_back(p);
         // AG3: V = U_phi M'
         p = b;
         p.M = np; p.N = d.rt * R; p.K = d.rp; p.a0 = d.uphi; p.b0 = o2[q]; p.c0 = o3[q];
-        add_tiles(tl[AG3], (int)pr[AG3].size(), p.M, p.N); pr[AG3].push_back(p);
+        pr[AG3].push_back(p);
         // AG4: F = U_theta V'
         p = b;
         p.M = nt; p.N = np * R; p.K = d.rt; p.a0 = d.uth; p.b0 = o3[q];
-        add_tiles(tl[AG4], (int)pr[AG4].size(), p.M, p.N); pr[AG4].push_back(p);
+        pr[AG4].push_back(p);
         // DG1a: P = U_theta^T conj(W g)
         p = b;
         p.M = d.rt; p.N = np * R; p.K = nt; p.a0 = d.uth; p.c0 = o3[q];
-        add_tiles(tl[DG1A], (int)pr[DG1A].size(), p.M, p.N); pr[DG1A].push_back(p);
+        pr[DG1A].push_back(p);
         // DG1b: H = P' U_phi
         p = b;
         p.M = d.rt * R; p.N = d.rp; p.K = np; p.a0 = d.uphi; p.b0 = o3[q]; p.c0 = o2[q];
-        add_tiles(tl[DG1B], (int)pr[DG1B].size(), p.M, p.N); pr[DG1B].push_back(p);
+        pr[DG1B].push_back(p);
         // DG2: S = C_(3) H
         p = b;
         p.M = d.rb; p.N = R; p.K = m; p.a0 = d.core; p.lda = d.ld_ab; p.b0 = o2[q]; p.c0 = o1[q];
-        add_tiles(tl[DG2], (int)pr[DG2].size(), p.M, p.N); pr[DG2].push_back(p);
+        pr[DG2].push_back(p);
     }
     for (int g = 0; g < P.G; ++g) {
         const TuckerItem& d0 = P.items[2 * g];
@@ -281,9 +311,13 @@ MrPlan* get_mr_plan(Plan& P, int R) {
         p.a0 = d0.ub; p.a1 = d1.ub; p.lda = d0.ld_nb;
         p.b0 = o1[2 * g]; p.b1 = o1[2 * g + 1];
         p.rwg = d0.rwg;
-        add_tiles(tl[DG3], (int)pr[DG3].size(), p.M, p.N); pr[DG3].push_back(p);
+        pr[DG3].push_back(p);
     }
-    for (int s = 0; s < 8; ++s) upload_stage(M.st[s], pr[s], tl[s]);
+    for (int s = 0; s < 8; ++s) {
+        std::vector<MrTile> tiles;
+        make_tiles(M.st[s], pr[s], tiles);
+        upload_stage(M.st[s], pr[s], tiles);
+    }
     P.mr.push_back(std::move(mp));
     return P.mr.back().get();
 }

@@ -239,3 +239,12 @@ def test_split_path_blocks(split):
     finally:
         tfmm.tfmm_plan_from_tucker = made
     assert (seen[0] == 0) == (split == 0)
+
+
+@pytest.mark.parametrize("R", [2, 4, 5, 16, 17, 32, 33, 64, 65])
+def test_fp32_chain_tile_shapes_and_few_columns(R):
+    """FP32 engine on groups too large for one CTA's shared memory: the columns' single-RHS kernels up to
+    four right-hand sides, then the chain with 64- and 32-row tiles of 64, 32 and 16 columns."""
+    nbetas = [63, 520, 130, 31]
+    ranks = [[(5, 4, 15), (16, 24, 16)], [(16, 24, 150), (17, 33, 65)], [(9, 17, 33), (3, 2, 64)], [(4, 8, 17), (2, 3, 6)]]
+    _check(8000 + R, 24, 48, nbetas, ranks, R, 0, 1e-5, pad=1)
