@@ -71,7 +71,8 @@ typedef struct {
     int32_t keep_dense;/* nonzero: also keep FP32 uncompressed tensors (Eqs. 3, 5) */
     int32_t max_rhs;   /* largest R later passed to the hot path (>= 1) */
     int32_t batch_groups; /* groups per setup batch (0 = automatic) */
-    int32_t mrhs_precision; /* engine for R > 1: 0 = grouped-GEMM chain in FP32 on CUDA cores;
+    int32_t mrhs_precision; /* engine for R > 1: 0 = FP32 on CUDA cores: the grouped-GEMM chain, or
+                               whichever other FP32 kernels are faster for the plan and R;
                                1 = the single-RHS kernels, one column after another (FP32);
                                2 or 3 = tensor cores with FP32 operands split into 2 or 3
                                BF16 terms (hi + lo [+ lo2]), FP32 accumulation */

@@ -167,8 +167,8 @@ void check_params(const tfmm_params& p) {
 //   small:   one CTA per (group, component) with everything in shared memory, for plans whose
 //            every item fits (small.cu), in place of columns and chain unless the tuning
 //            asks for one of the single-RHS paths;
-//   columns: the persistent single-RHS kernels, one column after the other (R = 1, or
-//            mrhs_precision 1, or TFMM_MR=loop);
+//   columns: the single-RHS kernels, one column after the other (R = 1, or mrhs_precision 1,
+//            or TFMM_MR=loop, or few columns of mrhs_precision 0);
 //   chain:   the grouped-GEMM chain on FP32 CUDA cores (mrhs_precision 0), also the
 //            fallback when a work item does not fit the single-RHS kernels;
 //   tc:      the split-BF16 tensor-core chain with `terms` terms (mrhs_precision 2, 3).
@@ -180,7 +180,13 @@ Engine engine_for(const Plan& P, int R, int* terms) {
     const char* e = std::getenv("TFMM_MR");
     const bool loop = e && std::strcmp(e, "loop") == 0;
     if (P.tuning.split == 0 && !loop && (R <= 1 ? P.small_one : P.small_ok && p <= 1)) return Engine::small;
-    if (P.hot_ok && (R <= 1 || loop || p == 1 || plan_is_svd(P))) return Engine::columns;
+    // Up to kColumnsMax columns the chain reads every factor about as slowly as for one tile's width, and
+    // the single-RHS kernels stream them once per column near the copy rate.  Measured, chain / columns
+    // (both stages, ms): 20-lambda sphere in 2-lambda boxes, 2 columns 2.95 / 1.50, 4 3.15 / 2.99, 6 3.39 / 4.49;
+    // 10-lambda sphere 4 columns 0.81 / 0.59, 8 0.95 / 1.16; 4-lambda boxes 4 columns 1.97 / 1.61.
+    constexpr int kColumnsMax = 4;
+    if (P.hot_ok && (R <= 1 || loop || p == 1 || plan_is_svd(P) || (p == 0 && R <= kColumnsMax)))
+        return Engine::columns;
     if (R > 1 && (p == 2 || p == 3)) {
         *terms = p;
         return Engine::tc;
