@@ -591,11 +591,14 @@ __global__ void __launch_bounds__(CH ? 2 * TTHREADS : TTHREADS)
 // (Fig. 2b step 2); then for each r of the block V_r = D1[:, (., r)] goes
 // TMEM -> registers -> shared memory (split into BF16 terms) as the A operand of
 // AG4, F_r[i_phi][i_theta] = sum_a V_r[i_phi][a] U_theta[i_theta][a] (Fig. 2b
-// steps 3-4), which leaves TMEM straight for the spectra.  The MMAs of r overlap
-// the spectra stores of r - 1 (two D2 accumulators).  What bounds it: one CTA per SM, whose
-// operand loads and AG3 nothing overlaps, and the chain V -> A operand -> MMA -> spectra of each r.
-// 30-lambda sphere, 128 columns: 6.45 ms with a lone issuing thread, 5.88 with the convergent MMA
-// warp (1.4 ms for the bytes); 10-lambda, 37 columns: 0.591 -> 0.443 ms.
+// steps 3-4), which leaves TMEM for the spectra.  V_(r + 1) is prepared and the spectra of r - 1
+// leave while the MMAs of r run (two A operands, two D2 accumulators, a set of warps for either side).
+// What bounds it, from cycle counts at n_theta = 40, r = (22, 34), 7 columns a tile, 36,000 cycles: the operand
+// loads (10,500, about one 16-byte chunk a cycle) and AG3 (6000), which nothing overlaps with one CTA per SM,
+// then 2300 a column, where the MMAs' operand reads (1350 cycles), V and the staged spectra together fill
+// the shared-memory port.  30-lambda sphere, 128 columns: 6.45 ms with a lone issuing thread, 5.88 with the
+// convergent MMA warp, 4.72 with the loads in the order of the layout, the two roles and the bulk store
+// (1.4 ms for the bytes); 10-lambda, 37 columns: 0.591, 0.443, 0.393 ms; 20-lambda, 16 columns: 0.372, 0.338, 0.280.
 struct F34Item {
     const bf16* uph; int64_t uph_ld, uph_ps;  // U_phi planes [i_phi][b]
     const bf16* uth; int64_t uth_ld, uth_ps;  // U_theta planes [i_theta][a]
@@ -613,18 +616,25 @@ __device__ __forceinline__ uint64_t make_desc_sbo(uint32_t addr, uint32_t sbo) {
     return d;
 }
 
-// 2T planes of `rows` rows (zero-filled from row `valid` and from column r8(kvalid))
-// of a K-major source into the canonical no-swizzle layout with depth K.
+// 2T planes of `rows` rows, rounded up to 8 (zero-filled from row `valid` and from column r8(kvalid))
+// of a K-major source into the canonical no-swizzle layout with depth K, of which the first `kuse`
+// columns are wanted; NTHR threads share the copies.  The chunks of 16 bytes are taken in the order of the
+// shared-memory layout (eight lanes write 128 bytes in a row, no bank twice) and the index of one serves
+// all planes: with the lanes along K and an index per chunk and plane, these loads took 11,000 to 14,000
+// cycles of a 41,000-cycle tile of the fused AG3 + AG4 kernel (7000 to 10,500 now).
 template <int T>
 __device__ __forceinline__ void load_planes(uint8_t* dst, int plane_bytes, int K, const bf16* src, int64_t ld,
-                                            int64_t ps, int rows, int valid, int kvalid) {
-    const int kc8 = K / 8, k8v = (kvalid + 7) / 8;
-    const int total = 2 * T * rows * kc8;
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-        const int pl = idx / (rows * kc8), rem = idx % (rows * kc8), r = rem / kc8, kc = rem % kc8;
+                                            int64_t ps, int rows, int valid, int kvalid, int kuse, int nthr) {
+    const int kc8 = K / 8, k8v = (kvalid + 7) / 8, k8u = kuse / 8;
+    const int total = ((rows + 7) >> 3) * 8 * kc8;
+    for (int idx = threadIdx.x; idx < total; idx += nthr) {
+        const int core = idx >> 3, rb = core / kc8, kc = core - rb * kc8, r = rb * 8 + (idx & 7);
+        if (kc >= k8u) continue;
         const bool ok = r < valid && kc < k8v;
-        const bf16* g = ok ? src + pl * ps + (int64_t)r * ld + kc * 8 : src;
-        cp16(dst + pl * plane_bytes + (r >> 3) * (K * 16) + kc * 128 + (r & 7) * 16, g, ok ? 16 : 0);
+        const bf16* g = ok ? src + (int64_t)r * ld + kc * 8 : src;
+        const int64_t step = ok ? ps : 0;
+#pragma unroll
+        for (int pl = 0; pl < 2 * T; ++pl) cp16(dst + pl * plane_bytes + idx * 16, g + pl * step, ok ? 16 : 0);
     }
 }
 
@@ -965,15 +975,18 @@ __global__ void __launch_bounds__(TMA_THREADS, 1)
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm), "r"(tcols));
 }
 
-constexpr int F34_WORKERS = 512;               // 16 warps, four per TMEM lane quarter
-constexpr int F34_THREADS = F34_WORKERS + 32;  // and one warp that only issues MMAs
+// Sixteen worker warps: eight turn AG3's columns into AG4's operands, eight take AG4's
+// results to the spectra (two of either per TMEM lane quarter), and one more warp that only issues MMAs.
+constexpr int F34_ROLE = 256, F34_WORKERS = 2 * F34_ROLE;
+constexpr int F34_THREADS = F34_WORKERS + 32;
 
-__device__ __forceinline__ void workers_sync() {
-    asm volatile("bar.sync 1, %0;" ::"n"(F34_WORKERS) : "memory");
+template <int ID, int N>
+__device__ __forceinline__ void named_sync() {
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(N) : "memory");
 }
 
 // mbarriers of the fused kernel
-enum { F34_D1 = 0, F34_A2 = 1, F34_D2 = 3, F34_EMPTY = 5, F34_NBAR = 7 };
+enum { F34_D1 = 0, F34_A2 = 1, F34_D2 = 3, F34_EMPTY = 5, F34_FREE = 7, F34_NBAR = 9 };
 
 template <int T>
 __global__ void __launch_bounds__(F34_THREADS) tc_ag34_kernel(const TcCtx c, const F34Item* __restrict__ items,
@@ -981,7 +994,7 @@ __global__ void __launch_bounds__(F34_THREADS) tc_ag34_kernel(const TcCtx c, con
                                                              int n_phi) {
     extern __shared__ __align__(1024) uint8_t smem[];
     // F34_D1: AG3 done; F34_A2 + b: A2[b] written; F34_D2 + b: AG4 into D2[b] done;
-    // F34_EMPTY + b: D2[b] read out
+    // F34_EMPTY + b: D2[b] read out; F34_FREE + b: the MMAs that read A2[b] done
     __shared__ __align__(8) uint64_t mbar[F34_NBAR];
     __shared__ uint32_t tmem_base;
     const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
@@ -991,9 +1004,8 @@ __global__ void __launch_bounds__(F34_THREADS) tc_ag34_kernel(const TcCtx c, con
     const int a1p = TBM * K1 * 2, b1p = sh.N1p * K1 * 2, b2p = sh.ntp * K2 * 2, a2p = TBM * K2 * 2;
     // U_phi and M' are dead once AG3 is done: the spectra staging reuses the first,
     // the two A operands of AG4 the second
-    const int r1 = max(2 * T * a1p, n_phi * nt * 8), r2 = max(2 * T * b1p, 2 * 2 * T * a2p);
+    const int r1 = max(2 * T * a1p, (n_phi * nt * 8 + 15) & ~15), r2 = max(2 * T * b1p, 2 * 2 * T * a2p);
     uint8_t* sA1 = smem;
-    float2* stage = reinterpret_cast<float2*>(smem);
     uint8_t* sB1 = smem + r1;
     uint8_t* sA2b = sB1;
     uint8_t* sB2 = sB1 + r2;  // 3T slots (-Im_q, Re_q, Im_q) of b2p bytes
@@ -1004,28 +1016,23 @@ __global__ void __launch_bounds__(F34_THREADS) tc_ag34_kernel(const TcCtx c, con
     }
     if (tid == 0)
         for (int b = 0; b < F34_NBAR; ++b) {
-            const int cnt = (b == F34_A2 || b == F34_A2 + 1 || b == F34_EMPTY || b == F34_EMPTY + 1) ? F34_WORKERS : 1;
+            const int cnt = (b == F34_A2 || b == F34_A2 + 1 || b == F34_EMPTY || b == F34_EMPTY + 1) ? F34_ROLE : 1;
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar[b])), "r"(cnt));
         }
     asm volatile("fence.mbarrier_init.release.cluster;");
     const int n1 = it.rt * t.nr, n1p = (n1 + 15) & ~15;
-    load_planes<T>(sA1, a1p, K1, it.uph, it.uph_ld, it.uph_ps, n_phi, n_phi, it.rp);
-    load_planes<T>(sB1, b1p, K1, it.m + (int64_t)it.rt * t.r0 * it.m_ld, it.m_ld, it.m_ps, n1p, n1, it.rp);
-    for (int q = 0; q < T; ++q) {  // Re_q -> slot 3q + 1, Im_q -> slot 3q + 2
-        load_planes<1>(sB2 + (3 * q + 1) * b2p, b2p, K2, it.uth + q * it.uth_ps, it.uth_ld, it.uth_ps * T, sh.ntp,
-                       nt, it.rt);
-    }
+    // K steps of 16 that hold any of this item's ranks
+    const int ks1 = (it.rp + 15) >> 4, ks2 = (it.rt + 15) >> 4;
+    load_planes<T>(sA1, a1p, K1, it.uph, it.uph_ld, it.uph_ps, n_phi, n_phi, it.rp, ks1 * 16, F34_THREADS);
+    load_planes<T>(sB1, b1p, K1, it.m + (int64_t)it.rt * t.r0 * it.m_ld, it.m_ld, it.m_ps, n1p, n1, it.rp, ks1 * 16,
+                   F34_THREADS);
     asm volatile("cp.async.commit_group;");
-    asm volatile("cp.async.wait_group 0;");
-    __syncthreads();
-    for (int q = 0; q < T; ++q) {  // slot 3q = -Im_q (bfloat16 sign bits flipped)
-        const uint4* src = reinterpret_cast<const uint4*>(sB2 + (3 * q + 2) * b2p);
-        uint4* dst = reinterpret_cast<uint4*>(sB2 + 3 * q * b2p);
-        for (int e = tid; e < b2p / 16; e += F34_THREADS) {
-            const uint4 v = src[e];
-            dst[e] = make_uint4(v.x ^ 0x80008000u, v.y ^ 0x80008000u, v.z ^ 0x80008000u, v.w ^ 0x80008000u);
-        }
-    }
+    if (tid < F34_WORKERS)  // waited for while AG3 runs
+        for (int q = 0; q < T; ++q)  // Re_q -> slot 3q + 1, Im_q -> slot 3q + 2
+            load_planes<1>(sB2 + (3 * q + 1) * b2p, b2p, K2, it.uth + q * it.uth_ps, it.uth_ld, it.uth_ps * T, sh.ntp,
+                           nt, it.rt, ks2 * 16, F34_WORKERS);
+    asm volatile("cp.async.commit_group;");
+    asm volatile("cp.async.wait_group 1;");
     asm volatile("fence.proxy.async.shared::cta;");
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
@@ -1039,9 +1046,9 @@ __global__ void __launch_bounds__(F34_THREADS) tc_ag34_kernel(const TcCtx c, con
         // ---- MMA warp (convergent, one lane issues): AG3 once, then AG4 for every r as soon as its
         // A2 is written
         const uint32_t lead = elect_lane();
-        const int nr = uniform(t.nr), n1u = uniform(n1p);
+        const int nr = uniform(t.nr), n1u = uniform(n1p), ks2u = uniform(ks2);
         auto wait = [&](uint64_t* bar, uint32_t parity) { return (bool)__all_sync(0xffffffffu, mbar_wait(bar, parity)); };
-        issue_products<T>(lead, tm, tm + sh.N1s, smem_u32(sA1), a1p, smem_u32(sB1), b1p, K1 * 16, K1 * 16, K1 / 16,
+        issue_products<T>(lead, tm, tm + sh.N1s, smem_u32(sA1), a1p, smem_u32(sB1), b1p, K1 * 16, K1 * 16, uniform(ks1),
                           idesc_bf16(n1u));
         commit_lead(lead, &mbar[F34_D1]);
         for (int j = 0; j < nr; ++j) {
@@ -1051,91 +1058,171 @@ __global__ void __launch_bounds__(F34_THREADS) tc_ag34_kernel(const TcCtx c, con
             asm volatile("tcgen05.fence::after_thread_sync;");
             const uint32_t dr = d2 + b * set;
             issue_products_cat<T>(lead, dr, dr + (sh.nacc - 1) * 2 * sh.ntp, smem_u32(sA2b + a * 2 * T * a2p), a2p,
-                                  smem_u32(sB2), b2p, K2 * 16, K2 * 16, K2 / 16, idesc_bf16(2 * sh.ntp));
+                                  smem_u32(sB2), b2p, K2 * 16, K2 * 16, ks2u, idesc_bf16(2 * sh.ntp));
+            commit_lead(lead, &mbar[F34_FREE + a]);
             commit_lead(lead, &mbar[F34_D2 + b]);
         }
     } else {
-        // ---- workers: warps w, w + 4, ... share lane quarter w & 3 and split the columns
-        const int phi = (warp & 3) * 32 + lane, grp = warp >> 2, ngrp = F34_WORKERS / 128;
+        // ---- workers: lane quarter w & 3; the two warps of a role and quarter split the columns
+        const int phi = (warp & 3) * 32 + lane, grp = (warp >> 2) & 1;
         const bool rows = (warp & 3) * 32 < n_phi;  // quarters past n_phi hold no direction
         const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
         const int64_t n_dir = c.n_dir;
+        // -Im_q of U_theta (bfloat16 sign bits flipped) while AG3 runs; A2's barrier tells the MMA warp
+        asm volatile("cp.async.wait_group 0;");
+        named_sync<1, F34_WORKERS>();
+        for (int q = 0; q < T; ++q) {
+            const uint4* src = reinterpret_cast<const uint4*>(sB2 + (3 * q + 2) * b2p);
+            uint4* dst = reinterpret_cast<uint4*>(sB2 + 3 * q * b2p);
+            for (int e = tid; e < b2p / 16; e += F34_WORKERS) {
+                const uint4 v = src[e];
+                dst[e] = make_uint4(v.x ^ 0x80008000u, v.y ^ 0x80008000u, v.z ^ 0x80008000u, v.w ^ 0x80008000u);
+            }
+        }
+        asm volatile("fence.proxy.async.shared::cta;");
+        named_sync<1, F34_WORKERS>();
         ok = mbar_wait(&mbar[F34_D1], 0);
         asm volatile("tcgen05.fence::after_thread_sync;");
-        for (int j = 0; j <= t.nr; ++j) {
-            if (j < t.nr) {
-                // V_j: TMEM columns (a + r_t j) -> BF16 planes of A2[j & 1], row i_phi, depth a
-                // (zeros past r_t); A2[j & 1] was last read by the MMAs of j - 2, waited below
+        if (warp < F34_ROLE / 32) {
+            // V_j: TMEM columns (a + r_t j) -> BF16 planes of A2[j & 1], row i_phi, depth a (zeros past r_t)
+            const int nk = 2 * ks2;
+            for (int j = 0; j < t.nr; ++j) {
                 uint8_t* sA2 = sA2b + (j & 1) * 2 * T * a2p;
-                if (rows)
-                    for (int kc = grp; kc < K2 / 8; kc += ngrp) {
-                        const int off = (phi >> 3) * (K2 * 16) + kc * 128 + (phi & 7) * 16;
-                        if (kc * 8 >= it.rt) {
+                auto put = [&](int kc, const uint32_t (&vr)[8], const uint32_t (&vi)[8]) {
+                    uint32_t w[2 * T][4];
 #pragma unroll
-                            for (int q = 0; q < 2 * T; ++q)
-                                *reinterpret_cast<uint4*>(sA2 + q * a2p + off) = make_uint4(0, 0, 0, 0);
-                            continue;
+                    for (int e = 0; e < 8; e += 2) {
+                        uint32_t pr[3], pi[3];
+                        const int k = kc * 8 + e;
+                        split_pack<T>(k < it.rt ? __uint_as_float(vr[e]) : 0.f, k + 1 < it.rt ? __uint_as_float(vr[e + 1]) : 0.f, pr);
+                        split_pack<T>(k < it.rt ? __uint_as_float(vi[e]) : 0.f, k + 1 < it.rt ? __uint_as_float(vi[e + 1]) : 0.f, pi);
+#pragma unroll
+                        for (int q = 0; q < T; ++q) {
+                            w[q][e / 2] = pr[q];
+                            w[T + q][e / 2] = pi[q];
                         }
-                        uint32_t vr[8], vi[8], w[2 * T][4];
-                        tmem_ld8(vr, tm + lanes + it.rt * j + kc * 8);
-                        tmem_ld8(vi, tm + lanes + sh.N1s + it.rt * j + kc * 8);
-                        asm volatile("tcgen05.wait::ld.sync.aligned;");
-#pragma unroll
-                        for (int e = 0; e < 8; e += 2) {
-                            uint32_t pr[3], pi[3];
-                            const int k = kc * 8 + e;
-                            split_pack<T>(k < it.rt ? __uint_as_float(vr[e]) : 0.f, k + 1 < it.rt ? __uint_as_float(vr[e + 1]) : 0.f, pr);
-                            split_pack<T>(k < it.rt ? __uint_as_float(vi[e]) : 0.f, k + 1 < it.rt ? __uint_as_float(vi[e + 1]) : 0.f, pi);
-#pragma unroll
-                            for (int q = 0; q < T; ++q) {
-                                w[q][e / 2] = pr[q];
-                                w[T + q][e / 2] = pi[q];
-                            }
-                        }
-#pragma unroll
-                        for (int q = 0; q < 2 * T; ++q)
-                            *reinterpret_cast<uint4*>(sA2 + q * a2p + off) = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
                     }
+                    const int off = (phi >> 3) * (K2 * 16) + kc * 128 + (phi & 7) * 16;
+#pragma unroll
+                    for (int q = 0; q < 2 * T; ++q)
+                        *reinterpret_cast<uint4*>(sA2 + q * a2p + off) = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
+                };
+                if (j >= 2) ok = mbar_wait(&mbar[F34_FREE + (j & 1)], ((j >> 1) - 1) & 1) && ok;
+                if (rows)
+                    for (int kc = grp; kc < nk; kc += 4) {  // two blocks of eight at a time
+                        const bool more = kc + 2 < nk;
+                        const uint32_t col = tm + lanes + it.rt * j + kc * 8;
+                        uint32_t vr[2][8], vi[2][8];
+                        // (a block that starts past r_t reads other columns and is stored as zeros)
+                        tmem_ld8(vr[0], col);
+                        tmem_ld8(vi[0], col + sh.N1s);
+                        if (more) {
+                            tmem_ld8(vr[1], col + 16);
+                            tmem_ld8(vi[1], col + 16 + sh.N1s);
+                        }
+                        asm volatile("tcgen05.wait::ld.sync.aligned;");
+                        put(kc, vr[0], vi[0]);
+                        if (more) put(kc + 2, vr[1], vi[1]);
+                    }
+                asm volatile("tcgen05.fence::before_thread_sync;");
                 asm volatile("fence.proxy.async.shared::cta;");
                 mbar_arrive(&mbar[F34_A2 + (j & 1)]);
             }
-            if (j > 0) {
-                // spectra of RHS r0 + j - 1: TMEM -> rows in shared memory -> one contiguous block
-                const int jj = j - 1, b = jj % nbuf;
-                ok = mbar_wait(&mbar[F34_D2 + b], (jj / nbuf) & 1) && ok;
+        } else {
+            // Spectra of RHS r0 + j: TMEM -> rows in shared memory -> one contiguous block.  One bulk copy takes
+            // them on to memory behind the next one's work, where its address and size allow (shared among
+            // the threads, the copy held them for 1050 cycles a column); with two staging buffers it has
+            // that long to read them.
+            const int tid2 = tid - F34_ROLE;
+            const int sbytes = (int)(n_dir * 8 + 15) & ~15;
+            const bool bulk = (n_dir & 1) == 0 && (reinterpret_cast<uintptr_t>(c.spec) & 15) == 0;
+            const bool two = 2 * sbytes <= r1;
+            // A row (i_phi) of the staged spectra is nt complex numbers and a warp stores 32 rows at once, pairs
+            // of theta for even nt.  Rows an even number of pairs apart share banks: such lanes take
+            // their four pairs of eight theta in another order (one, two or three on).
+            const int pairs = nt >> 1, turn = (phi >> (pairs & 1 ? 3 : pairs & 2 ? 2 : pairs & 4 ? 1 : 0)) & 3;
+            const int nk = (nt + 7) / 8;
+            for (int j = 0; j < t.nr; ++j) {
+                const int b = j % nbuf;
+                float2* stage = reinterpret_cast<float2*>(smem + (two && (j & 1) ? sbytes : 0));
+                ok = mbar_wait(&mbar[F34_D2 + b], (j / nbuf) & 1) && ok;
                 asm volatile("tcgen05.fence::after_thread_sync;");
-                const uint32_t dr = d2 + b * set;
-                for (int kc = grp; rows && kc < sh.ntp / 8; kc += ngrp) {
-                    uint32_t vr[8], vi[8], ur[8] = {}, ui[8] = {};
-                    tmem_ld8(vr, dr + lanes + kc * 8);
-                    tmem_ld8(vi, dr + lanes + sh.ntp + kc * 8);
-                    if (sh.nacc == 2) {
-                        tmem_ld8(ur, dr + lanes + 2 * sh.ntp + kc * 8);
-                        tmem_ld8(ui, dr + lanes + 3 * sh.ntp + kc * 8);
-                    }
-                    asm volatile("tcgen05.wait::ld.sync.aligned;");
-                    if (phi < n_phi) {
+                auto put = [&](int kc, const uint32_t (&vr)[8], const uint32_t (&vi)[8]) {
+                    if (phi >= n_phi) return;
+                    float4 v[4];
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2)
+                        v[e / 2] = make_float4(__uint_as_float(vr[e]), __uint_as_float(vi[e]), __uint_as_float(vr[e + 1]),
+                                               __uint_as_float(vi[e + 1]));
+                    float2* dst = stage + phi * nt + kc * 8;
+                    if ((nt & 1) == 0) {
+                        if (turn & 1) {
+                            const float4 f = v[0];
+                            v[0] = v[1], v[1] = v[2], v[2] = v[3], v[3] = f;
+                        }
+                        if (turn & 2) {
+                            const float4 f = v[0], g = v[1];
+                            v[0] = v[2], v[1] = v[3], v[2] = f, v[3] = g;
+                        }
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int pr = (e + turn) & 3;
+                            if (kc * 8 + 2 * pr < nt) reinterpret_cast<float4*>(dst)[pr] = v[e];
+                        }
+                    } else {
 #pragma unroll
                         for (int e = 0; e < 8; ++e)
-                            if (kc * 8 + e < nt)
-                                stage[phi * nt + kc * 8 + e] =
-                                    make_float2(__uint_as_float(vr[e]) + __uint_as_float(ur[e]),
-                                                __uint_as_float(vi[e]) + __uint_as_float(ui[e]));
+                            if (kc * 8 + e < nt) dst[e] = e & 1 ? make_float2(v[e / 2].z, v[e / 2].w)
+                                                                : make_float2(v[e / 2].x, v[e / 2].y);
                     }
+                };
+                for (int kc = grp; rows && kc < nk; kc += 4) {  // two blocks of eight at a time
+                    const bool more = kc + 2 < nk;
+                    const uint32_t col = d2 + b * set + lanes + kc * 8;
+                    uint32_t vr[2][8], vi[2][8];
+                    tmem_ld8(vr[0], col);
+                    tmem_ld8(vi[0], col + sh.ntp);
+                    if (more) {
+                        tmem_ld8(vr[1], col + 16);
+                        tmem_ld8(vi[1], col + 16 + sh.ntp);
+                    }
+                    asm volatile("tcgen05.wait::ld.sync.aligned;");
+                    if (sh.nacc == 2) {
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            if (u && !more) break;
+                            uint32_t ur[8], ui[8];
+                            tmem_ld8(ur, col + 16 * u + 2 * sh.ntp);
+                            tmem_ld8(ui, col + 16 * u + 3 * sh.ntp);
+                            asm volatile("tcgen05.wait::ld.sync.aligned;");
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) {
+                                vr[u][e] = __float_as_uint(__uint_as_float(vr[u][e]) + __uint_as_float(ur[e]));
+                                vi[u][e] = __float_as_uint(__uint_as_float(vi[u][e]) + __uint_as_float(ui[e]));
+                            }
+                        }
+                    }
+                    put(kc, vr[0], vi[0]);
+                    if (more) put(kc + 2, vr[1], vi[1]);
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;");
-                mbar_arrive(&mbar[F34_EMPTY + b]);  // set b may take the MMAs of jj + nbuf
-                workers_sync();
-                float2* F = c.spec + (((int64_t)(t.r0 + jj) * c.G + it.g) * 2 + it.alpha) * n_dir;
-                if ((n_dir & 1) == 0) {
-                    const float4* src = reinterpret_cast<const float4*>(stage);
-                    float4* dst = reinterpret_cast<float4*>(F);
-                    for (int e = tid; e < (int)(n_dir >> 1); e += F34_WORKERS) dst[e] = src[e];
-                } else {
-                    for (int e = tid; e < (int)n_dir; e += F34_WORKERS) F[e] = stage[e];
+                mbar_arrive(&mbar[F34_EMPTY + b]);  // set b may take the MMAs of j + nbuf
+                asm volatile("fence.proxy.async.shared::cta;");
+                if (bulk && tid2 == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // j - 1 read out
+                named_sync<2, F34_ROLE>();
+                float2* F = c.spec + (((int64_t)(t.r0 + j) * c.G + it.g) * 2 + it.alpha) * n_dir;
+                if (!bulk) {
+                    for (int e = tid2; e < (int)n_dir; e += F34_ROLE) F[e] = stage[e];
+                } else if (tid2 == 0) {
+                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(F),
+                                 "r"(smem_u32(stage)), "r"((uint32_t)(n_dir * 8))
+                                 : "memory");
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    if (!two) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 }
-                workers_sync();
+                if (!two) named_sync<2, F34_ROLE>();  // else the next one's barrier comes before this buffer's next use
             }
+            if (tid2 == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
         }
     }
     // every MMA was waited for (bounded) by the workers before TMEM is freed
@@ -1187,7 +1274,7 @@ __global__ void __launch_bounds__(D1_THREADS) tc_dg1a_kernel(const TcCtx c, cons
     if (tid == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar)), "r"(1));
     asm volatile("fence.mbarrier_init.release.cluster;");
     // A: U_theta^T, r_theta rows (lanes past r_theta hold no output)
-    load_planes<T>(sA, ap, K, it.uth, it.uth_ld, it.uth_ps, it.rt, it.rt, nt);
+    load_planes<T>(sA, ap, K, it.uth, it.uth_ld, it.uth_ps, it.rt, it.rt, nt, K, D1_THREADS);
     asm volatile("cp.async.commit_group;");
     // B: pair row p0 + i = i_phi + n_phi r, depth theta; conj(W g), zero past n_theta and n_phi R.
     // Every load of a thread is issued before the splits (memory-level parallelism).
@@ -2370,7 +2457,7 @@ constexpr size_t kMaxDynSmem = 225 * 1024;
 
 size_t f34_smem(int T, int K1, int K2, int N1p, int ntp, int nt, int np) {
     const size_t pl = (size_t)2 * T * 2;  // bytes per element over the 2T planes
-    return std::max(pl * TBM * K1, (size_t)np * nt * 8) + pl * std::max((size_t)N1p * K1, (size_t)2 * TBM * K2) +
+    return std::max(pl * TBM * K1, ((size_t)np * nt * 8 + 15) & ~(size_t)15) + pl * std::max((size_t)N1p * K1, (size_t)2 * TBM * K2) +
            (size_t)3 * T * 2 * ntp * K2;
 }
 
@@ -2424,14 +2511,14 @@ void plan_fused34(const Plan& P, TcPlan& M, const bf16* F, const std::vector<TcI
     constexpr size_t kSmemSM = 228 * 1024;
     const int ctas_tmem = 512 / f.tcols;
     if (kSmemSM / (f.smem + 2048) > (size_t)ctas_tmem) f.smem = std::min(kMaxDynSmem, kSmemSM / ctas_tmem - 2048);
-    // work list, most work first
-    std::vector<int> order(P.items.size());
-    std::iota(order.begin(), order.end(), 0);
-    auto cost = [&](int q) { return (double)P.items[q].rt * (P.items[q].rp + nt); };
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost(a) > cost(b); });
+    // work list, longest first: a tile's time goes with its right-hand sides (a small r_theta takes many)
     std::vector<F34Tile> tiles;
-    for (int q : order)
-        for (int r0 = 0; r0 < R; r0 += nr_of[q]) tiles.push_back(F34Tile{q, r0, std::min(nr_of[q], R - r0)});
+    for (size_t q = 0; q < P.items.size(); ++q)
+        for (int r0 = 0; r0 < R; r0 += nr_of[q]) tiles.push_back(F34Tile{(int)q, r0, std::min(nr_of[q], R - r0)});
+    auto longer = [&](const F34Tile& a, const F34Tile& b) {
+        return a.nr != b.nr ? a.nr > b.nr : P.items[a.item].rp > P.items[b.item].rp;
+    };
+    std::stable_sort(tiles.begin(), tiles.end(), longer);
     TFMM_CUDA_CHECK(device_malloc(&M.f34_items.p, sizeof(F34Item) * items.size()));
     TFMM_CUDA_CHECK(device_malloc(&M.f34_tiles.p, sizeof(F34Tile) * tiles.size()));
     TFMM_CUDA_CHECK(cudaMemcpy(M.f34_items.p, items.data(), sizeof(F34Item) * items.size(), cudaMemcpyHostToDevice));

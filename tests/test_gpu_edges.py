@@ -248,3 +248,15 @@ def test_fp32_chain_tile_shapes_and_few_columns(R):
     nbetas = [63, 520, 130, 31]
     ranks = [[(5, 4, 15), (16, 24, 16)], [(16, 24, 150), (17, 33, 65)], [(9, 17, 33), (3, 2, 64)], [(4, 8, 17), (2, 3, 6)]]
     _check(8000 + R, 24, 48, nbetas, ranks, R, 0, 1e-5, pad=1)
+
+
+@pytest.mark.parametrize("R", [2, 5, 19])
+@pytest.mark.parametrize("nt,npf,top", [(13, 25, (13, 14)), (13, 26, (12, 16)), (16, 32, (15, 18)), (20, 33, (16, 17)),
+                                        (24, 48, (17, 33)), (26, 52, (18, 30)), (40, 80, (33, 15)), (64, 128, (20, 15))])
+def test_aggregation_last_steps_forms(nt, npf, top, R):
+    """Odd and even N_theta by the powers of two in it (the order in which rows are staged), spectra of odd and
+    even length, one and two staging buffers, K steps that only the larger item has, the most lanes."""
+    rt, rp = top
+    nbetas = [140, 60]
+    ranks = [[(rt, rp, 70), (rt - 1, rp - 5, 40)], [(5, 7, 30), (rt, 4, 25)]]
+    _check(9000 + nt + R, nt, npf, nbetas, ranks, R, 3, 1e-6, pad=1)
