@@ -161,8 +161,9 @@ tfmm_status tfmm_plan_from_tucker(int64_t n_rwg, int32_t n_groups, int32_t n_the
 tfmm_status tfmm_plan_set_dense(tfmm_plan* plan, const tfmm_cdouble* tensors, void* stream);
 
 /* Engine of the R > 1 hot path (see tfmm_params.mrhs_precision): 0, 1, 2 or 3.
- * When the largest work item does not fit the single-RHS kernels (shared
- * memory), every R, R = 1 included, runs the FP32 grouped-GEMM chain.
+ * When the largest work item does not fit the persistent single-RHS kernels
+ * (shared memory), their split path runs (single_rhs_split of tfmm_tuning); when
+ * it does not fit that either, every R, R = 1 included, runs the FP32 grouped-GEMM chain.
  * Tensor-core modes build BF16 planes of the factors on first use (device
  * memory: 2 layouts x 2 or 3 terms of every factor).  INVALID_ARG otherwise. */
 tfmm_status tfmm_plan_set_mrhs_precision(tfmm_plan* plan, int32_t precision);
@@ -248,8 +249,9 @@ tfmm_status tfmm_matvec_host(tfmm_plan* plan, const tfmm_cfloat* x_host, tfmm_cf
  * EFIE (Eq. 2) for the x that tfmm_aggregate received.  Evaluated as a 3-D FFT
  * convolution over the zero-padded box grid, FP32 (the translation kernel's
  * transform is computed once in FP64).  The first call builds it (device memory
- * owned by the plan: the kernel's transform, N_grid x N_dir complex, and a work
- * grid of N_grid x 2 N_dir complex, N_grid >= (2K_x - 1)(2K_y - 1)(2K_z - 1));
+ * owned by the plan: the kernel's transform, N_grid x N_dir complex, and, for box
+ * grids of more than 18 a side, a work grid of N_grid x 2 N_dir complex, N_grid >=
+ * (2K_x - 1)(2K_y - 1)(2K_z - 1), or the cube of the longest side where that is near-cubic);
  * later calls allocate nothing.
  *   spectra_out  device, R x G x 2 x N_dir FP32 complex (as tfmm_aggregate writes it)
  *   spectra_in   device, same shape, overwritten; must not alias spectra_out
@@ -346,7 +348,10 @@ typedef struct {
                                        (0: 128 when it fits, else 64) */
     int32_t single_rhs_split;       /* single-RHS stages as three launches that spread every work
                                        item over many CTAs (for plans with few, large groups):
-                                       0 automatic (fewer work items than 2 x SMs), 1 always, 2 never */
+                                       0 automatic (fewer work items than 2 x SMs, the largest of more
+                                       than 700 KB, or items too large for the persistent kernels;
+                                       groups that fit one CTA's shared memory run in one launch of
+                                       their own), 1 always, 2 never */
     double agg_ms, dis_ms;          /* times the autotuner measured (0 if not tuned) */
 } tfmm_tuning;
 tfmm_status tfmm_plan_tuning_get(const tfmm_plan* plan, tfmm_tuning* t);

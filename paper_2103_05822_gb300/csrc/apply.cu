@@ -1087,8 +1087,16 @@ void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s) {
     // ran the grouped-GEMM chain on 64-column tiles for one column (50 groups of up to 7273 RWGs, both
     // stages: 5.26 -> 0.55 ms).
     P.persistent_ok = P.agg_sched.blocks > 0 && P.dis_sched.blocks > 0;
+    // Automatic: few items, of which the largest would keep one CTA streaming for longer than the split
+    // path's two further launches a stage take.  Measured (aggregation + disaggregation, persistent / split,
+    // us): 182 items of up to 0.48 MB 50 / 61, of 0.92 MB 72 / 74; 52 items of 0.55 MB 40.5 / 43.5; 262
+    // of 0.33 MB 43 / 63; the trihedral's 38 1330 / 110.
+    constexpr int64_t kSplitItem = 700 << 10;
+    int64_t largest = 0;
+    for (const TuckerItem& d : P.items) largest = std::max<int64_t>(largest, 8ll * d.rb * (d.n_beta + d.rt * d.rp));
+    const bool few_large = nI < 2 * P.num_sms && largest > kSplitItem;
     const bool want_split = !plan_is_svd(P) && split_fits(P) &&
-                            (t.split == 1 || (t.split == 0 && (nI < 2 * P.num_sms || !P.persistent_ok)));
+                            (t.split == 1 || (t.split == 0 && (few_large || !P.persistent_ok)));
     P.hot_ok = P.persistent_ok || want_split;
     if (want_split != (bool)P.split) {  // captured graphs point into the split path's scratch
         TFMM_REQUIRE(P.live_graphs == 0, "destroy the plan's graphs before changing the single-RHS path");
@@ -1099,16 +1107,22 @@ void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s) {
 }
 
 // Block sizes and shared memory of the split path's kernels.
+constexpr size_t kSplitSmem = 200 * 1024;
 void split_smem(const Plan& P, SplitPlan& S) {
     const int nI = P.G * 2, NT = 512;
-    // blocks of SA3 and SD1: about two CTAs per SM over all items, at least 8 directions or 4 columns each
-    const int parts = std::max(4, (2 * P.num_sms + nI - 1) / nI);
-    S.blk_phi = std::max(8, (P.n_phi + parts - 1) / parts);
-    S.blk_b = std::max(4, (P.max_rank[1] + parts - 1) / parts);
+    // blocks of SA3 and SD1: about two CTAs per SM over all items, at least 8 directions or 4 columns each,
+    // and more where one would not fit (a block repeats the theta / phi factors' staging: four for each of
+    // 182 items cost 66 us a matvec instead of 62)
+    const int least = std::max(1, (2 * P.num_sms + nI - 1) / nI);
+    for (int parts = least; parts <= std::max(least, 8); ++parts) {
+        S.blk_phi = std::max(8, (P.n_phi + parts - 1) / parts);
+        S.blk_b = std::max(4, (P.max_rank[1] + parts - 1) / parts);
+        S.smem_ag34 = sizeof(float2) * split_ag34_layout(P, S.blk_phi).total;
+        S.smem_dg1 = sizeof(float2) * split_dg1_layout(P, S.blk_b).total;
+        if (std::max(S.smem_ag34, S.smem_dg1) <= kSplitSmem) break;
+    }
     S.smem_ag1 = sizeof(float2) * al16(P.max_ldnb);
     S.smem_ag2 = sizeof(float4) * NT + sizeof(float2) * al16(P.max_rank[2]);
-    S.smem_ag34 = sizeof(float2) * split_ag34_layout(P, S.blk_phi).total;
-    S.smem_dg1 = sizeof(float2) * split_dg1_layout(P, S.blk_b).total;
     S.smem_dg2 = sizeof(float2) * al16(P.max_ldab);
     S.smem_dg3 = sizeof(float4) * (NT + kSplitCols) + sizeof(float2) * al16(P.max_rank[2]);
 }
