@@ -15,9 +15,10 @@
 // of bfloat16, "K-major": row = M (or N) index, K contiguous, leading dimension
 // a multiple of 8 and zero beyond K.  A CTA computes a 128-row x BN tile
 // (BN <= 128, multiple of 16); K goes in steps of 32 through a ring of shared
-// memory stages filled by cp.async (zero-fill at ragged edges) in the
+// memory stages, filled by TMA (64-byte rows, 64-byte swizzle; tc_gemm_tma_kernel) or by
+// cp.async (zero-fill at ragged edges; tc_gemm_kernel) in the
 // no-swizzle canonical layout (8 x 16-byte core matrices; the next core matrix
-// along K is 128 bytes on, the next 8 rows 512 bytes on).  One thread issues
+// along K is 128 bytes on, the next 8 rows 512 bytes on).  One thread or lane issues
 // the MMAs of a stage and commits them to that stage's mbarrier, which frees
 // the stage for the next load.  The epilogue reads Cr / Ci from TMEM (one row
 // per thread) and writes the next step's operand planes, or the FP32 spectra /
@@ -33,10 +34,11 @@
 //   DG1b H'  (r_t R x r_p)        = P''      . U_phi        A: P'' [a+r_t r][i_phi]  B: U_phi^T [b][i_phi]
 //   DG2  S   (r_b x R)            = C_(3)    . H            A: C_(3) [c][ab]  B: H [r][ab]
 //   DG3  y_g (n_b x R)            = conj(U_beta^(0) S^(0) + U_beta^(1) S^(1))  A: U_beta [n][c]  B: S [r][c]
-// The generic stage kernel (tc_gemm_kernel) runs these as listed.  Two kernels replace
+// The generic stage kernels (tc_gemm_tma_kernel, tc_gemm_kernel) run these as listed.  Others replace
 // steps when the shapes allow: tc_ag34_kernel fuses AG3 and AG4 (V'' never leaves the
-// SM), and tc_dg1a_kernel runs DG1a transposed, U_theta^T as A and 128 (i_phi, r)
-// pairs of the spectra as N, so that its MMAs are wide.
+// SM), tc_dg1_kernel DG1a and DG1b (nor does P'').  Where the latter does not fit, tc_cat_kernel
+// runs the two with the factor's terms stacked along N, or tc_dg1a_kernel runs DG1a transposed,
+// U_theta^T as A and 128 (i_phi, r) pairs of the spectra as N.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
