@@ -296,16 +296,16 @@ def launches_per_step(tfmm, plan, R, dev):
     """Kernels one aggregate + disaggregate pair launches: one persistent kernel per stage
     or one per stage with small groups wholly in shared memory (at least; by size class when
     there are many) for one RHS (three per stage on the split path, taken by plans with fewer
-    work items than twice the SMs, of more than 700 KB), the tensor-core chain for many (operand prep and three kernels
+    work items than twice the SMs, of more than about 1 MB and 0.5 MB), the tensor-core chain for many (operand prep and three kernels
     for aggregation; four and the reordering of y for disaggregation)."""
     import torch
     t = tfmm.tfmm_plan_tuning_get(plan)
     if R == 1:
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
         rt, rp, rb = plan.info["max_rank"]
-        large = 8 * rb * (plan.info["max_n_beta"] + rt * rp) > 700 << 10
-        split = t["single_rhs_split"] == 1 or (t["single_rhs_split"] == 0 and large and plan.info["n_groups"] < sms)
-        return 6 if split else 2
+        largest = 8 * rb * (plan.info["max_n_beta"] + rt * rp)
+        few = t["single_rhs_split"] == 0 and plan.info["n_groups"] < sms
+        return sum(3 if t["single_rhs_split"] == 1 or (few and largest > kb << 10) else 1 for kb in (960, 450))
     return 9
 
 

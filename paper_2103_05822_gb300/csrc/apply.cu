@@ -1088,20 +1088,26 @@ void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s) {
     // stages: 5.26 -> 0.55 ms).
     P.persistent_ok = P.agg_sched.blocks > 0 && P.dis_sched.blocks > 0;
     // Automatic: few items, of which the largest would keep one CTA streaming for longer than the split
-    // path's two further launches a stage take.  Measured (aggregation + disaggregation, persistent / split,
-    // us): 182 items of up to 0.48 MB 50 / 61, of 0.92 MB 72 / 74; 52 items of 0.55 MB 40.5 / 43.5; 262
-    // of 0.33 MB 43 / 63; the trihedral's 38 1330 / 110.
-    constexpr int64_t kSplitItem = 700 << 10;
+    // path's two further launches take; the disaggregation, one CTA per group, sooner.  Measured (persistent /
+    // split, us; largest item): aggregation 182 items of 0.48 MB 21 / 28, 192 of 0.92 MB 30.4 / 35.0, 52 of
+    // 1.04 MB 26.6 / 24.9, 112 of 2.8 MB 67 / 62; disaggregation 262 of 0.33 MB 25 / 31, 182 of 0.48 MB
+    // 29.6 / 28.9, 52 of 0.55 MB 24.8 / 22.8, 192 of 0.92 MB 45.5 / 37.2, 112 of 2.8 MB 109 / 67.
+    constexpr int64_t kSplitAgg = 960 << 10, kSplitDis = 450 << 10;
     int64_t largest = 0;
     for (const TuckerItem& d : P.items) largest = std::max<int64_t>(largest, 8ll * d.rb * (d.n_beta + d.rt * d.rp));
-    const bool few_large = nI < 2 * P.num_sms && largest > kSplitItem;
-    const bool want_split = !plan_is_svd(P) && split_fits(P) &&
-                            (t.split == 1 || (t.split == 0 && (few_large || !P.persistent_ok)));
+    const bool few = t.split == 0 && nI < 2 * P.num_sms;
+    const bool all = t.split == 1 || (t.split == 0 && !P.persistent_ok);
+    const bool split_agg = all || (few && largest > kSplitAgg), split_dis = all || (few && largest > kSplitDis);
+    const bool want_split = !plan_is_svd(P) && (split_agg || split_dis) && split_fits(P);
     P.hot_ok = P.persistent_ok || want_split;
     if (want_split != (bool)P.split) {  // captured graphs point into the split path's scratch
         TFMM_REQUIRE(P.live_graphs == 0, "destroy the plan's graphs before changing the single-RHS path");
         P.split.reset();
         if (want_split) configure_split(P, s);
+    }
+    if (P.split) {
+        P.split->agg = split_agg;
+        P.split->dis = split_dis;
     }
     TFMM_CUDA_CHECK(cudaStreamSynchronize(s));
 }
@@ -1296,7 +1302,7 @@ void launch_split_disaggregate(const Plan& P, const float2* spec, int R, int wei
 
 void launch_tucker_aggregate(const Plan& P, const float2* x, int R, int64_t ldx, float2* spec, cudaStream_t s) {
     TFMM_REQUIRE(P.hot_ok, "single-RHS kernels unavailable for this plan (work item exceeds one CTA)");
-    if (P.split) {
+    if (P.split && P.split->agg) {
         launch_split_aggregate(P, x, R, ldx, spec, s);
         return;
     }
@@ -1329,7 +1335,7 @@ void launch_tucker_aggregate(const Plan& P, const float2* x, int R, int64_t ldx,
 void launch_tucker_disaggregate(const Plan& P, const float2* spec, int R, int weights, float2 beta, float2* y,
                                 int64_t ldy, cudaStream_t s) {
     TFMM_REQUIRE(P.hot_ok, "single-RHS kernels unavailable for this plan (work item exceeds one CTA)");
-    if (P.split) {
+    if (P.split && P.split->dis) {
         launch_split_disaggregate(P, spec, R, weights, beta, y, ldy, s);
         return;
     }

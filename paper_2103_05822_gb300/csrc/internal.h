@@ -221,6 +221,7 @@ struct HotTuning {
 // Split path of the single-RHS stages (plans with few, large items): tile lists of the
 // row- and column-block launches and the items' intermediates.
 struct SplitPlan {
+    bool agg = true, dis = true;              // stages that run split
     DeviceBuffer t_ag1, t_ag2, t_ag34, t_dg1, t_dg2, t_dg3;  // SplitTile lists
     int n_ag1 = 0, n_ag2 = 0, n_ag34 = 0, n_dg1 = 0, n_dg2 = 0, n_dg3 = 0;
     int blk_phi = 0, blk_b = 0;               // phi directions per SA3 tile, columns of U_phi per SD1 tile

@@ -260,3 +260,9 @@ def test_aggregation_last_steps_forms(nt, npf, top, R):
     nbetas = [140, 60]
     ranks = [[(rt, rp, 70), (rt - 1, rp - 5, 40)], [(5, 7, 30), (rt, 4, 25)]]
     _check(9000 + nt + R, nt, npf, nbetas, ranks, R, 3, 1e-6, pad=1)
+
+
+@pytest.mark.parametrize("rb", [60, 100, 160])
+def test_split_by_stage(rb):
+    """Largest items of 0.4, 0.7 and 1.1 MB: no stage split, the disaggregation only, both."""
+    _check(9500 + rb, 20, 40, [600, 333], [[(14, 16, rb), (9, 11, 50)], [(12, 13, rb - 1), (5, 6, 25)]], 1, 0, 1e-5, pad=1)
