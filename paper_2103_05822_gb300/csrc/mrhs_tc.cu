@@ -160,9 +160,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     return done != 0;
 }
 
+// 16 bytes, of which the first `bytes` come from src and the rest are zeros
 __device__ __forceinline__ void cp16(void* dst, const void* src, int bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes));
 }
+
+// Bytes of the 16-byte chunk at column k that hold any of a row's K values.  What follows them in
+// a scratch plane is not zero: the planes of the two stages share buffers in different layouts (M' and H, V''
+// and P''), and a NaN left there by the other stage would meet the other operand's zeros.
+__device__ __forceinline__ int chunk_bytes(int K, int k) { return min(max(2 * (K - k), 0), 16); }
 
 // v = t0 + t1 (+ t2) in bfloat16 terms, two values at once, one 32-bit word per term
 // (x0's term in the low half, x1's in the high half): the hardware conversion rounds
@@ -254,7 +260,6 @@ __device__ __forceinline__ void load_stage(uint8_t* st, const TcCtx& c, const Tc
     const bool seg1 = kt >= kt0;
     const int k0 = (seg1 ? kt - kt0 : kt) * TBK;
     const int K = seg1 ? p.K1 : p.K0;
-    const int K8 = (K + 7) & ~7;
     const bf16* A = seg1 ? p.A1 : p.A0;
     const bf16* B = seg1 ? p.B1 : p.B0;
     const int64_t ald = seg1 ? p.a_ld1 : p.a_ld0, aps = seg1 ? p.a_ps1 : p.a_ps0;
@@ -267,18 +272,18 @@ __device__ __forceinline__ void load_stage(uint8_t* st, const TcCtx& c, const Tc
     for (int idx = threadIdx.x; idx < na; idx += NTHR) {
         const int pl = idx / (TBM * 4), rem = idx % (TBM * 4), r = rem >> 2, kc = rem & 3;
         const int m = m0 + r, k = k0 + kc * 8;
-        const bool ok = m < p.M && k < K8;
-        const bf16* src = ok ? A + pl * aps + (int64_t)m * ald + k : A;
-        cp16(st + pl * PLANE_TILE + (r >> 3) * 512 + kc * 128 + (r & 7) * 16, src, ok ? 16 : 0);
+        const int bytes = m < p.M ? chunk_bytes(K, k) : 0;
+        const bf16* src = bytes ? A + pl * aps + (int64_t)m * ald + k : A;
+        cp16(st + pl * PLANE_TILE + (r >> 3) * 512 + kc * 128 + (r & 7) * 16, src, bytes);
     }
     const int nb = 2 * T * p.BN * 4;
     uint8_t* sb = st + 2 * T * PLANE_TILE;
     for (int idx = threadIdx.x; idx < nb; idx += NTHR) {
         const int pl = idx / (p.BN * 4), rem = idx % (p.BN * 4), r = rem >> 2, kc = rem & 3;
         const int n = n0 + r, k = k0 + kc * 8;
-        const bool ok = n < p.N && k < K8;
-        const bf16* src = ok ? B + pl * bps + (int64_t)n * bld + k : B;
-        cp16(sb + pl * b_plane + (r >> 3) * 512 + kc * 128 + (r & 7) * 16, src, ok ? 16 : 0);
+        const int bytes = n < p.N ? chunk_bytes(K, k) : 0;
+        const bf16* src = bytes ? B + pl * bps + (int64_t)n * bld + k : B;
+        cp16(sb + pl * b_plane + (r >> 3) * 512 + kc * 128 + (r & 7) * 16, src, bytes);
     }
 }
 
@@ -618,7 +623,7 @@ __device__ __forceinline__ uint64_t make_desc_sbo(uint32_t addr, uint32_t sbo) {
     return d;
 }
 
-// 2T planes of `rows` rows, rounded up to 8 (zero-filled from row `valid` and from column r8(kvalid))
+// 2T planes of `rows` rows, rounded up to 8 (zero-filled from row `valid` and from column `kvalid`)
 // of a K-major source into the canonical no-swizzle layout with depth K, of which the first `kuse`
 // columns are wanted; NTHR threads share the copies.  The chunks of 16 bytes are taken in the order of the
 // shared-memory layout (eight lanes write 128 bytes in a row, no bank twice) and the index of one serves
@@ -627,16 +632,16 @@ __device__ __forceinline__ uint64_t make_desc_sbo(uint32_t addr, uint32_t sbo) {
 template <int T>
 __device__ __forceinline__ void load_planes(uint8_t* dst, int plane_bytes, int K, const bf16* src, int64_t ld,
                                             int64_t ps, int rows, int valid, int kvalid, int kuse, int nthr) {
-    const int kc8 = K / 8, k8v = (kvalid + 7) / 8, k8u = kuse / 8;
+    const int kc8 = K / 8, k8u = kuse / 8;
     const int total = ((rows + 7) >> 3) * 8 * kc8;
     for (int idx = threadIdx.x; idx < total; idx += nthr) {
         const int core = idx >> 3, rb = core / kc8, kc = core - rb * kc8, r = rb * 8 + (idx & 7);
         if (kc >= k8u) continue;
-        const bool ok = r < valid && kc < k8v;
-        const bf16* g = ok ? src + (int64_t)r * ld + kc * 8 : src;
-        const int64_t step = ok ? ps : 0;
+        const int bytes = r < valid ? chunk_bytes(kvalid, kc * 8) : 0;
+        const bf16* g = bytes ? src + (int64_t)r * ld + kc * 8 : src;
+        const int64_t step = bytes ? ps : 0;
 #pragma unroll
-        for (int pl = 0; pl < 2 * T; ++pl) cp16(dst + pl * plane_bytes + idx * 16, g + pl * step, ok ? 16 : 0);
+        for (int pl = 0; pl < 2 * T; ++pl) cp16(dst + pl * plane_bytes + idx * 16, g + pl * step, bytes);
     }
 }
 
@@ -1477,18 +1482,18 @@ __device__ __forceinline__ void cat_store_g(uint8_t* sA, const float2 (&v)[CAT_I
     }
 }
 
-// DG1b A: rows p0 .. p0 + 127 of the P'' planes, 16-byte chunks by cp.async (zero past the
-// item's rows and past the planes' leading dimension, whose padding columns are zero)
+// DG1b A: rows p0 .. p0 + 127 of the P'' planes, K deep, 16-byte chunks by cp.async (zero past the
+// item's rows and past K)
 template <int T>
-__device__ __forceinline__ void cat_load_planes(uint8_t* sA, const CatItem& it, int p0, int kc8, uint32_t sbo,
+__device__ __forceinline__ void cat_load_planes(uint8_t* sA, const CatItem& it, int p0, int K, int kc8, uint32_t sbo,
                                                 int planeA) {
     const int ntask = TBM * kc8;
     for (int task = threadIdx.x; task < 2 * T * ntask; task += CAT_THREADS) {
         const int q = task / ntask, rem = task % ntask, i = rem / kc8, kc = rem % kc8, m = p0 + i;
         uint8_t* dst = sA + q * planeA + canon_off(i, kc, sbo);
-        const bool ok = m < it.M && kc * 8 < it.a_ld;
-        const bf16* src = ok ? it.a + q * it.a_ps + (int64_t)m * it.a_ld + kc * 8 : it.a;
-        cp16(dst, src, ok ? 16 : 0);
+        const int bytes = m < it.M ? chunk_bytes(K, kc * 8) : 0;
+        const bf16* src = bytes ? it.a + q * it.a_ps + (int64_t)m * it.a_ld + kc * 8 : it.a;
+        cp16(dst, src, bytes);
     }
     asm volatile("cp.async.commit_group;");
 }
@@ -1627,7 +1632,7 @@ __global__ void __launch_bounds__(CAT_THREADS) tc_cat_kernel(const TcCtx c, cons
         cat_build_b<T>(sBp, sBn, it, K, kc8, sbo, threadIdx.x);
         cat_store_g<T>(sA, v, kc8, sbo, planeA);
     } else {
-        cat_load_planes<T>(sA, it, t.p0, kc8, sbo, planeA);
+        cat_load_planes<T>(sA, it, t.p0, K, kc8, sbo, planeA);
         cat_build_b<T>(sBp, sBn, it, K, kc8, sbo, threadIdx.x);
         asm volatile("cp.async.wait_group 0;");
     }

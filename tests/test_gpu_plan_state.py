@@ -1,0 +1,55 @@
+"""What one call, one plan or one refused request leaves behind for the next, on the GPU.
+
+Scratch planes, launch limits and launch shapes outlive a call: each test makes a call that could
+disturb them and compares what follows with the same call on its own, bit for bit where the same
+kernels run.  Oracle bounds are those of ``test_gpu_kernels.py``.
+"""
+import numpy as np
+import pytest
+
+from oracle import apply
+from paper_2103_05822_gb300.inputs import complex_gaussian
+from test_gpu_edges import _problem, _worst
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(plan, R, seed):
+    i = plan.info
+    x = torch.from_numpy(complex_gaussian((R, i["n_rwg"]), seed).astype(np.complex64)).cuda()
+    g = torch.from_numpy(complex_gaussian((R, i["n_groups"], 2, i["n_dir"]), seed + 1).astype(np.complex64)).cuda()
+    return x, g
+
+
+def _agg(tfmm, plan, x):
+    i = plan.info
+    spec = torch.full((len(x), i["n_groups"], 2, i["n_dir"]), float("nan"), dtype=torch.complex64, device="cuda")
+    tfmm.tfmm_aggregate(plan, x, spec, R=len(x))
+    return spec
+
+
+def _dis(tfmm, plan, g):
+    y = torch.full((len(g), plan.info["n_rwg"]), float("nan"), dtype=torch.complex64, device="cuda")
+    tfmm.tfmm_disaggregate(plan, g, y, R=len(g))
+    return y
+
+
+# (n_theta, n_phi, rank): fused AG3 + AG4 and DG1a + DG1b; n_phi past the fused AG3 + AG4's lanes; r_theta past
+# the fused DG1 and n_phi past the stacked DG1b; the stacked DG1b with odd n_phi
+@pytest.mark.parametrize("nt,npf,rank", [(12, 25, (5, 9, 20)), (66, 131, (5, 9, 20)), (66, 131, (33, 9, 20)),
+                                         (40, 75, (33, 17, 30))])
+@pytest.mark.parametrize("terms", [2, 3])
+def test_non_finite_data_does_not_outlive_its_call(nt, npf, rank, terms):
+    """The planes of the two stages share buffers in different layouts, so that one stage's values lie in the
+    padding of the other's: after a call on NaN, calls on finite data give what they gave before."""
+    nbetas = [40, 33]
+    tfmm, plan, *_ = _problem(41, nt, npf, nbetas, [[rank, (3, 5, 9)], [(2, 3, 7), rank]], 3, terms)
+    x, g = _inputs(plan, 3, 42)
+    spec, y = _agg(tfmm, plan, x), _dis(tfmm, plan, g)
+    assert torch.isfinite(torch.view_as_real(spec)).all() and torch.isfinite(torch.view_as_real(y)).all()
+    _dis(tfmm, plan, torch.full_like(g, float("nan")))
+    assert torch.equal(_agg(tfmm, plan, x), spec)
+    _agg(tfmm, plan, torch.full_like(x, float("nan")))
+    assert torch.equal(_dis(tfmm, plan, g), y)
+    tfmm.tfmm_sync(plan)
