@@ -927,18 +927,27 @@ SmemLayout split_dg1_layout(const Plan& P, int blk) {
     return L;
 }
 
+// The dynamic shared memory a CTA of `kernel` may have on this device, and the kernel's limit raised
+// to it.  The limit belongs to the kernel, not to a plan: set to a plan's own need, a smaller plan made
+// later would lower it under a larger one's launches.
+size_t allow_all_smem(const void* kernel) {
+    int dev = 0, opt_in = 0;
+    TFMM_CUDA_CHECK(cudaGetDevice(&dev));
+    TFMM_CUDA_CHECK(cudaDeviceGetAttribute(&opt_in, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    cudaFuncAttributes fa{};
+    TFMM_CUDA_CHECK(cudaFuncGetAttributes(&fa, kernel));
+    const size_t room = (size_t)opt_in - fa.sharedSizeBytes;
+    TFMM_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room));
+    return room;
+}
+
 template <class K>
 Schedule make_schedule(K kernel, int NT, size_t smem, int num_sms, int n_items, int ctas_per_sm = 0) {
     Schedule s;
     s.threads = NT;
     s.smem = smem;
     s.blocks = 0;  // 0: the largest work item does not fit one CTA
-    int dev = 0, opt_in = 0;
-    TFMM_CUDA_CHECK(cudaGetDevice(&dev));
-    TFMM_CUDA_CHECK(cudaDeviceGetAttribute(&opt_in, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    if (smem > (size_t)opt_in) return s;
-    if (smem > 48 * 1024)
-        TFMM_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > allow_all_smem((const void*)kernel)) return s;
     int per_sm = 0;
     TFMM_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, smem));
     if (per_sm < 1) return s;
@@ -1112,7 +1121,7 @@ void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s) {
     TFMM_CUDA_CHECK(cudaStreamSynchronize(s));
 }
 
-// Block sizes and shared memory of the split path's kernels.
+// Block sizes and shared memory of the split path's kernels; split_fits also raises their limits.
 constexpr size_t kSplitSmem = 200 * 1024;
 void split_smem(const Plan& P, SplitPlan& S) {
     const int nI = P.G * 2, NT = 512;
@@ -1136,10 +1145,13 @@ void split_smem(const Plan& P, SplitPlan& S) {
 bool split_fits(const Plan& P) {
     SplitPlan S;
     split_smem(P, S);
-    int dev = 0, opt_in = 0;
-    TFMM_CUDA_CHECK(cudaGetDevice(&dev));
-    TFMM_CUDA_CHECK(cudaDeviceGetAttribute(&opt_in, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    return std::max({S.smem_ag1, S.smem_ag2, S.smem_ag34, S.smem_dg1, S.smem_dg2, S.smem_dg3}) <= (size_t)opt_in;
+    const std::pair<const void*, size_t> need[] = {
+        {(const void*)split_ag1_kernel, S.smem_ag1},   {(const void*)split_ag2_kernel, S.smem_ag2},
+        {(const void*)split_ag34_kernel, S.smem_ag34}, {(const void*)split_dg1_kernel, S.smem_dg1},
+        {(const void*)split_dg2_kernel, S.smem_dg2},   {(const void*)split_dg3_kernel, S.smem_dg3}};
+    bool fits = true;
+    for (const auto& [kernel, smem] : need) fits = smem <= allow_all_smem(kernel) && fits;
+    return fits;
 }
 
 // Tile lists, scratch and shared-memory sizes of the split path.
@@ -1190,15 +1202,6 @@ void configure_split(Plan& P, cudaStream_t s) {
     TFMM_CUDA_CHECK(device_malloc(&SP->scratch.p, sizeof(float2) * std::max<int64_t>(tot, 1)));
     TFMM_CUDA_CHECK(device_malloc(&SP->scr_off.p, sizeof(int64_t) * nI));
     TFMM_CUDA_CHECK(cudaMemcpyAsync(SP->scr_off.p, off.data(), sizeof(int64_t) * nI, cudaMemcpyHostToDevice, s));
-    auto allow = [](const void* k, size_t bytes) {
-        if (bytes > 48 * 1024) TFMM_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    };
-    allow((const void*)split_ag1_kernel, SP->smem_ag1);
-    allow((const void*)split_ag2_kernel, SP->smem_ag2);
-    allow((const void*)split_ag34_kernel, SP->smem_ag34);
-    allow((const void*)split_dg1_kernel, SP->smem_dg1);
-    allow((const void*)split_dg2_kernel, SP->smem_dg2);
-    allow((const void*)split_dg3_kernel, SP->smem_dg3);
     P.split = std::move(SP);
 }
 

@@ -53,3 +53,23 @@ def test_non_finite_data_does_not_outlive_its_call(nt, npf, rank, terms):
     _agg(tfmm, plan, torch.full_like(x, float("nan")))
     assert torch.equal(_dis(tfmm, plan, g), y)
     tfmm.tfmm_sync(plan)
+
+
+@pytest.mark.parametrize("split", [1, 2])
+def test_a_smaller_plan_leaves_a_larger_ones_launches_alone(split):
+    """A kernel's shared-memory limit is one for all plans: one of 136 KB runs on after one of 72 KB was made."""
+    def make(nb, seed):
+        tfmm, plan, n, members, T, w = _problem(seed, 6, 12, [nb, 40], [[(3, 4, 9)] * 2] * 2, 1, 0)
+        tfmm.tfmm_plan_tuning_set(plan, single_rhs_split=split)
+        return tfmm, plan, n, members, T, w
+
+    tfmm, large, n, members, T, w = make(16000, 51)
+    small = make(8000, 53)[1]
+    x, g = _inputs(large, 1, 54)
+    spec, y = _agg(tfmm, large, x).cpu().numpy()[0], _dis(tfmm, large, g).cpu().numpy()[0]
+    ref = apply.aggregate_all(T, members, x.cpu().numpy()[0].astype(np.complex128))
+    for i in range(2):
+        for a in range(2):
+            assert _worst(spec[i, a], ref[i, a]) <= 1e-5
+    assert _worst(y, apply.disaggregate_all(T, members, g.cpu().numpy()[0].astype(np.complex128), n, w)) <= 1e-5
+    del small
