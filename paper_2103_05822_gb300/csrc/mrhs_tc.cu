@@ -2115,14 +2115,23 @@ __global__ void planes_kernel(const float2* __restrict__ src, int rows, int cols
 // 972,000 RWGs in random order x 128 columns: 2.53 -> 0.72 ms (floor 0.37 ms: 1.0 GB read,
 // 1.5 GB written).
 constexpr int kXTile = 512, kXCols = 4;
+
+// Calls launch(first column, rows of column blocks) over R columns, a launch's grid.y being 65535 at most.
+template <class F>
+void by_column_blocks(int R, F&& launch) {
+    constexpr int64_t most = (int64_t)65535 * kXCols;
+    for (int64_t r0 = 0; r0 < R; r0 += most)
+        launch((int)r0, (unsigned)((std::min<int64_t>(R - r0, most) + kXCols - 1) / kXCols));
+}
+
 template <int T>
 __global__ void __launch_bounds__(kXTile / 2) prep_x_kernel(const float2* __restrict__ x, int64_t ldx,
                                                             const int* __restrict__ grp_rwg,
                                                             const TcProb* __restrict__ probs,
-                                                            const MrTile* __restrict__ tiles, int R) {
+                                                            const MrTile* __restrict__ tiles, int first, int R) {
     const MrTile t = tiles[blockIdx.x];
     const TcProb& p = probs[t.prob];  // AG1 problem of (g, alpha = 0): B0 points at the group's X planes
-    const int nb = p.K0, n = t.n0 + 2 * (int)threadIdx.x, r0 = blockIdx.y * kXCols;
+    const int nb = p.K0, n = t.n0 + 2 * (int)threadIdx.x, r0 = first + blockIdx.y * kXCols;
     if (n >= nb) return;
     const int64_t ld = p.b_ld0, ps = p.b_ps0;
     bf16* dst = const_cast<bf16*>(p.B0);
@@ -2159,11 +2168,11 @@ __global__ void __launch_bounds__(kXTile / 2) prep_x_kernel(const float2* __rest
 // order x 128 columns: DG3 5.55 ms -> 2.64 + 0.52 ms; 108,000 x 37 (y fits L2): 0.389 ->
 // 0.210 + 0.020 ms; 432,000 x 16: 1.22 -> 1.16 + 0.03 ms, so every size takes this way.
 __global__ void __launch_bounds__(256) order_y_kernel(const float2* __restrict__ ybuf, const int* __restrict__ pos,
-                                                      int64_t N, int R, float2 beta, float2* __restrict__ y,
-                                                      int64_t ldy) {
+                                                      int64_t N, int first, int R, float2 beta,
+                                                      float2* __restrict__ y, int64_t ldy) {
     const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (n >= N) return;
-    const int r0 = blockIdx.y * kXCols, nc = min(kXCols, R - r0);
+    const int r0 = first + blockIdx.y * kXCols, nc = min(kXCols, R - r0);
     const float2* src = ybuf + (int64_t)r0 * N + pos[n];
     float2* dst = y + n + ldy * r0;
     float2 v[kXCols], o[kXCols];
@@ -2929,10 +2938,12 @@ void tc_aggregate_t(Plan& P, TcPlan& M, const float2* x, int R, int64_t ldx, flo
     TcCtx c{};
     c.R = R; c.G = P.G; c.n_theta = P.n_theta; c.n_dir = P.n_dir; c.err = static_cast<int*>(P.tc_err.p);
     c.spec = spec;
-    const dim3 gx(M.n_xtiles, (R + kXCols - 1) / kXCols);
-    prep_x_kernel<T><<<gx, kXTile / 2, 0, s>>>(x, ldx, P.d_grp_rwg, reinterpret_cast<const TcProb*>(M.st[TAG1].d_probs),
-                                               static_cast<const MrTile*>(M.x_tiles.p), R);
-    TFMM_CUDA_CHECK(cudaGetLastError());
+    by_column_blocks(R, [&](int first, unsigned rows) {
+        prep_x_kernel<T><<<dim3(M.n_xtiles, rows), kXTile / 2, 0, s>>>(
+            x, ldx, P.d_grp_rwg, reinterpret_cast<const TcProb*>(M.st[TAG1].d_probs),
+            static_cast<const MrTile*>(M.x_tiles.p), first, R);
+        TFMM_CUDA_CHECK(cudaGetLastError());
+    });
     launch_tc<T, TAG1>(M.st[TAG1], c, P.num_sms, s);
     launch_tc<T, TAG2>(M.st[TAG2], c, P.num_sms, s);
     if (M.fused34) {
@@ -2976,9 +2987,11 @@ void tc_disaggregate_t(Plan& P, TcPlan& M, const float2* spec, int R, int weight
     c.ybuf = static_cast<float2*>(M.ybuf.p);
     c.N = P.N;
     launch_tc<T, TDG3>(M.st[TDG3], c, P.num_sms, s);
-    const dim3 gy((unsigned)((P.N + 255) / 256), (R + kXCols - 1) / kXCols);
-    order_y_kernel<<<gy, 256, 0, s>>>(c.ybuf, static_cast<const int*>(M.y_pos.p), P.N, R, beta, y, ldy);
-    TFMM_CUDA_CHECK(cudaGetLastError());
+    by_column_blocks(R, [&](int first, unsigned rows) {
+        order_y_kernel<<<dim3((unsigned)((P.N + 255) / 256), rows), 256, 0, s>>>(
+            c.ybuf, static_cast<const int*>(M.y_pos.p), P.N, first, R, beta, y, ldy);
+        TFMM_CUDA_CHECK(cudaGetLastError());
+    });
 }
 
 }  // namespace

@@ -73,3 +73,19 @@ def test_a_smaller_plan_leaves_a_larger_ones_launches_alone(split):
             assert _worst(spec[i, a], ref[i, a]) <= 1e-5
     assert _worst(y, apply.disaggregate_all(T, members, g.cpu().numpy()[0].astype(np.complex128), n, w)) <= 1e-5
     del small
+
+
+def test_more_columns_than_one_launch_of_the_gather_takes():
+    """262,148 columns on the tensor cores: past 65,535 blocks of four."""
+    R = 4 * 65535 + 8
+    tfmm, plan, n, members, T, w = _problem(61, 3, 5, [6], [[(2, 3, 4), (3, 2, 5)]], R, 3)
+    i = plan.info
+    few = complex_gaussian((7, n), 62).astype(np.complex64)
+    g7 = complex_gaussian((7, 1, 2, i["n_dir"]), 63).astype(np.complex64)
+    spec = _agg(tfmm, plan, torch.from_numpy(np.resize(few, (R, n))).cuda()).cpu().numpy()
+    y = _dis(tfmm, plan, torch.from_numpy(np.resize(g7, (R, 1, 2, i["n_dir"]))).cuda()).cpu().numpy()
+    for r in range(7):
+        ref = apply.aggregate_all(T, members, few[r].astype(np.complex128))
+        assert max(_worst(spec[r, 0, a], ref[0, a]) for a in range(2)) <= 1e-6
+        assert _worst(y[r], apply.disaggregate_all(T, members, g7[r].astype(np.complex128), n, w)) <= 1e-6
+        assert (spec[r::7] == spec[r]).all() and (y[r::7] == y[r]).all()
