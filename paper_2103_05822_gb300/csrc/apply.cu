@@ -1045,19 +1045,62 @@ void finalize_hot_layout(Plan& P, cudaStream_t s) {
     configure_hot(P, P.tuning, s);
 }
 
-void configure_split(Plan& P, cudaStream_t s);
+std::unique_ptr<SplitPlan> make_split(const Plan& P, cudaStream_t s);
 bool split_fits(const Plan& P);
 
-// Queue orders (0: most factor bytes first, the LPT rule; 1: group order) and
-// persistent grids (threads per CTA, CTAs per SM capped by occupancy) of the
-// two single-RHS kernels.
-void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s) {
+// What a tuning makes of the single-RHS stages: persistent grids (threads per CTA, CTAs per SM capped by
+// occupancy) and the stages that run split.  Changes nothing of the plan.
+HotShape plan_hot(const Plan& P, const HotTuning& t) {
     const int nI = P.G * 2;
     auto ok_threads = [](int nt) { return nt >= 64 && nt <= 512 && nt % 32 == 0; };
     TFMM_REQUIRE(ok_threads(t.agg_threads) && ok_threads(t.dis_threads), "threads per CTA must be 64..512, a multiple of 32");
     TFMM_REQUIRE(t.agg_ctas_per_sm >= 0 && t.dis_ctas_per_sm >= 0, "CTAs per SM must be >= 0");
     TFMM_REQUIRE((t.agg_order == 0 || t.agg_order == 1) && (t.dis_order == 0 || t.dis_order == 1), "order must be 0 or 1");
     TFMM_REQUIRE(t.split >= 0 && t.split <= 2, "split must be 0 (automatic), 1 (always) or 2 (never)");
+    HotShape h;
+    if (plan_is_svd(P)) {
+        h.agg = make_schedule(tucker_aggregate_kernel<true>, t.agg_threads,
+                              sizeof(float2) * svd_agg_layout(P, t.agg_threads).total, P.num_sms, nI,
+                              t.agg_ctas_per_sm);
+        h.dis = make_schedule(tucker_disaggregate_kernel<true>, t.dis_threads,
+                              sizeof(float2) * svd_dis_layout(P, t.dis_threads).total, P.num_sms, P.G,
+                              t.dis_ctas_per_sm);
+    } else {
+        h.agg = make_schedule(tucker_aggregate_kernel<false>, t.agg_threads,
+                              sizeof(float2) * agg_layout(P, t.agg_threads).total, P.num_sms, nI, t.agg_ctas_per_sm);
+        h.dis = make_schedule(tucker_disaggregate_kernel<false>, t.dis_threads,
+                              sizeof(float2) * dis_layout(P, t.dis_threads).total, P.num_sms, P.G, t.dis_ctas_per_sm);
+    }
+    // The split path needs less shared memory than the persistent kernels (a block of the theta /
+    // phi work at a time), so it also takes the plans whose items do not fit those: 4-lambda boxes, which
+    // ran the grouped-GEMM chain on 64-column tiles for one column (50 groups of up to 7273 RWGs, both
+    // stages: 5.26 -> 0.55 ms).
+    h.persistent = h.agg.blocks > 0 && h.dis.blocks > 0;
+    // Automatic: few items, of which the largest would keep one CTA streaming for longer than the split
+    // path's two further launches take; the disaggregation, one CTA per group, sooner.  Measured (persistent /
+    // split, us; largest item): aggregation 182 items of 0.48 MB 21 / 28, 192 of 0.92 MB 30.4 / 35.0, 52 of
+    // 1.04 MB 26.6 / 24.9, 112 of 2.8 MB 67 / 62; disaggregation 262 of 0.33 MB 25 / 31, 182 of 0.48 MB
+    // 29.6 / 28.9, 52 of 0.55 MB 24.8 / 22.8, 192 of 0.92 MB 45.5 / 37.2, 112 of 2.8 MB 109 / 67.
+    constexpr int64_t kSplitAgg = 960 << 10, kSplitDis = 450 << 10;
+    int64_t largest = 0;
+    for (const TuckerItem& d : P.items) largest = std::max<int64_t>(largest, 8ll * d.rb * (d.n_beta + d.rt * d.rp));
+    const bool few = t.split == 0 && nI < 2 * P.num_sms;
+    const bool all = t.split == 1 || (t.split == 0 && !h.persistent);
+    h.split_agg = all || (few && largest > kSplitAgg);
+    h.split_dis = all || (few && largest > kSplitDis);
+    h.split = !plan_is_svd(P) && (h.split_agg || h.split_dis) && split_fits(P);
+    return h;
+}
+
+// Queue orders (0: most factor bytes first, the LPT rule; 1: group order), persistent grids and split
+// path of the single-RHS stages.  The checks come first: a tuning that is refused changes nothing.
+void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s) {
+    const int nI = P.G * 2;
+    const HotShape h = plan_hot(P, t);
+    if (h.split != (bool)P.split)  // captured graphs point into the split path's scratch
+        TFMM_REQUIRE(P.live_graphs == 0, "destroy the plan's graphs before changing the single-RHS path");
+    std::unique_ptr<SplitPlan> split;
+    if (h.split && !P.split) split = make_split(P, s);
     auto bytes = [&](const TuckerItem& d) {
         return (double)d.rb * d.ld_nb + (double)d.rb * d.ld_ab + (double)P.n_phi * d.rp + (double)P.n_theta * d.rt;
     };
@@ -1075,48 +1118,16 @@ void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s) {
     // stream-ordered: launches already queued keep reading the old order until these copies land
     TFMM_CUDA_CHECK(cudaMemcpyAsync(P.d_agg_order, agg.data(), sizeof(int) * nI, cudaMemcpyHostToDevice, s));
     TFMM_CUDA_CHECK(cudaMemcpyAsync(P.d_dis_order, dis.data(), sizeof(int) * P.G, cudaMemcpyHostToDevice, s));
-    if (plan_is_svd(P)) {
-        P.agg_sched = make_schedule(tucker_aggregate_kernel<true>, t.agg_threads,
-                                    sizeof(float2) * svd_agg_layout(P, t.agg_threads).total, P.num_sms, nI,
-                                    t.agg_ctas_per_sm);
-        P.dis_sched = make_schedule(tucker_disaggregate_kernel<true>, t.dis_threads,
-                                    sizeof(float2) * svd_dis_layout(P, t.dis_threads).total, P.num_sms, P.G,
-                                    t.dis_ctas_per_sm);
-    } else {
-        P.agg_sched = make_schedule(tucker_aggregate_kernel<false>, t.agg_threads,
-                                    sizeof(float2) * agg_layout(P, t.agg_threads).total, P.num_sms, nI,
-                                    t.agg_ctas_per_sm);
-        P.dis_sched = make_schedule(tucker_disaggregate_kernel<false>, t.dis_threads,
-                                    sizeof(float2) * dis_layout(P, t.dis_threads).total, P.num_sms, P.G,
-                                    t.dis_ctas_per_sm);
-    }
+    P.agg_sched = h.agg;
+    P.dis_sched = h.dis;
     P.tuning = t;
-    // The split path needs less shared memory than the persistent kernels (a block of the theta /
-    // phi work at a time), so it also takes the plans whose items do not fit those: 4-lambda boxes, which
-    // ran the grouped-GEMM chain on 64-column tiles for one column (50 groups of up to 7273 RWGs, both
-    // stages: 5.26 -> 0.55 ms).
-    P.persistent_ok = P.agg_sched.blocks > 0 && P.dis_sched.blocks > 0;
-    // Automatic: few items, of which the largest would keep one CTA streaming for longer than the split
-    // path's two further launches take; the disaggregation, one CTA per group, sooner.  Measured (persistent /
-    // split, us; largest item): aggregation 182 items of 0.48 MB 21 / 28, 192 of 0.92 MB 30.4 / 35.0, 52 of
-    // 1.04 MB 26.6 / 24.9, 112 of 2.8 MB 67 / 62; disaggregation 262 of 0.33 MB 25 / 31, 182 of 0.48 MB
-    // 29.6 / 28.9, 52 of 0.55 MB 24.8 / 22.8, 192 of 0.92 MB 45.5 / 37.2, 112 of 2.8 MB 109 / 67.
-    constexpr int64_t kSplitAgg = 960 << 10, kSplitDis = 450 << 10;
-    int64_t largest = 0;
-    for (const TuckerItem& d : P.items) largest = std::max<int64_t>(largest, 8ll * d.rb * (d.n_beta + d.rt * d.rp));
-    const bool few = t.split == 0 && nI < 2 * P.num_sms;
-    const bool all = t.split == 1 || (t.split == 0 && !P.persistent_ok);
-    const bool split_agg = all || (few && largest > kSplitAgg), split_dis = all || (few && largest > kSplitDis);
-    const bool want_split = !plan_is_svd(P) && (split_agg || split_dis) && split_fits(P);
-    P.hot_ok = P.persistent_ok || want_split;
-    if (want_split != (bool)P.split) {  // captured graphs point into the split path's scratch
-        TFMM_REQUIRE(P.live_graphs == 0, "destroy the plan's graphs before changing the single-RHS path");
-        P.split.reset();
-        if (want_split) configure_split(P, s);
-    }
+    P.persistent_ok = h.persistent;
+    P.hot_ok = h.persistent || h.split;
+    if (split) P.split = std::move(split);
+    if (!h.split) P.split.reset();
     if (P.split) {
-        P.split->agg = split_agg;
-        P.split->dis = split_dis;
+        P.split->agg = h.split_agg;
+        P.split->dis = h.split_dis;
     }
     TFMM_CUDA_CHECK(cudaStreamSynchronize(s));
 }
@@ -1155,7 +1166,7 @@ bool split_fits(const Plan& P) {
 }
 
 // Tile lists, scratch and shared-memory sizes of the split path.
-void configure_split(Plan& P, cudaStream_t s) {
+std::unique_ptr<SplitPlan> make_split(const Plan& P, cudaStream_t s) {
     auto SP = std::make_unique<SplitPlan>();
     const int nI = P.G * 2;
     split_smem(P, *SP);
@@ -1202,7 +1213,7 @@ void configure_split(Plan& P, cudaStream_t s) {
     TFMM_CUDA_CHECK(device_malloc(&SP->scratch.p, sizeof(float2) * std::max<int64_t>(tot, 1)));
     TFMM_CUDA_CHECK(device_malloc(&SP->scr_off.p, sizeof(int64_t) * nI));
     TFMM_CUDA_CHECK(cudaMemcpyAsync(SP->scr_off.p, off.data(), sizeof(int64_t) * nI, cudaMemcpyHostToDevice, s));
-    P.split = std::move(SP);
+    return SP;
 }
 
 void finalize_dense_layout(Plan& P) {

@@ -244,6 +244,14 @@ struct Schedule {
     size_t smem = 0;      // dynamic shared memory per CTA
 };
 
+// Single-RHS stages as a tuning makes them (plan_hot).
+struct HotShape {
+    Schedule agg, dis;
+    bool persistent = false;                  // the largest work item fits the persistent kernels
+    bool split = false;                       // the split path runs, for the stages below
+    bool split_agg = false, split_dis = false;
+};
+
 // ----------------------------------------------------------------------- plan
 struct HostFactors64 {     // FP64 factors of one (g, alpha), device memory (inside an arena)
     double2* base = nullptr;  // U_theta | U_phi | U_beta | core (column-major, back to back)
@@ -364,6 +372,7 @@ void launch_dense_aggregate(const Plan& P, const float2* x, int R, int64_t ldx, 
 void launch_dense_disaggregate(const Plan& P, const float2* spec, int R, int weights, float2 beta, float2* y,
                                int64_t ldy, cudaStream_t s);
 void pack_factors_fp32(Plan& P, cudaStream_t s);  // from P.f64 into P.d_factors
+HotShape plan_hot(const Plan& P, const HotTuning& t);
 void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s);  // orders and schedules of the 1-RHS kernels
 // small.cu
 void configure_small(Plan& P, cudaStream_t s);  // after the items are known

@@ -388,24 +388,23 @@ tfmm_status tfmm_plan_tuning_set(tfmm_plan* plan, const tfmm_tuning* t, void* st
                      "tc_dg1a_pairs must be 0, 64 or 128");
         TFMM_REQUIRE(t->single_rhs_split >= 0 && t->single_rhs_split <= 2,
                      "single_rhs_split must be 0 (automatic), 1 (always) or 2 (never)");
-        if (t->tc_f34_n1 != plan->p.tc_f34_n1 || t->tc_dg1a_pairs != plan->p.tc_dg1a_pairs) {
-            TFMM_REQUIRE(plan->p.live_graphs == 0, "destroy the plan's graphs before changing tile shapes");
-            plan->p.tc_f34_n1 = t->tc_f34_n1;
-            plan->p.tc_dg1a_pairs = t->tc_dg1a_pairs;
-            tc_replan_shapes(plan->p);
-        }
+        Plan& P = plan->p;
         HotTuning h;
         h.agg_threads = t->agg_threads; h.agg_ctas_per_sm = t->agg_ctas_per_sm; h.agg_order = t->agg_order;
         h.dis_threads = t->dis_threads; h.dis_ctas_per_sm = t->dis_ctas_per_sm; h.dis_order = t->dis_order;
         h.split = t->single_rhs_split;
-        const HotTuning old = plan->p.tuning;
-        const bool was_ok = plan->p.persistent_ok;
-        configure_hot(plan->p, h, (cudaStream_t)stream);
-        if (was_ok && !plan->p.persistent_ok) {
-            configure_hot(plan->p, old, (cudaStream_t)stream);
-            fail(TFMM_INVALID_ARG, "launch shape leaves no room for the largest work item");
+        // every check before the first change
+        const bool tiles = t->tc_f34_n1 != P.tc_f34_n1 || t->tc_dg1a_pairs != P.tc_dg1a_pairs;
+        if (tiles) TFMM_REQUIRE(P.live_graphs == 0, "destroy the plan's graphs before changing tile shapes");
+        if (P.persistent_ok)
+            TFMM_REQUIRE(plan_hot(P, h).persistent, "launch shape leaves no room for the largest work item");
+        configure_hot(P, h, (cudaStream_t)stream);
+        if (tiles) {
+            P.tc_f34_n1 = t->tc_f34_n1;
+            P.tc_dg1a_pairs = t->tc_dg1a_pairs;
+            tc_replan_shapes(P);
         }
-        plan->p.params.mrhs_precision = t->mrhs_precision;
+        P.params.mrhs_precision = t->mrhs_precision;
     });
 }
 
@@ -455,8 +454,8 @@ tfmm_status tfmm_autotune(tfmm_plan* plan, int32_t R, double budget_ms, int32_t 
                             (stage == 0 ? t.agg_threads : t.dis_threads) = nt;
                             (stage == 0 ? t.agg_ctas_per_sm : t.dis_ctas_per_sm) = c;
                             (stage == 0 ? t.agg_order : t.dis_order) = order;
+                            if (P.persistent_ok && !plan_hot(P, t).persistent) continue;  // no room for the largest item
                             configure_hot(P, t, s);
-                            if (!P.hot_ok) continue;
                             const Schedule& sc = stage == 0 ? P.agg_sched : P.dis_sched;
                             if (std::find(seen.begin(), seen.end(), std::make_pair(nt * 2 + order, sc.blocks)) !=
                                 seen.end())

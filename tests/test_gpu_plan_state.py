@@ -89,3 +89,54 @@ def test_more_columns_than_one_launch_of_the_gather_takes():
         assert max(_worst(spec[r, 0, a], ref[0, a]) for a in range(2)) <= 1e-6
         assert _worst(y[r], apply.disaggregate_all(T, members, g7[r].astype(np.complex128), n, w)) <= 1e-6
         assert (spec[r::7] == spec[r]).all() and (y[r::7] == y[r]).all()
+
+
+def _large_item_plan(threads=64):
+    """One group whose items fit the persistent kernels with 64 threads a CTA and not with 512 (their scratch)."""
+    tfmm, plan, *_ = _problem(71, 3, 6, [28500], [[(1, 1, 1), (2, 3, 2)]], 1, 0)
+    assert tfmm.tfmm_plan_tuning_get(plan)["dis_blocks"] == 0
+    tfmm.tfmm_plan_tuning_set(plan, agg_threads=threads, dis_threads=threads, single_rhs_split=0)
+    assert tfmm.tfmm_plan_tuning_get(plan)["dis_blocks"] > 0
+    return tfmm, plan
+
+
+@pytest.mark.parametrize("change", [{"agg_threads": 512}, {"dis_threads": 512}, {"single_rhs_split": 1},
+                                    {"single_rhs_split": 1, "mrhs_precision": 3},
+                                    {"agg_threads": 96, "tc_dg1a_pairs": 64}])
+@pytest.mark.parametrize("graph", [True, False])
+def test_a_refused_tuning_changes_nothing(change, graph):
+    tfmm, plan = _large_item_plan()
+    x, g = _inputs(plan, 1, 72)
+    spec, y = _agg(tfmm, plan, x), _dis(tfmm, plan, g)
+    before = tfmm.tfmm_plan_tuning_get(plan)
+    if graph:
+        out = torch.zeros_like(spec)
+        held = tfmm.tfmm_graph_capture(plan, 1, out, x=x)
+    elif 512 not in change.values():
+        return  # only a graph that is still held forbids the others
+    with pytest.raises(tfmm.TfmmError) as e:
+        tfmm.tfmm_plan_tuning_set(plan, **change)
+    assert e.value.status == tfmm.INVALID_ARG
+    assert tfmm.tfmm_plan_tuning_get(plan) == before
+    assert torch.equal(_agg(tfmm, plan, x), spec) and torch.equal(_dis(tfmm, plan, g), y)
+    if graph:
+        out.zero_()
+        held.launch()
+        torch.cuda.synchronize()
+        assert torch.equal(out, spec)
+        tfmm.tfmm_graph_destroy(held)
+
+
+def test_autotuning_beside_a_graph_skips_shapes_without_room():
+    tfmm, plan = _large_item_plan()
+    x, g = _inputs(plan, 1, 73)
+    spec = _agg(tfmm, plan, x)
+    out = torch.zeros_like(spec)
+    held = tfmm.tfmm_graph_capture(plan, 1, out, x=x)
+    t = tfmm.tfmm_autotune(plan, R=1, budget_ms=500.0)
+    assert t["agg_blocks"] > 0 and t["dis_blocks"] > 0 and t["single_rhs_split"] == 0
+    _agg(tfmm, plan, x), _dis(tfmm, plan, g)
+    held.launch()
+    torch.cuda.synchronize()
+    assert torch.equal(out, spec)
+    tfmm.tfmm_graph_destroy(held)
