@@ -73,7 +73,8 @@ typedef struct {
     int32_t batch_groups; /* groups per setup batch (0 = automatic) */
     int32_t mrhs_precision; /* engine for R > 1: 0 = FP32 on CUDA cores: the grouped-GEMM chain, or
                                whichever other FP32 kernels are faster for the plan and R;
-                               1 = the single-RHS kernels, one column after another (FP32);
+                               1 = the kernels of R = 1, one column after another (FP32), so that
+                               each column has the bits of a call of its own;
                                2 or 3 = tensor cores with FP32 operands split into 2 or 3
                                BF16 terms (hi + lo [+ lo2]), FP32 accumulation */
     int32_t compression; /* 0 = Tucker (Eq. 6, gamma / sqrt(3) per mode); 1 = truncated SVD of

@@ -367,7 +367,7 @@ void with_cols(int cols, F&& f) {
 // Columns per pass: the most, up to R, with which three CTAs fit an SM, else two, else one.
 template <class Work>
 int pick_cols(const Plan& P, const SmallClass& k, int R, Work work) {
-    if (R == 1) return 1;
+    if (R == 1 || P.params.mrhs_precision == 1) return 1;  // 1: every column as a call of its own
     for (size_t room : {kThirdSM, kHalfSM, P.small_room})
         for (int c : kBlocks)
             if ((c < 2 * R || c == 4) && c > 1 && sizeof(float2) * work(P, k, c).total <= room) return c;

@@ -166,7 +166,9 @@ void check_params(const tfmm_params& p) {
 // The engine that applies one call with R columns:
 //   small:   one CTA per (group, component) with everything in shared memory, for plans whose
 //            every item fits (small.cu), in place of columns and chain unless the tuning
-//            asks for one of the single-RHS paths;
+//            asks for one of the single-RHS paths; mrhs_precision 1 takes it one column
+//            at a time and only where a one-column call does, so that its columns have
+//            the bits of one-column calls;
 //   columns: the single-RHS kernels, one column after the other (R = 1, or mrhs_precision 1,
 //            or TFMM_MR=loop, or few columns of mrhs_precision 0);
 //   chain:   the grouped-GEMM chain on FP32 CUDA cores (mrhs_precision 0), also the
@@ -179,7 +181,7 @@ Engine engine_for(const Plan& P, int R, int* terms) {
     const int p = P.params.mrhs_precision;
     const char* e = std::getenv("TFMM_MR");
     const bool loop = e && std::strcmp(e, "loop") == 0;
-    if (P.tuning.split == 0 && !loop && (R <= 1 ? P.small_one : P.small_ok && p <= 1)) return Engine::small;
+    if (P.tuning.split == 0 && !loop && (R <= 1 || p == 1 ? P.small_one : P.small_ok && p == 0)) return Engine::small;
     // Up to kColumnsMax columns the chain reads every factor about as slowly as for one tile's width, and
     // the single-RHS kernels stream them once per column near the copy rate.  Measured, chain / columns
     // (both stages, ms): 20-lambda sphere in 2-lambda boxes, 2 columns 2.95 / 1.50, 4 3.15 / 2.99, 6 3.39 / 4.49;

@@ -140,3 +140,19 @@ def test_autotuning_beside_a_graph_skips_shapes_without_room():
     torch.cuda.synchronize()
     assert torch.equal(out, spec)
     tfmm.tfmm_graph_destroy(held)
+
+
+@pytest.mark.parametrize("G,nb", [(3, 60), (400, 24), (3, 2500)])
+def test_one_column_after_another_gives_the_bits_of_one_column_calls(G, nb):
+    """mrhs_precision 1 on groups that fit one CTA's shared memory, few (one launch a column there) and many
+    (the persistent kernels), and on groups that do not."""
+    rng = np.random.default_rng(81)
+    ranks = [[(5, 7, min(nb, 20)), (4, 9, min(nb, 17))] for _ in range(G)]
+    nbetas = [int(v) for v in rng.integers(max(1, nb - 3), nb + 1, G)]
+    ranks = [[(a, b, min(c, n)) for a, b, c in r] for r, n in zip(ranks, nbetas)]
+    tfmm, plan, *_ = _problem(82, 10, 21, nbetas, ranks, 5, 1)
+    x, g = _inputs(plan, 5, 83)
+    spec, y = _agg(tfmm, plan, x), _dis(tfmm, plan, g)
+    for r in range(5):
+        assert torch.equal(spec[r], _agg(tfmm, plan, x[r:r + 1])[0])
+        assert torch.equal(y[r], _dis(tfmm, plan, g[r:r + 1])[0])
