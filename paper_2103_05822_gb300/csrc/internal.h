@@ -376,6 +376,7 @@ HotShape plan_hot(const Plan& P, const HotTuning& t);
 void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s);  // orders and schedules of the 1-RHS kernels
 // small.cu
 void configure_small(Plan& P, cudaStream_t s);  // after the items are known
+bool small_takes(const Plan& P, bool aggregation, int R);  // where these kernels are the faster ones
 void launch_small_aggregate(const Plan& P, const float2* x, int R, int64_t ldx, float2* spec, cudaStream_t s);
 void launch_small_disaggregate(const Plan& P, const float2* spec, int R, int weights, float2 beta, float2* y,
                                int64_t ldy, cudaStream_t s);

@@ -365,13 +365,34 @@ void with_cols(int cols, F&& f) {
 }
 
 // Columns per pass: the most, up to R, with which three CTAs fit an SM, else two, else one.
+struct SmallPass {
+    int cols, per_sm;
+};
 template <class Work>
-int pick_cols(const Plan& P, const SmallClass& k, int R, Work work) {
-    if (R == 1 || P.params.mrhs_precision == 1) return 1;  // 1: every column as a call of its own
-    for (size_t room : {kThirdSM, kHalfSM, P.small_room})
+SmallPass pick_pass(const Plan& P, const SmallClass& k, int R, Work work) {
+    if (R == 1 || P.params.mrhs_precision == 1) return {1, 1};  // 1: every column as a call of its own
+    const size_t room[3] = {kThirdSM, kHalfSM, P.small_room};
+    for (int i = 0; i < 3; ++i)
         for (int c : kBlocks)
-            if ((c < 2 * R || c == 4) && c > 1 && sizeof(float2) * work(P, k, c).total <= room) return c;
-    return 1;
+            if ((c < 2 * R || c == 4) && c > 1 && sizeof(float2) * work(P, k, c).total <= room[i]) return {c, 3 - i};
+    return {1, 1};
+}
+
+// Columns in blocks pay where a pass takes four at least: with one, a pass costs as much as a column of
+// the persistent kernels and more.  Past 48 columns the passes of one CTA also lose to the chain where
+// the CTAs do not fill the SMs, or where four columns fill an SM's shared memory.  Measured (us, this /
+// chain), one column a pass: 300 groups of 200 KB disaggregation, 16 columns 567 / 264, 100 3446 / 1325;
+// 40 groups of 54 KB, 48 columns 68 + 77 / 60 + 77, 100 136 + 169 / 93 + 110 (110 groups 181 + 229 /
+// 207 + 239); four columns to an SM: 80 groups of 198 KB aggregation, 12 columns 71 / 75, 48 257 / 205, 100
+// 560 / 361, 400 of 161 KB disaggregation, 8 columns 252 / 250, 48 1392 / 975, 100 2884 / 1886.
+template <class Work>
+bool blocks_pay(const Plan& P, int R, Work work) {
+    for (const SmallClass& k : P.small_classes) {
+        const SmallPass p = pick_pass(P, k, R, work);
+        if (p.cols == 1) return false;
+        if (R > 48 && (2 * P.G <= P.num_sms || (p.cols <= 4 && p.per_sm == 1))) return false;
+    }
+    return true;
 }
 
 SmallArgs small_args(const Plan& P, const SmallClass& k, int R, const SmallLayout& l) {
@@ -462,9 +483,15 @@ void configure_small(Plan& P, cudaStream_t s) {
     P.small_one = 2 * P.G <= 3 * P.num_sms;
 }
 
+bool small_takes(const Plan& P, bool aggregation, int R) {
+    if (R <= 1 || P.params.mrhs_precision == 1) return P.small_one;
+    return P.small_ok && P.params.mrhs_precision == 0 &&
+           (aggregation ? blocks_pay(P, R, agg_work) : blocks_pay(P, R, dis_work));
+}
+
 void launch_small_aggregate(const Plan& P, const float2* x, int R, int64_t ldx, float2* spec, cudaStream_t s) {
     for (const SmallClass& k : P.small_classes)
-        with_cols(pick_cols(P, k, R, agg_work), [&](auto n) {
+        with_cols(pick_pass(P, k, R, agg_work).cols, [&](auto n) {
             constexpr int COLS = decltype(n)::value;
             const SmallLayout l = agg_work(P, k, COLS);
             SmallArgs a = small_args(P, k, R, l);
@@ -479,7 +506,7 @@ void launch_small_aggregate(const Plan& P, const float2* x, int R, int64_t ldx, 
 void launch_small_disaggregate(const Plan& P, const float2* spec, int R, int weights, float2 beta, float2* y,
                                int64_t ldy, cudaStream_t s) {
     for (const SmallClass& k : P.small_classes)
-        with_cols(pick_cols(P, k, R, dis_work), [&](auto n) {
+        with_cols(pick_pass(P, k, R, dis_work).cols, [&](auto n) {
             constexpr int COLS = decltype(n)::value;
             const SmallLayout l = dis_work(P, k, COLS);
             SmallArgs a = small_args(P, k, R, l);

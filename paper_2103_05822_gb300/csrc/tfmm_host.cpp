@@ -163,12 +163,12 @@ void check_params(const tfmm_params& p) {
     TFMM_REQUIRE(p.compression == 0 || p.compression == 1, "compression must be 0 (Tucker) or 1 (SVD)");
 }
 
-// The engine that applies one call with R columns:
+// The engine that applies one stage with R columns:
 //   small:   one CTA per (group, component) with everything in shared memory, for plans whose
-//            every item fits (small.cu), in place of columns and chain unless the tuning
-//            asks for one of the single-RHS paths; mrhs_precision 1 takes it one column
-//            at a time and only where a one-column call does, so that its columns have
-//            the bits of one-column calls;
+//            every item fits (small.cu), in place of columns and chain where it is faster
+//            (small_takes) and the tuning does not ask for one of the single-RHS paths;
+//            mrhs_precision 1 takes it one column at a time and only where a one-column
+//            call does, so that its columns have the bits of one-column calls;
 //   columns: the single-RHS kernels, one column after the other (R = 1, or mrhs_precision 1,
 //            or TFMM_MR=loop, or few columns of mrhs_precision 0);
 //   chain:   the grouped-GEMM chain on FP32 CUDA cores (mrhs_precision 0), also the
@@ -176,12 +176,12 @@ void check_params(const tfmm_params& p) {
 //   tc:      the split-BF16 tensor-core chain with `terms` terms (mrhs_precision 2, 3).
 enum class Engine { small, columns, chain, tc };
 
-Engine engine_for(const Plan& P, int R, int* terms) {
+Engine engine_for(const Plan& P, bool aggregation, int R, int* terms) {
     *terms = 0;
     const int p = P.params.mrhs_precision;
     const char* e = std::getenv("TFMM_MR");
     const bool loop = e && std::strcmp(e, "loop") == 0;
-    if (P.tuning.split == 0 && !loop && (R <= 1 || p == 1 ? P.small_one : P.small_ok && p == 0)) return Engine::small;
+    if (P.tuning.split == 0 && !loop && small_takes(P, aggregation, R)) return Engine::small;
     // Up to kColumnsMax columns the chain reads every factor about as slowly as for one tile's width, and
     // the single-RHS kernels stream them once per column near the copy rate.  Measured, chain / columns
     // (both stages, ms): 20-lambda sphere in 2-lambda boxes, 2 columns 2.95 / 1.50, 4 3.15 / 2.99, 6 3.39 / 4.49;
@@ -205,7 +205,7 @@ struct NvtxRange {
 void run_aggregate(Plan& P, const float2* x, int R, int64_t ldx, float2* spec, cudaStream_t s) {
     NvtxRange nvtx("tfmm_aggregate");
     int T = 0;
-    switch (engine_for(P, R, &T)) {
+    switch (engine_for(P, true, R, &T)) {
         case Engine::small: launch_small_aggregate(P, x, R, ldx, spec, s); break;
         case Engine::tc: launch_tc_aggregate(P, T, x, R, ldx, spec, s); break;
         case Engine::chain: launch_mr_aggregate(P, x, R, ldx, spec, s); break;
@@ -217,7 +217,7 @@ void run_disaggregate(Plan& P, const float2* spec, int R, int weights, float2 be
                       cudaStream_t s) {
     NvtxRange nvtx("tfmm_disaggregate");
     int T = 0;
-    switch (engine_for(P, R, &T)) {
+    switch (engine_for(P, false, R, &T)) {
         case Engine::small: launch_small_disaggregate(P, spec, R, weights, beta, y, ldy, s); break;
         case Engine::tc: launch_tc_disaggregate(P, T, spec, R, weights, beta, y, ldy, s); break;
         case Engine::chain: launch_mr_disaggregate(P, spec, R, weights, beta, y, ldy, s); break;

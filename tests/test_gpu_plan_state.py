@@ -156,3 +156,18 @@ def test_one_column_after_another_gives_the_bits_of_one_column_calls(G, nb):
     for r in range(5):
         assert torch.equal(spec[r], _agg(tfmm, plan, x[r:r + 1])[0])
         assert torch.equal(y[r], _dis(tfmm, plan, g[r:r + 1])[0])
+
+
+@pytest.mark.parametrize("nt,npf,nbetas,rank,R,stages", [
+    (17, 34, [70, 70, 66], (14, 19, 66), 6, "d"),    # one column a pass in the disaggregation: the chain
+    (17, 34, [70, 70, 66], (14, 19, 66), 3, "d"),    # the same, few columns: the persistent kernels
+    (14, 28, [60, 55, 31], (9, 13, 31), 64, "ad"),   # many columns for three groups' CTAs: the chain
+])
+def test_small_groups_leave_what_others_do_faster(nt, npf, nbetas, rank, R, stages):
+    """The stages that take the kernels of single_rhs_split 2 (never the small-group ones) have their bits."""
+    tfmm, plan, *_ = _problem(91, nt, npf, nbetas, [[rank, (3, 5, 9)]] * 3, R, 0)
+    x, g = _inputs(plan, R, 92)
+    spec, y = _agg(tfmm, plan, x), _dis(tfmm, plan, g)
+    tfmm.tfmm_plan_tuning_set(plan, single_rhs_split=2)
+    assert torch.equal(_agg(tfmm, plan, x), spec) == ("a" in stages)
+    assert torch.equal(_dis(tfmm, plan, g), y) == ("d" in stages)
