@@ -334,6 +334,19 @@ struct Plan {
 };
 
 // tfmm_host.cpp
+// The engine that applies one stage with R columns:
+//   small:   one CTA per (group, component) with everything in shared memory, for plans whose
+//            every item fits (small.cu), in place of columns and chain where it is faster
+//            (small_takes) and the tuning does not ask for one of the single-RHS paths;
+//            mrhs_precision 1 takes it one column at a time and only where a one-column
+//            call does, so that its columns have the bits of one-column calls;
+//   columns: the single-RHS kernels, one column after the other (R = 1, or mrhs_precision 1,
+//            or TFMM_MR=loop, or few columns of mrhs_precision 0);
+//   chain:   the grouped-GEMM chain on FP32 CUDA cores (mrhs_precision 0), also the
+//            fallback when a work item does not fit the single-RHS kernels;
+//   tc:      the split-BF16 tensor-core chain with `terms` terms (mrhs_precision 2, 3).
+enum class Engine { small, columns, chain, tc };
+Engine engine_for(const Plan& P, bool aggregation, int R, int* terms);
 std::string& last_error();  // message of the calling thread's last failure
 void upload_common(Plan& P, cudaStream_t s);
 

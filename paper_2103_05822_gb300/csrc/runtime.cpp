@@ -3,6 +3,7 @@
 // capture of the two stages, and the autotuner that picks launch shapes, queue
 // orders and the multi-RHS engine by timing them on the plan's own data.
 #include <algorithm>
+#include <array>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -438,18 +439,25 @@ tfmm_status tfmm_autotune(tfmm_plan* plan, int32_t R, double budget_ms, int32_t 
         auto agg = [&] { run_stages(plan, 1, x, R, P.N, sp, 1, zero, y, P.N, s); };
         auto dis = [&] { run_stages(plan, 2, x, R, P.N, sp, 1, zero, y, P.N, s); };
         if (R == 1 && P.hot_ok) {
-            // launch shape x queue order, one stage at a time; the other stage keeps its setting
+            // launch shape x queue order of the persistent kernels, one stage at a time; the other stage keeps
+            // its setting.  A stage that runs other kernels (small groups, split path) is timed as it is.
             HotTuning best = P.tuning;
-            double best_ms[2] = {1e30, 1e30};
+            double best_ms[2];
             const int threads[3] = {512, 384, 256};
             const int ctas[3] = {0, 2, 1};
             for (int stage = 0; stage < 2; ++stage) {
-                std::vector<std::pair<int, int>> seen;  // (threads and order, blocks) already timed
+                int terms = 0;
+                best_ms[stage] = stage == 0 ? time_ms(agg, 5, s, tm) : time_ms(dis, 5, s, tm);
+                if (engine_for(P, stage == 0, 1, &terms) != Engine::columns) continue;
+                if (P.split && (stage == 0 ? P.split->agg : P.split->dis)) continue;
+                // (threads and order, blocks) already timed
+                std::vector<std::pair<int, int>> seen = {
+                    stage == 0 ? std::make_pair(best.agg_threads * 2 + best.agg_order, P.agg_sched.blocks)
+                               : std::make_pair(best.dis_threads * 2 + best.dis_order, P.dis_sched.blocks)};
                 for (int order = 0; order < 2; ++order)
                     for (int nt : threads)
                         for (int c : ctas) {
-                            // the budget stops the search once this stage has one timing
-                            if (spent() > budget_ms * (stage + 1) / 2 && best_ms[stage] < 1e30) continue;
+                            if (spent() > budget_ms * (stage + 1) / 2) continue;
                             HotTuning t = best;
                             (stage == 0 ? t.agg_threads : t.dis_threads) = nt;
                             (stage == 0 ? t.agg_ctas_per_sm : t.dis_ctas_per_sm) = c;
@@ -479,9 +487,17 @@ tfmm_status tfmm_autotune(tfmm_plan* plan, int32_t R, double budget_ms, int32_t 
             if (allow_two_term) cand.push_back(2);
             int best = P.params.mrhs_precision;
             double best_ms = 1e30, ba = 0, bd = 0;
+            // engines of both stages, terms and columns per pass already timed: several values can mean one engine
+            std::vector<std::array<int, 4>> seen;
             for (int prec : cand) {
                 if (spent() > budget_ms && best_ms < 1e30) break;
                 P.params.mrhs_precision = prec;
+                int terms = 0;
+                const Engine ea = engine_for(P, true, R, &terms), ed = engine_for(P, false, R, &terms);
+                const std::array<int, 4> key = {(int)ea, (int)ed, terms,
+                                                prec == 1 && (ea == Engine::small || ed == Engine::small)};
+                if (std::find(seen.begin(), seen.end(), key) != seen.end()) continue;
+                seen.push_back(key);
                 const double a = time_ms(agg, 2, s, tm);
                 const double d = time_ms(dis, 2, s, tm);
                 if (a + d < best_ms) {

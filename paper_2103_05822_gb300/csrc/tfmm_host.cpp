@@ -163,39 +163,6 @@ void check_params(const tfmm_params& p) {
     TFMM_REQUIRE(p.compression == 0 || p.compression == 1, "compression must be 0 (Tucker) or 1 (SVD)");
 }
 
-// The engine that applies one stage with R columns:
-//   small:   one CTA per (group, component) with everything in shared memory, for plans whose
-//            every item fits (small.cu), in place of columns and chain where it is faster
-//            (small_takes) and the tuning does not ask for one of the single-RHS paths;
-//            mrhs_precision 1 takes it one column at a time and only where a one-column
-//            call does, so that its columns have the bits of one-column calls;
-//   columns: the single-RHS kernels, one column after the other (R = 1, or mrhs_precision 1,
-//            or TFMM_MR=loop, or few columns of mrhs_precision 0);
-//   chain:   the grouped-GEMM chain on FP32 CUDA cores (mrhs_precision 0), also the
-//            fallback when a work item does not fit the single-RHS kernels;
-//   tc:      the split-BF16 tensor-core chain with `terms` terms (mrhs_precision 2, 3).
-enum class Engine { small, columns, chain, tc };
-
-Engine engine_for(const Plan& P, bool aggregation, int R, int* terms) {
-    *terms = 0;
-    const int p = P.params.mrhs_precision;
-    const char* e = std::getenv("TFMM_MR");
-    const bool loop = e && std::strcmp(e, "loop") == 0;
-    if (P.tuning.split == 0 && !loop && small_takes(P, aggregation, R)) return Engine::small;
-    // Up to kColumnsMax columns the chain reads every factor about as slowly as for one tile's width, and
-    // the single-RHS kernels stream them once per column near the copy rate.  Measured, chain / columns
-    // (both stages, ms): 20-lambda sphere in 2-lambda boxes, 2 columns 2.95 / 1.50, 4 3.15 / 2.99, 6 3.39 / 4.49;
-    // 10-lambda sphere 4 columns 0.81 / 0.59, 8 0.95 / 1.16; 4-lambda boxes 4 columns 1.97 / 1.61.
-    constexpr int kColumnsMax = 4;
-    if (P.hot_ok && (R <= 1 || loop || p == 1 || plan_is_svd(P) || (p == 0 && R <= kColumnsMax)))
-        return Engine::columns;
-    if (R > 1 && (p == 2 || p == 3)) {
-        *terms = p;
-        return Engine::tc;
-    }
-    return Engine::chain;
-}
-
 // An NVTX range around one hot-path call (seen by profilers, free otherwise).
 struct NvtxRange {
     explicit NvtxRange(const char* name) { nvtxRangePushA(name); }
@@ -236,6 +203,26 @@ void check_hot(const Plan& P, const void* a, const void* b, int R, int64_t ld) {
 }  // namespace tfmm
 
 namespace tfmm {
+
+Engine engine_for(const Plan& P, bool aggregation, int R, int* terms) {
+    *terms = 0;
+    const int p = P.params.mrhs_precision;
+    const char* e = std::getenv("TFMM_MR");
+    const bool loop = e && std::strcmp(e, "loop") == 0;
+    if (P.tuning.split == 0 && !loop && small_takes(P, aggregation, R)) return Engine::small;
+    // Up to kColumnsMax columns the chain reads every factor about as slowly as for one tile's width, and
+    // the single-RHS kernels stream them once per column near the copy rate.  Measured, chain / columns
+    // (both stages, ms): 20-lambda sphere in 2-lambda boxes, 2 columns 2.95 / 1.50, 4 3.15 / 2.99, 6 3.39 / 4.49;
+    // 10-lambda sphere 4 columns 0.81 / 0.59, 8 0.95 / 1.16; 4-lambda boxes 4 columns 1.97 / 1.61.
+    constexpr int kColumnsMax = 4;
+    if (P.hot_ok && (R <= 1 || loop || p == 1 || plan_is_svd(P) || (p == 0 && R <= kColumnsMax)))
+        return Engine::columns;
+    if (R > 1 && (p == 2 || p == 3)) {
+        *terms = p;
+        return Engine::tc;
+    }
+    return Engine::chain;
+}
 
 namespace {
 // Allocations left before the one the test hook fails (0: disarmed).

@@ -171,3 +171,19 @@ def test_small_groups_leave_what_others_do_faster(nt, npf, nbetas, rank, R, stag
     tfmm.tfmm_plan_tuning_set(plan, single_rhs_split=2)
     assert torch.equal(_agg(tfmm, plan, x), spec) == ("a" in stages)
     assert torch.equal(_dis(tfmm, plan, g), y) == ("d" in stages)
+
+
+@pytest.mark.parametrize("kernels", ["small", "split"])
+def test_autotuning_leaves_a_launch_shape_alone_that_does_not_run(kernels):
+    """One column on the small-group kernels or the split path: their time is reported and the persistent
+    kernels' shape, which nothing was measured with, stays."""
+    nbetas = [60, 50] if kernels == "small" else [2500, 900]
+    rank = (5, 7, 20) if kernels == "small" else (20, 30, 120)
+    tfmm, plan, *_ = _problem(95, 21, 42, nbetas, [[rank, rank]] * 2, 1, 0)
+    shape = ("agg_threads", "agg_ctas_per_sm", "agg_order", "dis_threads", "dis_ctas_per_sm", "dis_order")
+    for threads in (96, 448):
+        tfmm.tfmm_plan_tuning_set(plan, agg_threads=threads, dis_threads=threads)
+        before = tfmm.tfmm_plan_tuning_get(plan)
+        t = tfmm.tfmm_autotune(plan, R=1, budget_ms=300.0)
+        assert [t[k] for k in shape] == [before[k] for k in shape]
+        assert 0 < t["agg_ms"] < 10 and 0 < t["dis_ms"] < 10
