@@ -200,22 +200,24 @@ __device__ __forceinline__ void rowdot_rows(const float4* __restrict__ M, int ld
 }
 
 // out[j] (float4 = two complex columns) = sum_c M[c][j] s[c]; `part` holds
-// blockDim float4 of scratch for the split-row case.
-template <class Emit>
+// blockDim float4 of scratch for the split-row case.  DEPTH loads in flight per column: eight in the
+// persistent kernels (two CTAs of 64 registers an SM), four in the dense kernel, which has three CTAs of 40:
+// 56 groups, 882 directions 87 us with four and 109 with eight, 8 groups, 2312 directions 1267 and 1658.
+template <int DEPTH, class Emit>
 __device__ __forceinline__ void rowaxpy(const float4* __restrict__ M, int ld2, int nrows, const float2* s,
                                         float4* part, Emit emit) {
     const int NT = blockDim.x, tid = threadIdx.x;
-    // rows c0, c0 + st, ... of column j, eight loads in flight
+    // rows c0, c0 + st, ... of column j
     auto column = [&](int j, int c0, int st) {
         float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
         const float4* col = M + j;
         int c = c0;
-        for (; c + 7 * st < nrows; c += 8 * st) {
-            float4 m[8];
+        for (; c + (DEPTH - 1) * st < nrows; c += DEPTH * st) {
+            float4 m[DEPTH];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) m[i] = ld_stream(col + (int64_t)(c + i * st) * ld2);
+            for (int i = 0; i < DEPTH; ++i) m[i] = ld_stream(col + (int64_t)(c + i * st) * ld2);
 #pragma unroll
-            for (int i = 0; i < 8; i += 2) {
+            for (int i = 0; i < DEPTH; i += 2) {
                 cfma2(a0, m[i], s[c + i * st]);
                 cfma2(a1, m[i + 1], s[c + (i + 1) * st]);
             }
@@ -343,7 +345,7 @@ __global__ void __launch_bounds__(512, 2) tucker_aggregate_kernel(const AggArgs 
             if (SVD) {
                 // F[i] = sum_c B[i, c] t[c], i = i_theta + n_theta i_phi (the core's column index)
                 float2* out = a.spec + (((int64_t)r * a.G + d.g) * 2 + d.alpha) * a.n_dir;
-                rowaxpy(reinterpret_cast<const float4*>(Cc), d.ld_ab / 2, d.rb, s_t, s_part, [&](int j, float4 v) {
+                rowaxpy<8>(reinterpret_cast<const float4*>(Cc), d.ld_ab / 2, d.rb, s_t, s_part, [&](int j, float4 v) {
                     out[2 * j] = make_float2(v.x, v.y);
                     if (2 * j + 1 < a.n_dir) out[2 * j + 1] = make_float2(v.z, v.w);
                 });
@@ -351,7 +353,7 @@ __global__ void __launch_bounds__(512, 2) tucker_aggregate_kernel(const AggArgs 
                 continue;
             }
             // AG2: M[ab] = sum_c C_(3)[c, ab] t[c]
-            rowaxpy(reinterpret_cast<const float4*>(Cc), d.ld_ab / 2, d.rb, s_t, s_part,
+            rowaxpy<8>(reinterpret_cast<const float4*>(Cc), d.ld_ab / 2, d.rb, s_t, s_part,
                     [&](int j, float4 v) { reinterpret_cast<float4*>(s_M)[j] = v; });
             __syncthreads();
             // AG3: V[i_phi, a] = sum_b U_phi[i_phi, b] M[a, b]
@@ -470,7 +472,7 @@ __global__ void __launch_bounds__(512, 2) tucker_disaggregate_kernel(const DisAr
                     prefetch_head_l2(a.fac + d1.core, (int64_t)d1.rb * d1.ld_ab * 8);
                 }
                 // DG3: y_n += conj(sum_c U_beta[n, c] s[c])
-                rowaxpy(reinterpret_cast<const float4*>(Ub), d.ld_nb / 2, d.rb, s_s, s_part, [&](int j, float4 v) {
+                rowaxpy<8>(reinterpret_cast<const float4*>(Ub), d.ld_nb / 2, d.rb, s_s, s_part, [&](int j, float4 v) {
                     float4 o = s_y4[j];
                     s_y4[j] = make_float4(o.x + v.x, o.y - v.y, o.z + v.z, o.w - v.w);
                 });
@@ -523,7 +525,7 @@ __global__ void __launch_bounds__(512) dense_aggregate_kernel(const DenseAggArgs
             __syncthreads();
             float2* out = a.spec + (((int64_t)r * a.G + d.g) * 2 + d.alpha) * a.n_dir;
             const int ld2 = a.ld_dir / 2;
-            rowaxpy(reinterpret_cast<const float4*>(a.A + d.a), ld2, d.n_beta, s_x, s_part, [&](int j, float4 v) {
+            rowaxpy<4>(reinterpret_cast<const float4*>(a.A + d.a), ld2, d.n_beta, s_x, s_part, [&](int j, float4 v) {
                 out[2 * j] = make_float2(v.x, v.y);
                 if (2 * j + 1 < a.n_dir) out[2 * j + 1] = make_float2(v.z, v.w);
             });
