@@ -714,8 +714,9 @@ struct SplitArgs {
 };
 
 // out[j0 + j] = sum_{c < nrows} M[c][j0 + j] s[c] for j < cbv (float4 columns): the CTA
-// splits into NT / kSplitCols slices of rows, summed through `part` (NT float4).
-template <class Emit>
+// splits into NT / kSplitCols slices of rows, summed through `part` (NT float4).  FOUR: four loads in
+// flight (eight cost a resident CTA: slower), else two.
+template <bool FOUR, class Emit>
 __device__ __forceinline__ void colblock_axpy(const float4* __restrict__ M, int64_t ld2, int j0, int cbv, int nrows,
                                               const float2* s, float4* part, Emit emit) {
     const int tid = threadIdx.x, S = blockDim.x / kSplitCols;
@@ -724,17 +725,28 @@ __device__ __forceinline__ void colblock_axpy(const float4* __restrict__ M, int6
     if (j < cbv && sl < S) {
         const float4* col = M + j0 + j;
         int c = sl;
-        for (; c + 3 * S < nrows; c += 4 * S) {  // four loads in flight (eight cost a resident CTA: slower)
-            float4 m[4];
+        if constexpr (FOUR) {
+            for (; c + 3 * S < nrows; c += 4 * S) {
+                float4 m[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) m[i] = ld_stream(col + (int64_t)(c + i * S) * ld2);
+                for (int i = 0; i < 4; ++i) m[i] = ld_stream(col + (int64_t)(c + i * S) * ld2);
 #pragma unroll
-            for (int i = 0; i < 4; i += 2) {
-                cfma2(a0, m[i], s[c + i * S]);
-                cfma2(a1, m[i + 1], s[c + (i + 1) * S]);
+                for (int i = 0; i < 4; i += 2) {
+                    cfma2(a0, m[i], s[c + i * S]);
+                    cfma2(a1, m[i + 1], s[c + (i + 1) * S]);
+                }
             }
+            for (; c < nrows; c += S) cfma2(a0, ld_stream(col + (int64_t)c * ld2), s[c]);
+        } else {
+#pragma unroll 2
+            for (; c + S < nrows; c += 2 * S) {
+                const float4 m0 = ld_stream(col + (int64_t)c * ld2);
+                const float4 m1 = ld_stream(col + (int64_t)(c + S) * ld2);
+                cfma2(a0, m0, s[c]);
+                cfma2(a1, m1, s[c + S]);
+            }
+            if (c < nrows) cfma2(a0, ld_stream(col + (int64_t)c * ld2), s[c]);
         }
-        for (; c < nrows; c += S) cfma2(a0, ld_stream(col + (int64_t)c * ld2), s[c]);
     }
     if (sl < S) part[sl * kSplitCols + j] = add4(a0, a1);
     __syncthreads();
@@ -751,19 +763,21 @@ __global__ void __launch_bounds__(512) split_ag1_kernel(const SplitArgs a) {
     float2* s_x = reinterpret_cast<float2*>(smem4);
     const SplitTile t = a.tiles[blockIdx.x];
     const TuckerItem d = a.items[t.item];
-    const int rows = min(kSplitRows, d.rb - t.start);
-    if (threadIdx.x == 0)  // the rows start towards L2 while x is gathered
-        prefetch_head_l2(a.fac + d.ub + (int64_t)t.start * d.ld_nb, (int64_t)rows * d.ld_nb * 8);
     for (int n = threadIdx.x; n < d.ld_nb; n += blockDim.x)
         s_x[n] = n < d.n_beta ? a.x[(int64_t)a.grp_rwg[d.rwg + n] + a.ldx * a.r] : make_float2(0.f, 0.f);
     __syncthreads();
     float2* tout = a.scratch + a.scr_off[t.item];
+    const int rows = min(kSplitRows, d.rb - t.start);
     rowdot<false>(reinterpret_cast<const float4*>(a.fac + d.ub) + (int64_t)t.start * (d.ld_nb / 2), d.ld_nb / 2, rows,
                   reinterpret_cast<const float4*>(s_x), [&](int c, float2 v) { tout[t.start + c] = v; });
 }
 
-// SA2: M[ab] = sum_c C_(3)[c, ab] t[c] for the column pairs of one tile
-__global__ void __launch_bounds__(512, 3) split_ag2_kernel(const SplitArgs a) {
+// SA2: M[ab] = sum_c C_(3)[c, ab] t[c] for the column pairs of one tile.  FOUR: three CTAs an SM with
+// four loads in flight each, while they take all tiles at once; else four CTAs with two.  Measured (us, two /
+// four): 40 tiles 9.7 / 7.8, 152 17.5 / 15.8 (268 rows), 304 25.8 / 23.4; 480 21.7 / 25.9, 608 25.7 / 30.1, 1200 29.1 /
+// 32.0, 2400 88.9 / 94.0, though 800 37.0 / 35.0.
+template <bool FOUR>
+__global__ void __launch_bounds__(512, FOUR ? 3 : 4) split_ag2_kernel(const SplitArgs a) {
     extern __shared__ float4 smem4[];
     float4* s_part = smem4;
     float2* s_t = reinterpret_cast<float2*>(smem4 + blockDim.x);
@@ -774,13 +788,15 @@ __global__ void __launch_bounds__(512, 3) split_ag2_kernel(const SplitArgs a) {
     __syncthreads();
     float4* mout = reinterpret_cast<float4*>(a.scratch + a.scr_off[t.item] + round_up_dev(d.rb, 2));
     const int ld2 = d.ld_ab / 2;
-    colblock_axpy(reinterpret_cast<const float4*>(a.fac + d.core), ld2, t.start, min(kSplitCols, ld2 - t.start), d.rb,
+    colblock_axpy<FOUR>(reinterpret_cast<const float4*>(a.fac + d.core), ld2, t.start, min(kSplitCols, ld2 - t.start), d.rb,
                   s_t, s_part, [&](int j, float4 v) { mout[j] = v; });
 }
 
 // SA3: AG3 + AG4 of a.blk phi directions of one item from its M.  The directions are
 // independent, so a plan of few items spreads them over the SMs: with one CTA per item the trihedral's 38
-// items took 14 us for latency alone (SA3 and SD1 alike), in blocks 9 and 12 us.
+// items took 14 us for latency alone (SA3 and SD1 alike), in blocks 9 and 12 us.  WHOLE: all directions,
+// larger register tiles.
+template <bool WHOLE>
 __global__ void __launch_bounds__(512) split_ag34_kernel(const SplitArgs a) {
     extern __shared__ float4 smem4[];
     float2* sm = reinterpret_cast<float2*>(smem4);
@@ -800,20 +816,22 @@ __global__ void __launch_bounds__(512) split_ag34_kernel(const SplitArgs a) {
     __syncthreads();
     {
         const int ldp = a.L.ldp, ldv = a.L.ldv, rt = d.rt;
-        smem_gemm<1, 2>(np, rt, d.rp, [&](int ip, int b) { return s_up[ip + ldp * b]; },
+        smem_gemm<WHOLE ? 2 : 1, 2>(np, rt, d.rp, [&](int ip, int b) { return s_up[ip + ldp * b]; },
                         [&](int b, int aa) { return s_M[aa + rt * b]; },
                         [&](int ip, int aa, float2 v) { s_V[ip + ldv * aa] = v; });
     }
     __syncthreads();
     float2* out = a.spec_out + (((int64_t)a.r * a.G + d.g) * 2 + d.alpha) * a.n_dir + (int64_t)a.n_theta * p0;
     const int ldt = a.L.ldt, ldv = a.L.ldv, nth = a.n_theta;
-    smem_gemm<1, 2>(nth, np, d.rt, [&](int it, int aa) { return s_ut[it + ldt * aa]; },
+    smem_gemm<WHOLE ? 2 : 1, WHOLE ? 4 : 2>(nth, np, d.rt, [&](int it, int aa) { return s_ut[it + ldt * aa]; },
                     [&](int aa, int ip) { return s_V[ip + ldv * aa]; },
                     [&](int it, int ip, float2 v) { out[it + nth * ip] = v; });
 }
 
 // SD1: columns b of H = U_theta^T (conj(W g) U_phi) for a.blk columns of U_phi of one item; the
 // last block zero-pads H to ld_ab.  (U_phi first: a block then needs all of g but a share of the work.)
+// WHOLE: all columns, U_theta first, larger register tiles (300 items of 38 x 75 directions 24.3 -> 20.4 us).
+template <bool WHOLE>
 __global__ void __launch_bounds__(512) split_dg1_kernel(const SplitArgs a) {
     extern __shared__ float4 smem4[];
     float2* sm = reinterpret_cast<float2*>(smem4);
@@ -837,14 +855,25 @@ __global__ void __launch_bounds__(512) split_dg1_kernel(const SplitArgs a) {
     for (int e = tid; e < a.n_phi * nb; e += NT) s_up[(e % a.n_phi) + a.L.ldp * (e / a.n_phi)] = Up[e];
     __syncthreads();
     const int ldt = a.L.ldt, ldg = a.L.ldg, ldp = a.L.ldp, rt = d.rt, ldq = a.L.ldv;
-    smem_gemm<1, 1>(a.n_theta, nb, a.n_phi, [&](int it, int ip) { return s_G[it + ldg * ip]; },
-                    [&](int ip, int b) { return s_up[ip + ldp * b]; },
-                    [&](int it, int b, float2 v) { s_Q[it + ldq * b] = v; });
-    __syncthreads();
     float2* hout = a.scratch + a.scr_off[q] + round_up_dev(d.rb, 2);
-    smem_gemm<1, 1>(rt, nb, a.n_theta, [&](int aa, int it) { return s_ut[it + ldt * aa]; },
-                    [&](int it, int b) { return s_Q[it + ldq * b]; },
-                    [&](int aa, int b, float2 v) { hout[aa + rt * (b0 + b)] = v; });
+    if constexpr (WHOLE) {
+        float2* s_P = s_Q;  // U_theta^T conj(W g)
+        smem_gemm<2, 4>(rt, a.n_phi, a.n_theta, [&](int aa, int it) { return s_ut[it + ldt * aa]; },
+                        [&](int it, int ip) { return s_G[it + ldg * ip]; },
+                        [&](int aa, int ip, float2 v) { s_P[aa + rt * ip] = v; });
+        __syncthreads();
+        smem_gemm<2, 2>(rt, nb, a.n_phi, [&](int aa, int ip) { return s_P[aa + rt * ip]; },
+                        [&](int ip, int b) { return s_up[ip + ldp * b]; },
+                        [&](int aa, int b, float2 v) { hout[aa + rt * b] = v; });
+    } else {
+        smem_gemm<1, 1>(a.n_theta, nb, a.n_phi, [&](int it, int ip) { return s_G[it + ldg * ip]; },
+                        [&](int ip, int b) { return s_up[ip + ldp * b]; },
+                        [&](int it, int b, float2 v) { s_Q[it + ldq * b] = v; });
+        __syncthreads();
+        smem_gemm<1, 1>(rt, nb, a.n_theta, [&](int aa, int it) { return s_ut[it + ldt * aa]; },
+                        [&](int it, int b) { return s_Q[it + ldq * b]; },
+                        [&](int aa, int b, float2 v) { hout[aa + rt * (b0 + b)] = v; });
+    }
     if (b0 + nb == d.rp)
         for (int o = rt * d.rp + tid; o < d.ld_ab; o += NT) hout[o] = make_float2(0.f, 0.f);
 }
@@ -880,7 +909,7 @@ __global__ void __launch_bounds__(512, 3) split_dg3_kernel(const SplitArgs a) {
         const float2* sin_ = a.scratch + a.scr_off[2 * g + al];
         for (int c = threadIdx.x; c < d.rb; c += blockDim.x) s_s[c] = sin_[c];
         __syncthreads();
-        colblock_axpy(reinterpret_cast<const float4*>(a.fac + d.ub), ld2, t.start, cbv, d.rb, s_s, s_part,
+        colblock_axpy<true>(reinterpret_cast<const float4*>(a.fac + d.ub), ld2, t.start, cbv, d.rb, s_s, s_part,
                       [&](int j, float4 v) {
                           const int jj = j - t.start;
                           s_acc[jj] = al == 0 ? v : add4(s_acc[jj], v);
@@ -924,7 +953,8 @@ SmemLayout split_dg1_layout(const Plan& P, int blk) {
     L.o_a = o; o += al16(L.ldt * P.max_rank[0]);
     L.o_b = o; o += al16(L.ldp * blk);
     L.o_f = o; o += al16(L.ldg * P.n_phi);
-    L.o_g = o; o += al16(L.ldv * blk);
+    // U_theta^T conj(W g) of a whole item, or conj(W g) U_phi for a block of columns
+    L.o_g = o; o += al16(blk >= P.max_rank[1] ? P.max_rank[0] * P.n_phi : L.ldv * blk);
     L.total = o;
     return L;
 }
@@ -1138,29 +1168,47 @@ void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s) {
 constexpr size_t kSplitSmem = 200 * 1024;
 void split_smem(const Plan& P, SplitPlan& S) {
     const int nI = P.G * 2, NT = 512;
-    // blocks of SA3 and SD1: about two CTAs per SM over all items, at least 8 directions or 4 columns each,
-    // and more where one would not fit (a block repeats the theta / phi factors' staging: four for each of
-    // 182 items cost 66 us a matvec instead of 62)
-    const int least = std::max(1, (2 * P.num_sms + nI - 1) / nI);
-    for (int parts = least; parts <= std::max(least, 8); ++parts) {
-        S.blk_phi = std::max(8, (P.n_phi + parts - 1) / parts);
-        S.blk_b = std::max(4, (P.max_rank[1] + parts - 1) / parts);
+    // Parts of SA3 and SD1: as many as the SMs take at once, two CTAs each (at least 8 directions or 4
+    // columns), and more where one would not fit.  A block repeats the theta / phi factors' staging and has
+    // less work per thread, so SD1 starts with three, and past the SMs' room whole items are faster.  Measured
+    // (us, whole / parts; 40 x 80 directions): SA3 10 items 14.4 / 7.9, 38 14.9 / 9.1, 76 in 4 15.3 / 11.2, 152 in
+    // 2 15.5 / 15.1, 240 in 2 20.4 / 26.6; SD1 38 items 16.1 / 11.7, 76 in 4 16.0 / 13.6, 152 in 2 16.2 / 18.8, 300 in 2
+    // 21.9 / 28.8.
+    const int room = std::max(1, 2 * P.num_sms / nI);
+    for (int parts = room;; ++parts) {
+        S.blk_phi = std::max(std::min(8, P.n_phi), (P.n_phi + parts - 1) / parts);
         S.smem_ag34 = sizeof(float2) * split_ag34_layout(P, S.blk_phi).total;
-        S.smem_dg1 = sizeof(float2) * split_dg1_layout(P, S.blk_b).total;
-        if (std::max(S.smem_ag34, S.smem_dg1) <= kSplitSmem) break;
+        if (S.smem_ag34 <= kSplitSmem || S.blk_phi <= 8) break;
     }
+    for (int parts = room >= 3 ? room : 1;; ++parts) {
+        S.blk_b = std::max(std::min(4, P.max_rank[1]), (P.max_rank[1] + parts - 1) / parts);
+        S.smem_dg1 = sizeof(float2) * split_dg1_layout(P, S.blk_b).total;
+        if (S.smem_dg1 <= kSplitSmem || S.blk_b <= 4) break;
+    }
+    int64_t tiles = 0;
+    for (const TuckerItem& d : P.items) tiles += (d.ld_ab / 2 + kSplitCols - 1) / kSplitCols;
+    S.ag2_four = tiles <= 3 * P.num_sms;
     S.smem_ag1 = sizeof(float2) * al16(P.max_ldnb);
     S.smem_ag2 = sizeof(float4) * NT + sizeof(float2) * al16(P.max_rank[2]);
     S.smem_dg2 = sizeof(float2) * al16(P.max_ldab);
     S.smem_dg3 = sizeof(float4) * (NT + kSplitCols) + sizeof(float2) * al16(P.max_rank[2]);
 }
 
+using SplitKernel = void (*)(SplitArgs);
+SplitKernel ag2_kernel(const SplitPlan& S) { return S.ag2_four ? split_ag2_kernel<true> : split_ag2_kernel<false>; }
+SplitKernel ag34_kernel(const Plan& P, const SplitPlan& S) {
+    return S.blk_phi >= P.n_phi ? split_ag34_kernel<true> : split_ag34_kernel<false>;
+}
+SplitKernel dg1_kernel(const Plan& P, const SplitPlan& S) {
+    return S.blk_b >= P.max_rank[1] ? split_dg1_kernel<true> : split_dg1_kernel<false>;
+}
+
 bool split_fits(const Plan& P) {
     SplitPlan S;
     split_smem(P, S);
     const std::pair<const void*, size_t> need[] = {
-        {(const void*)split_ag1_kernel, S.smem_ag1},   {(const void*)split_ag2_kernel, S.smem_ag2},
-        {(const void*)split_ag34_kernel, S.smem_ag34}, {(const void*)split_dg1_kernel, S.smem_dg1},
+        {(const void*)split_ag1_kernel, S.smem_ag1},   {(const void*)ag2_kernel(S), S.smem_ag2},
+        {(const void*)ag34_kernel(P, S), S.smem_ag34}, {(const void*)dg1_kernel(P, S), S.smem_dg1},
         {(const void*)split_dg2_kernel, S.smem_dg2},   {(const void*)split_dg3_kernel, S.smem_dg3}};
     bool fits = true;
     for (const auto& [kernel, smem] : need) fits = smem <= allow_all_smem(kernel) && fits;
@@ -1189,15 +1237,19 @@ std::unique_ptr<SplitPlan> make_split(const Plan& P, cudaStream_t s) {
     }
     for (int g = 0; g < P.G; ++g)
         for (int j = 0; j < P.items[2 * g].ld_nb / 2; j += kSplitCols) d3.push_back(SplitTile{g, j});
-    // Most bytes first: nearly all tiles of a launch are resident at once, dealt to the SMs in order,
+    // Most bytes first where nearly all tiles of a launch are resident at once, dealt to the SMs in order,
     // so that each SM gets its share of the long rows (a tile of the trihedral's streams 10 to 600 KB).
-    auto by_bytes = [&](std::vector<SplitTile>& v, auto bytes) {
+    // Past that the order of the items is the better one (us, by bytes / by item: SA1 540 tiles 18.5 / 18.4, 646
+    // 33.0 / 35.2, 900 19.4 / 18.8, 1292 50.3 / 45.0, 2584 87.6 / 77.8; SA2 800 tiles 39.0 / 36.9; the
+    // disaggregation of 60 uneven groups, 1400 and 850 tiles, 147 / 142).
+    auto by_bytes = [&](std::vector<SplitTile>& v, size_t most, auto bytes) {
+        if (v.size() > most) return;
         std::stable_sort(v.begin(), v.end(), [&](const SplitTile& x, const SplitTile& y) { return bytes(x) > bytes(y); });
     };
-    by_bytes(a1, [&](const SplitTile& t) { return (int64_t)std::min(kSplitRows, P.items[t.item].rb - t.start) * P.items[t.item].ld_nb; });
-    by_bytes(d2, [&](const SplitTile& t) { return (int64_t)std::min(kSplitRows, P.items[t.item].rb - t.start) * P.items[t.item].ld_ab; });
-    by_bytes(a2, [&](const SplitTile& t) { return (int64_t)std::min(kSplitCols, P.items[t.item].ld_ab / 2 - t.start) * P.items[t.item].rb; });
-    by_bytes(d3, [&](const SplitTile& t) {
+    by_bytes(a1, 4 * P.num_sms, [&](const SplitTile& t) { return (int64_t)std::min(kSplitRows, P.items[t.item].rb - t.start) * P.items[t.item].ld_nb; });
+    by_bytes(d2, 6 * P.num_sms, [&](const SplitTile& t) { return (int64_t)std::min(kSplitRows, P.items[t.item].rb - t.start) * P.items[t.item].ld_ab; });
+    by_bytes(a2, 3 * P.num_sms, [&](const SplitTile& t) { return (int64_t)std::min(kSplitCols, P.items[t.item].ld_ab / 2 - t.start) * P.items[t.item].rb; });
+    by_bytes(d3, 6 * P.num_sms, [&](const SplitTile& t) {
         const TuckerItem &x = P.items[2 * t.item], &y = P.items[2 * t.item + 1];
         return (int64_t)std::min(kSplitCols, x.ld_nb / 2 - t.start) * (x.rb + y.rb);
     });
@@ -1283,11 +1335,11 @@ void launch_split_aggregate(const Plan& P, const float2* x, int R, int64_t ldx, 
         a.tiles = static_cast<const SplitTile*>(S.t_ag1.p);
         split_ag1_kernel<<<S.n_ag1, 512, S.smem_ag1, s>>>(a);
         a.tiles = static_cast<const SplitTile*>(S.t_ag2.p);
-        split_ag2_kernel<<<S.n_ag2, 512, S.smem_ag2, s>>>(a);
+        ag2_kernel(S)<<<S.n_ag2, 512, S.smem_ag2, s>>>(a);
         a.tiles = static_cast<const SplitTile*>(S.t_ag34.p);
         a.blk = S.blk_phi;
         a.L = split_ag34_layout(P, S.blk_phi);
-        split_ag34_kernel<<<S.n_ag34, 512, S.smem_ag34, s>>>(a);
+        ag34_kernel(P, S)<<<S.n_ag34, 512, S.smem_ag34, s>>>(a);
         TFMM_CUDA_CHECK(cudaGetLastError());
     }
 }
@@ -1305,7 +1357,7 @@ void launch_split_disaggregate(const Plan& P, const float2* spec, int R, int wei
         a.tiles = static_cast<const SplitTile*>(S.t_dg1.p);
         a.blk = S.blk_b;
         a.L = split_dg1_layout(P, S.blk_b);
-        split_dg1_kernel<<<S.n_dg1, 512, S.smem_dg1, s>>>(a);
+        dg1_kernel(P, S)<<<S.n_dg1, 512, S.smem_dg1, s>>>(a);
         a.tiles = static_cast<const SplitTile*>(S.t_dg2.p);
         split_dg2_kernel<<<S.n_dg2, 512, S.smem_dg2, s>>>(a);
         a.tiles = static_cast<const SplitTile*>(S.t_dg3.p);

@@ -225,6 +225,7 @@ struct SplitPlan {
     DeviceBuffer t_ag1, t_ag2, t_ag34, t_dg1, t_dg2, t_dg3;  // SplitTile lists
     int n_ag1 = 0, n_ag2 = 0, n_ag34 = 0, n_dg1 = 0, n_dg2 = 0, n_dg3 = 0;
     int blk_phi = 0, blk_b = 0;               // phi directions per SA3 tile, columns of U_phi per SD1 tile
+    bool ag2_four = false;                    // SA2 with four loads in flight
     DeviceBuffer scratch;                     // per item: r_beta (padded to 2) + ld_ab complex
     DeviceBuffer scr_off;                     // per item: offset of its slot (complex elements)
     size_t smem_ag1 = 0, smem_ag2 = 0, smem_ag34 = 0, smem_dg1 = 0, smem_dg2 = 0, smem_dg3 = 0;

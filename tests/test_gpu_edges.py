@@ -266,3 +266,24 @@ def test_aggregation_last_steps_forms(nt, npf, top, R):
 def test_split_by_stage(rb):
     """Largest items of 0.4, 0.7 and 1.1 MB: no stage split, the disaggregation only, both."""
     _check(9500 + rb, 20, 40, [600, 333], [[(14, 16, rb), (9, 11, 50)], [(12, 13, rb - 1), (5, 6, 25)]], 1, 0, 1e-5, pad=1)
+
+
+@pytest.mark.parametrize("per_sm", [(1, 2), (2, 3), (1, 1), (1, 1, 1)])
+def test_split_path_parts_by_item_count(per_sm, monkeypatch):
+    """Items for four, three, two and one part of the theta / phi steps (one: whole items, larger register
+    tiles), column tiles of the second step up to and past three to an SM (four and two loads in flight)."""
+    from paper_2103_05822_gb300 import tfmm
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    items = {(1, 2): sms // 2, (2, 3): 2 * sms // 3, (1, 1): sms, (1, 1, 1): sms + 2}[per_sm]
+    made = tfmm.tfmm_plan_from_tucker
+
+    def split(*args, **kw):
+        plan = made(*args, **kw)
+        tfmm.tfmm_plan_tuning_set(plan, single_rhs_split=1)
+        return plan
+
+    monkeypatch.setattr(tfmm, "tfmm_plan_from_tucker", split)
+    rng = np.random.default_rng(items)
+    nbetas = [int(n) for n in rng.integers(18, 60, items // 2)]
+    ranks = [[(12, 23, int(rng.integers(1, 18))), (12, int(rng.integers(22, 24)), 17)] for _ in nbetas]
+    _check(9700 + items, 13, 26, nbetas, ranks, 1, 0, 1e-5, pad=1)
