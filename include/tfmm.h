@@ -351,7 +351,8 @@ typedef struct {
                                        item over many CTAs (for plans with few, large groups):
                                        0 automatic (fewer work items than 2 x SMs, the largest of more
                                        than 960 KB for the aggregation and 450 KB for the
-                                       disaggregation, or items too large for the persistent kernels;
+                                       disaggregation (225 KB up to an item per SM), or items too
+                                       large for the persistent kernels;
                                        groups that fit one CTA's shared memory run in one launch of
                                        their own), 1 always, 2 never */
     double agg_ms, dis_ms;          /* times the autotuner measured (0 if not tuned) */

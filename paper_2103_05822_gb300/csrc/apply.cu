@@ -1112,8 +1112,11 @@ HotShape plan_hot(const Plan& P, const HotTuning& t) {
     // path's two further launches take; the disaggregation, one CTA per group, sooner.  Measured (persistent /
     // split, us; largest item): aggregation 182 items of 0.48 MB 21 / 28, 192 of 0.92 MB 30.4 / 35.0, 52 of
     // 1.04 MB 26.6 / 24.9, 112 of 2.8 MB 67 / 62; disaggregation 262 of 0.33 MB 25 / 31, 182 of 0.48 MB
-    // 29.6 / 28.9, 52 of 0.55 MB 24.8 / 22.8, 192 of 0.92 MB 45.5 / 37.2, 112 of 2.8 MB 109 / 67.
-    constexpr int64_t kSplitAgg = 960 << 10, kSplitDis = 450 << 10;
+    // 29.6 / 28.9, 52 of 0.55 MB 24.8 / 22.8, 192 of 0.92 MB 45.5 / 37.2, 112 of 2.8 MB 109 / 67; and up to an
+    // item per SM from smaller ones on: 10 items of 0.27 MB 23.7 / 19.9, 38 23.7 / 21.5, 100 24.8 / 23.4, 152 25.8 /
+    // 25.6, but 200 26.2 / 29.9.
+    constexpr int64_t kSplitAgg = 960 << 10;
+    const int64_t kSplitDis = (nI <= P.num_sms ? 225 : 450) << 10;
     int64_t largest = 0;
     for (const TuckerItem& d : P.items) largest = std::max<int64_t>(largest, 8ll * d.rb * (d.n_beta + d.rt * d.rp));
     const bool few = t.split == 0 && nI < 2 * P.num_sms;
