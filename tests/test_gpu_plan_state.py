@@ -92,8 +92,9 @@ def test_more_columns_than_one_launch_of_the_gather_takes():
 
 
 def _large_item_plan(threads=64):
-    """One group whose items fit the persistent kernels with 64 threads a CTA and not with 512 (their scratch)."""
-    tfmm, plan, *_ = _problem(71, 3, 6, [28500], [[(1, 1, 1), (2, 3, 2)]], 1, 0)
+    """One group whose items fit the persistent kernels with 64 threads a CTA and not with 512 (their scratch),
+    and of less bytes than the automatic choice splits."""
+    tfmm, plan, *_ = _problem(71, 3, 6, [28500], [[(1, 1, 1)] * 2], 1, 0)
     assert tfmm.tfmm_plan_tuning_get(plan)["dis_blocks"] == 0
     tfmm.tfmm_plan_tuning_set(plan, agg_threads=threads, dis_threads=threads, single_rhs_split=0)
     assert tfmm.tfmm_plan_tuning_get(plan)["dis_blocks"] > 0
