@@ -395,9 +395,10 @@ struct DisArgs {
 };
 
 // Disaggregation (Fig. 3b) of one group (both alpha) per work item.  SVD (see the
-// aggregation): H is conj(W g) itself, then DG2 and DG3.
-template <bool SVD>
-__global__ void __launch_bounds__(512, 2) tucker_disaggregate_kernel(const DisArgs a) {
+// aggregation): H is conj(W g) itself, then DG2 and DG3.  THREE: three CTAs of 512 threads an SM, with one row
+// per warp and four loads in flight in 40 registers (see plan_hot).
+template <bool SVD, bool THREE = false>
+__global__ void __launch_bounds__(512, THREE ? 3 : 2) tucker_disaggregate_kernel(const DisArgs a) {
     extern __shared__ float4 smem4[];
     float2* sm = reinterpret_cast<float2*>(smem4);
     __shared__ int s_item;
@@ -464,15 +465,20 @@ __global__ void __launch_bounds__(512, 2) tucker_disaggregate_kernel(const DisAr
                 __syncthreads();
                 }
                 // DG2: s[c] = sum_ab C_(3)[c, ab] H[ab]
-                rowdot_rows<false>(reinterpret_cast<const float4*>(Cc), d.ld_ab / 2, d.rb,
-                              reinterpret_cast<const float4*>(s_H), [&](int c, float2 v) { s_s[c] = v; });
+                auto put_s = [&](int c, float2 v) { s_s[c] = v; };
+                if constexpr (THREE)
+                    rowdot<false>(reinterpret_cast<const float4*>(Cc), d.ld_ab / 2, d.rb,
+                                  reinterpret_cast<const float4*>(s_H), put_s);
+                else
+                    rowdot_rows<false>(reinterpret_cast<const float4*>(Cc), d.ld_ab / 2, d.rb,
+                                       reinterpret_cast<const float4*>(s_H), put_s);
                 __syncthreads();
                 if (tid == 0 && al == 0) {  // the next component's C while this one's U_beta streams
                     const TuckerItem d1 = a.items[2 * g + 1];
                     prefetch_head_l2(a.fac + d1.core, (int64_t)d1.rb * d1.ld_ab * 8);
                 }
                 // DG3: y_n += conj(sum_c U_beta[n, c] s[c])
-                rowaxpy<8>(reinterpret_cast<const float4*>(Ub), d.ld_nb / 2, d.rb, s_s, s_part, [&](int j, float4 v) {
+                rowaxpy<THREE ? 4 : 8>(reinterpret_cast<const float4*>(Ub), d.ld_nb / 2, d.rb, s_s, s_part, [&](int j, float4 v) {
                     float4 o = s_y4[j];
                     s_y4[j] = make_float4(o.x + v.x, o.y - v.y, o.z + v.z, o.w - v.w);
                 });
@@ -1058,6 +1064,8 @@ void pack_factors_fp32(Plan& P, cudaStream_t s) {
     finalize_hot_layout(P, s);
 }
 
+constexpr int64_t kThreeAgg = 2 << 20, kThreeDis = 900 << 10;
+bool between_two_and_three(const Plan& P, int n) { return n > 2 * P.num_sms && n <= 3 * P.num_sms; }  // per SM
 void finalize_hot_layout(Plan& P, cudaStream_t s) {
     const int nI = P.G * 2;
     if (P.d_items) cudaFree(P.d_items);
@@ -1074,6 +1082,13 @@ void finalize_hot_layout(Plan& P, cudaStream_t s) {
     const int64_t item = (int64_t)sizeof(float2) * P.factor_elems / nI;
     P.tuning.agg_threads = item <= 448 * 1024 && nI >= 4 * P.num_sms ? 256 : 512;
     P.tuning.dis_threads = item <= 300 * 1024 && P.G >= 4 * P.num_sms ? 256 : 512;
+    // Between two and three items per SM two CTAs of 512 threads leave the third item of an SM to a second
+    // round; three of 320 take all at once, until the items are long enough to want the warps (the
+    // disaggregation then takes three of 512, see plan_hot).  Measured, 512 / 320 threads (us): aggregation, 308
+    // items of 0.19 MB 23.8 / 19.8, 456 of 1.1 MB 99 / 94, 360 of 1.8 MB 134 / 121, but 360 of 3 MB 204 / 209;
+    // disaggregation, 310 groups of 0.19 MB items 50 / 42, 380 of 0.75 MB 148 / 122, but 380 of 1.1 MB 191 / 191.
+    if (between_two_and_three(P, nI) && item <= kThreeAgg) P.tuning.agg_threads = 320;
+    if (between_two_and_three(P, P.G) && item <= kThreeDis) P.tuning.dis_threads = 320;
     configure_hot(P, P.tuning, s);
 }
 
@@ -1102,6 +1117,16 @@ HotShape plan_hot(const Plan& P, const HotTuning& t) {
                               sizeof(float2) * agg_layout(P, t.agg_threads).total, P.num_sms, nI, t.agg_ctas_per_sm);
         h.dis = make_schedule(tucker_disaggregate_kernel<false>, t.dis_threads,
                               sizeof(float2) * dis_layout(P, t.dis_threads).total, P.num_sms, P.G, t.dis_ctas_per_sm);
+        // Between two and three groups per SM: three CTAs of 512 threads where their shared memory fits, with half
+        // the loads in flight (us, two / three): 310 groups of 1.1 MB items 174 / 157, 380 191 / 176, 340 of 1.8 MB
+        // 265 / 236, 456 303 / 291.
+        if (between_two_and_three(P, P.G) && t.dis_threads == 512 && t.dis_ctas_per_sm == 0) {
+            const Schedule three = make_schedule(tucker_disaggregate_kernel<false, true>, 512, h.dis.smem, P.num_sms, P.G);
+            if (three.blocks > h.dis.blocks) {
+                h.dis = three;
+                h.dis_three = true;
+            }
+        }
     }
     // The split path needs less shared memory than the persistent kernels (a block of the theta /
     // phi work at a time), so it also takes the plans whose items do not fit those: 4-lambda boxes, which
@@ -1155,6 +1180,7 @@ void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s) {
     TFMM_CUDA_CHECK(cudaMemcpyAsync(P.d_dis_order, dis.data(), sizeof(int) * P.G, cudaMemcpyHostToDevice, s));
     P.agg_sched = h.agg;
     P.dis_sched = h.dis;
+    P.dis_three = h.dis_three;
     P.tuning = t;
     P.persistent_ok = h.persistent;
     P.hot_ok = h.persistent || h.split;
@@ -1433,7 +1459,8 @@ void launch_tucker_disaggregate(const Plan& P, const float2* spec, int R, int we
         tucker_disaggregate_kernel<true><<<P.dis_sched.blocks, P.dis_sched.threads, P.dis_sched.smem, s>>>(a);
     } else {
         a.L = dis_layout(P, P.dis_sched.threads);
-        tucker_disaggregate_kernel<false><<<P.dis_sched.blocks, P.dis_sched.threads, P.dis_sched.smem, s>>>(a);
+        (P.dis_three ? tucker_disaggregate_kernel<false, true> : tucker_disaggregate_kernel<false>)
+            <<<P.dis_sched.blocks, P.dis_sched.threads, P.dis_sched.smem, s>>>(a);
     }
     TFMM_CUDA_CHECK(cudaGetLastError());
 }

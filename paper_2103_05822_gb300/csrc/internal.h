@@ -251,6 +251,7 @@ struct HotShape {
     bool persistent = false;                  // the largest work item fits the persistent kernels
     bool split = false;                       // the split path runs, for the stages below
     bool split_agg = false, split_dis = false;
+    bool dis_three = false;                   // three CTAs of 512 threads an SM in the disaggregation
 };
 
 // ----------------------------------------------------------------------- plan
@@ -296,6 +297,7 @@ struct Plan {
     int tc_dg1a_pairs = 0;             // (i_phi, r) pairs per CTA of the DG1a kernel (0: 128 when it fits, else 64)
     bool persistent_ok = false;        // the persistent single-RHS kernels fit (shared memory of the largest item)
     bool hot_ok = false;               // they or the split path run
+    bool dis_three = false;            // form of the persistent disaggregation kernel
     bool small_ok = false;             // every item's factors and one column fit one CTA's shared memory
     bool small_one = false;            // and that is the faster way for one right-hand side
     std::vector<SmallClass> small_classes;

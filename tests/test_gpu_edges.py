@@ -287,3 +287,25 @@ def test_split_path_parts_by_item_count(per_sm, monkeypatch):
     nbetas = [int(n) for n in rng.integers(18, 60, items // 2)]
     ranks = [[(12, 23, int(rng.integers(1, 18))), (12, int(rng.integers(22, 24)), 17)] for _ in nbetas]
     _check(9700 + items, 13, 26, nbetas, ranks, 1, 0, 1e-5, pad=1)
+
+
+@pytest.mark.parametrize("threads", [0, 512])
+def test_between_two_and_three_groups_per_sm(threads, monkeypatch):
+    """All groups at once on three CTAs an SM: of 320 threads (the default for small items), and of 512 in the
+    form with fewer registers."""
+    from paper_2103_05822_gb300 import tfmm
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    made = tfmm.tfmm_plan_from_tucker
+
+    def persistent(*args, **kw):
+        plan = made(*args, **kw)
+        tfmm.tfmm_plan_tuning_set(plan, single_rhs_split=2, **({"dis_threads": threads} if threads else {}))
+        t = tfmm.tfmm_plan_tuning_get(plan)
+        assert t["dis_threads"] == (threads or 320) and t["dis_blocks"] == 2 * sms + 6
+        return plan
+
+    monkeypatch.setattr(tfmm, "tfmm_plan_from_tucker", persistent)
+    rng = np.random.default_rng(41)
+    nbetas = [int(n) for n in rng.integers(2, 90, 2 * sms + 6)]
+    ranks = [_small_ranks(rng, 9, 18, nb, 70) for nb in nbetas]
+    _check(9800 + threads, 9, 18, nbetas, ranks, 1, 0, 1e-5, pad=1)
