@@ -245,6 +245,15 @@ struct Schedule {
     size_t smem = 0;      // dynamic shared memory per CTA
 };
 
+// Mean point and central moments m(j, k) of the triangle rule, for the plane waves' expansion up to
+// kDegree (planewave_kernel).
+struct PlanewaveRule {
+    static constexpr int kDegree = 8;
+    static constexpr int kTerms = (kDegree - 1) * (kDegree + 4) / 2;  // (n, k), 2 <= n <= kDegree, 0 <= k <= n
+    double u, v, m00, m20, m11, m02;
+    float cp[kTerms], cq[kTerms], cr[kTerms];  // (-1)^(n/2) C(n, k) / n! times m(k, n-k), m(k+1, n-k), m(k, n-k+1)
+};
+
 // Single-RHS stages as a tuning makes them (plan_hot).
 struct HotShape {
     Schedule agg, dis;
@@ -317,6 +326,7 @@ struct Plan {
     // device: geometry for recomputation / excitation
     RwgGeom* d_geom = nullptr;         // N, global RWG order
     std::vector<RwgGeom> geom;
+    PlanewaveRule pw{};                // with the geometry
     // FP64 factors (exports)
     std::vector<HostFactors64> f64;    // G x 2, pointers into f64_arenas
     std::vector<double2*> f64_arenas;  // owned device allocations
@@ -376,6 +386,7 @@ void build_tucker_setup(Plan& P, const Mesh& M, cudaStream_t s);
 void farfield_group_host(const Plan& P, int g, double2* At, double2* Ap, cudaStream_t s);
 void planewave_rhs(const Plan& P, const double* khat, const double* pol, int R, float2* V, cudaStream_t s);
 void planewave_rhs_noalloc(const Plan& P, const double* khat, const double* pol, int R, float2* V, cudaStream_t s);
+void upload_geometry(Plan& P, cudaStream_t s);  // P.geom to the device, and what the excitations need beside it
 void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w);
 
 // apply.cu

@@ -130,6 +130,7 @@ std::unique_ptr<tfmm_plan> load_plan(const char* path, cudaStream_t s) {
     bad(P.n_theta < 1 || P.n_theta > 4096 || P.n_phi < 1 || P.n_phi > 8192, "grid");
     bad(P.G < 1 || P.G > (1 << 26) || P.N < 1 || P.N >= ((int64_t)1 << 31), "sizes");
     bad(P.params.max_rhs < 1, "params");
+    bad(P.params.quad_order < 1 || P.params.quad_order > 10, "params");
     P.n_dir = P.n_theta * P.n_phi;
     P.ld_dir = (int)round_up(P.n_dir, 2);
     {
@@ -206,10 +207,7 @@ std::unique_ptr<tfmm_plan> load_plan(const char* path, cudaStream_t s) {
     F.get(tail, 8);
     bad(std::memcmp(tail, kTrailer, 8) != 0, "trailer");
     if (std::fgetc(F.f) != EOF) fail(TFMM_IO, "trailing bytes after the checkpoint: " + F.path);
-    if (P.has_geometry) {
-        TFMM_CUDA_CHECK(device_malloc(&P.d_geom, sizeof(RwgGeom) * P.N));
-        TFMM_CUDA_CHECK(cudaMemcpyAsync(P.d_geom, P.geom.data(), sizeof(RwgGeom) * P.N, cudaMemcpyHostToDevice, s));
-    }
+    if (P.has_geometry) upload_geometry(P, s);
     pack_factors_fp32(P, s);
     TFMM_CUDA_CHECK(cudaStreamSynchronize(s));
     return h;

@@ -225,8 +225,7 @@ __global__ void to_f32_kernel(const double2* __restrict__ in, int64_t n, int64_t
 // Against 64 bits the unrounded sum is off by 7e-10 on a lambda/10 mesh (rounding V to FP32:
 // 2.55e-8, as before) and 1.3e-9 at the limit kPWSpread.  1.8 ms for the same block (0.02 ms
 // for the bytes); the 28 FP64 operations left per side and incidence are what bounds it.
-constexpr int kPWDegree = 8;
-constexpr int kPWTerms = (kPWDegree - 1) * (kPWDegree + 4) / 2;  // (n, k), 2 <= n <= 8, 0 <= k <= n
+constexpr int kPWDegree = PlanewaveRule::kDegree, kPWTerms = PlanewaveRule::kTerms;
 constexpr int kPWTable = 256;    // steps per turn of the phase table
 constexpr int kPWCols = 64;      // incidences per block: a side's constants cost as much FP64 as three of them
 constexpr int kPWThreads = 128;
@@ -234,7 +233,7 @@ constexpr int kPWThreads = 128;
 // triangle that spreads further takes the points one by one
 constexpr float kPWSpread = 0.5f;
 
-struct PWArgs {
+struct PWArgs : PlanewaveRule {
     const RwgGeom* geom;
     const double* khat;  // R x 3
     const double* pol;   // R x 3
@@ -242,8 +241,6 @@ struct PWArgs {
     double k;
     int64_t n;
     int R, nq;
-    double u, v, m00, m20, m11, m02;  // mean point and central moments of the rule
-    float cp[kPWTerms], cq[kPWTerms], cr[kPWTerms];  // (-1)^(n/2) C(n, k) / n! times m(k, n-k), m(k+1, n-k), m(k, n-k+1)
 };
 
 // The points one by one, all FP64.
@@ -432,20 +429,15 @@ void triangle_rule(int order, std::vector<double>& qu, std::vector<double>& qv, 
         }
 }
 
-void launch_planewave(const Plan& P, const double* khat, const double* pol, int R, float2* V, cudaStream_t s) {
-    PWArgs a{};
-    a.geom = P.d_geom;
-    a.khat = khat;
-    a.pol = pol;
-    a.V = V;
-    a.k = P.k;
-    a.n = P.N;
-    a.R = R;
-    a.nq = P.params.quad_order * P.params.quad_order;
+// The moments depend on the rule alone and are laid out with the plan: computed in every call they took 8
+// (order 1) to 250 us (order 10) of the host, more than the kernel on most meshes.
+PlanewaveRule planewave_rule(int order) {
+    PlanewaveRule a{};
+    const int nq = order * order;
     std::vector<double> qu, qv, qw;
-    triangle_rule(P.params.quad_order, qu, qv, qw);
+    triangle_rule(order, qu, qv, qw);
     double su = 0.0, sv = 0.0;
-    for (int q = 0; q < a.nq; ++q) {
+    for (int q = 0; q < nq; ++q) {
         a.m00 += qw[q];
         su += qw[q] * qu[q];
         sv += qw[q] * qv[q] * (1.0 - qu[q]);
@@ -454,7 +446,7 @@ void launch_planewave(const Plan& P, const double* khat, const double* pol, int 
     a.v = sv / a.m00;
     auto moment = [&](int j, int k) {
         double m = 0.0;
-        for (int q = 0; q < a.nq; ++q) m += qw[q] * std::pow(qu[q] - a.u, j) * std::pow(qv[q] * (1.0 - qu[q]) - a.v, k);
+        for (int q = 0; q < nq; ++q) m += qw[q] * std::pow(qu[q] - a.u, j) * std::pow(qv[q] * (1.0 - qu[q]) - a.v, k);
         return m;
     };
     a.m20 = moment(2, 0);
@@ -472,6 +464,20 @@ void launch_planewave(const Plan& P, const double* khat, const double* pol, int 
             ++i;
         }
     }
+    return a;
+}
+
+void launch_planewave(const Plan& P, const double* khat, const double* pol, int R, float2* V, cudaStream_t s) {
+    PWArgs a{};
+    static_cast<PlanewaveRule&>(a) = P.pw;
+    a.geom = P.d_geom;
+    a.khat = khat;
+    a.pol = pol;
+    a.V = V;
+    a.k = P.k;
+    a.n = P.N;
+    a.R = R;
+    a.nq = P.params.quad_order * P.params.quad_order;
     for (int c0 = 0; c0 < R; c0 += 65535 * kPWCols) {  // grid.y limit
         PWArgs b = a;
         b.khat += 3 * (int64_t)c0;
@@ -1132,8 +1138,7 @@ void build_tucker_setup(Plan& P, const Mesh& M, cudaStream_t s) {
     const int nq = prm.quad_order * prm.quad_order;
 
     // geometry and directions
-    TFMM_CUDA_CHECK(device_malloc(&P.d_geom, sizeof(RwgGeom) * std::max<int64_t>(P.N, 1)));
-    TFMM_CUDA_CHECK(cudaMemcpyAsync(P.d_geom, P.geom.data(), sizeof(RwgGeom) * P.N, cudaMemcpyHostToDevice, s));
+    upload_geometry(P, s);
     const std::vector<double> dirs = direction_table(P);
     DevBuf d_dirs(sizeof(double) * dirs.size());
     TFMM_CUDA_CHECK(cudaMemcpyAsync(d_dirs.p, dirs.data(), sizeof(double) * dirs.size(), cudaMemcpyHostToDevice, s));
@@ -1284,6 +1289,12 @@ void farfield_group_host(const Plan& P, int g, double2* At, double2* Ap, cudaStr
     TFMM_CUDA_CHECK(cudaMemcpyAsync(Ap, d_A.as<double2>() + (int64_t)nd * nb, sizeof(double2) * (int64_t)nd * nb,
                                     cudaMemcpyDeviceToHost, s));
     TFMM_CUDA_CHECK(cudaStreamSynchronize(s));
+}
+
+void upload_geometry(Plan& P, cudaStream_t s) {
+    TFMM_CUDA_CHECK(device_malloc(&P.d_geom, sizeof(RwgGeom) * std::max<int64_t>(P.N, 1)));
+    TFMM_CUDA_CHECK(cudaMemcpyAsync(P.d_geom, P.geom.data(), sizeof(RwgGeom) * P.N, cudaMemcpyHostToDevice, s));
+    P.pw = planewave_rule(P.params.quad_order);
 }
 
 void planewave_rhs(const Plan& P, const double* khat, const double* pol, int R, float2* V, cudaStream_t s) {

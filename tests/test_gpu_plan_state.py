@@ -188,3 +188,29 @@ def test_autotuning_leaves_a_launch_shape_alone_that_does_not_run(kernels):
         t = tfmm.tfmm_autotune(plan, R=1, budget_ms=300.0)
         assert [t[k] for k in shape] == [before[k] for k in shape]
         assert 0 < t["agg_ms"] < 10 and 0 < t["dis_ms"] < 10
+
+
+def test_planewave_call_does_not_pay_for_the_rules_moments():
+    """The allocation-free entry point only queues work: its host time at 100 points a triangle is that at one
+    point and the rule itself (7 us; the moments, if computed in the call, take 250)."""
+    import time
+    from paper_2103_05822_gb300 import tfmm
+    from paper_2103_05822_gb300.inputs import icosphere
+    v, f = icosphere(1.0, 6)
+    mesh = tfmm.tfmm_mesh_create(v, f)
+    kh, pol = np.array([[0.0, 0.0, 1.0]]), np.array([[1.0, 0.0, 0.0]])
+
+    def host_us(order):
+        plan = tfmm.tfmm_plan_create(mesh, tfmm.tfmm_params_default(box=0.5, digits=1.0, tol=1e-1, quad_order=order))
+        V = torch.empty((1, plan.info["n_rwg"]), dtype=torch.complex64, device="cuda")
+        best = 1e9
+        for _ in range(30):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            for _ in range(4):
+                tfmm.tfmm_planewave_noalloc(plan, kh, pol, V)
+            best = min(best, (time.perf_counter() - t0) / 4 * 1e6)
+        return best
+
+    one = host_us(1)
+    assert host_us(10) <= one + 80
