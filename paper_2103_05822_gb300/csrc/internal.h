@@ -327,6 +327,8 @@ struct Plan {
     RwgGeom* d_geom = nullptr;         // N, global RWG order
     std::vector<RwgGeom> geom;
     PlanewaveRule pw{};                // with the geometry
+    bool pw_coarse = false;            // many triangles spread the phase past the expansion's limit
+    DeviceBuffer pw_table;             // phase table of the excitations
     // FP64 factors (exports)
     std::vector<HostFactors64> f64;    // G x 2, pointers into f64_arenas
     std::vector<double2*> f64_arenas;  // owned device allocations

@@ -227,7 +227,7 @@ __global__ void to_f32_kernel(const double2* __restrict__ in, int64_t n, int64_t
 // for the bytes); the 28 FP64 operations left per side and incidence are what bounds it.
 constexpr int kPWDegree = PlanewaveRule::kDegree, kPWTerms = PlanewaveRule::kTerms;
 constexpr int kPWTable = 256;    // steps per turn of the phase table
-constexpr int kPWCols = 64;      // incidences per block: a side's constants cost as much FP64 as three of them
+constexpr int kPWCols = 64;      // most incidences per block: a side's constants cost as much FP64 as three of them
 constexpr int kPWThreads = 128;
 // largest |phase - phase at c| over a triangle for the expansion (0.40 on a lambda/10 mesh); a
 // triangle that spreads further takes the points one by one
@@ -238,17 +238,17 @@ struct PWArgs : PlanewaveRule {
     const double* khat;  // R x 3
     const double* pol;   // R x 3
     float2* V;
+    const double2* table;  // (cos, -sin)(2 pi i / kPWTable)
     double k;
     int64_t n;
-    int R, nq;
+    int R, nq, cols;
 };
 
-// The points one by one, all FP64.
-__device__ __noinline__ double2 planewave_points(const RwgGeom* gp, const double* kh, const double* p, double k,
-                                                 int nq) {
-    const RwgGeom g = *gp;
+// The points of sides [first, last) one by one, all FP64.
+__device__ __forceinline__ double2 planewave_sum(const RwgGeom& g, int first, int last, const double* kh,
+                                                 const double* p, double k, int nq) {
     double vr = 0.0, vi = 0.0;
-    for (int side = 0; side < 2; ++side) {
+    for (int side = first; side < last; ++side) {
         const double* pv = side ? g.pm : g.pp;
         const double sgn = side ? -1.0 : 1.0;
         for (int q = 0; q < nq; ++q) {
@@ -256,7 +256,7 @@ __device__ __noinline__ double2 planewave_points(const RwgGeom* gp, const double
             double r3[3], dot = 0.0, ph = 0.0;
             for (int c = 0; c < 3; ++c) {
                 r3[c] = pv[c] + u * (g.q1[c] - pv[c]) + v * (1.0 - u) * (g.q2[c] - pv[c]);
-                dot += sgn * g.l * w * (r3[c] - pv[c]) * p[c];
+                dot += sgn * w * g.l * (r3[c] - pv[c]) * p[c];
                 ph += kh[c] * r3[c];
             }
             double sn, cs;
@@ -266,6 +266,31 @@ __device__ __noinline__ double2 planewave_points(const RwgGeom* gp, const double
         }
     }
     return make_double2(vr, vi);
+}
+__device__ __noinline__ double2 planewave_points(const RwgGeom* gp, int side, const double* kh, const double* p,
+                                                 double k, int nq) {
+    const RwgGeom g = *gp;
+    return planewave_sum(g, side, side + 1, kh, p, k, nq);
+}
+
+// One RWG and incidence per thread by the points: where many triangles are too large for the expansion, and
+// one-point rules of few results.
+struct PWPointArgs {
+    const RwgGeom* geom;
+    const double* khat;
+    const double* pol;
+    float2* V;
+    double k;
+    int64_t n;
+    int nq;
+};
+__global__ void planewave_points_kernel(const PWPointArgs a) {
+    const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int r = blockIdx.y;
+    if (m >= a.n) return;
+    const RwgGeom g = a.geom[m];
+    const double2 v = planewave_sum(g, 0, 2, a.khat + 3 * r, a.pol + 3 * r, a.k, a.nq);
+    a.V[m + a.n * r] = make_float2((float)v.x, (float)v.y);
 }
 
 struct PWSide {        // one triangle of an RWG
@@ -360,17 +385,16 @@ __device__ __forceinline__ bool planewave_side_sum(const PWSide& s, const PWInc&
 }
 
 // One side of an RWG per thread (two neighbouring lanes an RWG: both sides in one thread
-// spilled), kPWCols incidences per block, their table in shared memory.
+// spilled), a.cols incidences per block, their table in shared memory.
 __global__ void __launch_bounds__(kPWThreads, 4) planewave_kernel(const __grid_constant__ PWArgs a) {
     __shared__ double2 tab[kPWTable];
     __shared__ float2 tabf[kPWTable];
     __shared__ PWInc inc[kPWCols];
-    const int r0 = blockIdx.y * kPWCols, nr = min(kPWCols, a.R - r0);
+    const int r0 = blockIdx.y * a.cols, nr = min(a.cols, a.R - r0);
     for (int i = threadIdx.x; i < kPWTable; i += kPWThreads) {
-        double sn, cs;
-        sincospi(2.0 * i / kPWTable, &sn, &cs);
-        tab[i] = make_double2(cs, -sn);
-        tabf[i] = make_float2((float)cs, (float)-sn);
+        const double2 t = a.table[i];
+        tab[i] = t;
+        tabf[i] = make_float2((float)t.x, (float)t.y);
     }
     if (threadIdx.x < nr) {
         PWInc& v = inc[threadIdx.x];
@@ -402,18 +426,22 @@ __global__ void __launch_bounds__(kPWThreads, 4) planewave_kernel(const __grid_c
     for (int r = 0; r < nr; ++r) {
         double re = 0.0, im = 0.0;
         bool ok = planewave_side_sum(side, inc[r], a, tab, tabf, re, im);
+        ok = __shfl_xor_sync(0xffffffffu, (int)ok, 1) && ok;  // the pair takes one way
+        if (!ok) {
+            const double2 v = planewave_points(gp, minus, a.khat + 3 * (r0 + r), a.pol + 3 * (r0 + r), a.k, a.nq);
+            re = -v.x;
+            im = -v.y;
+        }
         re = -(re + __shfl_xor_sync(0xffffffffu, re, 1));
         im = -(im + __shfl_xor_sync(0xffffffffu, im, 1));
-        ok = __shfl_xor_sync(0xffffffffu, (int)ok, 1) && ok;
-        if (live && !minus) {
-            if (!ok) {
-                const double2 v = planewave_points(gp, a.khat + 3 * (r0 + r), a.pol + 3 * (r0 + r), a.k, a.nq);
-                re = v.x;
-                im = v.y;
-            }
-            a.V[m + a.n * (r0 + r)] = make_float2((float)re, (float)im);
-        }
+        if (live && !minus) a.V[m + a.n * (r0 + r)] = make_float2((float)re, (float)im);
     }
+}
+
+__global__ void planewave_table_kernel(double2* table) {
+    double sn, cs;
+    sincospi(2.0 * threadIdx.x / kPWTable, &sn, &cs);
+    table[threadIdx.x] = make_double2(cs, -sn);
 }
 
 // The rule's points on the triangle's (u, v (1 - u)) and their weights (sum 1/2).
@@ -468,23 +496,50 @@ PlanewaveRule planewave_rule(int order) {
 }
 
 void launch_planewave(const Plan& P, const double* khat, const double* pol, int R, float2* V, cudaStream_t s) {
+    const int nq = P.params.quad_order * P.params.quad_order;
+    // A one-point rule costs two sincos a result, about what a side's constants cost: by the points up to
+    // three incidences and where the results are few (us, points / expansion: 108,000 RWGs, one incidence 38 / 66,
+    // three 84 / 92; 1080 RWGs x 65 39 / 48, 4320 x 20 38 / 40; 38,880 x 65 516 / 335).
+    if (P.pw_coarse || (nq == 1 && (R <= 3 || R * P.N <= 140000))) {
+        for (int64_t c0 = 0; c0 < R; c0 += 65535) {  // grid.y limit
+            const dim3 grid((unsigned)((P.N + 255) / 256), (unsigned)std::min<int64_t>(R - c0, 65535));
+            planewave_points_kernel<<<grid, 256, 0, s>>>(
+                PWPointArgs{P.d_geom, khat + 3 * c0, pol + 3 * c0, V + P.N * c0, P.k, P.N, nq});
+            TFMM_CUDA_CHECK(cudaGetLastError());
+        }
+        return;
+    }
     PWArgs a{};
     static_cast<PlanewaveRule&>(a) = P.pw;
     a.geom = P.d_geom;
     a.khat = khat;
     a.pol = pol;
     a.V = V;
+    a.table = static_cast<const double2*>(P.pw_table.p);
     a.k = P.k;
     a.n = P.N;
     a.R = R;
-    a.nq = P.params.quad_order * P.params.quad_order;
-    for (int c0 = 0; c0 < R; c0 += 65535 * kPWCols) {  // grid.y limit
+    a.nq = nq;
+    // Incidences per block.  A block's constants cost what three incidences do; alone on an SM it takes 1.6 us
+    // for each, and together the blocks of an SM 1.3 us each: the least of that over the columns (us, with 25
+    // points a triangle: 270 and 4320 RWGs x 65, 64 to a block 124 and 124, now 27 and 55).
+    const int64_t blocks = (2 * P.N + kPWThreads - 1) / kPWThreads;
+    int64_t best = INT64_MAX;
+    for (int c = std::min(R, kPWCols); c >= 1; --c) {
+        const int64_t per_sm = (blocks * ((R + c - 1) / c) + P.num_sms - 1) / P.num_sms;
+        const int64_t cost = (per_sm == 1 ? 16 : 13 * per_sm) * (3 + c);
+        if (cost < best) {
+            best = cost;
+            a.cols = c;
+        }
+    }
+    for (int64_t c0 = 0; c0 < R; c0 += (int64_t)65535 * a.cols) {  // grid.y limit
         PWArgs b = a;
-        b.khat += 3 * (int64_t)c0;
-        b.pol += 3 * (int64_t)c0;
+        b.khat += 3 * c0;
+        b.pol += 3 * c0;
         b.V += a.n * c0;
-        b.R = std::min(R - c0, 65535 * kPWCols);
-        const dim3 grid((unsigned)((2 * P.N + kPWThreads - 1) / kPWThreads), (unsigned)((b.R + kPWCols - 1) / kPWCols));
+        b.R = (int)std::min<int64_t>(R - c0, (int64_t)65535 * a.cols);
+        const dim3 grid((unsigned)blocks, (unsigned)((b.R + a.cols - 1) / a.cols));
         planewave_kernel<<<grid, kPWThreads, 0, s>>>(b);
         TFMM_CUDA_CHECK(cudaGetLastError());
     }
@@ -1295,6 +1350,29 @@ void upload_geometry(Plan& P, cudaStream_t s) {
     TFMM_CUDA_CHECK(device_malloc(&P.d_geom, sizeof(RwgGeom) * std::max<int64_t>(P.N, 1)));
     TFMM_CUDA_CHECK(cudaMemcpyAsync(P.d_geom, P.geom.data(), sizeof(RwgGeom) * P.N, cudaMemcpyHostToDevice, s));
     P.pw = planewave_rule(P.params.quad_order);
+    // Coarse: half of the RWGs have a triangle with a vertex this far from its mean point, so that nearly every
+    // warp holds a pair past kPWSpread and would go through the expansion and the points (us, points / both: spheres with edges of 0.23 wavelength, 4
+    // points a triangle, 5880 RWGs x 360 1584 / 2024, 0.18 wavelength, 9720 RWGs 2591 / 2832).
+    const double limit = P.params.quad_order == 1 ? 0.5 : 0.6;
+    int64_t wide = 0;
+    for (const RwgGeom& g : P.geom) {
+        double far2 = 0.0;
+        for (const double* p : {g.pp, g.pm}) {
+            double d2[3] = {0.0, 0.0, 0.0};
+            for (int c = 0; c < 3; ++c) {
+                const double e1 = g.q1[c] - p[c], e2 = g.q2[c] - p[c], m = P.pw.u * e1 + P.pw.v * e2;
+                d2[0] += m * m;
+                d2[1] += (e1 - m) * (e1 - m);
+                d2[2] += (e2 - m) * (e2 - m);
+            }
+            far2 = std::max(far2, std::max(d2[0], std::max(d2[1], d2[2])));
+        }
+        wide += P.k * std::sqrt(far2) > limit;
+    }
+    P.pw_coarse = 2 * wide > P.N;
+    TFMM_CUDA_CHECK(device_malloc(&P.pw_table.p, sizeof(double2) * kPWTable));
+    planewave_table_kernel<<<1, kPWTable, 0, s>>>(static_cast<double2*>(P.pw_table.p));
+    TFMM_CUDA_CHECK(cudaGetLastError());
 }
 
 void planewave_rhs(const Plan& P, const double* khat, const double* pol, int R, float2* V, cudaStream_t s) {
