@@ -2612,9 +2612,19 @@ void launch_dg1a(const Plan& P, const TcPlan& M, const TcCtx& c, cudaStream_t s)
     TFMM_CUDA_CHECK(cudaGetLastError());
 }
 
-// The stacked-term form of DG1a (MODE CAT_DG1A) or DG1b (CAT_DG1B) when the stacked N
-// (2 T r8(rank)) fits one MMA and both operands fit shared memory; TFMM_TC_CAT=0 keeps
-// the other forms (for comparisons), as does a DG1a pair count set by the tuning.
+// Shared memory of the stacked-term form of DG1a (mode CAT_DG1A) or DG1b (CAT_DG1B), 0 where its
+// stacked N (2 T r8(rank)) does not fit one MMA or its operands not shared memory.
+size_t cat_smem(const Plan& P, int T, int mode) {
+    const int K16 = ((mode == CAT_DG1A ? P.n_theta : P.n_phi) + 15) & ~15;
+    const int n8max = (int)r8(P.max_rank[mode == CAT_DG1A ? 0 : 1]);
+    if (2 * T * n8max > 256 || (mode == CAT_DG1A && TBM * (K16 / 8) > 4 * CAT_THREADS)) return 0;
+    const size_t sbo = (size_t)K16 * 16;
+    const size_t smem = (size_t)2 * T * (TBM / 8) * sbo + (size_t)2 * (2 * T * n8max / 8) * sbo;
+    return smem <= kMaxDynSmem ? smem : 0;
+}
+
+// The stacked-term form when it fits; TFMM_TC_CAT=0 keeps the other forms (for comparisons),
+// as does a DG1a pair count set by the tuning.
 template <class VOff, class MOff>
 void plan_cat(const Plan& P, TcPlan& M, int mode, bf16* Vb, VOff voff, bf16* Mb, MOff moff) {
     CatPlan& C = mode == CAT_DG1A ? M.cat1a : M.cat1b;
@@ -2624,11 +2634,8 @@ void plan_cat(const Plan& P, TcPlan& M, int mode, bf16* Vb, VOff voff, bf16* Mb,
     const int T = M.T, R = M.R, nt = P.n_theta, np = P.n_phi;
     const int K = mode == CAT_DG1A ? nt : np, K16 = (K + 15) & ~15;
     const int n8max = (int)r8(P.max_rank[mode == CAT_DG1A ? 0 : 1]);
-    if (2 * T * n8max > 256) return;
-    if (mode == CAT_DG1A && TBM * (K16 / 8) > 4 * CAT_THREADS) return;
-    const size_t sbo = (size_t)K16 * 16;
-    const size_t smem = (size_t)2 * T * (TBM / 8) * sbo + (size_t)2 * (2 * T * n8max / 8) * sbo;
-    if (smem > kMaxDynSmem) return;
+    const size_t smem = cat_smem(P, T, mode);
+    if (smem == 0) return;
     std::vector<CatItem> items(P.items.size());
     std::vector<D1Tile> tiles;
     for (size_t q = 0; q < P.items.size(); ++q) {
@@ -2662,8 +2669,9 @@ void plan_cat(const Plan& P, TcPlan& M, int mode, bf16* Vb, VOff voff, bf16* Mb,
 }
 
 // The fused DG1a + DG1b when r_theta <= 32, both accumulators fit TMEM and the operands shared
-// memory (every workload up to 2-lambda boxes); larger ranks keep the two kernels, as do
-// TFMM_TC_CAT=0 and a DG1a pair count set by the tuning.
+// memory, and the separate kernels would not be the more precise ones (every workload up to
+// 2-lambda boxes); larger ranks keep the two kernels, as do TFMM_TC_CAT=0 and a DG1a pair count
+// set by the tuning.
 template <class MOff>
 void plan_dg1(const Plan& P, TcPlan& M, const bf16* F, const std::vector<TcItem>& tci, bf16* Mb, MOff moff) {
     Dg1Plan& D = M.dg1;
@@ -2672,6 +2680,12 @@ void plan_dg1(const Plan& P, TcPlan& M, const bf16* F, const std::vector<TcItem>
     if (P.tc_dg1a_pairs != 0 || !fused_enabled() || !tc_split_accumulators()) return;
     const int T = M.T, R = M.R, nt = P.n_theta, np = P.n_phi;
     if (P.max_rank[0] > 32) return;
+    // One accumulator takes all of n_phi here.  Where the separate DG1b restarts its accumulator every chunk
+    // (more than a chunk of directions, and too large for the stacked form, which does not), TMEM's rounding
+    // towards zero would show: 128 directions, r_phi = 64, an error of 5.3e-7 instead of 4.3e-7; 96, 4.6e-7
+    // instead of 4.0e-7.
+    const int chunk = tc_chunk_ktiles() * TBK;
+    if (chunk > 0 && np > chunk && cat_smem(P, T, CAT_DG1B) == 0) return;
     Dg1Shape sh{};
     sh.PC = P.max_rank[0] <= 16 ? 16 : 32;
     sh.NS = DG1_SLABS;
