@@ -192,8 +192,6 @@ struct TcPlan {             // per (R, terms): problem lists of the 8 steps and 
     int n_xtiles = 0;
     DeviceBuffer ybuf;      // DG3 output in group order (R x N complex)
     DeviceBuffer y_pos;     // position of every RWG in group order
-    // per item: element offsets of its M' and V'' / P'' scratch planes (for re-planning)
-    std::vector<int64_t> m_off, v_off;
     ~TcPlan();
 };
 
@@ -412,7 +410,7 @@ void launch_small_disaggregate(const Plan& P, const float2* spec, int R, int wei
 // mrhs_tc.cu
 void build_tc_factors(Plan& P, int T, cudaStream_t s);
 TcPlan* get_tc_plan(Plan& P, int R, int T, cudaStream_t s);
-void tc_replan_shapes(Plan& P);  // re-plans the fused AG3+AG4 and DG1a kernels of every chain after a preference change
+void tc_replan_shapes(Plan& P, cudaStream_t s);  // plans every chain anew after a preference change
 void launch_tc_aggregate(Plan& P, int T, const float2* x, int R, int64_t ldx, float2* spec, cudaStream_t s);
 void launch_tc_disaggregate(Plan& P, int T, const float2* spec, int R, int weights, float2 beta, float2* y,
                             int64_t ldy, cudaStream_t s);

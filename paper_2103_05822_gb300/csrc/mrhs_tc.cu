@@ -2791,7 +2791,7 @@ TcPlan* get_tc_plan(Plan& P, int R, int T, cudaStream_t s) {
         // M' ([a + r_t r][b]) and H ([r][a + r_t b]) share a buffer
         o.ldm = std::max(r8(d.rp), r8(m));
         o.m = sz[BM]; sz[BM] += (int64_t)2 * T * std::max<int64_t>((int64_t)d.rt * R * r8(d.rp), (int64_t)R * r8(m));
-        // V'' ([i_phi + n_phi r][a]) and P'' ([a + r_t r][i_phi]) share a buffer
+        // V'' ([i_phi + n_phi r][a]) and P'' ([a + r_t r][i_phi]) share a buffer (if either is written)
         o.v = sz[BV]; sz[BV] += (int64_t)2 * T * std::max<int64_t>((int64_t)np * R * r8(d.rt), (int64_t)d.rt * R * r8(np));
         o.ldg = r8(nt); o.g = fused_enabled() ? 0 : sz[BG]; sz[BG] += (int64_t)2 * T * np * R * o.ldg;
         for (int b = 0; b < NB; ++b) sz[b] = (sz[b] + 63) & ~int64_t(63);
@@ -2804,15 +2804,23 @@ TcPlan* get_tc_plan(Plan& P, int R, int T, cudaStream_t s) {
         TFMM_CUDA_CHECK(device_malloc(&M.y_pos.p, sizeof(int) * P.N));
         TFMM_CUDA_CHECK(cudaMemcpy(M.y_pos.p, pos.data(), sizeof(int) * P.N, cudaMemcpyHostToDevice));
     }
-    for (int b = 0; b < NB; ++b) {
+    auto scratch = [&](int b) {
         TFMM_CUDA_CHECK(device_malloc(&M.buf[b], sizeof(bf16) * std::max<int64_t>(sz[b], 1)));
         TFMM_CUDA_CHECK(cudaMemset(M.buf[b], 0, sizeof(bf16) * std::max<int64_t>(sz[b], 1)));
-    }
-    bf16* X = reinterpret_cast<bf16*>(M.buf[BX]);
-    bf16* Tb = reinterpret_cast<bf16*>(M.buf[BT]);
-    bf16* Mb = reinterpret_cast<bf16*>(M.buf[BM]);
-    bf16* Vb = reinterpret_cast<bf16*>(M.buf[BV]);
-    bf16* Gb = reinterpret_cast<bf16*>(M.buf[BG]);
+        return reinterpret_cast<bf16*>(M.buf[b]);
+    };
+    bf16* X = scratch(BX);
+    bf16* Tb = scratch(BT);
+    bf16* Mb = scratch(BM);
+    // The fused kernels first: with both, nothing reads or writes V'' and P'' (6 GB for 128 columns of the
+    // 30-lambda sphere).
+    const auto voff = [&](int q) { return of[q].v; };
+    const auto moff = [&](int q) { return of[q].m; };
+    plan_fused34(P, M, F, tci, Mb, moff);
+    plan_dg1(P, M, F, tci, Mb, moff);
+    if (M.fused34 && M.dg1.on) sz[BV] = 0;
+    bf16* Vb = scratch(BV);
+    bf16* Gb = scratch(BG);
     std::vector<TcProb> pr[8];
     std::vector<MrTile> tl[8];
     for (int q = 0; q < nI; ++q) {
@@ -2904,45 +2912,23 @@ TcPlan* get_tc_plan(Plan& P, int R, int T, cudaStream_t s) {
         TFMM_CUDA_CHECK(device_malloc(&M.x_tiles.p, sizeof(MrTile) * xt.size()));
         TFMM_CUDA_CHECK(cudaMemcpy(M.x_tiles.p, xt.data(), sizeof(MrTile) * xt.size(), cudaMemcpyHostToDevice));
     }
-    M.m_off.resize(nI);
-    M.v_off.resize(nI);
-    for (int q = 0; q < nI; ++q) {
-        M.m_off[q] = of[q].m;
-        M.v_off[q] = of[q].v;
+    if (!M.dg1.on) {
+        plan_cat(P, M, CAT_DG1A, Vb, voff, Mb, moff);
+        if (!M.cat1a.on) plan_dg1a(P, M, F, tci, Vb, voff);
+        plan_cat(P, M, CAT_DG1B, Vb, voff, Mb, moff);
     }
-    plan_fused34(P, M, F, tci, Mb, [&](int q) { return M.m_off[q]; });
-    const auto voff = [&](int q) { return M.v_off[q]; };
-    const auto moff = [&](int q) { return M.m_off[q]; };
-    plan_dg1(P, M, F, tci, Mb, moff);
-    plan_cat(P, M, CAT_DG1A, Vb, voff, Mb, moff);
-    if (!M.cat1a.on) plan_dg1a(P, M, F, tci, Vb, voff);
-    plan_cat(P, M, CAT_DG1B, Vb, voff, Mb, moff);
     P.tc.push_back(std::move(tp));
     return P.tc.back().get();
 }
 
-void tc_replan_shapes(Plan& P) {
+// Makes every chain anew: a preference can change which kernels run and with them the scratch.
+void tc_replan_shapes(Plan& P, cudaStream_t s) {
     TFMM_REQUIRE(P.live_graphs == 0, "captured graphs use the current tile lists: destroy them first");
     TFMM_CUDA_CHECK(cudaDeviceSynchronize());  // no launch may still read the old lists
-    for (auto& mp : P.tc) {
-        TcPlan& M = *mp;
-        for (DeviceBuffer* b : {&M.f34_items, &M.f34_tiles, &M.dg1a_items, &M.dg1a_tiles, &M.cat1a.items,
-                                &M.cat1a.tiles, &M.dg1.items, &M.dg1.units}) {
-            if (b->p) cudaFree(b->p);
-            b->p = nullptr;
-        }
-        const bf16* F = reinterpret_cast<const bf16*>(P.tc_fac[M.T].p);
-        const std::vector<TcItem>& tci = P.tc_items[M.T];
-        bf16* Mb = reinterpret_cast<bf16*>(M.buf[2]);
-        bf16* Vb = reinterpret_cast<bf16*>(M.buf[3]);
-        plan_fused34(P, M, F, tci, Mb, [&](int q) { return M.m_off[q]; });
-        const auto voff = [&](int q) { return M.v_off[q]; };
-        const auto moff = [&](int q) { return M.m_off[q]; };
-        plan_dg1(P, M, F, tci, Mb, moff);
-        plan_cat(P, M, CAT_DG1A, Vb, voff, Mb, moff);
-        M.dg1a = false;
-        if (!M.cat1a.on) plan_dg1a(P, M, F, tci, Vb, voff);
-    }
+    std::vector<std::pair<int, int>> chains;
+    for (const auto& m : P.tc) chains.emplace_back(m->R, m->T);
+    P.tc.clear();
+    for (const auto& [R, T] : chains) get_tc_plan(P, R, T, s);
 }
 
 namespace {

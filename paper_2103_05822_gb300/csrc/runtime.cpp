@@ -401,7 +401,7 @@ tfmm_status tfmm_plan_tuning_set(tfmm_plan* plan, const tfmm_tuning* t, void* st
         if (tiles) {
             P.tc_f34_n1 = t->tc_f34_n1;
             P.tc_dg1a_pairs = t->tc_dg1a_pairs;
-            tc_replan_shapes(P);
+            tc_replan_shapes(P, (cudaStream_t)stream);
         }
         P.params.mrhs_precision = t->mrhs_precision;
     });
@@ -517,7 +517,7 @@ tfmm_status tfmm_autotune(tfmm_plan* plan, int32_t R, double budget_ms, int32_t 
                         if (n1 == bn1 && pairs == bpairs) continue;
                         P.tc_f34_n1 = n1;
                         P.tc_dg1a_pairs = pairs;
-                        tc_replan_shapes(P);
+                        tc_replan_shapes(P, s);
                         const double a = time_ms(agg, 2, s, tm);
                         const double d = time_ms(dis, 2, s, tm);
                         if (a + d < best_ms) {
@@ -531,7 +531,7 @@ tfmm_status tfmm_autotune(tfmm_plan* plan, int32_t R, double budget_ms, int32_t 
                 if (P.tc_f34_n1 != bn1 || P.tc_dg1a_pairs != bpairs) {
                     P.tc_f34_n1 = bn1;
                     P.tc_dg1a_pairs = bpairs;
-                    tc_replan_shapes(P);
+                    tc_replan_shapes(P, s);
                 }
             }
         }

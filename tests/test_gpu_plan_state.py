@@ -232,3 +232,34 @@ def test_first_step_of_the_disaggregation_keeps_its_precision_on_fine_grids(nt, 
             y = _dis(tfmm, plan, g).cpu().numpy()
             total[pairs] += sum(np.linalg.norm(y[r] - ref[r]) / np.linalg.norm(ref[r]) for r in range(8))
     assert total[0] <= 1.1 * total[64]
+
+
+def test_fused_tensor_core_kernels_take_no_planes_for_what_they_keep_on_chip():
+    """V'' and P'' of 128 columns would be 153 MB here; X, T, M', y and the factor planes are about 70 MB, and
+    allocations come in steps of 2 MB.  A tile preference that turns the fused kernels off brings them back."""
+    nt, npf, rank, R, G = 26, 52, (12, 14, 30), 128, 60
+    planes = 2 * G * 12 * npf * R * 16  # 2 x 3 terms of 2 bytes, r_theta rounded up to 8
+    tfmm, first, *_ = _problem(101, nt, npf, [40, 40], [[rank, rank]] * 2, R, 3)
+    x, g = _inputs(first, R, 102)
+    _agg(tfmm, first, x), _dis(tfmm, first, g)  # the kernels are loaded
+    tfmm, plan, *_ = _problem(103, nt, npf, [40] * G, [[rank, rank]] * G, R, 3)
+    x, g = _inputs(plan, R, 104)
+    spec, y = torch.empty_like(g), torch.empty_like(x)
+
+    def call():
+        tfmm.tfmm_aggregate(plan, x, spec)
+        tfmm.tfmm_disaggregate(plan, g, y)
+        torch.cuda.synchronize()
+
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    call()
+    assert free - torch.cuda.mem_get_info()[0] < 0.75 * planes
+    fused = y.clone()
+    tfmm.tfmm_plan_tuning_set(plan, tc_dg1a_pairs=64)
+    call()
+    assert free - torch.cuda.mem_get_info()[0] > planes
+    assert torch.linalg.vector_norm(y - fused) <= 2e-6 * torch.linalg.vector_norm(fused)
+    tfmm.tfmm_plan_tuning_set(plan, tc_dg1a_pairs=0)
+    call()
+    assert torch.equal(y, fused)
