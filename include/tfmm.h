@@ -250,9 +250,10 @@ tfmm_status tfmm_matvec_host(tfmm_plan* plan, const tfmm_cfloat* x_host, tfmm_cf
  * EFIE (Eq. 2) for the x that tfmm_aggregate received.  Evaluated as a 3-D FFT
  * convolution over the zero-padded box grid, FP32 (the translation kernel's
  * transform is computed once in FP64).  The first call builds it (device memory
- * owned by the plan: the kernel's transform, N_grid x N_dir complex, and, for box
- * grids of more than 18 a side, a work grid of N_grid x 2 N_dir complex, N_grid >=
- * (2K_x - 1)(2K_y - 1)(2K_z - 1), or the cube of the longest side where that is near-cubic);
+ * owned by the plan: the kernel's transform, N_grid x N_dir complex, N_grid >= (2K_x - 1)
+ * (2K_y - 1)(2K_z - 1), or the cube over the longest side where that has at most twice as
+ * many points and K <= 18; other box grids, those of one or two boxes a side among them, also
+ * take a work grid of N_grid x 2 N_dir complex);
  * later calls allocate nothing.
  *   spectra_out  device, R x G x 2 x N_dir FP32 complex (as tfmm_aggregate writes it)
  *   spectra_in   device, same shape, overwritten; must not alias spectra_out

@@ -143,7 +143,8 @@ __global__ void gather_kernel(const float2* __restrict__ grid, const int* __rest
 // Register FFTs: a thread transforms one line of N = A B points (A, B <= 8) held in
 // registers, X[k1 + A k2] = sum_b W_B^(b k2) W_N^(b k1) sum_a W_A^(a k1) x[B a + b].  Every
 // loop unrolls, so that the line stays in registers and the twiddles are constant operands.
-constexpr int kCubeSizes[] = {4, 6, 8, 10, 12, 15, 16, 18, 20, 24, 25, 30, 32, 36};
+// (no 4: for up to two boxes a side its volume is past twice cuFFT's grid; no 16: 15 serves eight boxes, 18 nine)
+constexpr int kCubeSizes[] = {6, 8, 10, 12, 15, 18, 20, 24, 25, 30, 32, 36};
 constexpr int kCubeMax = 36;
 __constant__ float2 c_tw[kCubeMax * (kCubeMax + 1) / 2];  // W_n^k = exp(-2 pi i k / n) at n (n - 1) / 2 + k
 
@@ -215,8 +216,7 @@ __device__ __forceinline__ void dft(float2 (&v)[R]) {
 
 template <int N>
 __host__ __device__ constexpr int fft_a() {  // first factor of N
-    return N == 4 ? 2 : N == 6 ? 2 : N == 8 ? 2 : N == 10 ? 2 : N == 12 ? 3 : N == 15 ? 3 : N == 16 ? 4
-         : N == 18 ? 3 : N == 20 ? 4 : N == 24 ? 4 : N == 25 ? 5 : N == 30 ? 5 : N == 32 ? 4 : 6;
+    return N == 6 ? 2 : N == 8 ? 2 : N == 10 ? 2 : N == 12 ? 3 : N == 15 ? 3 : N == 18 ? 3 : N == 20 ? 4 : N == 24 ? 4 : N == 25 ? 5 : N == 30 ? 5 : N == 32 ? 4 : 6;
 }
 
 template <int N>
@@ -358,8 +358,8 @@ template <class F>
 void with_cube_size(int n, F&& f) {
     switch (n) {
 #define TFMM_CUBE(N) case N: f(std::integral_constant<int, N>{}); break;
-        TFMM_CUBE(4) TFMM_CUBE(6) TFMM_CUBE(8) TFMM_CUBE(10) TFMM_CUBE(12) TFMM_CUBE(15) TFMM_CUBE(16)
-        TFMM_CUBE(18) TFMM_CUBE(20) TFMM_CUBE(24) TFMM_CUBE(25) TFMM_CUBE(30) TFMM_CUBE(32) TFMM_CUBE(36)
+        TFMM_CUBE(6) TFMM_CUBE(8) TFMM_CUBE(10) TFMM_CUBE(12) TFMM_CUBE(15) TFMM_CUBE(18) TFMM_CUBE(20)
+        TFMM_CUBE(24) TFMM_CUBE(25) TFMM_CUBE(30) TFMM_CUBE(32) TFMM_CUBE(36)
 #undef TFMM_CUBE
         default: fail(TFMM_CUDA, "no cube kernel of this size");
     }
