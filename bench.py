@@ -293,20 +293,22 @@ def run_reference(args, w, world, rank):
 
 # --------------------------------------------------------------------- ours
 def launches_per_step(tfmm, plan, R, dev):
-    """Kernels one aggregate + disaggregate pair launches: one persistent kernel per stage
-    or one per stage with small groups wholly in shared memory (at least; by size class when
-    there are many) for one RHS (three per stage on the split path, taken by plans with fewer
-    work items than twice the SMs, of more than about 1 MB and 0.5 MB), the tensor-core chain for many (operand prep and three kernels
-    for aggregation; four and the reordering of y for disaggregation)."""
+    """Kernels one aggregate + disaggregate pair launches, at least.  One RHS: one persistent kernel per stage,
+    or one per stage with small groups wholly in shared memory, or three per stage on the split path (plans
+    with fewer work items than twice the SMs, of more than 960 KB in the aggregation, 450 KB in the
+    disaggregation, 225 KB there up to an item per SM).  Many: the tensor-core chain's operand prep, AG1, AG2
+    and the fused AG3 + AG4; the fused DG1, DG2, DG3 and the reordering of y."""
     import torch
     t = tfmm.tfmm_plan_tuning_get(plan)
     if R == 1:
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
         rt, rp, rb = plan.info["max_rank"]
         largest = 8 * rb * (plan.info["max_n_beta"] + rt * rp)
-        few = t["single_rhs_split"] == 0 and plan.info["n_groups"] < sms
-        return sum(3 if t["single_rhs_split"] == 1 or (few and largest > kb << 10) else 1 for kb in (960, 450))
-    return 9
+        items = 2 * plan.info["n_groups"]
+        few = t["single_rhs_split"] == 0 and items < 2 * sms
+        kbs = (960, 225 if items <= sms else 450)
+        return sum(3 if t["single_rhs_split"] == 1 or (few and largest > kb << 10) else 1 for kb in kbs)
+    return 8
 
 
 def traffic_record(kernel, factor_bytes):

@@ -74,3 +74,24 @@ def test_group_time_extrapolation_is_exact_for_an_affine_cost():
     assert abs(total - float(np.sum(a + b * sizes))) <= 1e-9 * total
     # a degenerate sample (one size) falls back to the groups' share of RWGs
     assert abs(bench.scale_group_times([100, 100], [1.0, 1.0], [100, 300]) - 4.0) < 1e-12
+
+
+def test_launch_count_per_pair_of_stages(monkeypatch):
+    """One persistent or three split launches a stage for one column, eight for the tensor-core chain."""
+    import types
+
+    import pytest
+    torch = pytest.importorskip("torch")
+    monkeypatch.setattr(torch.cuda, "get_device_properties", lambda dev: types.SimpleNamespace(multi_processor_count=152))
+
+    def count(groups, n_beta, rank, R=1, split=0):
+        plan = types.SimpleNamespace(info={"n_groups": groups, "max_n_beta": n_beta, "max_rank": rank})
+        tfmm = types.SimpleNamespace(tfmm_plan_tuning_get=lambda p: {"single_rhs_split": split})
+        return bench.launches_per_step(tfmm, plan, R, 0)
+
+    assert count(1034, 1972, [25, 36, 268]) == 2          # 30-lambda sphere: persistent
+    assert count(19, 6000, [25, 36, 268]) == 6            # trihedral: split
+    assert count(100, 300, [13, 17, 65]) == 2             # 271 KB items, more than one per SM
+    assert count(50, 300, [13, 17, 65]) == 4              # the same, fewer: the disaggregation splits
+    assert count(1034, 1972, [25, 36, 268], split=1) == 6
+    assert count(1034, 1972, [25, 36, 268], R=128) == 8
