@@ -20,6 +20,7 @@
 // r_phi intermediates never leave the SM.
 #include <algorithm>
 #include <cmath>
+#include <functional>
 #include <numeric>
 
 #include "internal.h"
@@ -1064,8 +1065,35 @@ void pack_factors_fp32(Plan& P, cudaStream_t s) {
     finalize_hot_layout(P, s);
 }
 
+// Complex elements that one work item streams.
+double item_elems(const Plan& P, const TuckerItem& d) {
+    return (double)d.rb * d.ld_nb + (double)d.rb * d.ld_ab + (double)P.n_phi * d.rp + (double)P.n_theta * d.rt;
+}
+
 constexpr int64_t kThreeAgg = 2 << 20, kThreeDis = 900 << 10;
-bool between_two_and_three(const Plan& P, int n) { return n > 2 * P.num_sms && n <= 3 * P.num_sms; }  // per SM
+
+// Between two and three work items per SM: whether three CTAs an SM, which take all items at once, beat two.
+// Two leave a second item to some slots, three share the SM's rate; so the longest queue of two (longest
+// items first, bytes) is held against the longest item.  Uneven groups balance on two: 416 of the
+// 10-lambda sphere, disaggregation 87 us on two, 105 on three.
+template <class Bytes>
+bool three_pay(const Plan& P, int n, Bytes bytes) {
+    if (n <= 2 * P.num_sms || n > 3 * P.num_sms) return false;
+    std::vector<double> item(n);
+    for (int i = 0; i < n; ++i) item[i] = bytes(i);
+    std::sort(item.begin(), item.end(), std::greater<double>());
+    std::vector<double> slot(item.begin(), item.begin() + 2 * P.num_sms);  // a heap, least load first
+    std::make_heap(slot.begin(), slot.end(), std::greater<double>());
+    for (int i = 2 * P.num_sms; i < n; ++i) {
+        std::pop_heap(slot.begin(), slot.end(), std::greater<double>());
+        slot.back() += item[i];
+        std::push_heap(slot.begin(), slot.end(), std::greater<double>());
+    }
+    return 3.0 * item[0] <= 2.0 * *std::max_element(slot.begin(), slot.end());
+}
+bool three_groups_pay(const Plan& P) {
+    return three_pay(P, P.G, [&](int g) { return item_elems(P, P.items[2 * g]) + item_elems(P, P.items[2 * g + 1]); });
+}
 void finalize_hot_layout(Plan& P, cudaStream_t s) {
     const int nI = P.G * 2;
     if (P.d_items) cudaFree(P.d_items);
@@ -1083,12 +1111,13 @@ void finalize_hot_layout(Plan& P, cudaStream_t s) {
     P.tuning.agg_threads = item <= 448 * 1024 && nI >= 4 * P.num_sms ? 256 : 512;
     P.tuning.dis_threads = item <= 300 * 1024 && P.G >= 4 * P.num_sms ? 256 : 512;
     // Between two and three items per SM two CTAs of 512 threads leave the third item of an SM to a second
-    // round; three of 320 take all at once, until the items are long enough to want the warps (the
-    // disaggregation then takes three of 512, see plan_hot).  Measured, 512 / 320 threads (us): aggregation, 308
+    // round; three of 320 take all at once, where the items are even (three_pay) and until they are long
+    // enough to want the warps (the disaggregation then takes three of 512, see plan_hot).  Measured on items
+    // whose sizes differ by a factor of two at most, 512 / 320 threads (us): aggregation, 308
     // items of 0.19 MB 23.8 / 19.8, 456 of 1.1 MB 99 / 94, 360 of 1.8 MB 134 / 121, but 360 of 3 MB 204 / 209;
     // disaggregation, 310 groups of 0.19 MB items 50 / 42, 380 of 0.75 MB 148 / 122, but 380 of 1.1 MB 191 / 191.
-    if (between_two_and_three(P, nI) && item <= kThreeAgg) P.tuning.agg_threads = 320;
-    if (between_two_and_three(P, P.G) && item <= kThreeDis) P.tuning.dis_threads = 320;
+    if (item <= kThreeAgg && three_pay(P, nI, [&](int q) { return item_elems(P, P.items[q]); })) P.tuning.agg_threads = 320;
+    if (item <= kThreeDis && three_groups_pay(P)) P.tuning.dis_threads = 320;
     configure_hot(P, P.tuning, s);
 }
 
@@ -1117,10 +1146,10 @@ HotShape plan_hot(const Plan& P, const HotTuning& t) {
                               sizeof(float2) * agg_layout(P, t.agg_threads).total, P.num_sms, nI, t.agg_ctas_per_sm);
         h.dis = make_schedule(tucker_disaggregate_kernel<false>, t.dis_threads,
                               sizeof(float2) * dis_layout(P, t.dis_threads).total, P.num_sms, P.G, t.dis_ctas_per_sm);
-        // Between two and three groups per SM: three CTAs of 512 threads where their shared memory fits, with half
+        // Between two and three even groups per SM: three CTAs of 512 threads where their shared memory fits, with half
         // the loads in flight (us, two / three): 310 groups of 1.1 MB items 174 / 157, 380 191 / 176, 340 of 1.8 MB
         // 265 / 236, 456 303 / 291.
-        if (between_two_and_three(P, P.G) && t.dis_threads == 512 && t.dis_ctas_per_sm == 0) {
+        if (t.dis_threads == 512 && t.dis_ctas_per_sm == 0 && three_groups_pay(P)) {
             const Schedule three = make_schedule(tucker_disaggregate_kernel<false, true>, 512, h.dis.smem, P.num_sms, P.G);
             if (three.blocks > h.dis.blocks) {
                 h.dis = three;
@@ -1161,9 +1190,7 @@ void configure_hot(Plan& P, const HotTuning& t, cudaStream_t s) {
         TFMM_REQUIRE(P.live_graphs == 0, "destroy the plan's graphs before changing the single-RHS path");
     std::unique_ptr<SplitPlan> split;
     if (h.split && !P.split) split = make_split(P, s);
-    auto bytes = [&](const TuckerItem& d) {
-        return (double)d.rb * d.ld_nb + (double)d.rb * d.ld_ab + (double)P.n_phi * d.rp + (double)P.n_theta * d.rt;
-    };
+    auto bytes = [&](const TuckerItem& d) { return item_elems(P, d); };
     std::vector<int> agg(nI), dis(P.G);
     std::iota(agg.begin(), agg.end(), 0);
     std::iota(dis.begin(), dis.end(), 0);

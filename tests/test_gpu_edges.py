@@ -306,6 +306,6 @@ def test_between_two_and_three_groups_per_sm(threads, monkeypatch):
 
     monkeypatch.setattr(tfmm, "tfmm_plan_from_tucker", persistent)
     rng = np.random.default_rng(41)
-    nbetas = [int(n) for n in rng.integers(2, 90, 2 * sms + 6)]
-    ranks = [_small_ranks(rng, 9, 18, nb, 70) for nb in nbetas]
+    nbetas = [int(n) for n in rng.integers(60, 68, 2 * sms + 6)]  # even enough for three (uneven groups run on two)
+    ranks = [[(9, 17 + i % 2, 57 + i % 3), (8 + i % 2, 18, 59)] for i in range(len(nbetas))]
     _check(9800 + threads, 9, 18, nbetas, ranks, 1, 0, 1e-5, pad=1)
