@@ -1674,7 +1674,8 @@ __global__ void __launch_bounds__(CAT_THREADS) tc_cat_kernel(const TcCtx c, cons
 //                    (a, r) as its rows: an MN-major operand, 16 bytes = 8 values of a at one i_phi
 //   4 H warps        H from TMEM (lane = (a, r)) -> the planes [r][a + r_t b] that DG2 reads
 // S1 of a tile runs while P of the one before is split, S2 while the next P leaves TMEM.
-// What bounds it: the tensor pipe (narrow N: r_theta, r_phi <= 48) and the splits' issue.
+// What bounds it: the chain slab -> P -> H of a tile and its hand-overs; nothing is full (10-lambda sphere, 128
+// columns: tensor pipe 17 %, 2.0 of 4 instructions a cycle, shared-memory wavefronts 26 %, DRAM 16 %).
 // 30-lambda sphere, 128 columns: DG1a + DG1b 8.6 + 3.3 ms -> 5.0 ms (1.4 ms for the bytes).
 struct Dg1Item {
     const float2* uth;                        // U_theta, n_theta x r_theta column-major (FP32)

@@ -223,8 +223,8 @@ __global__ void to_f32_kernel(const double2* __restrict__ in, int64_t n, int64_t
 // n = 1 (bilinear in khat and pol, a symmetric 3 x 3 matrix per side).  Terms n = 2 .. 8, at
 // most a few percent of the sum, and the rotation by the rest of the phase (under 0.0123 rad) are FP32.
 // Against 64 bits the unrounded sum is off by 7e-10 on a lambda/10 mesh (rounding V to FP32:
-// 2.55e-8, as before) and 1.3e-9 at the limit kPWSpread.  1.8 ms for the same block (0.02 ms
-// for the bytes); the 28 FP64 operations left per side and incidence are what bounds it.
+// 2.55e-8, as before) and 1.3e-9 at the limit kPWSpread.  1.6 ms for the same block (0.02 ms
+// for the bytes); the 28 FP64 operations left per side and incidence are what bounds it (1.3 ms).
 constexpr int kPWDegree = PlanewaveRule::kDegree, kPWTerms = PlanewaveRule::kTerms;
 constexpr int kPWTable = 256;    // steps per turn of the phase table
 constexpr int kPWCols = 64;      // most incidences per block: a side's constants cost as much FP64 as three of them

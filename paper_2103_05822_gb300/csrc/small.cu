@@ -14,7 +14,7 @@
 // the half to two thirds of the issue slots that three CTAs' barriers leave.  20-lambda sphere in
 // half-wavelength boxes (7240 groups, 16 columns, ranks to (9, 13, 35)): aggregation 3.59 -> 0.86 ms,
 // disaggregation 4.01 -> 1.46 ms (0.18 ms each for the bytes).  One column of the 2-lambda sphere
-// (56 groups), both stages in a graph: 25.9 -> 18.7 us.
+// (56 groups), both stages in a graph: 25.9 -> 20.0 us.
 #include <cooperative_groups.h>
 
 #include <algorithm>
